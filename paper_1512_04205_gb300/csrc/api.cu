@@ -82,7 +82,7 @@ static cdmd_status fail_clip(cdmd_status st, int clip) {
     return fail(st, "clip %d: %s", clip, msg);
 }
 
-constexpr int kMaxSharedRun = 8;   // clips per cdmd_run_shared / cdmd_run_host_shared call
+constexpr int kMaxSharedRun = kMaxSolveClips;   // clips per cdmd_run_shared / cdmd_run_host_shared call
 
 }  // namespace cdmd
 
@@ -301,12 +301,8 @@ cdmd_status cdmd_sketch_gather(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n
     return launch_sketch_gather(ctx, D, m, n, ldd, meas, DY, static_cast<cudaStream_t>(stream));
 }
 
-cdmd_status cdmd_decompose(cdmd_ctx* ctx, const double* DY, int k, int n, int r, int K, cdmd_selector selector,
-                           double* sigma, double* lambda, double* G, double* PhiY, double* beta, int32_t* sel,
-                           int32_t* nsel, void* stream) {
-    clear_error();
-    CDMD_REQUIRE(ctx != nullptr, "ctx is NULL");
-    CDMD_REQUIRE(DY && sigma && lambda && G && beta && sel && nsel, "a required pointer is NULL");
+static cdmd_status check_decompose(const cdmd_ctx* ctx, int k, int n, int r, int K,
+                                   cdmd_selector selector) {
     CDMD_REQUIRE(n >= 2 && n <= 512, "n must be in [2, 512] (got %d)", n);
     CDMD_REQUIRE(k >= 1, "k must be >= 1");
     CDMD_REQUIRE(r >= 1 && r <= 32 && r <= k && r <= n - 1, "r must be in [1, min(32, k, n-1)] (got %d)", r);
@@ -315,9 +311,20 @@ cdmd_status cdmd_decompose(cdmd_ctx* ctx, const double* DY, int k, int n, int r,
                  "unknown selector %d", static_cast<int>(selector));
     CDMD_REQUIRE(selector != CDMD_SEL_MLP || ctx->selector_loaded,
                  "CDMD_SEL_MLP needs a model (cdmd_selector_load)");
+    return CDMD_OK;
+}
+
+cdmd_status cdmd_decompose(cdmd_ctx* ctx, const double* DY, int k, int n, int r, int K, cdmd_selector selector,
+                           double* sigma, double* lambda, double* G, double* PhiY, double* beta, int32_t* sel,
+                           int32_t* nsel, void* stream) {
+    clear_error();
+    CDMD_REQUIRE(ctx != nullptr, "ctx is NULL");
+    CDMD_REQUIRE(DY && sigma && lambda && G && beta && sel && nsel, "a required pointer is NULL");
+    cdmd_status st = check_decompose(ctx, k, n, r, K, selector);
+    if (st != CDMD_OK) return st;
     DeviceGuard g(ctx->device);
-    return launch_decompose(ctx, DY, k, n, r, K, selector, sigma, lambda, G, PhiY, beta, sel, nsel,
-                            static_cast<cudaStream_t>(stream));
+    const DecomposeIO io = {DY, nullptr, n, sigma, lambda, G, PhiY, beta, sel, nsel};
+    return launch_decompose(ctx, 1, &io, k, r, K, selector, static_cast<cudaStream_t>(stream));
 }
 
 cdmd_status cdmd_decompose_auto(cdmd_ctx* ctx, const double* DY, int k, int n, int r_max, int K,
@@ -336,8 +343,8 @@ cdmd_status cdmd_decompose_auto(cdmd_ctx* ctx, const double* DY, int k, int n, i
     CDMD_REQUIRE(selector != CDMD_SEL_MLP || ctx->selector_loaded,
                  "CDMD_SEL_MLP needs a model (cdmd_selector_load)");
     DeviceGuard g(ctx->device);
-    return launch_decompose_auto(ctx, DY, k, n, r_max, K, selector, sigma, lambda, G, PhiY, beta, sel, nsel, r_out,
-                                 tau_out, static_cast<cudaStream_t>(stream));
+    const DecomposeIO io = {DY, nullptr, n, sigma, lambda, G, PhiY, beta, sel, nsel};
+    return launch_decompose_auto(ctx, io, k, r_max, K, selector, r_out, tau_out, static_cast<cudaStream_t>(stream));
 }
 
 cdmd_status cdmd_snapshot_gram(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, int64_t ldd, double* R,
@@ -369,8 +376,8 @@ cdmd_status cdmd_decompose_gram(cdmd_ctx* ctx, const double* R, int n, int r, in
     cdmd_status st = check_exact_selector(selector);
     if (st != CDMD_OK) return st;
     DeviceGuard g(ctx->device);
-    return launch_decompose_gram(ctx, R, n, r, K, selector, sigma, lambda, G, beta, sel, nsel,
-                                 static_cast<cudaStream_t>(stream));
+    const DecomposeIO io = {nullptr, R, n, sigma, lambda, G, nullptr, beta, sel, nsel};
+    return launch_decompose(ctx, 1, &io, 0, r, K, selector, static_cast<cudaStream_t>(stream));
 }
 
 cdmd_status cdmd_lift(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, int64_t ldd, const double* G, int r,
@@ -440,50 +447,87 @@ cdmd_status check_run(const uint8_t* D, int64_t m, int n, int64_t ldd, const cdm
     return CDMD_OK;
 }
 
-// Steps 4-9 of cdmd_run on a sketch DY already in device memory, or, with
-// DY NULL, of exact DMD on the snapshot Gram R (the context's small-solve and
-// Phi buffers are reused, stream-ordered).
-cdmd_status run_from(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, int64_t ldd, const cdmd_params* p,
-                     double* DY, const double* R, uint32_t* mask, void* stream) {
+// Lift and subtract of one clip after its small solves (io): OMP and the
+// learned selector lift and subtract only the selected modes (sel, -1
+// padded); with LSTSQ every mode carries an amplitude, so all r are used.
+cdmd_status run_apply(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int64_t ldd, const cdmd_params* p,
+                      const DecomposeIO& io, int r, uint32_t* mask, void* stream) {
+    const bool all = p->selector == CDMD_SEL_LSTSQ;
+    const int ncols = all ? r : std::min<int>(p->K, r);
+    const int32_t* cols = all ? nullptr : io.sel;
+    cdmd_status st = cdmd_lift(ctx, D, m, io.n, ldd, io.G, r, cols, ncols, p->prec, ctx->run_Phi, stream);
+    if (st != CDMD_OK) return st;
+    return cdmd_subtract(ctx, D, m, io.n, ldd, ctx->run_Phi, ncols, cols, io.beta, io.lambda, r, p->tau, p->bgmode,
+                         mask, nullptr, stream);
+}
+
+// Steps 4-9 of cdmd_run on sketches DY[i] already in device memory, or, with
+// DY NULL, of exact DMD on the snapshot Gram R of one clip.  With a fixed rank
+// the small solves of all clips run side by side; the lift and the subtract
+// then go clip by clip (one Phi buffer, stream-ordered).  An automatic rank
+// synchronises once per clip, so there everything goes clip by clip.
+cdmd_status run_from(cdmd_ctx* ctx, int nclips, const uint8_t* const* D, int64_t m, const int* n, const int64_t* ldd,
+                     const cdmd_params* p, double* const* DY, const double* R, uint32_t* const* mask, void* stream) {
     const int k = p->k, K = p->K;
+    const bool auto_rank = p->r == 0;
     // r == 0: the rank comes from the optimal hard threshold (Remark 2), at
     // most min(32, k, n-1); buffers are sized for that bound
-    const bool auto_rank = p->r == 0;
-    int r = auto_rank ? std::min(32, std::min(k, n - 1)) : p->r;
-    const int p1 = n - 1;
-    const int ncols_max = (p->selector == CDMD_SEL_LSTSQ) ? r : K;
+    DecomposeIO io[kMaxSolveClips];
+    size_t off[kMaxSolveClips + 1] = {0};
+    int r[kMaxSolveClips], rmax = 0;
+    for (int i = 0; i < nclips; ++i) {
+        r[i] = auto_rank ? std::min(32, std::min(k, n[i] - 1)) : p->r;
+        rmax = std::max(rmax, r[i]);
+        const size_t rr = r[i];
+        const size_t doubles = rr + 2 * rr + 2 * static_cast<size_t>(n[i] - 1) * rr + 2 * rr + 8;
+        off[i + 1] = off[i] + (doubles * sizeof(double) + (rr + 8) * sizeof(int32_t) + 255) / 256 * 256;
+    }
     void* v = nullptr;
-    const size_t n_small = static_cast<size_t>(r) + 2 * r + 2 * static_cast<size_t>(p1) * r + 2 * r + 8;
-    cdmd_status st = ensure_buffer(ctx, BUF_RUN_SMALL, n_small * sizeof(double) + (r + 8) * sizeof(int32_t), &v);
+    cdmd_status st = ensure_buffer(ctx, BUF_RUN_SMALL, off[nclips], &v);
     if (st != CDMD_OK) return st;
-    double* sigma = static_cast<double*>(v);
-    double* lambda = sigma + r;
-    double* Gm = lambda + 2 * r;
-    double* beta = Gm + 2 * static_cast<size_t>(p1) * r;
-    int32_t* sel = reinterpret_cast<int32_t*>(beta + 2 * r + 8);
-    int32_t* nsel = sel + r + 4;
+    for (int i = 0; i < nclips; ++i) {
+        DecomposeIO& q = io[i];
+        q.DY = DY != nullptr ? DY[i] : nullptr;
+        q.R = DY != nullptr ? nullptr : R;
+        q.n = n[i];
+        q.sigma = reinterpret_cast<double*>(static_cast<char*>(v) + off[i]);
+        q.lambda = q.sigma + r[i];
+        q.G = q.lambda + 2 * r[i];
+        q.PhiY = nullptr;
+        q.beta = q.G + 2 * static_cast<size_t>(n[i] - 1) * r[i];
+        q.sel = reinterpret_cast<int32_t*>(q.beta + 2 * r[i] + 8);
+        q.nsel = q.sel + r[i] + 4;
+    }
+    const int ncols_max = (p->selector == CDMD_SEL_LSTSQ) ? rmax : K;
     st = ensure_buffer(ctx, BUF_RUN_PHI, static_cast<size_t>(m) * ncols_max * 2 * sizeof(float), &v);
     if (st != CDMD_OK) return st;
-    float* Phi = static_cast<float*>(v);
-    ctx->run_DY = DY; ctx->run_sigma = sigma; ctx->run_lambda = lambda; ctx->run_G = Gm;
-    ctx->run_beta = beta; ctx->run_sel = sel; ctx->run_nsel = nsel; ctx->run_Phi = Phi;
+    const DecomposeIO& last = io[nclips - 1];
+    ctx->run_DY = const_cast<double*>(last.DY); ctx->run_sigma = last.sigma; ctx->run_lambda = last.lambda;
+    ctx->run_G = last.G; ctx->run_beta = last.beta; ctx->run_sel = last.sel; ctx->run_nsel = last.nsel;
+    ctx->run_Phi = static_cast<float*>(v);
 
-    if (DY != nullptr && auto_rank)
-        st = cdmd_decompose_auto(ctx, DY, k, n, r, K, p->selector, sigma, lambda, Gm, nullptr, beta, sel, nsel, &r,
-                                 nullptr, stream);
-    else if (DY != nullptr)
-        st = cdmd_decompose(ctx, DY, k, n, r, K, p->selector, sigma, lambda, Gm, nullptr, beta, sel, nsel, stream);
-    else
-        st = cdmd_decompose_gram(ctx, R, n, r, K, p->selector, sigma, lambda, Gm, beta, sel, nsel, stream);
-    if (st != CDMD_OK) return st;
-    const int ncols = (p->selector == CDMD_SEL_LSTSQ) ? r : std::min(K, r);
-    // OMP: lift and subtract only the selected modes (sel, -1 padded);
-    // LSTSQ: every mode carries an amplitude, so all r are used.
-    const int32_t* cols = (p->selector == CDMD_SEL_LSTSQ) ? nullptr : sel;
-    st = cdmd_lift(ctx, D, m, n, ldd, Gm, r, cols, ncols, p->prec, Phi, stream);
-    if (st != CDMD_OK) return st;
-    return cdmd_subtract(ctx, D, m, n, ldd, Phi, ncols, cols, beta, lambda, r, p->tau, p->bgmode, mask, nullptr,
-                         stream);
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (!auto_rank) {
+        if (DY != nullptr) {
+            for (int i = 0; i < nclips; ++i) {
+                st = check_decompose(ctx, k, n[i], p->r, K, p->selector);
+                if (st != CDMD_OK) return st;
+            }
+        }
+        st = launch_decompose(ctx, nclips, io, k, p->r, K, p->selector, s);
+        if (st != CDMD_OK) return st;
+    }
+    for (int i = 0; i < nclips; ++i) {
+        if (auto_rank) {
+            const DecomposeIO& q = io[i];
+            st = cdmd_decompose_auto(ctx, q.DY, k, q.n, r[i], K, p->selector, q.sigma, q.lambda, q.G, nullptr, q.beta,
+                                     q.sel, q.nsel, &r[i], nullptr, stream);
+            if (st != CDMD_OK) return st;
+        }
+        st = run_apply(ctx, D[i], m, ldd[i], p, io[i], r[i], mask[i], stream);
+        if (st != CDMD_OK) return st;
+    }
+    return CDMD_OK;
 }
 
 }  // namespace
@@ -501,7 +545,7 @@ cdmd_status cdmd_run(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, int64_t 
     double* DY = static_cast<double*>(v);
     st = cdmd_sketch(ctx, D, m, n, ldd, p->ctype, p->k, p->seed, p->prec, DY, stream);
     if (st != CDMD_OK) return st;
-    return run_from(ctx, D, m, n, ldd, p, DY, nullptr, mask, stream);
+    return run_from(ctx, 1, &D, m, &n, &ldd, p, &DY, nullptr, &mask, stream);
 }
 
 cdmd_status cdmd_run_exact(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, int64_t ldd, const cdmd_params* p,
@@ -521,7 +565,7 @@ cdmd_status cdmd_run_exact(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, in
     double* R = static_cast<double*>(v);
     st = cdmd_snapshot_gram(ctx, D, m, n, ldd, R, stream);
     if (st != CDMD_OK) return st;
-    return run_from(ctx, D, m, n, ldd, p, nullptr, R, mask, stream);
+    return run_from(ctx, 1, &D, m, &n, &ldd, p, nullptr, R, &mask, stream);
 }
 
 cdmd_status cdmd_run_shared(cdmd_ctx* ctx, int nclips, const uint8_t* const* D, int64_t m, const int* n,
@@ -546,11 +590,7 @@ cdmd_status cdmd_run_shared(cdmd_ctx* ctx, int nclips, const uint8_t* const* D, 
     for (int i = 0; i < nclips; ++i) DYs[i] = static_cast<double*>(v) + off[i];
     st = cdmd_sketch_shared(ctx, nclips, D, m, n, ldd, p->ctype, p->k, p->seed, p->prec, DYs, stream);
     if (st != CDMD_OK) return st;
-    for (int i = 0; i < nclips; ++i) {
-        st = run_from(ctx, D[i], m, n[i], ldd[i], p, DYs[i], nullptr, mask[i], stream);
-        if (st != CDMD_OK) return st;
-    }
-    return CDMD_OK;
+    return run_from(ctx, nclips, D, m, n, ldd, p, DYs, nullptr, mask, stream);
 }
 
 cdmd_status cdmd_run_host(cdmd_ctx* ctx, const uint8_t* D_host, int64_t m, int n, const cdmd_params* p,

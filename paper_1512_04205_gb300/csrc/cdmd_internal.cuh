@@ -231,18 +231,21 @@ struct cdmd_ctx {
 
 namespace cdmd {
 
-// Selector buffer: model blob (FP32, 2 KB slot), pick order (32 int32),
-// accept flag (int), fallback count (uint64).
+constexpr int kMaxSolveClips = 8;   // clips whose small solves run side by side (cdmd_run_shared's limit)
+
+// Selector buffer: model blob (FP32, 2 KB slot), per clip of a call the pick
+// order (32 int32) and the accept flag (int), fallback count (uint64).
 constexpr size_t kSelOrderOff = 2048;
-constexpr size_t kSelAcceptOff = 2176;
-constexpr size_t kSelFallbackOff = 2184;
-constexpr size_t kSelBytes = 2304;
+constexpr size_t kSelAcceptOff = kSelOrderOff + kMaxSolveClips * 32 * sizeof(int32_t);
+constexpr size_t kSelFallbackOff = kSelAcceptOff + kMaxSolveClips * sizeof(int32_t);
+constexpr size_t kSelBytes = kSelFallbackOff + 96;
+static_assert(kSelFallbackOff % 8 == 0, "the fallback count is a 64-bit atomic");
 inline float* selector_blob(cdmd_ctx* ctx) { return static_cast<float*>(ctx->buf[BUF_SELECTOR].ptr); }
-inline int32_t* selector_order(cdmd_ctx* ctx) {
-    return reinterpret_cast<int32_t*>(static_cast<char*>(ctx->buf[BUF_SELECTOR].ptr) + kSelOrderOff);
+inline int32_t* selector_order(cdmd_ctx* ctx, int clip) {
+    return reinterpret_cast<int32_t*>(static_cast<char*>(ctx->buf[BUF_SELECTOR].ptr) + kSelOrderOff) + 32 * clip;
 }
-inline int* selector_accept(cdmd_ctx* ctx) {
-    return reinterpret_cast<int*>(static_cast<char*>(ctx->buf[BUF_SELECTOR].ptr) + kSelAcceptOff);
+inline int* selector_accept(cdmd_ctx* ctx, int clip) {
+    return reinterpret_cast<int*>(static_cast<char*>(ctx->buf[BUF_SELECTOR].ptr) + kSelAcceptOff) + clip;
 }
 inline unsigned long long* selector_fallbacks(cdmd_ctx* ctx) {
     return reinterpret_cast<unsigned long long*>(static_cast<char*>(ctx->buf[BUF_SELECTOR].ptr) + kSelFallbackOff);
@@ -287,13 +290,21 @@ cdmd_status launch_selftest_wait(cdmd_ctx* ctx, uint64_t limit_ns, cudaStream_t 
 cdmd_status launch_selftest_recip(const double* a, int64_t n, double* r, double* q, cudaStream_t stream);
 cdmd_status launch_gram_tc(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, int64_t ldd, double* R,
                            cudaStream_t stream);
-cdmd_status launch_decompose_auto(cdmd_ctx* ctx, const double* DY, int k, int n, int r_max, int K,
-                                  cdmd_selector selector, double* sigma, double* lambda, double* G, double* PhiY,
-                                  double* beta, int32_t* sel, int32_t* nsel, int* r_out, double* tau_out,
-                                  cudaStream_t stream);
-cdmd_status launch_decompose_gram(cdmd_ctx* ctx, const double* R, int n, int r, int K, cdmd_selector selector,
-                                  double* sigma, double* lambda, double* G, double* beta, int32_t* sel,
-                                  int32_t* nsel, cudaStream_t stream);
+// One clip's small solves: its sketch DY (k x n), or its n x n Gram R (then DY
+// and PhiY are NULL), and the outputs of cdmd_decompose.
+struct DecomposeIO {
+    const double* DY;
+    const double* R;
+    int n;
+    double *sigma, *lambda, *G, *PhiY, *beta;
+    int32_t *sel, *nsel;
+};
+// The small solves of 1..kMaxSolveClips clips with the same k, r and K, side
+// by side; all from sketches or all from Grams.
+cdmd_status launch_decompose(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int k, int r, int K,
+                             cdmd_selector selector, cudaStream_t stream);
+cdmd_status launch_decompose_auto(cdmd_ctx* ctx, const DecomposeIO& io, int k, int r_max, int K,
+                                  cdmd_selector selector, int* r_out, double* tau_out, cudaStream_t stream);
 cdmd_status launch_median3x3(const uint32_t* mask, int64_t W, int64_t H, int n, uint32_t* out,
                              cudaStream_t stream);
 cdmd_status launch_sketch_gather(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, int64_t ldd,
@@ -303,10 +314,6 @@ cdmd_status launch_measure_sparse_count(cdmd_ctx* ctx, int64_t m, int k, uint64_
 cdmd_status launch_measure_build(cdmd_ctx* ctx, cdmd_measure* meas, cudaStream_t stream);
 cdmd_status launch_sketch_srft(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, int64_t ldd,
                                const cdmd_measure* meas, double* DY, cudaStream_t stream);
-cdmd_status launch_decompose(cdmd_ctx* ctx, const double* DY, int k, int n, int r, int K,
-                             cdmd_selector selector, double* sigma, double* lambda, double* G,
-                             double* PhiY, double* beta, int32_t* sel, int32_t* nsel,
-                             cudaStream_t stream);
 cdmd_status launch_lift_fp32(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, int64_t ldd,
                              const double* G, int r, const int32_t* cols, int ncols, float* Phi,
                              cudaStream_t stream);
@@ -326,7 +333,7 @@ cdmd_status launch_selector_relabel(cdmd_ctx* ctx, const double* DY, int k, int 
                                     const double* lambda, int r, const double* y_target, int K, int32_t* sel,
                                     cudaStream_t stream);
 cdmd_status launch_mlp_select(cdmd_ctx* ctx, const double* lambda, const double* M, const double* cvec,
-                              const double* R, int r, int K, cudaStream_t stream);
+                              const double* R, int r, int K, int32_t* order, cudaStream_t stream);
 cdmd_status launch_mlp_forward(cdmd_ctx* ctx, const float* blob, const float* X, int64_t N, int bf16,
                                float* s, float* p, cudaStream_t stream);
 cdmd_status launch_mlp_train(cdmd_ctx* ctx, int apply, float* blob, float* m, float* v, int step, float lr,

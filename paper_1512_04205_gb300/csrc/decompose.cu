@@ -54,6 +54,31 @@ constexpr double kRankTol = 64.0;
 constexpr int kMaxR = 32;
 constexpr size_t kMaxOptInSmem = 232448;      // opt-in shared memory per CTA
 
+// One launch of each kernel below serves every clip of a call (up to
+// kMaxSolveClips clips under one C, their own n, the same k, r, K): the chain
+// is bound by dependent FP64 latency and leaves the device mostly idle, so the
+// clips of a shared run go through it side by side, one clip per grid slice
+// (blockIdx.z, or .y where z is taken), in the time of one.
+struct SolveClip {
+    const double* DY;    // k x n sketch; NULL when R is given
+    const double* R;     // n x n Gram
+    int n, p;            // frames, p = n - 1
+    double *gpart, *Rw;  // Gram partials; the Gram's own storage (NULL when R is given)
+    double *Hv, *htau, *dd, *ee;                  // reflectors and the tridiagonal form
+    double *lamT, *Z, *V, *B, *At, *W, *M, *WR, *lamR, *cvec;
+    float2 *lam32, *W32;
+    int* flag;           // eigen-solver fallback
+    double *sigma, *lambda, *G, *PhiY, *beta;     // the caller's outputs
+    int32_t *sel, *nsel;
+    int32_t* order;      // learned pick order and its verdict
+    int* accept;
+};
+struct SolveBatch {
+    SolveClip c[kMaxSolveClips];
+    int k, r, K;
+    int* status;
+};
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -110,10 +135,16 @@ __device__ __forceinline__ cd shfl_cd(cd v, int src) {
 constexpr int kGT = 32;
 
 __global__ void __launch_bounds__(256)
-gram_partial_kernel(const double* __restrict__ DY, int k, int n, int kchunk,
-                    double* __restrict__ part) {
-    const int ta = blockIdx.y, tb = blockIdx.x;
-    if (ta > tb) return;
+gram_partial_kernel(const __grid_constant__ SolveBatch sb, int kchunk) {
+    const SolveClip& q = sb.c[blockIdx.y];
+    const double* DY = q.DY;
+    const int k = sb.k, n = q.n;
+    // blockIdx.x counts the tile pairs ta <= tb row by row
+    const int ntiles = (n + kGT - 1) / kGT;
+    int ta = 0, tb = blockIdx.x;
+    while (ta < ntiles && tb >= ntiles - ta) { tb -= ntiles - ta; ++ta; }
+    if (ta >= ntiles) return;
+    tb += ta;
     __shared__ double As[kGT][kGT + 1];
     __shared__ double Bs[kGT][kGT + 1];
     const int tid = threadIdx.x;
@@ -134,28 +165,30 @@ gram_partial_kernel(const double* __restrict__ DY, int k, int n, int kchunk,
         for (int ii = 0; ii < kGT; ++ii) {
             const double bv = Bs[ii][tx];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] = fma(As[ii][ty + 8 * q], bv, acc[q]);
+            for (int e = 0; e < 4; ++e) acc[e] = fma(As[ii][ty + 8 * e], bv, acc[e]);
         }
         __syncthreads();
     }
-    double* dst = part + static_cast<int64_t>(blockIdx.z) * n * n;
+    double* dst = q.gpart + static_cast<int64_t>(blockIdx.z) * n * n;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int a = a0 + ty + 8 * q, b = b0 + tx;
-        if (a < n && b < n) dst[a * n + b] = acc[q];
+    for (int e = 0; e < 4; ++e) {
+        const int a = a0 + ty + 8 * e, b = b0 + tx;
+        if (a < n && b < n) dst[a * n + b] = acc[e];
     }
 }
 
-__global__ void gram_reduce_kernel(const double* __restrict__ part, int splits, int n,
-                                   double* __restrict__ R, int* status) {
+__global__ void gram_reduce_kernel(const __grid_constant__ SolveBatch sb, int splits) {
+    const SolveClip& q = sb.c[blockIdx.y];
+    const double* part = q.gpart;
+    const int n = q.n;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= n * n) return;
     int a = idx / n, b = idx % n;
     if (a / kGT > b / kGT) { const int t = a; a = b; b = t; }
     double s = 0.0;
     for (int sp = 0; sp < splits; ++sp) s += part[static_cast<int64_t>(sp) * n * n + a * n + b];
-    if (!isfinite(s)) record_status(status, CDMD_ERR_NONFINITE);
-    R[idx] = s;
+    if (!isfinite(s)) record_status(sb.status, CDMD_ERR_NONFINITE);
+    q.Rw[idx] = s;
 }
 
 // ---------------------------------------------------------------------------
@@ -220,8 +253,11 @@ __device__ void tri_reflector_warp(cg::cluster_group& cluster, int P, const doub
 }
 
 __global__ void __launch_bounds__(kTriThreads)
-tridiag_kernel(const double* __restrict__ R, int n, int p, double* __restrict__ Hv,
-               double* __restrict__ htau, double* __restrict__ dd, double* __restrict__ ee) {
+tridiag_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& q = sb.c[blockIdx.z];
+    const double* R = q.R;
+    const int n = q.n, p = q.p;
+    double *Hv = q.Hv, *htau = q.htau, *dd = q.dd, *ee = q.ee;
     cg::cluster_group cluster = cg::this_cluster();
     const int P = static_cast<int>(cluster.num_blocks());
     const int rank = static_cast<int>(cluster.block_rank());
@@ -245,7 +281,8 @@ tridiag_kernel(const double* __restrict__ R, int n, int p, double* __restrict__ 
     // every CTA of the cluster has started (and loaded its rows) before any
     // CTA writes into another's shared memory
     cluster.sync();
-    if (rank == 0 && wid == 0) {
+    // p <= 2: already tridiagonal, no reflectors
+    if (rank == 0 && wid == 0 && p >= 3) {
         double tp = 0.0;
         for (int l = 2 + lane; l < p; l += 32) tp = fma(Aloc[l], Aloc[l], tp);
         tri_reflector_warp(cluster, P, Aloc, 0, p, tp, vbuf, tau_slot, 0, Hv, htau, dd, ee);
@@ -280,7 +317,7 @@ tridiag_kernel(const double* __restrict__ R, int n, int p, double* __restrict__ 
             __syncthreads();
             if (tid < P) {
                 double t = 0.0;
-                for (int q = 0; q < nwarps; ++q) t += red[q];
+                for (int w = 0; w < nwarps; ++w) t += red[w];
                 *cluster.map_shared_rank(slot + rank, tid) = t;
             }
         }
@@ -290,7 +327,7 @@ tridiag_kernel(const double* __restrict__ R, int n, int p, double* __restrict__ 
         const int li_next = nxt / P;
         if (tau != 0.0) {
             double vtu = 0.0;
-            for (int q = 0; q < P; ++q) vtu += slot[q];
+            for (int w = 0; w < P; ++w) vtu += slot[w];
             const double kc = 0.5 * tau * tau * vtu;
             for (int l = j + 1 + tid; l < p; l += kTriThreads) wv[l] = fma(tau, ubuf[l], -kc * v[l]);
             __syncthreads();
@@ -341,15 +378,6 @@ tridiag_kernel(const double* __restrict__ R, int n, int p, double* __restrict__ 
     }
 }
 
-// p <= 2: the leading block of R is already tridiagonal (no reflectors).
-__global__ void tiny_tridiag_kernel(const double* R, int n, int p, double* dd, double* ee, double* htau) {
-    for (int i = 0; i < p; ++i) {
-        dd[i] = R[i * n + i];
-        if (i + 1 < p) ee[i] = R[i * n + i + 1];
-        htau[i] = 0.0;
-    }
-}
-
 // ---------------------------------------------------------------------------
 // 3. Eigenpairs of the symmetric tridiagonal T (d, e), the r largest.
 // Sturm count N(x) = #eigenvalues < x = sign changes in the leading minors
@@ -393,8 +421,12 @@ __device__ __forceinline__ void sturm_count2(const double* d, const double* e2, 
 constexpr int kShifts = 64;   // shifts tested per multisection pass (two per lane)
 
 __global__ void __launch_bounds__(32)
-tridiag_eigpair_kernel(const double* __restrict__ dd, const double* __restrict__ ee, int p, int r, double* lam,
-                       double* Z, int* status) {
+tridiag_eigpair_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& q = sb.c[blockIdx.z];
+    const double *dd = q.dd, *ee = q.ee;
+    const int p = q.p;
+    double *lam = q.lamT, *Z = q.Z;
+    int* status = sb.status;
     extern __shared__ double tsm[];
     double* d = tsm;            // p
     double* e = d + p;          // p (e[p-1] = 0)
@@ -611,7 +643,9 @@ gd_rank_kernel(const double* __restrict__ dd, const double* __restrict__ ee, int
 // taken in parallel (one warp each).  Z is not __restrict__: threads read
 // entries other threads wrote, ordered by __syncthreads.
 __global__ void __launch_bounds__(1024)
-orthonormalise_kernel(double* Z, int p, int r) {
+orthonormalise_kernel(const __grid_constant__ SolveBatch sb) {
+    double* Z = sb.c[blockIdx.z].Z;
+    const int p = sb.c[blockIdx.z].p, r = sb.r;
     // classical Gram-Schmidt, twice, on the r columns held in shared memory
     extern __shared__ double osm[];
     double* Zs = osm;                         // r columns of p
@@ -665,9 +699,12 @@ orthonormalise_kernel(double* Z, int p, int r) {
 // kBtPer: reflector entries per lane, 8 for p <= 256 and 16 up to p = 511
 template <int kBtPer>
 __global__ void __launch_bounds__(32)
-backtransform_kernel(const double* __restrict__ Z, const double* __restrict__ Hv,
-                     const double* __restrict__ htau, const double* __restrict__ lam, int p, int r,
-                     double* __restrict__ V, double* __restrict__ sigma, int* status) {
+backtransform_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& clip = sb.c[blockIdx.z];
+    const double *Z = clip.Z, *Hv = clip.Hv, *htau = clip.htau, *lam = clip.lamT;
+    const int p = clip.p;
+    double *V = clip.V, *sigma = clip.sigma;
+    int* status = sb.status;
     extern __shared__ double ysm[];   // p
     const int c = blockIdx.x;
     const int lane = threadIdx.x;
@@ -725,11 +762,15 @@ backtransform_kernel(const double* __restrict__ Z, const double* __restrict__ Hv
 
 // 4c. B[a][c] = sum_b R[a][b+1] V[b][c] = ((Y^T Y') V)[a][c]; one warp per entry.
 __global__ void __launch_bounds__(256)
-bmat_kernel(const double* __restrict__ R, const double* __restrict__ V, int n, int p, double* __restrict__ B) {
+bmat_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& q = sb.c[blockIdx.z];
+    const double *R = q.R, *V = q.V;
+    const int n = q.n, p = q.p;
+    double* B = q.B;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int a = blockIdx.x * 8 + wid;
     const int c = blockIdx.y;
-    if (a >= p) return;
+    if (a >= p) return;   // also the rows a shorter clip does not have
     const double* row = R + static_cast<int64_t>(a) * n + 1;
     const double* vc = V + static_cast<int64_t>(c) * p;
     double s0 = 0.0, s1 = 0.0;
@@ -745,8 +786,11 @@ bmat_kernel(const double* __restrict__ R, const double* __restrict__ V, int n, i
 
 // 5. A~[a][c] = V[:,a]^T B[:,c] / (sigma_a sigma_c), one CTA per column c.
 __global__ void __launch_bounds__(32)
-atilde_kernel(const double* __restrict__ V, const double* __restrict__ B,
-              const double* __restrict__ sigma, int p, int r, double* __restrict__ At) {
+atilde_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& q = sb.c[blockIdx.z];
+    const double *V = q.V, *B = q.B, *sigma = q.sigma;
+    const int p = q.p, r = sb.r;
+    double* At = q.At;
     const int c = blockIdx.x;
     const int lane = threadIdx.x;
     const double* bc = B + static_cast<int64_t>(c) * p;
@@ -804,8 +848,12 @@ __device__ __forceinline__ cf fsqrtc(cf a) {
 }
 
 __global__ void __launch_bounds__(32)
-eig_f32_kernel(const double* __restrict__ At, int r, float2* __restrict__ lam32, float2* __restrict__ W32,
-               int* fallback) {
+eig_f32_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& clip = sb.c[blockIdx.z];
+    const double* At = clip.At;
+    const int r = sb.r;
+    float2 *lam32 = clip.lam32, *W32 = clip.W32;
+    int* fallback = clip.flag;
     __shared__ float Hr[kMaxR][kMaxR + 1];
     __shared__ float Q[kMaxR][kMaxR + 1];
     __shared__ cf T[kMaxR][kMaxR + 1];
@@ -976,8 +1024,13 @@ eig_f32_kernel(const double* __restrict__ At, int r, float2* __restrict__ lam32,
 }
 
 __global__ void __launch_bounds__(32)
-eig_refine_kernel(const double* __restrict__ At, int r, const float2* __restrict__ lam32,
-                  const float2* __restrict__ W32, double* __restrict__ lamR, double* __restrict__ WR, int* fallback) {
+eig_refine_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& clip = sb.c[blockIdx.z];
+    const double* At = clip.At;
+    const int r = sb.r;
+    const float2 *lam32 = clip.lam32, *W32 = clip.W32;
+    double *lamR = clip.lamR, *WR = clip.WR;
+    int* fallback = clip.flag;
     __shared__ double A[kMaxR][kMaxR + 1];
     __shared__ cd Mx[kMaxR][kMaxR + 1];
     __shared__ cd wv[kMaxR];
@@ -1120,7 +1173,12 @@ constexpr int kQrThreads = 64;
 constexpr size_t kQrSmem = 2 * kMaxR * (kMaxR + 1) * sizeof(double) + 3 * kMaxR * (kMaxR + 1) * sizeof(cd);
 
 __global__ void __launch_bounds__(kQrThreads)
-eig_qr64_kernel(const double* __restrict__ At, int r, double* lamR, double* WR, int* fallback, int* status) {
+eig_qr64_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& clip = sb.c[blockIdx.z];
+    const double* At = clip.At;
+    const int r = sb.r;
+    double *lamR = clip.lamR, *WR = clip.WR;
+    int *fallback = clip.flag, *status = sb.status;
     extern __shared__ double qsm[];
     typedef double RowD[kMaxR + 1];
     typedef cd RowC[kMaxR + 1];
@@ -1319,8 +1377,11 @@ eig_qr64_kernel(const double* __restrict__ At, int r, double* lamR, double* WR, 
 }
 
 __global__ void __launch_bounds__(32)
-eig_order_kernel(const double* __restrict__ lamR, const double* __restrict__ WR, int r, double* __restrict__ lam_out,
-                 double* __restrict__ W_out) {
+eig_order_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& clip = sb.c[blockIdx.z];
+    const double *lamR = clip.lamR, *WR = clip.WR;
+    const int r = sb.r;
+    double *lam_out = clip.lambda, *W_out = clip.W;
     __shared__ int order[kMaxR];
     const int lane = threadIdx.x;
     if (lane == 0) {
@@ -1404,8 +1465,11 @@ eig_order_kernel(const double* __restrict__ lamR, const double* __restrict__ WR,
 }
 
 // 7. G[t][c] = sum_a V[t][a] / sigma_a * W[a][c]   (column-major complex)
-__global__ void gmat_kernel(const double* __restrict__ V, const double* __restrict__ sigma,
-                            const double* __restrict__ W, int p, int r, double* __restrict__ G) {
+__global__ void gmat_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& q = sb.c[blockIdx.z];
+    const double *V = q.V, *sigma = q.sigma, *W = q.W;
+    const int p = q.p, r = sb.r;
+    double* G = q.G;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= p * r) return;
     const int t = idx % p, c = idx / p;
@@ -1422,8 +1486,11 @@ __global__ void gmat_kernel(const double* __restrict__ V, const double* __restri
 // 8. h = (Y'^T Y') G[:, c];  M[a][c] = G[:,a]^H h;  cvec[c] = G[:,c]^H (Y'^T y1).
 // One CTA of 16 warps per column c, one warp per row of h, then per entry.
 __global__ void __launch_bounds__(512)
-hmat_kernel(const double* __restrict__ R, const double* __restrict__ G, int n, int p, int r,
-            double* __restrict__ M, double* __restrict__ cvec) {
+hmat_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& q = sb.c[blockIdx.z];
+    const double *R = q.R, *G = q.G;
+    const int n = q.n, p = q.p, r = sb.r;
+    double *M = q.M, *cvec = q.cvec;
     extern __shared__ double hsm[];   // h: 2p
     const int c = blockIdx.x;
     const double* gc = G + 2 * static_cast<int64_t>(c) * p;
@@ -1480,12 +1547,9 @@ hmat_kernel(const double* __restrict__ R, const double* __restrict__ G, int n, i
 // on the selected set solves M_SS beta = c_S through a Cholesky factor
 // M_SS = L L^H grown by one row per pick; every triangular solve is
 // right-looking (one row per lane, one broadcast per step).
-__global__ void __launch_bounds__(32)
-omp_kernel(const double* __restrict__ M, const double* __restrict__ cvec, const double* __restrict__ R,
-           const double* __restrict__ lam, int r, int K, int lstsq, double* __restrict__ beta,
-           int32_t* __restrict__ sel, int32_t* __restrict__ nsel_out, int* status,
-           const int32_t* __restrict__ order, const float* __restrict__ blob, int* accept,
-           unsigned long long* fallbacks) {
+__device__ void omp_warp(const double* M, const double* cvec, const double* R, const double* lam, int r, int K,
+                         int lstsq, double* beta, int32_t* sel, int32_t* nsel_out, int* status,
+                         const int32_t* order, const float* blob, int* accept, unsigned long long* fallbacks) {
     // Modes of operation:
     //   order == nullptr, accept == nullptr   greedy OMP (or lstsq over all r)
     //   order != nullptr                      least squares on the learned pick
@@ -1607,9 +1671,30 @@ omp_kernel(const double* __restrict__ M, const double* __restrict__ cvec, const 
     if (lane == 0) *nsel_out = ns;
 }
 
+// learned: 0 = OMP or lstsq, 1 = least squares on the learned pick order,
+// 2 = OMP unless that order was accepted
+__global__ void __launch_bounds__(32)
+omp_kernel(const __grid_constant__ SolveBatch sb, int lstsq, int learned, const float* blob,
+           unsigned long long* fallbacks) {
+    const SolveClip& q = sb.c[blockIdx.z];
+    omp_warp(q.M, q.cvec, q.R, q.lambda, sb.r, sb.K, lstsq, q.beta, q.sel, q.nsel, sb.status,
+             learned == 1 ? q.order : nullptr, blob, learned != 0 ? q.accept : nullptr, fallbacks);
+}
+
+// OMP against another target (cvec and ||y||^2 of it) on the last decomposition
+__global__ void __launch_bounds__(32)
+relabel_omp_kernel(const double* M, const double* cvec, const double* y2, const double* lam, int r, int K,
+                   double* beta, int32_t* sel, int32_t* nsel, int* status) {
+    omp_warp(M, cvec, y2, lam, r, K, 0, beta, sel, nsel, status, nullptr, nullptr, nullptr, nullptr);
+}
+
 // 10. Phi_Y[i][c] = sum_t DY[(t+1)*k + i] G[t][c]
-__global__ void phiy_kernel(const double* __restrict__ DY, const double* __restrict__ G, int k, int p,
-                            int r, double* __restrict__ PhiY) {
+__global__ void phiy_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& q = sb.c[blockIdx.z];
+    if (q.PhiY == nullptr || q.DY == nullptr) return;
+    const double *DY = q.DY, *G = q.G;
+    const int k = sb.k, p = q.p, r = sb.r;
+    double* PhiY = q.PhiY;
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (idx >= static_cast<int64_t>(k) * r) return;
     const int i = static_cast<int>(idx % k), c = static_cast<int>(idx / k);
@@ -1680,85 +1765,110 @@ cdmd_status launch_selector_relabel(cdmd_ctx* ctx, const double* DY, int k, int 
     int32_t* nsel_t = reinterpret_cast<int32_t*>(y2_t + 1);
     relabel_target_kernel<<<1, 256, 0, stream>>>(DY, k, p, G, r, y_target, u, cvec_t, y2_t);
     CDMD_CHECK_LAUNCH("relabel_target_kernel");
-    omp_kernel<<<1, 32, 0, stream>>>(ctx->last_M, cvec_t, y2_t, lambda, r, K, 0, beta_t, sel, nsel_t,
-                                     ctx->d_status, nullptr, nullptr, nullptr, nullptr);
-    CDMD_CHECK_LAUNCH("omp_kernel");
+    relabel_omp_kernel<<<1, 32, 0, stream>>>(ctx->last_M, cvec_t, y2_t, lambda, r, K, beta_t, sel, nsel_t,
+                                             ctx->d_status);
+    CDMD_CHECK_LAUNCH("relabel_omp_kernel");
     return CDMD_OK;
 }
 
 namespace {
 
-// Steps 4-7 and 9 from the Gram of the sketch DY (k x n), or, when Rin is
-// given, from that n x n Gram directly (DY and PhiY unused).
+// Steps 4-7 and 9 of every clip in io from the Gram of its sketch DY (k x n),
+// or from the n x n Gram R directly when that is given (DY and PhiY unused).
 struct AutoRank {
     int* r_host;        // receives the chosen rank
     double* tau_host;   // receives the threshold (may be NULL)
 };
 
-cdmd_status decompose_impl(cdmd_ctx* ctx, const double* DY, int k, const double* Rin, int n, int r, int K,
-                           cdmd_selector selector, double* sigma, double* lambda, double* G, double* PhiY,
-                           double* beta, int32_t* sel, int32_t* nsel, cudaStream_t stream,
-                           const AutoRank* autor = nullptr) {
-    const int p = n - 1;
-    // ---- workspace layout (doubles) ----
-    const int ntiles = (n + kGT - 1) / kGT;
+cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int k, int r, int K,
+                           cdmd_selector selector, cudaStream_t stream, const AutoRank* autor = nullptr) {
+    if (nclips < 1 || nclips > kMaxSolveClips) return fail(CDMD_ERR_INVALID_ARG, "%d clips in one solve", nclips);
+    // ---- workspace layout (doubles), one region per clip ----
     const int kchunk = 128;
-    const int splits = Rin != nullptr ? 0 : (k + kchunk - 1) / kchunk;
-    const size_t n_gram_part = static_cast<size_t>(splits) * n * n;
-    const size_t n_R = static_cast<size_t>(n) * n;
-    const size_t n_Hv = static_cast<size_t>(p) * p;
-    const size_t n_vec = static_cast<size_t>(p);
-    const size_t n_Z = static_cast<size_t>(p) * r;
-    const size_t n_small = static_cast<size_t>(r) * r * 2;
-    const size_t total = n_gram_part + n_R + n_Hv + 3 * n_vec + r + 3 * n_Z + 5 * n_small + 6 * r + 64;
-    // + one slot for the eigen-solver's fallback flag and two for the rank
-    // threshold's result; with an automatic rank, r is its upper bound here
+    const int splits = io[0].R != nullptr ? 0 : (k + kchunk - 1) / kchunk;
+    size_t off[kMaxSolveClips + 1] = {0};
+    int nmax = 0;
+    for (int i = 0; i < nclips; ++i) {
+        const size_t n = io[i].n, p = n - 1, rr = r;
+        const size_t total = static_cast<size_t>(splits) * n * n + n * n + p * p + 3 * p + rr + 3 * p * rr +
+                             10 * rr * rr + 6 * rr + 64;
+        // + one slot for the eigen-solver's fallback flag and two for the rank
+        // threshold's result; with an automatic rank, r is its upper bound here
+        off[i + 1] = off[i] + total + 3;
+        nmax = std::max(nmax, io[i].n);
+    }
     double* ws = nullptr;
-    cdmd_status st = ensure_buffer(ctx, BUF_EIG, (total + 3) * sizeof(double), reinterpret_cast<void**>(&ws));
+    cdmd_status st = ensure_buffer(ctx, BUF_EIG, off[nclips] * sizeof(double), reinterpret_cast<void**>(&ws));
     if (st != CDMD_OK) return st;
-    int* eig_flag = reinterpret_cast<int*>(ws + total);   // written by eig_f32_kernel before any read
-    int* gd_r = reinterpret_cast<int*>(ws + total + 1);
-    double* gd_tau = ws + total + 2;
-    double* gpart = ws;
-    double* Rws = gpart + n_gram_part;
-    const double* R = Rin != nullptr ? Rin : Rws;
-    double* Hv = Rws + n_R;
-    double* htau = Hv + n_Hv;
-    double* dd = htau + n_vec;
-    double* ee = dd + n_vec;
-    double* lamT = ee + n_vec;
-    // the regions below depend on r; with an automatic rank they are laid out
-    // again once the rank is known (a smaller r fits the same allocation)
-    double *Z, *V, *B, *At, *W, *M, *WR, *lamR, *cvec;
-    float *lam32, *W32;
+    SolveBatch sb = {};
+    sb.k = k;
+    sb.status = ctx->d_status;
+    bool want_phiy = false;
+    // the regions from lamT on depend on r; with an automatic rank they are
+    // laid out again once the rank is known (a smaller r fits the allocation)
     auto lay_out = [&](int rr) {
-        const size_t nz = static_cast<size_t>(p) * rr, ns = static_cast<size_t>(rr) * rr * 2;
-        Z = lamT + rr;
-        V = Z + nz;
-        B = V + nz;
-        At = B + nz;
-        W = At + ns;
-        M = W + ns;
-        WR = M + ns;
-        lamR = WR + ns;
-        cvec = lamR + 2 * rr;
-        lam32 = reinterpret_cast<float*>(cvec + 2 * rr);    // 2r floats
-        W32 = reinterpret_cast<float*>(cvec + 4 * rr);      // 2r^2 floats (ns/2 doubles)
+        for (int i = 0; i < nclips; ++i) {
+            SolveClip& q = sb.c[i];
+            const size_t nz = static_cast<size_t>(q.p) * rr, ns = static_cast<size_t>(rr) * rr * 2;
+            q.Z = q.lamT + rr;
+            q.V = q.Z + nz;
+            q.B = q.V + nz;
+            q.At = q.B + nz;
+            q.W = q.At + ns;
+            q.M = q.W + ns;
+            q.WR = q.M + ns;
+            q.lamR = q.WR + ns;
+            q.cvec = q.lamR + 2 * rr;
+            q.lam32 = reinterpret_cast<float2*>(q.cvec + 2 * rr);    // 2r floats
+            q.W32 = reinterpret_cast<float2*>(q.cvec + 4 * rr);      // 2r^2 floats (ns/2 doubles)
+        }
+        sb.r = rr;
     };
+    for (int i = 0; i < nclips; ++i) {
+        SolveClip& q = sb.c[i];
+        q.DY = io[i].DY;
+        q.n = io[i].n;
+        q.p = q.n - 1;
+        q.gpart = ws + off[i];
+        q.Rw = q.gpart + static_cast<size_t>(splits) * q.n * q.n;
+        q.R = io[i].R != nullptr ? io[i].R : q.Rw;
+        q.Hv = q.Rw + static_cast<size_t>(q.n) * q.n;
+        q.htau = q.Hv + static_cast<size_t>(q.p) * q.p;
+        q.dd = q.htau + q.p;
+        q.ee = q.dd + q.p;
+        q.lamT = q.ee + q.p;
+        q.flag = reinterpret_cast<int*>(ws + off[i + 1] - 3);   // written by eig_f32_kernel before any read
+        q.sigma = io[i].sigma;
+        q.lambda = io[i].lambda;
+        q.G = io[i].G;
+        q.PhiY = io[i].PhiY;
+        q.beta = io[i].beta;
+        q.sel = io[i].sel;
+        q.nsel = io[i].nsel;
+        if (selector == CDMD_SEL_MLP) {
+            q.order = selector_order(ctx, i);
+            q.accept = selector_accept(ctx, i);
+        }
+        want_phiy = want_phiy || (q.PhiY != nullptr && q.DY != nullptr);
+    }
     lay_out(r);
+    sb.K = K;
+    const int p = nmax - 1;                          // the longest clip sizes the launches
+    const unsigned nc = static_cast<unsigned>(nclips);
 
     // 1. Gram
-    if (Rin == nullptr) {
-        gram_partial_kernel<<<dim3(ntiles, ntiles, splits), 256, 0, stream>>>(DY, k, n, kchunk, gpart);
+    if (splits > 0) {
+        const int ntiles = (nmax + kGT - 1) / kGT;
+        gram_partial_kernel<<<dim3(ntiles * (ntiles + 1) / 2, nc, splits), 256, 0, stream>>>(sb, kchunk);
         CDMD_CHECK_LAUNCH("gram_partial_kernel");
-        gram_reduce_kernel<<<(n * n + 255) / 256, 256, 0, stream>>>(gpart, splits, n, Rws, ctx->d_status);
+        gram_reduce_kernel<<<dim3((nmax * nmax + 255) / 256, nc), 256, 0, stream>>>(sb, splits);
         CDMD_CHECK_LAUNCH("gram_reduce_kernel");
     }
 
     // 2. tridiagonalisation on a cluster of 8 CTAs (else 4).  A cluster must
     // fit in one GPC beside other clips' full-data passes: 8 CTAs gave 3.8 %
     // more clips/s than 16 with clips in flight, at 2 % more latency
-    if (p >= 3) {
+    {
         // cluster size: 8 CTAs first (fits one GPC beside other clips' passes),
         // else 16 (non-portable; large n), else 4
         const int csize_pref = 8;
@@ -1776,7 +1886,7 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, const double* DY, int k, const double*
             if (csize > 8)
                 CDMD_CHECK_CUDA(cudaFuncSetAttribute(tridiag_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
             cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(csize, 1, 1);
+            cfg.gridDim = dim3(csize, 1, nc);
             cfg.blockDim = dim3(kTriThreads, 1, 1);
             cfg.dynamicSmemBytes = smem;
             cfg.stream = stream;
@@ -1793,23 +1903,21 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, const double* DY, int k, const double*
                 (void)cudaGetLastError();
                 continue;
             }
-            CDMD_CHECK_CUDA(cudaLaunchKernelEx(&cfg, tridiag_kernel, static_cast<const double*>(R), n, p, Hv,
-                                               htau, dd, ee));
+            CDMD_CHECK_CUDA(cudaLaunchKernelEx(&cfg, tridiag_kernel, sb));
             launched = true;
         }
         if (!launched) return fail(CDMD_ERR_UNSUPPORTED, "no cluster size fits the tridiagonalisation of p = %d", p);
-    } else {
-        tiny_tridiag_kernel<<<1, 1, 0, stream>>>(R, n, p, dd, ee, htau);
-        CDMD_CHECK_LAUNCH("tiny_tridiag_kernel");
     }
     // 2b. optional automatic rank (Remark 2): the one host synchronisation of
     // the decomposition, since the launches below are sized by r
-    if (autor != nullptr) {
+    if (autor != nullptr) {   // one clip
+        int* gd_r = sb.c[0].flag + 2;
+        double* gd_tau = reinterpret_cast<double*>(sb.c[0].flag + 4);
         const int q = k < p ? k : p;
         const double bq = static_cast<double>(q) / static_cast<double>(k > p ? k : p);
         const double omega = ((0.56 * bq - 0.95) * bq + 1.82) * bq + 1.43;
-        gd_rank_kernel<<<1, 32, 2 * static_cast<size_t>(p) * sizeof(double), stream>>>(dd, ee, p, q, omega, r, gd_r,
-                                                                                         gd_tau, ctx->d_status);
+        gd_rank_kernel<<<1, 32, 2 * static_cast<size_t>(p) * sizeof(double), stream>>>(sb.c[0].dd, sb.c[0].ee, p, q, omega, r,
+                                                                                 gd_r, gd_tau, ctx->d_status);
         CDMD_CHECK_LAUNCH("gd_rank_kernel");
         int hr = 0;
         double ht = 0.0;
@@ -1818,9 +1926,10 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, const double* DY, int k, const double*
         CDMD_CHECK_CUDA(cudaStreamSynchronize(stream));
         if (hr < 1 || hr > r) return fail(CDMD_ERR_CUDA, "rank threshold returned %d (bound %d)", hr, r);
         // picks past the capped K read as "no mode"
-        CDMD_CHECK_CUDA(cudaMemsetAsync(sel, 0xff, static_cast<size_t>(K) * sizeof(int32_t), stream));
+        CDMD_CHECK_CUDA(cudaMemsetAsync(sb.c[0].sel, 0xff, static_cast<size_t>(K) * sizeof(int32_t), stream));
         r = hr;
         if (K > r) K = r;
+        sb.K = K;
         *autor->r_host = r;
         if (autor->tau_host != nullptr) *autor->tau_host = ht;
         lay_out(r);
@@ -1830,68 +1939,64 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, const double* DY, int k, const double*
         const size_t esm = 10 * static_cast<size_t>(p) * sizeof(double);
         CDMD_CHECK_CUDA(cudaFuncSetAttribute(tridiag_eigpair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(kMaxOptInSmem)));
-        tridiag_eigpair_kernel<<<r, 32, esm, stream>>>(dd, ee, p, r, lamT, Z, ctx->d_status);
+        tridiag_eigpair_kernel<<<dim3(r, 1, nc), 32, esm, stream>>>(sb);
         CDMD_CHECK_LAUNCH("tridiag_eigpair_kernel");
     }
     {
         const size_t osm = (static_cast<size_t>(r) * p + 64) * sizeof(double);
         CDMD_CHECK_CUDA(cudaFuncSetAttribute(orthonormalise_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(kMaxOptInSmem)));
-        orthonormalise_kernel<<<1, 1024, osm, stream>>>(Z, p, r);
+        orthonormalise_kernel<<<dim3(1, 1, nc), 1024, osm, stream>>>(sb);
     }
     CDMD_CHECK_LAUNCH("orthonormalise_kernel");
     static_assert(32 * 16 >= 511, "the back-transform covers p = n - 1 <= 511 (n <= 512)");
     if (p <= 256)
-        backtransform_kernel<8><<<r, 32, p * sizeof(double), stream>>>(Z, Hv, htau, lamT, p, r, V, sigma,
-                                                                       ctx->d_status);
+        backtransform_kernel<8><<<dim3(r, 1, nc), 32, p * sizeof(double), stream>>>(sb);
     else
-        backtransform_kernel<16><<<r, 32, p * sizeof(double), stream>>>(Z, Hv, htau, lamT, p, r, V, sigma,
-                                                                        ctx->d_status);
+        backtransform_kernel<16><<<dim3(r, 1, nc), 32, p * sizeof(double), stream>>>(sb);
     CDMD_CHECK_LAUNCH("backtransform_kernel");
     // 4. A~ and its eigen-decomposition
-    bmat_kernel<<<dim3((p + 7) / 8, r), 256, 0, stream>>>(R, V, n, p, B);
+    bmat_kernel<<<dim3((p + 7) / 8, r, nc), 256, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("bmat_kernel");
-    atilde_kernel<<<r, 32, 0, stream>>>(V, B, sigma, p, r, At);
+    atilde_kernel<<<dim3(r, 1, nc), 32, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("atilde_kernel");
-    eig_f32_kernel<<<1, 32, 0, stream>>>(At, r, reinterpret_cast<float2*>(lam32), reinterpret_cast<float2*>(W32),
-                                         eig_flag);
+    eig_f32_kernel<<<dim3(1, 1, nc), 32, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("eig_f32_kernel");
-    eig_refine_kernel<<<r, 32, 0, stream>>>(At, r, reinterpret_cast<const float2*>(lam32),
-                                            reinterpret_cast<const float2*>(W32), lamR, WR, eig_flag);
+    eig_refine_kernel<<<dim3(r, 1, nc), 32, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("eig_refine_kernel");
     CDMD_CHECK_CUDA(cudaFuncSetAttribute(eig_qr64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(kQrSmem)));
-    eig_qr64_kernel<<<1, kQrThreads, kQrSmem, stream>>>(At, r, lamR, WR, eig_flag, ctx->d_status);
+    eig_qr64_kernel<<<dim3(1, 1, nc), kQrThreads, kQrSmem, stream>>>(sb);
     CDMD_CHECK_LAUNCH("eig_qr64_kernel");
-    eig_order_kernel<<<1, 32, 0, stream>>>(lamR, WR, r, lambda, W);
+    eig_order_kernel<<<dim3(1, 1, nc), 32, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("eig_order_kernel");
     // 5. G, Gram-form quantities, selection
-    gmat_kernel<<<(p * r + 127) / 128, 128, 0, stream>>>(V, sigma, W, p, r, G);
+    gmat_kernel<<<dim3((p * r + 127) / 128, 1, nc), 128, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("gmat_kernel");
-    hmat_kernel<<<r, 512, 2 * p * sizeof(double), stream>>>(R, G, n, p, r, M, cvec);
+    hmat_kernel<<<dim3(r, 1, nc), 512, 2 * p * sizeof(double), stream>>>(sb);
     CDMD_CHECK_LAUNCH("hmat_kernel");
-    ctx->last_M = M;
-    ctx->last_cvec = cvec;
-    ctx->last_R = R;
+    const SolveClip& last = sb.c[nclips - 1];
+    ctx->last_M = last.M;
+    ctx->last_cvec = last.cvec;
+    ctx->last_R = last.R;
     ctx->last_r = r;
     if (selector == CDMD_SEL_MLP) {
         // learned pick order -> least squares on it -> OMP only if rejected
-        st = launch_mlp_select(ctx, lambda, M, cvec, R, r, K, stream);
-        if (st != CDMD_OK) return st;
-        omp_kernel<<<1, 32, 0, stream>>>(M, cvec, R, lambda, r, K, 0, beta, sel, nsel, ctx->d_status,
-                                         selector_order(ctx), selector_blob(ctx), selector_accept(ctx),
-                                         selector_fallbacks(ctx));
+        for (int i = 0; i < nclips; ++i) {
+            const SolveClip& q = sb.c[i];
+            st = launch_mlp_select(ctx, q.lambda, q.M, q.cvec, q.R, r, K, q.order, stream);
+            if (st != CDMD_OK) return st;
+        }
+        omp_kernel<<<dim3(1, 1, nc), 32, 0, stream>>>(sb, 0, 1, selector_blob(ctx), selector_fallbacks(ctx));
         CDMD_CHECK_LAUNCH("omp_kernel");
-        omp_kernel<<<1, 32, 0, stream>>>(M, cvec, R, lambda, r, K, 0, beta, sel, nsel, ctx->d_status, nullptr,
-                                         nullptr, selector_accept(ctx), nullptr);
+        omp_kernel<<<dim3(1, 1, nc), 32, 0, stream>>>(sb, 0, 2, nullptr, nullptr);
     } else {
-        omp_kernel<<<1, 32, 0, stream>>>(M, cvec, R, lambda, r, K, selector == CDMD_SEL_LSTSQ ? 1 : 0, beta, sel,
-                                         nsel, ctx->d_status, nullptr, nullptr, nullptr, nullptr);
+        omp_kernel<<<dim3(1, 1, nc), 32, 0, stream>>>(sb, selector == CDMD_SEL_LSTSQ ? 1 : 0, 0, nullptr, nullptr);
     }
     CDMD_CHECK_LAUNCH("omp_kernel");
-    if (PhiY != nullptr && DY != nullptr) {
+    if (want_phiy) {
         const int64_t tot = static_cast<int64_t>(k) * r;
-        phiy_kernel<<<static_cast<unsigned>((tot + 127) / 128), 128, 0, stream>>>(DY, G, k, p, r, PhiY);
+        phiy_kernel<<<dim3(static_cast<unsigned>((tot + 127) / 128), 1, nc), 128, 0, stream>>>(sb);
         CDMD_CHECK_LAUNCH("phiy_kernel");
     }
     return CDMD_OK;
@@ -1899,26 +2004,15 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, const double* DY, int k, const double*
 
 }  // namespace
 
-cdmd_status launch_decompose(cdmd_ctx* ctx, const double* DY, int k, int n, int r, int K,
-                             cdmd_selector selector, double* sigma, double* lambda, double* G,
-                             double* PhiY, double* beta, int32_t* sel, int32_t* nsel,
-                             cudaStream_t stream) {
-    return decompose_impl(ctx, DY, k, nullptr, n, r, K, selector, sigma, lambda, G, PhiY, beta, sel, nsel, stream);
+cdmd_status launch_decompose(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int k, int r, int K,
+                             cdmd_selector selector, cudaStream_t stream) {
+    return decompose_impl(ctx, nclips, io, k, r, K, selector, stream);
 }
 
-cdmd_status launch_decompose_auto(cdmd_ctx* ctx, const double* DY, int k, int n, int r_max, int K,
-                                  cdmd_selector selector, double* sigma, double* lambda, double* G, double* PhiY,
-                                  double* beta, int32_t* sel, int32_t* nsel, int* r_out, double* tau_out,
-                                  cudaStream_t stream) {
+cdmd_status launch_decompose_auto(cdmd_ctx* ctx, const DecomposeIO& io, int k, int r_max, int K,
+                                  cdmd_selector selector, int* r_out, double* tau_out, cudaStream_t stream) {
     const AutoRank a{r_out, tau_out};
-    return decompose_impl(ctx, DY, k, nullptr, n, r_max, K, selector, sigma, lambda, G, PhiY, beta, sel, nsel, stream,
-                          &a);
-}
-
-cdmd_status launch_decompose_gram(cdmd_ctx* ctx, const double* R, int n, int r, int K, cdmd_selector selector,
-                                  double* sigma, double* lambda, double* G, double* beta, int32_t* sel,
-                                  int32_t* nsel, cudaStream_t stream) {
-    return decompose_impl(ctx, nullptr, 0, R, n, r, K, selector, sigma, lambda, G, nullptr, beta, sel, nsel, stream);
+    return decompose_impl(ctx, 1, &io, k, r_max, K, selector, stream, &a);
 }
 
 }  // namespace cdmd

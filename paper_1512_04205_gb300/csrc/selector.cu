@@ -232,8 +232,8 @@ cdmd_status launch_selector_features(cdmd_ctx* ctx, const double* lambda, const 
 }
 
 cdmd_status launch_mlp_select(cdmd_ctx* ctx, const double* lambda, const double* M, const double* cvec,
-                              const double* R, int r, int K, cudaStream_t stream) {
-    mlp_select_kernel<<<1, 32, 0, stream>>>(selector_blob(ctx), lambda, M, cvec, R, r, K, selector_order(ctx));
+                              const double* R, int r, int K, int32_t* order, cudaStream_t stream) {
+    mlp_select_kernel<<<1, 32, 0, stream>>>(selector_blob(ctx), lambda, M, cvec, R, r, K, order);
     CDMD_CHECK_LAUNCH("mlp_select_kernel");
     return CDMD_OK;
 }

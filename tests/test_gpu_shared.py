@@ -160,3 +160,29 @@ def test_batch_pairs_clips_that_share_c(C):
         a, b = C.unpack_mask(batch.masks[i], clip.m), C.unpack_mask(mk, clip.m)
         assert np.mean(a != b) <= 2e-4
     batch.close()
+
+
+@pytest.mark.parametrize("ns,r,K,selector", [((40, 3, 64, 9), 2, 2, "omp"), ((33, 120, 61), 12, 6, "mlp"),
+                                             ((30, 260), 16, 16, "lstsq"), ((50,) * 8, 10, 4, "omp")])
+def test_run_shared_solves_side_by_side_equal_solo_solves(C, ctx, ns, r, K, selector):
+    # FP32 sketches are per clip, so every stage of a shared run sees the
+    # solo run's inputs and must give its bits, whatever lengths share the
+    # launches (n - 1 = 2 has no reflectors; 260 frames need other tile counts)
+    from paper_1512_04205_gb300 import selector as S
+    w, h, k = 96, 64, 64
+    clips = _clips(w, h, ns, seed0=17)
+    Ds = [torch.from_numpy(c.frames).cuda() for c in clips]
+    c2 = C.Context(0)
+    if selector == "mlp":
+        C.cdmd_selector_load(c2, torch.from_numpy(S.load_model()[0].copy()).cuda())
+    p = C.make_params(k, r, K, 25.0, seed=5, prec="fp32", selector=selector)
+    masks = C.cdmd_run_shared(c2, Ds, p)
+    cols = r if selector == "lstsq" else K
+    got = C.workspace_tensors(c2, clips[0].m, ns[-1], k, r, cols)
+    for D, mk in zip(Ds, masks):
+        assert torch.equal(mk, C.cdmd_run(c2, D, p))
+    want = C.workspace_tensors(c2, clips[0].m, ns[-1], k, r, cols)
+    C.cdmd_status_sync(c2)
+    for q in ("DY", "sigma", "lam", "G", "beta", "nsel", "Phi"):
+        assert torch.equal(got[q], want[q]), q
+    assert torch.equal(got["sel"][:K], want["sel"][:K])
