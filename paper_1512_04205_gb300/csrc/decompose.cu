@@ -64,10 +64,10 @@ struct SolveClip {
     const double* R;     // n x n Gram
     int n, p;            // frames, p = n - 1
     double *gpart, *Rw;  // Gram partials; the Gram's own storage (NULL when R is given)
-    double *Hv, *htau, *dd, *ee;                  // reflectors and the tridiagonal form
+    double *Hv, *htau, *Tw, *dd, *ee;             // reflectors, their block factors, the tridiagonal form
     double *lamT, *Z, *V, *B, *At, *W, *M, *WR, *lamR, *cvec;
     float2 *lam32, *W32;
-    int* flag;           // eigen-solver fallback
+    int* flag;           // [0] eigen-solver fallback, [1] eigenvectors of T not orthogonal to kOrthTol
     double *sigma, *lambda, *G, *PhiY, *beta;     // the caller's outputs
     int32_t *sel, *nsel;
     int32_t* order;      // learned pick order and its verdict
@@ -89,6 +89,19 @@ __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
+}
+
+// Sums of four values over the warp: lanes 8 e .. 8 e + 7 end with s[e]'s.
+// Six additions; four warp_sums take twenty.
+__device__ __forceinline__ double warp_sum4(const double s[4]) {
+    const int lane = threadIdx.x & 31;
+    const bool hi = (lane & 16) != 0, mid = (lane & 8) != 0;
+    const double t0 = (hi ? s[2] : s[0]) + __shfl_xor_sync(0xffffffffu, hi ? s[0] : s[2], 16);
+    const double t1 = (hi ? s[3] : s[1]) + __shfl_xor_sync(0xffffffffu, hi ? s[1] : s[3], 16);
+    double t = (mid ? t1 : t0) + __shfl_xor_sync(0xffffffffu, mid ? t0 : t1, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
 }
 
 // Block-wide sum; `red` holds >= 32 doubles of shared scratch.  All threads
@@ -458,40 +471,99 @@ __device__ __forceinline__ void sturm_count2(const double* d, const double* e2, 
     n1 = c1;
 }
 
-constexpr int kShifts = 64;   // shifts tested per multisection pass (two per lane)
+// The same count in FP32, for a first bracket only: entries scaled by a power
+// of two below 1, rescaled every four steps (products of four stay in range).
+__device__ __forceinline__ int sturm_count_f32(const float* d, const float* e2, int p, float x) {
+    float a = d[0] - x, b = 1.0f;
+    int c = static_cast<int>(__float_as_uint(a) >> 31);
+    for (int i = 1; i < p; ++i) {
+        const float t = fmaf(d[i] - x, a, -e2[i - 1] * b);
+        c += static_cast<int>((__float_as_uint(t) ^ __float_as_uint(a)) >> 31);
+        b = a;
+        a = t;
+        if ((i & 3) == 0) {
+            const int ex = static_cast<int>(__float_as_uint(a) >> 23) & 0xff;
+            if (ex > 127 + 16 || (ex > 0 && ex < 127 - 16)) {
+                const float s = __uint_as_float(static_cast<uint32_t>(254 - ex) << 23);
+                a *= s;
+                b *= s;
+            }
+        }
+    }
+    return c;
+}
 
-__global__ void __launch_bounds__(32)
-tridiag_eigpair_kernel(const __grid_constant__ SolveBatch sb) {
-    const SolveClip& q = sb.c[blockIdx.z];
+__device__ __forceinline__ int sturm_count(const double* d, const double* e2, int p, double x) {
+    double a = d[0] - x, b = 1.0;
+    int c = static_cast<int>(static_cast<unsigned>(__double2hiint(a)) >> 31);
+    for (int i = 1; i < p; ++i) {
+        const double t = fma(d[i] - x, a, -e2[i - 1] * b);
+        c += static_cast<int>(static_cast<unsigned>(__double2hiint(t) ^ __double2hiint(a)) >> 31);
+        b = a;
+        a = t;
+        if ((i & 7) == 0) rescale_pair(a, b);
+    }
+    return c;
+}
+
+constexpr int kEigThreads = 128;   // one warp per scheduler; one shift per thread
+
+// The first of the block's kEigThreads flags that is set (kEigThreads if
+// none); `ball` holds four words, alternating between calls (`turn`).
+__device__ __forceinline__ int first_set(bool flag, unsigned* ball, int turn) {
+    const unsigned b = __ballot_sync(0xffffffffu, flag);
+    unsigned* w = ball + 4 * (turn & 1);
+    if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = b;
+    __syncthreads();
+    int f = kEigThreads;
+#pragma unroll
+    for (int i = 3; i >= 0; --i)
+        if (w[i]) f = 32 * i + __ffs(w[i]) - 1;
+    return f;
+}
+
+// Eigenpair `w` (descending) of T, one CTA of four warps, one per scheduler:
+// a DP instruction holds its scheduler 64 clocks whatever its lanes do, so four
+// warps of one shift each run a Sturm pass over 128 shifts in the time one
+// warp takes over 32.  Three passes in FP32 narrow the interval to 2 units of
+// 1e-6 of the norm (margin: 16 eps32, above the count's backward error);
+// FP64 passes, the first of which tests both ends of that bracket (else
+// everything is repeated from the Gershgorin interval), go on to eps.
+// Inverse iteration: LU with partial pivoting and two solves by one thread,
+// each step one or two dependent DP instructions; everything that is not on
+// that chain (d - mu, the scaled rows of U, the divisions by the pivots) is
+// done by all threads between the chains.
+__device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm) {
     const double *dd = q.dd, *ee = q.ee;
     const int p = q.p;
-    double *lam = q.lamT, *Z = q.Z;
-    int* status = sb.status;
-    extern __shared__ double tsm[];
     double* d = tsm;            // p
     double* e = d + p;          // p (e[p-1] = 0)
     double* e2 = e + p;         // p
     double* lmul = e2 + p;      // p: elimination multipliers
-    double* udg = lmul + p;     // p: U diagonal
+    double* udg = lmul + p;     // p: T's shifted diagonal
     double* u1 = udg + p;       // p: U first super-diagonal
     double* u2 = u1 + p;        // p: U second super-diagonal
     double* invd = u2 + p;      // p: 1 / U diagonal
     double* z = invd + p;       // p: iterate
-    int* piv = reinterpret_cast<int*>(z + p);   // p
-    const int w = blockIdx.x;
-    const int lane = threadIdx.x;
-    for (int i = lane; i < p; i += 32) {
-        d[i] = dd[i];
-        e[i] = (i + 1 < p) ? ee[i] : 0.0;
-        e2[i] = e[i] * e[i];
-    }
-    __syncwarp();
+    int* piv = reinterpret_cast<int*>(z + p);          // p
+    float* d32 = reinterpret_cast<float*>(piv + p);    // p
+    float* e32 = d32 + p;                              // p
+    __shared__ double red[12];
+    __shared__ unsigned ball[8];
+    __shared__ int flags[4];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     double lo = 1e300, hi = -1e300, tn = 0.0;
-    for (int i = lane; i < p; i += 32) {
-        const double rad = fabs(e[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0);
-        lo = fmin(lo, d[i] - rad);
-        hi = fmax(hi, d[i] + rad);
-        tn = fmax(tn, fabs(d[i]) + rad);
+    for (int i = tid; i < p; i += kEigThreads) {
+        const double di = dd[i];
+        const double en = (i + 1 < p) ? ee[i] : 0.0;
+        const double ep = i > 0 ? fabs(ee[i - 1]) : 0.0;
+        d[i] = di;
+        e[i] = en;
+        e2[i] = en * en;
+        const double rad = fabs(en) + ep;
+        lo = fmin(lo, di - rad);
+        hi = fmax(hi, di + rad);
+        tn = fmax(tn, fabs(di) + rad);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -499,109 +571,273 @@ tridiag_eigpair_kernel(const __grid_constant__ SolveBatch sb) {
         hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
         tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
     }
+    if (lane == 0) { red[wid] = lo; red[4 + wid] = hi; red[8 + wid] = tn; }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        lo = fmin(lo, red[i]);
+        hi = fmax(hi, red[4 + i]);
+        tn = fmax(tn, red[8 + i]);
+    }
     const double pad = 2.0 * kEps * tn + 1e-300;
-    lo -= pad;
-    hi += pad;
+    const double glo = lo - pad, ghi = hi + pad;
     const int idx = p - 1 - w;   // ascending index of the target eigenvalue
+    int turn = 0;
+
+    // FP32 bracket (skipped when the scale factor would leave the range)
+    const int ex = (__double2hiint(tn) >> 20) & 0x7ff;
+    bool bracket = ex > 64 && ex < 1983;
+    if (bracket) {
+        const double sc = __hiloint2double((2046 - ex - 1) << 20, 0);     // tn sc in [1/2, 1)
+        const double isc = __hiloint2double((ex + 1) << 20, 0);
+        for (int i = tid; i < p; i += kEigThreads) {
+            const float ef = static_cast<float>(e[i] * sc);
+            d32[i] = static_cast<float>(d[i] * sc);
+            e32[i] = ef * ef;
+        }
+        __syncthreads();
+        float flo = static_cast<float>(glo * sc), fhi = static_cast<float>(ghi * sc);
+        for (int it = 0; it < 3; ++it) {
+            const float step = (fhi - flo) * (1.0f / (kEigThreads + 1));
+            const bool above = sturm_count_f32(d32, e32, p, fmaf(step, static_cast<float>(tid + 1), flo)) > idx;
+            const int f = first_set(above, ball, turn++);
+            const float nlo = (f == 0) ? flo : fmaf(step, static_cast<float>(f), flo);
+            fhi = (f == kEigThreads) ? fhi : fmaf(step, static_cast<float>(f + 1), flo);
+            flo = nlo;
+        }
+        const double margin = 16.0 * 1.1920929e-07;
+        lo = (static_cast<double>(flo) - margin) * isc;
+        hi = (static_cast<double>(fhi) + margin) * isc;
+        // the ends of the bracket and 126 shifts between them
+        const double step = (hi - lo) * (1.0 / (kEigThreads - 1));
+        const bool above = sturm_count(d, e2, p, fma(step, static_cast<double>(tid), lo)) > idx;
+        const int f = first_set(above, ball, turn++);
+        bracket = f > 0 && f < kEigThreads;
+        if (bracket) {
+            hi = fma(step, static_cast<double>(f), lo);
+            lo = fma(step, static_cast<double>(f - 1), lo);
+        }
+    }
+    if (!bracket) {
+        lo = glo;
+        hi = ghi;
+    }
     bool converged = false;
     for (int it = 0; it < 40; ++it) {
         const double width = hi - lo;
         if (width <= 2.0 * kEps * fmax(fabs(lo), fabs(hi)) + kEps * tn + 1e-300) { converged = true; break; }
-        const double step = width * (1.0 / (kShifts + 1));
-        int n0, n1;
-        sturm_count2(d, e2, p, fma(step, static_cast<double>(lane + 1), lo),
-                     fma(step, static_cast<double>(lane + 33), lo), n0, n1);
-        const unsigned b0 = __ballot_sync(0xffffffffu, n0 > idx);
-        const unsigned b1 = __ballot_sync(0xffffffffu, n1 > idx);
-        const int f = b0 ? __ffs(b0) - 1 : (b1 ? 32 + __ffs(b1) - 1 : kShifts);
+        const double step = width * (1.0 / (kEigThreads + 1));
+        const bool above = sturm_count(d, e2, p, fma(step, static_cast<double>(tid + 1), lo)) > idx;
+        const int f = first_set(above, ball, turn++);
         const double nlo = (f == 0) ? lo : fma(step, static_cast<double>(f), lo);
-        const double nhi = (f == kShifts) ? hi : fma(step, static_cast<double>(f + 1), lo);
+        const double nhi = (f == kEigThreads) ? hi : fma(step, static_cast<double>(f + 1), lo);
         if (nlo >= nhi || (nlo == lo && nhi == hi)) { converged = true; break; }
         lo = nlo;
         hi = nhi;
     }
     const double lambda = 0.5 * (lo + hi);
-    if (!converged && lane == 0) record_status(status, CDMD_ERR_NOT_CONVERGED);
-    if (lane == 0) lam[w] = lambda;
+    if (!converged && tid == 0) record_status(status, CDMD_ERR_NOT_CONVERGED);
+    if (tid == 0) q.lamT[w] = lambda;
+    double* Z = q.Z + static_cast<int64_t>(w) * p;
     if (!(lambda > kRankTol * static_cast<double>(p) * kEps * tn)) {
         // a numerically zero eigenvalue: sigma_r of the sketch vanishes
-        if (lane == 0) record_status(status, CDMD_ERR_RANK_DEFICIENT);
-        for (int i = lane; i < p; i += 32) Z[static_cast<int64_t>(w) * p + i] = (i == w) ? 1.0 : 0.0;
+        if (tid == 0) record_status(status, CDMD_ERR_RANK_DEFICIENT);
+        for (int i = tid; i < p; i += kEigThreads) Z[i] = (i == w) ? 1.0 : 0.0;
         return;
     }
     // inverse iteration: LU with partial pivoting of T - mu I, reciprocal pivots
     const double mu = lambda + kEps * tn;   // keeps T - mu I away from exact singularity
     const double tiny = kEps * tn + 1e-300;
-    for (int i = lane; i < p; i += 32) {
+    for (int i = tid; i < p; i += kEigThreads) {
         udg[i] = d[i] - mu;
-        lmul[i] = e[i];
-        u1[i] = e[i];
-        u2[i] = 0.0;
-        piv[i] = 0;
-        // start vector: 1 + a hash of (i, w) in [0, 1)
+        // start vector: 1 + a hash of (i, w) in [0, 1); its product with the
+        // eigenvector of T is positive in the result (two solves), which fixes
+        // the sign of the singular vector
         uint32_t h = (static_cast<uint32_t>(i) + 1u) * 0x9E3779B9u ^ (static_cast<uint32_t>(w) + 1u) * 0x85EBCA6Bu;
         h ^= h >> 15;
         h *= 0x2C1B3C6Du;
         h ^= h >> 12;
         z[i] = 1.0 + static_cast<double>(h & 0xffff) * (1.0 / 65536.0);
     }
-    __syncwarp();
-    if (lane == 0) {
+    __syncthreads();
+    if (tid == 0) {
+        // row i of U: (pivot, u1, u2); `cur`, `sup` are the reduced row i
+        double cur = udg[0], sup = e[0];
+        int anyp = 0;
         for (int i = 0; i + 1 < p; ++i) {
-            if (fabs(udg[i]) >= fabs(lmul[i])) {
-                if (udg[i] == 0.0) udg[i] = tiny;
-                const double inv = rcp64(udg[i]);
+            const double sub = e[i], nd = udg[i + 1], ns = e[i + 1];
+            // |cur| >= |sub| by the high words: at most 2^-20 off an exact comparison
+            if ((__double2hiint(cur) & 0x7fffffff) >= (__double2hiint(sub) & 0x7fffffff)) {
+                if ((__double2hiint(cur) & 0x7fffffff) == 0 && __double2loint(cur) == 0) cur = tiny;
+                const double inv = rcp64(cur);
+                const double f = sub * inv;
+                cur = fma(-f, sup, nd);
                 invd[i] = inv;
-                const double fct = lmul[i] * inv;
-                lmul[i] = fct;
-                udg[i + 1] = fma(-fct, u1[i], udg[i + 1]);
+                lmul[i] = f;
+                u1[i] = sup;
+                u2[i] = 0.0;
+                piv[i] = 0;
+                sup = ns;
             } else {
-                const double inv = rcp64(lmul[i]);
+                const double inv = rcp64(sub);
+                const double f = cur * inv;
+                cur = fma(-f, nd, sup);
                 invd[i] = inv;
-                const double fct = udg[i] * inv;
-                udg[i] = lmul[i];
-                lmul[i] = fct;
-                const double tmp = u1[i];
-                u1[i] = udg[i + 1];
-                udg[i + 1] = fma(-fct, udg[i + 1], tmp);
-                if (i + 2 < p) {
-                    u2[i] = u1[i + 1];
-                    u1[i + 1] = -fct * u1[i + 1];
-                }
+                lmul[i] = f;
+                u1[i] = nd;
+                u2[i] = ns;
                 piv[i] = 1;
+                anyp = 1;
+                sup = -f * ns;
             }
         }
-        if (udg[p - 1] == 0.0) udg[p - 1] = tiny;
-        invd[p - 1] = rcp64(udg[p - 1]);
+        if ((__double2hiint(cur) & 0x7fffffff) == 0 && __double2loint(cur) == 0) cur = tiny;
+        invd[p - 1] = rcp64(cur);
+        u1[p - 1] = u2[p - 1] = 0.0;
+        flags[0] = anyp;
+        flags[1] = 0;
+    }
+    __syncthreads();
+    const bool anyp = flags[0] != 0;
+    for (int i = tid; i < p; i += kEigThreads) {
+        u1[i] *= invd[i];
+        u2[i] *= invd[i];
     }
     for (int itr = 0; itr < 2; ++itr) {
-        if (lane == 0) {
+        __syncthreads();
+        if (tid == 0) {
+            double cur = z[0];
+#pragma unroll 4
             for (int i = 0; i + 1 < p; ++i) {
-                if (piv[i] == 0) {
-                    z[i + 1] = fma(-lmul[i], z[i], z[i + 1]);
-                } else {
-                    const double tmp = z[i];
-                    z[i] = z[i + 1];
-                    z[i + 1] = fma(-lmul[i], z[i], tmp);
+                const double zn = z[i + 1];
+                const bool sw = piv[i] != 0;
+                const double top = sw ? zn : cur, bot = sw ? cur : zn;
+                z[i] = top;
+                cur = fma(-lmul[i], top, bot);
+            }
+            z[p - 1] = cur;
+        }
+        __syncthreads();
+        for (int i = tid; i < p; i += kEigThreads) z[i] *= invd[i];
+        __syncthreads();
+        if (tid == 0) {
+            double n1 = z[p - 1], n2 = 0.0;
+            if (anyp) {
+#pragma unroll 4
+                for (int i = p - 2; i >= 0; --i) {
+                    const double t = fma(-u1[i], n1, fma(-u2[i], n2, z[i]));
+                    z[i] = t;
+                    n2 = n1;
+                    n1 = t;
+                }
+            } else {
+#pragma unroll 4
+                for (int i = p - 2; i >= 0; --i) {
+                    n1 = fma(-u1[i], n1, z[i]);
+                    z[i] = n1;
                 }
             }
-            z[p - 1] *= invd[p - 1];
-            if (p > 1) z[p - 2] = fma(-u1[p - 2], z[p - 1], z[p - 2]) * invd[p - 2];
-            for (int i = p - 3; i >= 0; --i) z[i] = fma(-u2[i], z[i + 2], fma(-u1[i], z[i + 1], z[i])) * invd[i];
         }
-        __syncwarp();
-        double s0 = 0.0;
-        for (int i = lane; i < p; i += 32) s0 = fma(z[i], z[i], s0);
-        const double nrm2 = warp_sum(s0);
-        if (!(nrm2 > 0.0) || !isfinite(nrm2)) {
-            if (lane == 0) record_status(status, CDMD_ERR_NOT_CONVERGED);
-            break;
+        __syncthreads();
+        if (itr == 0) {
+            // to around 1, by a power of two
+            int top = 0;
+            for (int i = tid; i < p; i += kEigThreads) top = max(top, (__double2hiint(z[i]) >> 20) & 0x7ff);
+            top = __reduce_max_sync(0xffffffffu, top);
+            if (lane == 0) atomicMax(&flags[1], top);
+            __syncthreads();
+            top = min(max(flags[1], 1), 2045);
+            const double sc = __hiloint2double((2046 - top) << 20, 0);
+            for (int i = tid; i < p; i += kEigThreads) z[i] *= sc;
         }
-        const double inv = rsqrt64(nrm2);
-        for (int i = lane; i < p; i += 32) z[i] *= inv;
-        __syncwarp();
     }
-    for (int i = lane; i < p; i += 32) Z[static_cast<int64_t>(w) * p + i] = z[i];
+    double s0 = 0.0;
+    for (int i = tid; i < p; i += kEigThreads) s0 = fma(z[i], z[i], s0);
+    s0 = warp_sum(s0);
+    if (lane == 0) red[wid] = s0;
+    __syncthreads();
+    const double nrm2 = (red[0] + red[1]) + (red[2] + red[3]);
+    if (!(nrm2 > 0.0) || !isfinite(nrm2)) {
+        if (tid == 0) record_status(status, CDMD_ERR_NOT_CONVERGED);
+        for (int i = tid; i < p; i += kEigThreads) Z[i] = z[i];
+        return;
+    }
+    const double inv = rsqrt64(nrm2);
+    for (int i = tid; i < p; i += kEigThreads) Z[i] = z[i] * inv;
+}
+
+// Reflectors j0 .. j0 + NB - 1 as one block I - V T V^T (compact WY form,
+// Schreiber and Van Loan): T is the inverse of the upper triangular matrix
+// with 1 / tau_j on its diagonal and v_i . v_j above it.  One CTA of four
+// warps per block, beside the eigenpairs, which take several times as long.
+template <int NB>
+__device__ void wy_cta(const SolveClip& q, int blk, double* tsm) {
+    const int p = q.p;
+    const int j0 = blk * NB;
+    double* S = tsm;                 // NB x NB: v_i . v_j (i < j)
+    double* Ts = S + NB * NB;        // NB x NB
+    double* Vb = Ts + NB * NB;       // NB x p
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    for (int idx = tid; idx < NB * p; idx += kEigThreads) {
+        const int b = idx / p, l = idx % p, j = j0 + b;
+        Vb[idx] = (j + 2 < p && l > j) ? q.Hv[static_cast<int64_t>(j) * p + l] : 0.0;
+    }
+    __syncthreads();
+    // four products v_i . v_j .. v_i . v_{j+3} per warp and turn
+    for (int g = wid; g < NB * (NB / 4); g += 4) {
+        const int i = g / (NB / 4), jb = 4 * (g % (NB / 4));
+        if (jb + 3 <= i) continue;
+        const double* vi = Vb + static_cast<size_t>(i) * p;
+        const double* vj = Vb + static_cast<size_t>(jb) * p;
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+        for (int l = j0 + 1 + lane; l < p; l += 32) {
+            const double x = vi[l];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[e] = fma(x, vj[static_cast<size_t>(e) * p + l], s[e]);
+        }
+        __syncwarp();
+        const double t = warp_sum4(s);
+        if ((lane & 7) == 0) S[i * NB + jb + (lane >> 3)] = t;
+    }
+    __syncthreads();
+    // row q of T from the rows below it: T_q. = tau_q (e_q - sum_{u > q} S_qu T_u.)
+    // right-looking: row u, once known, is added into the sums of the rows above
+    const bool col = lane < NB;
+    double acc[NB / 4];
+#pragma unroll
+    for (int a = 0; a < NB / 4; ++a) acc[a] = 0.0;
+#pragma unroll
+    for (int u = NB - 1; u >= 0; --u) {
+        if ((u & 3) == wid) {
+            const int j = j0 + u;
+            const double tau = (j + 2 < p) ? q.htau[j] : 0.0;
+            const double t = lane > u ? -tau * acc[u >> 2] : lane == u ? tau : 0.0;
+            if (col) Ts[u * NB + lane] = t;
+        }
+        __syncthreads();
+        if (u > 0) {
+            const double t = col ? Ts[u * NB + lane] : 0.0;
+#pragma unroll
+            for (int a = 0; a < NB / 4; ++a)
+                if (4 * a < u) acc[a] = fma((4 * a + wid < u) ? S[(4 * a + wid) * NB + u] : 0.0, t, acc[a]);
+        }
+    }
+    // transposed: the back-transform's lanes run over rows
+    double* T = q.Tw + static_cast<size_t>(blk) * NB * NB;
+    for (int idx = tid; idx < NB * NB; idx += kEigThreads) T[idx] = Ts[(idx % NB) * NB + idx / NB];
+}
+
+// blockIdx.x < r: eigenpair blockIdx.x; above: block blockIdx.x - r of reflectors
+template <int NB>
+__global__ void __launch_bounds__(kEigThreads)
+tridiag_eigpair_kernel(const __grid_constant__ SolveBatch sb) {
+    extern __shared__ double tsm[];
+    const SolveClip& q = sb.c[blockIdx.z];
+    const int b = static_cast<int>(blockIdx.x);
+    if (b == 0 && threadIdx.x == 0) q.flag[1] = 0;      // set by orthogonality_kernel
+    if (b < sb.r) eigpair_cta(q, b, sb.status, tsm);
+    else if ((b - sb.r) * NB + 2 < q.p) wy_cta<NB>(q, b - sb.r, tsm);
 }
 
 // ---------------------------------------------------------------------------
@@ -611,6 +847,8 @@ tridiag_eigpair_kernel(const __grid_constant__ SolveBatch sb) {
 // largest by multisection on Sturm counts, sets tau = omega * median and
 // counts the eigenvalues above tau^2 with one more Sturm count.
 // ---------------------------------------------------------------------------
+constexpr int kShifts = 64;   // shifts tested per multisection pass (two per lane)
+
 __device__ double kth_eigenvalue(const double* d, const double* e2, int p, int idx, double lo, double hi, double tn,
                                  int* status) {
     const int lane = threadIdx.x & 31;
@@ -678,48 +916,101 @@ gd_rank_kernel(const double* __restrict__ dd, const double* __restrict__ ee, int
     }
 }
 
-// 4a. Classical Gram-Schmidt over the r columns of Z (descending eigenvalue
-// order), applied twice: the dots of a column with all earlier columns are
-// taken in parallel (one warp each).  Z is not __restrict__: threads read
-// entries other threads wrote, ordered by __syncthreads.
-__global__ void __launch_bounds__(1024)
-orthonormalise_kernel(const __grid_constant__ SolveBatch sb) {
-    double* Z = sb.c[blockIdx.z].Z;
-    const int p = sb.c[blockIdx.z].p, r = sb.r;
-    // classical Gram-Schmidt, twice, on the r columns held in shared memory
-    extern __shared__ double osm[];
-    double* Zs = osm;                         // r columns of p
-    double* dots = Zs + static_cast<size_t>(r) * p;   // 32
-    double* red = dots + 32;                  // 32
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < r * p; i += blockDim.x) Zs[i] = Z[i];
+// 4a. The eigenvectors of T come out of the inverse iteration orthogonal to
+// about eps / gap, so one first-order step of Gram-Schmidt,
+//   z_c <- z_c - sum_{q < c} (z_q . z_c) z_q,
+// leaves an error of the square of the largest product.  Every column needs
+// only the original ones: one CTA per column, no chain over columns.  Products
+// above kOrthTol (a cluster of eigenvalues) raise flag[1], and the
+// back-transform then runs classical Gram-Schmidt, twice, instead.
+constexpr double kOrthTol = 1e-9;
+constexpr int kOrthThreads = 256;
+
+__global__ void __launch_bounds__(kOrthThreads)
+orthogonality_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& q = sb.c[blockIdx.z];
+    const int p = q.p, c = blockIdx.x;
+    __shared__ double dots[kMaxR];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const double* Z = q.Z;
+    const double* zc = Z + static_cast<int64_t>(c) * p;
+    // products with columns 4 wid .. 4 wid + 3 (r <= 32)
+    const int q0 = 4 * wid;
+    if (q0 < c) {
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+        const double* zq[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) zq[e] = Z + static_cast<int64_t>(min(q0 + e, c)) * p;
+#pragma unroll 1
+        for (int i = lane; i < p; i += 32) {
+            const double x = zc[i];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[e] = fma(zq[e][i], x, s[e]);
+        }
+        __syncwarp();
+        const double t = warp_sum4(s);
+        const int col = q0 + (lane >> 3);
+        if ((lane & 7) == 0 && col < c) {
+            dots[col] = t;
+            if (!(fabs(t) <= kOrthTol)) q.flag[1] = 1;
+        }
+    }
     __syncthreads();
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int c = 0; c < r; ++c) {
-            double* zc = Zs + static_cast<size_t>(c) * p;
-            if (wid < c) {
-                const double* zq = Zs + static_cast<size_t>(wid) * p;
-                double s0 = 0.0, s1 = 0.0;
-                int i = lane;
-                for (; i + 32 < p; i += 64) {
-                    s0 = fma(zq[i], zc[i], s0);
-                    s1 = fma(zq[i + 32], zc[i + 32], s1);
+    double* out = q.B + static_cast<int64_t>(c) * p;      // B's space: written again by bmat after the back-transform
+#pragma unroll 1
+    for (int i = tid; i < p; i += kOrthThreads) {
+        double a = zc[i];
+#pragma unroll 4
+        for (int u = 0; u < c; ++u) a = fma(-dots[u], Z[static_cast<int64_t>(u) * p + i], a);
+        out[i] = a;
+    }
+}
+
+// Columns 0 .. c_last of Z, a cluster among them, to orthonormal eigenvectors
+// in shared memory (descending eigenvalue order); every column's CTA repeats
+// the earlier ones.  The cluster's vectors come nearly parallel out of the
+// inverse iteration, and classical Gram-Schmidt, twice, amplifies their
+// rounding errors outside the cluster's space; one product with T damps those
+// (by the ratio of the eigenvalues, all of them below the cluster's), and
+// Gram-Schmidt makes the columns orthonormal again.
+__device__ void gram_schmidt_cta(const SolveClip& q, int c_last, double* Zs, double* dots, double* red) {
+    const int p = q.p;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int i = threadIdx.x; i < (c_last + 1) * p; i += blockDim.x) Zs[i] = q.Z[i];
+    __syncthreads();
+    for (int pass = 0; pass < 4; ++pass) {
+        if (pass == 2) {
+            for (int c = 0; c <= c_last; ++c) {
+                double* z = Zs + static_cast<size_t>(c) * p;
+                double t[2] = {0.0, 0.0};            // p < 512 = 2 kOrthThreads
+                for (int u = 0; u < 2; ++u) {
+                    const int i = threadIdx.x + u * kOrthThreads;
+                    if (i < p) {
+                        t[u] = q.dd[i] * z[i];
+                        if (i > 0) t[u] = fma(q.ee[i - 1], z[i - 1], t[u]);
+                        if (i + 1 < p) t[u] = fma(q.ee[i], z[i + 1], t[u]);
+                    }
                 }
-                if (i < p) s0 = fma(zq[i], zc[i], s0);
-                const double s = warp_sum(s0 + s1);
-                if (lane == 0) dots[wid] = s;
+                __syncthreads();
+                for (int u = 0; u < 2; ++u)
+                    if (threadIdx.x + u * kOrthThreads < p) z[threadIdx.x + u * kOrthThreads] = t[u];
+            }
+            __syncthreads();
+        }
+        for (int c = 0; c <= c_last; ++c) {
+            double* zc = Zs + static_cast<size_t>(c) * p;
+            for (int u = wid; u < c; u += nw) {
+                const double* zq = Zs + static_cast<size_t>(u) * p;
+                double s = 0.0;
+                for (int i = lane; i < p; i += 32) s = fma(zq[i], zc[i], s);
+                s = warp_sum(s);
+                if (lane == 0) dots[u] = s;
             }
             __syncthreads();
             double nacc = 0.0;
             for (int i = threadIdx.x; i < p; i += blockDim.x) {
-                double a0 = zc[i], a1 = 0.0;
-                int q = 0;
-                for (; q + 1 < c; q += 2) {
-                    a0 = fma(-dots[q], Zs[static_cast<size_t>(q) * p + i], a0);
-                    a1 = fma(-dots[q + 1], Zs[static_cast<size_t>(q + 1) * p + i], a1);
-                }
-                if (q < c) a0 = fma(-dots[q], Zs[static_cast<size_t>(q) * p + i], a0);
-                const double a = a0 + a1;
+                double a = zc[i];
+                for (int u = 0; u < c; ++u) a = fma(-dots[u], Zs[static_cast<size_t>(u) * p + i], a);
                 zc[i] = a;
                 nacc = fma(a, a, nacc);
             }
@@ -729,74 +1020,107 @@ orthonormalise_kernel(const __grid_constant__ SolveBatch sb) {
             __syncthreads();
         }
     }
-    for (int i = threadIdx.x; i < r * p; i += blockDim.x) Z[i] = Zs[i];
 }
 
-// 4b. V[:, c] = Q z_c (apply H_{p-3}, ..., H_0) and sigma_c = sqrt(lambda_c);
-// one CTA (one warp) per column, four partial sums per lane.  Each lane
-// holds its entries of the next reflector in registers, loaded one step
-// ahead, so the L2 latency of the reflector rows is off the critical path.
-// kBtPer: reflector entries per lane, 8 for p <= 256 and 16 up to p = 511
-template <int kBtPer>
-__global__ void __launch_bounds__(32)
-backtransform_kernel(const __grid_constant__ SolveBatch sb) {
-    const SolveClip& clip = sb.c[blockIdx.z];
-    const double *Z = clip.Z, *Hv = clip.Hv, *htau = clip.htau, *lam = clip.lamT;
-    const int p = clip.p;
-    double *V = clip.V, *sigma = clip.sigma;
-    int* status = sb.status;
-    extern __shared__ double ysm[];   // p
-    const int c = blockIdx.x;
-    const int lane = threadIdx.x;
-    for (int i = lane; i < p; i += 32) ysm[i] = Z[static_cast<int64_t>(c) * p + i];
-    __syncwarp();
-    // entry q of lane: index lane + 32 q of the reflector row
-    double cur[kBtPer], nxt[kBtPer];
-    double tau_cur = 0.0, tau_nxt = 0.0;
-    int j = p - 3;
-    if (j >= 0) {
-        tau_cur = htau[j];
-#pragma unroll
-        for (int q = 0; q < kBtPer; ++q) {
-            const int l = lane + 32 * q;
-            cur[q] = (l > j && l < p) ? Hv[static_cast<int64_t>(j) * p + l] : 0.0;
+// 4b. V[:, c] = Q z_c and sigma_c = sqrt(lambda_c), one CTA per column: the
+// reflectors are applied NB at a time, last block first, as I - V T V^T (three
+// products with a barrier between them, where one reflector at a time is a
+// chain of p reductions).  The next block's rows are copied to the other
+// buffer (cp.async) while the present one is applied.
+template <int NB>
+__device__ __forceinline__ void load_reflectors(const double* Hv, int p, int j0, double* buf) {
+    for (int idx = threadIdx.x; idx < NB * p; idx += kOrthThreads) {
+        const int b = idx / p, l = idx % p, j = j0 + b;
+        double* dst = buf + idx;
+        if (j + 2 < p && l > j) {
+            const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(s), "l"(Hv + static_cast<int64_t>(j) * p + l)
+                         : "memory");
+        } else {
+            *dst = 0.0;
         }
     }
-    for (; j >= 0; --j) {
-        if (j > 0) {
-            tau_nxt = htau[j - 1];
-#pragma unroll
-            for (int q = 0; q < kBtPer; ++q) {
-                const int l = lane + 32 * q;
-                nxt[q] = (l > j - 1 && l < p) ? Hv[static_cast<int64_t>(j - 1) * p + l] : 0.0;
-            }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+template <int NB>
+__global__ void __launch_bounds__(kOrthThreads)
+backtransform_kernel(const __grid_constant__ SolveBatch sb) {
+    constexpr int kWarps = kOrthThreads / 32;
+    static_assert(NB % kWarps == 0 && NB <= 32, "rows per warp");
+    const SolveClip& clip = sb.c[blockIdx.z];
+    const int p = clip.p, c = blockIdx.x;
+    extern __shared__ double ysm[];
+    double* y = ysm;                              // p
+    double* buf0 = y + p;                         // 2 x NB x p
+    double* buf1 = buf0 + static_cast<size_t>(NB) * p;
+    __shared__ double Ts[NB * NB];
+    __shared__ double dots[32], xs[32], red[32], red4[4][NB];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int nblk = p > 2 ? (p - 2 + NB - 1) / NB : 0;
+    if (clip.flag[1] != 0) {
+        gram_schmidt_cta(clip, c, buf0, dots, red);     // c + 1 <= 2 NB columns fit the two buffers
+        for (int i = tid; i < p; i += kOrthThreads) y[i] = buf0[static_cast<size_t>(c) * p + i];
+        __syncthreads();
+    } else {
+        const double* zc = clip.B + static_cast<int64_t>(c) * p;
+        for (int i = tid; i < p; i += kOrthThreads) y[i] = zc[i];
+    }
+    if (nblk > 0) load_reflectors<NB>(clip.Hv, p, (nblk - 1) * NB, ((nblk - 1) & 1) ? buf1 : buf0);
+    for (int b = nblk - 1; b >= 0; --b) {
+        const double* Vb = (b & 1) ? buf1 : buf0;
+        const int j0 = b * NB;
+        const double* T = clip.Tw + static_cast<size_t>(b) * NB * NB;
+        for (int i = tid; i < NB * NB; i += kOrthThreads) Ts[i] = T[i];
+        if (b > 0) {
+            load_reflectors<NB>(clip.Hv, p, (b - 1) * NB, ((b - 1) & 1) ? buf1 : buf0);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
-        if (tau_cur != 0.0) {
-            double s0 = 0.0, s1 = 0.0;
+        __syncthreads();
+        // V^T y: NB / 8 rows per warp
+        {
+            constexpr int kR = NB / kWarps;
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            const double* row = Vb + static_cast<size_t>(wid) * kR * p;
+#pragma unroll 1
+            for (int l = j0 + 1 + lane; l < p; l += 32) {
+                const double x = y[l];
 #pragma unroll
-            for (int q = 0; q < kBtPer; q += 2) {
-                const int l0 = lane + 32 * q, l1 = l0 + 32;
-                if (l0 < p) s0 = fma(cur[q], ysm[l0], s0);
-                if (l1 < p) s1 = fma(cur[q + 1], ysm[l1], s1);
-            }
-            const double s = warp_sum(s0 + s1) * tau_cur;
-#pragma unroll
-            for (int q = 0; q < kBtPer; ++q) {
-                const int l = lane + 32 * q;
-                if (l > j && l < p) ysm[l] = fma(-s, cur[q], ysm[l]);
+                for (int e = 0; e < kR; ++e) s[e] = fma(row[static_cast<size_t>(e) * p + l], x, s[e]);
             }
             __syncwarp();
+            const double t = warp_sum4(s);
+            if ((lane & 7) == 0 && (lane >> 3) < kR) dots[wid * kR + (lane >> 3)] = t;
         }
+        __syncthreads();
+        // T (V^T y): four warps take a quarter of the columns each
+        if (wid < 4 && lane < NB) {
+            double t = 0.0;
 #pragma unroll
-        for (int q = 0; q < kBtPer; ++q) cur[q] = nxt[q];
-        tau_cur = tau_nxt;
+            for (int u = 0; u < NB / 4; ++u) t = fma(Ts[(wid * (NB / 4) + u) * NB + lane], dots[wid * (NB / 4) + u], t);
+            red4[wid][lane] = t;
+        }
+        __syncthreads();
+        if (tid < NB) xs[tid] = (red4[0][tid] + red4[1][tid]) + (red4[2][tid] + red4[3][tid]);
+        __syncthreads();
+#pragma unroll 1
+        for (int l = j0 + 1 + tid; l < p; l += kOrthThreads) {
+            double a = y[l];
+#pragma unroll
+            for (int u = 0; u < NB; ++u) a = fma(-xs[u], Vb[static_cast<size_t>(u) * p + l], a);
+            y[l] = a;
+        }
+        __syncthreads();
     }
-    for (int i = lane; i < p; i += 32) V[static_cast<int64_t>(c) * p + i] = ysm[i];
-    if (lane == 0) {
-        const double l0 = lam[0];
-        const double lc = lam[c];
-        if (!(lc > kRankTol * static_cast<double>(p) * kEps * fabs(l0))) record_status(status, CDMD_ERR_RANK_DEFICIENT);
-        sigma[c] = lc > 0.0 ? lc * rsqrt64(lc) : 0.0;
+    for (int i = tid; i < p; i += kOrthThreads) clip.V[static_cast<int64_t>(c) * p + i] = y[i];
+    if (tid == 0) {
+        const double l0 = clip.lamT[0];
+        const double lc = clip.lamT[c];
+        if (!(lc > kRankTol * static_cast<double>(p) * kEps * fabs(l0)))
+            record_status(sb.status, CDMD_ERR_RANK_DEFICIENT);
+        clip.sigma[c] = lc > 0.0 ? lc * rsqrt64(lc) : 0.0;
     }
 }
 
@@ -1830,8 +2154,8 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
     int nmax = 0;
     for (int i = 0; i < nclips; ++i) {
         const size_t n = io[i].n, p = n - 1, rr = r;
-        const size_t total = static_cast<size_t>(splits) * n * n + n * n + p * p + 3 * p + rr + 3 * p * rr +
-                             10 * rr * rr + 6 * rr + 64;
+        const size_t total = static_cast<size_t>(splits) * n * n + n * n + p * p + 32 * p + 1024 + 3 * p + rr +
+                             3 * p * rr + 10 * rr * rr + 6 * rr + 64;
         // + one slot for the eigen-solver's fallback flag and two for the rank
         // threshold's result; with an automatic rank, r is its upper bound here
         off[i + 1] = off[i] + total + 3;
@@ -1874,7 +2198,8 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
         q.R = io[i].R != nullptr ? io[i].R : q.Rw;
         q.Hv = q.Rw + static_cast<size_t>(q.n) * q.n;
         q.htau = q.Hv + static_cast<size_t>(q.p) * q.p;
-        q.dd = q.htau + q.p;
+        q.Tw = q.htau + q.p;                         // ceil((p - 2) / NB) blocks of NB x NB, NB = 16 or 32
+        q.dd = q.Tw + 32 * static_cast<size_t>(q.p) + 1024;
         q.ee = q.dd + q.p;
         q.lamT = q.ee + q.p;
         q.flag = reinterpret_cast<int*>(ws + off[i + 1] - 3);   // written by eig_f32_kernel before any read
@@ -1976,27 +2301,27 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
         if (autor->tau_host != nullptr) *autor->tau_host = ht;
         lay_out(r);
     }
-    // 3. eigenpairs of T, orthonormalisation, back-transform
+    // 3. eigenpairs of T and, beside them, the reflectors' block factors; one
+    // step of orthogonalisation; back-transform.  Blocks of 32 reflectors while
+    // two of them fit the shared memory (p <= 256), else 16
+    const bool wide = p <= 256;
     {
-        const size_t esm = 10 * static_cast<size_t>(p) * sizeof(double);
-        CDMD_CHECK_CUDA(cudaFuncSetAttribute(tridiag_eigpair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(kMaxOptInSmem)));
-        tridiag_eigpair_kernel<<<dim3(r, 1, nc), 32, esm, stream>>>(sb);
+        const int nb = wide ? 32 : 16;
+        const int nblk = p > 2 ? (p - 2 + nb - 1) / nb : 0;
+        const size_t esm = std::max(84 * static_cast<size_t>(p),
+                                    (2 * nb + static_cast<size_t>(p)) * nb * sizeof(double));
+        const size_t bsm = (2 * nb + 1) * static_cast<size_t>(p) * sizeof(double);
+        void (*ek)(SolveBatch) = wide ? tridiag_eigpair_kernel<32> : tridiag_eigpair_kernel<16>;
+        void (*bk)(SolveBatch) = wide ? backtransform_kernel<32> : backtransform_kernel<16>;
+        for (auto kern : {ek, bk})
+            CDMD_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
+        ek<<<dim3(r + nblk, 1, nc), kEigThreads, esm, stream>>>(sb);
         CDMD_CHECK_LAUNCH("tridiag_eigpair_kernel");
+        orthogonality_kernel<<<dim3(r, 1, nc), kOrthThreads, 0, stream>>>(sb);
+        CDMD_CHECK_LAUNCH("orthogonality_kernel");
+        bk<<<dim3(r, 1, nc), kOrthThreads, bsm, stream>>>(sb);
+        CDMD_CHECK_LAUNCH("backtransform_kernel");
     }
-    {
-        const size_t osm = (static_cast<size_t>(r) * p + 64) * sizeof(double);
-        CDMD_CHECK_CUDA(cudaFuncSetAttribute(orthonormalise_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(kMaxOptInSmem)));
-        orthonormalise_kernel<<<dim3(1, 1, nc), 1024, osm, stream>>>(sb);
-    }
-    CDMD_CHECK_LAUNCH("orthonormalise_kernel");
-    static_assert(32 * 16 >= 511, "the back-transform covers p = n - 1 <= 511 (n <= 512)");
-    if (p <= 256)
-        backtransform_kernel<8><<<dim3(r, 1, nc), 32, p * sizeof(double), stream>>>(sb);
-    else
-        backtransform_kernel<16><<<dim3(r, 1, nc), 32, p * sizeof(double), stream>>>(sb);
-    CDMD_CHECK_LAUNCH("backtransform_kernel");
     // 4. A~ and its eigen-decomposition
     bmat_kernel<<<dim3((p + 7) / 8, r, nc), 256, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("bmat_kernel");
