@@ -1183,7 +1183,7 @@ atilde_kernel(const __grid_constant__ SolveBatch sb) {
 //     positive; eigenvalues ordered by descending modulus, conjugate pairs
 //     adjacent with the positive imaginary part first.
 // ---------------------------------------------------------------------------
-struct cf {
+struct alignas(8) cf {
     float x, y;
 };
 __device__ __forceinline__ cf fmulc(cf a, cf b) { return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
@@ -1191,16 +1191,20 @@ __device__ __forceinline__ cf faddc(cf a, cf b) { return {a.x + b.x, a.y + b.y};
 __device__ __forceinline__ cf fsubc(cf a, cf b) { return {a.x - b.x, a.y - b.y}; }
 __device__ __forceinline__ cf fconjc(cf a) { return {a.x, -a.y}; }
 __device__ __forceinline__ float fabs2c(cf a) { return a.x * a.x + a.y * a.y; }
-__device__ __forceinline__ float fabsc(cf a) { return hypotf(a.x, a.y); }
-__device__ __forceinline__ cf fdivc(cf a, cf b) {
-    const float s = fabsf(b.x) + fabsf(b.y);
-    const cf as = {a.x / s, a.y / s}, bs = {b.x / s, b.y / s};
-    const float den = bs.x * bs.x + bs.y * bs.y;
-    return {(as.x * bs.x + as.y * bs.y) / den, (as.y * bs.x - as.x * bs.y) / den};
+__device__ __forceinline__ float fabs1c(cf a) { return fabsf(a.x) + fabsf(a.y); }
+__device__ __forceinline__ cf finvc(cf a) {   // 1 / a, scaled so that the squares neither overflow nor vanish
+    const float s = fabs1c(a);
+    const float is = 1.0f / s;
+    const cf b = {a.x * is, a.y * is};
+    const float den = is / fabs2c(b);
+    return {b.x * den, -b.y * den};
 }
 __device__ __forceinline__ cf fsqrtc(cf a) {
-    const float m = fabsc(a);
-    if (m == 0.0f) return {0.0f, 0.0f};
+    const float s = fabs1c(a);
+    if (s == 0.0f) return {0.0f, 0.0f};
+    const float is = 1.0f / s;
+    const cf b = {a.x * is, a.y * is};
+    const float m = s * sqrtf(fabs2c(b));
     float re = sqrtf(0.5f * (m + fabsf(a.x)));
     float im = 0.5f * a.y / re;
     if (a.x < 0.0f) {
@@ -1210,220 +1214,231 @@ __device__ __forceinline__ cf fsqrtc(cf a) {
     }
     return {re, im};
 }
+__device__ __forceinline__ cf shfl_cf(cf v, int src) {
+    return {__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src)};
+}
 
-__global__ void __launch_bounds__(32)
+constexpr int kEig32Threads = 128;
+
+// Four warps; warp 0 runs the serial parts (Hessenberg reduction and QR
+// iteration), all four the products with the eigenvectors.  Latency-bound:
+// the reduction keeps a column (then a row) of H per lane in registers, and a
+// rotation's successor takes its two entries by shuffle from the lanes that
+// have just computed them, not through shared memory.  Square roots and
+// divisions on the rotation chain are one approximate reciprocal square root:
+// the result only starts the FP64 Newton iteration of 6b.
+__global__ void __launch_bounds__(kEig32Threads)
 eig_f32_kernel(const __grid_constant__ SolveBatch sb) {
     const SolveClip& clip = sb.c[blockIdx.z];
     const double* At = clip.At;
     const int r = sb.r;
-    float2 *lam32 = clip.lam32, *W32 = clip.W32;
-    int* fallback = clip.flag;
     __shared__ float Hr[kMaxR][kMaxR + 1];
     __shared__ float Q[kMaxR][kMaxR + 1];
     __shared__ cf T[kMaxR][kMaxR + 1];
     __shared__ cf Zs[kMaxR][kMaxR + 1];
     __shared__ cf X[kMaxR][kMaxR + 1];
     __shared__ float hv[kMaxR];
-    const int lane = threadIdx.x;
-    for (int idx = lane; idx < r * r; idx += 32) {
-        const int i = idx % r, c = idx / r;
-        Hr[i][c] = static_cast<float>(At[static_cast<int64_t>(c) * r + i]);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    for (int idx = tid; idx < kMaxR * kMaxR; idx += kEig32Threads) {
+        const int i = idx % kMaxR, c = idx / kMaxR;
+        Hr[i][c] = (i < r && c < r) ? static_cast<float>(At[static_cast<int64_t>(c) * r + i]) : 0.0f;
         Q[i][c] = (i == c) ? 1.0f : 0.0f;
-    }
-    __syncwarp();
-    for (int j = 0; j + 2 < r; ++j) {
-        const float hj = (lane > j && lane < r) ? Hr[lane][j] : 0.0f;
-        float nrm2 = hj * hj;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) nrm2 += __shfl_xor_sync(0xffffffffu, nrm2, o);
-        const float nrm = sqrtf(nrm2);
-        const float x0 = Hr[j + 1][j];
-        const float v0 = x0 + (x0 >= 0.0f ? nrm : -nrm);
-        // ||v||^2 = v0^2 + (nrm^2 - x0^2)
-        const float vn = fmaf(v0, v0, fmaxf(nrm2 - x0 * x0, 0.0f));
-        const float beta = (nrm > 0.0f && vn > 0.0f) ? 2.0f / vn : 0.0f;
-        __syncwarp();
-        if (lane > j && lane < r) hv[lane] = (lane == j + 1) ? v0 : hj;
-        __syncwarp();
-        if (beta != 0.0f) {
-            if (lane < r) {
-                float s = 0.0f;
-                for (int i = j + 1; i < r; ++i) s += hv[i] * Hr[i][lane];
-                s *= beta;
-                for (int i = j + 1; i < r; ++i) Hr[i][lane] -= s * hv[i];
-            }
-            __syncwarp();
-            if (lane < r) {
-                float s = 0.0f, sq = 0.0f;
-                for (int c = j + 1; c < r; ++c) {
-                    s += Hr[lane][c] * hv[c];
-                    sq += Q[lane][c] * hv[c];
-                }
-                s *= beta;
-                sq *= beta;
-                for (int c = j + 1; c < r; ++c) {
-                    Hr[lane][c] -= s * hv[c];
-                    Q[lane][c] -= sq * hv[c];
-                }
-            }
-            __syncwarp();
-            if (lane >= j + 2 && lane < r) Hr[lane][j] = 0.0f;
-        }
-        __syncwarp();
-    }
-    for (int idx = lane; idx < r * r; idx += 32) {
-        const int i = idx % r, c = idx / r;
-        T[i][c] = {Hr[i][c], 0.0f};
         Zs[i][c] = {(i == c) ? 1.0f : 0.0f, 0.0f};
     }
-    __syncwarp();
-    const float eps32 = 1.1920929e-07f;
-    int hi = r - 1, its = 0, total = 0;
-    bool failed = false;
-    while (hi > 0) {
-        // deflation: the largest lo <= hi with a negligible T[lo][lo-1] (or 0)
-        bool small = false;
-        if (lane >= 1 && lane <= hi) {
-            const float sc = fabsc(T[lane - 1][lane - 1]) + fabsc(T[lane][lane]);
-            small = fabsc(T[lane][lane - 1]) <= eps32 * sc;
+    __syncthreads();
+    if (wid == 0) {
+        float qr[kMaxR];                       // row `lane` of Q
+#pragma unroll
+        for (int c = 0; c < kMaxR; ++c) qr[c] = (c == lane) ? 1.0f : 0.0f;
+        for (int j = 0; j + 2 < r; ++j) {
+            const float hj = (lane > j) ? Hr[lane][j] : 0.0f;
+            float nrm2 = hj * hj;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) nrm2 += __shfl_xor_sync(0xffffffffu, nrm2, o);
+            const float nrm = sqrtf(nrm2);
+            const float x0 = __shfl_sync(0xffffffffu, hj, j + 1);
+            const float v0 = x0 + (x0 >= 0.0f ? nrm : -nrm);
+            // ||v||^2 = v0^2 + (nrm^2 - x0^2)
+            const float vn = fmaf(v0, v0, fmaxf(nrm2 - x0 * x0, 0.0f));
+            const float beta = (nrm > 0.0f && vn > 0.0f) ? 2.0f / vn : 0.0f;
+            hv[lane] = (lane == j + 1) ? v0 : hj;          // zero up to j and past r
+            __syncwarp();
+            if (beta != 0.0f) {
+                float h[kMaxR], v[kMaxR];
+                float s0 = 0.0f, s1 = 0.0f;
+#pragma unroll
+                for (int i = 0; i < kMaxR; i += 2) {       // column `lane` of H
+                    v[i] = hv[i];
+                    v[i + 1] = hv[i + 1];
+                    h[i] = Hr[i][lane];
+                    h[i + 1] = Hr[i + 1][lane];
+                    s0 = fmaf(v[i], h[i], s0);
+                    s1 = fmaf(v[i + 1], h[i + 1], s1);
+                }
+                const float s = (s0 + s1) * beta;
+#pragma unroll
+                for (int i = 0; i < kMaxR; ++i) Hr[i][lane] = fmaf(-s, v[i], h[i]);
+                __syncwarp();
+                float t0 = 0.0f, t1 = 0.0f, u0 = 0.0f, u1 = 0.0f;
+#pragma unroll
+                for (int c = 0; c < kMaxR; c += 2) {       // row `lane` of H and of Q
+                    h[c] = Hr[lane][c];
+                    h[c + 1] = Hr[lane][c + 1];
+                    t0 = fmaf(h[c], v[c], t0);
+                    t1 = fmaf(h[c + 1], v[c + 1], t1);
+                    u0 = fmaf(qr[c], v[c], u0);
+                    u1 = fmaf(qr[c + 1], v[c + 1], u1);
+                }
+                const float t = (t0 + t1) * beta, u = (u0 + u1) * beta;
+#pragma unroll
+                for (int c = 0; c < kMaxR; ++c) {
+                    Hr[lane][c] = (c == j && lane >= j + 2) ? 0.0f : fmaf(-t, v[c], h[c]);
+                    qr[c] = fmaf(-u, v[c], qr[c]);
+                }
+            }
+            __syncwarp();
         }
-        const unsigned sm_mask = __ballot_sync(0xffffffffu, small);
-        const int lo = sm_mask ? 31 - __clz(sm_mask) : 0;
-        if (lo > 0 && lane == 0) T[lo][lo - 1] = {0.0f, 0.0f};
+#pragma unroll
+        for (int c = 0; c < kMaxR; ++c) {
+            Q[lane][c] = qr[c];
+            T[lane][c] = {Hr[lane][c], 0.0f};
+        }
         __syncwarp();
-        if (lo == hi) { --hi; its = 0; continue; }
-        ++its;
-        ++total;
-        if (its > 60 || total > 60 * r) { failed = true; break; }
-        cf mu;
-        {
-            const cf a = T[hi - 1][hi - 1], b = T[hi - 1][hi], c = T[hi][hi - 1], dv = T[hi][hi];
-            if (its % 11 == 0) {
-                mu = {dv.x + fabsc(c), dv.y};
-            } else {
-                const cf half = {0.5f * (a.x - dv.x), 0.5f * (a.y - dv.y)};
-                const cf bc = fmulc(b, c);
-                const cf disc = fsqrtc(faddc(fmulc(half, half), bc));
-                const cf s1 = faddc(half, disc), s2 = fsubc(half, disc);
-                cf mu1 = dv, mu2 = dv;
-                if (fabs2c(s1) > 0.0f) mu1 = fsubc(dv, fdivc(bc, s1));
-                if (fabs2c(s2) > 0.0f) mu2 = fsubc(dv, fdivc(bc, s2));
-                mu = (fabs2c(fsubc(mu1, dv)) <= fabs2c(fsubc(mu2, dv))) ? mu1 : mu2;
-            }
-        }
-        // bulge chase: rotation q acts on rows q, q+1 (lanes = columns), then
-        // on columns q, q+1 (lanes = rows) and on Z; the entry T[q+1][q-1]
-        // the row rotation zeroes is written 0 by its lane
-        for (int q = lo; q < hi; ++q) {
-            cf x, y;
-            if (q == lo) { x = fsubc(T[lo][lo], mu); y = T[lo + 1][lo]; }
-            else { x = T[q][q - 1]; y = T[q + 1][q - 1]; }
-            const float rr = sqrtf(fabs2c(x) + fabs2c(y));
-            cf cg_ = {1.0f, 0.0f}, sg = {0.0f, 0.0f};
-            if (rr > 0.0f) {
-                const float inv = 1.0f / rr;
-                cg_ = {x.x * inv, x.y * inv};
-                sg = {y.x * inv, y.y * inv};
-            }
+        const float eps32 = 1.1920929e-07f;
+        int hi = r - 1, its = 0, total = 0;
+        bool failed = false;
+        while (hi > 0) {
+            // deflation: the largest lo <= hi with a negligible T[lo][lo-1] (or 0)
+            bool small = false;
+            if (lane >= 1 && lane <= hi)
+                small = fabs1c(T[lane][lane - 1]) <= eps32 * (fabs1c(T[lane - 1][lane - 1]) + fabs1c(T[lane][lane]));
+            const unsigned sm_mask = __ballot_sync(0xffffffffu, small);
+            const int lo = sm_mask ? 31 - __clz(sm_mask) : 0;
+            if (lo > 0 && lane == 0) T[lo][lo - 1] = {0.0f, 0.0f};
             __syncwarp();
-            const int col0 = max(q - 1, 0);
-            if (lane >= col0 && lane < r) {
-                const cf t0 = T[q][lane], t1 = T[q + 1][lane];
-                T[q][lane] = faddc(fmulc(fconjc(cg_), t0), fmulc(fconjc(sg), t1));
-                T[q + 1][lane] = (q > lo && lane == q - 1) ? cf{0.0f, 0.0f} : fsubc(fmulc(cg_, t1), fmulc(sg, t0));
+            if (lo == hi) { --hi; its = 0; continue; }
+            ++its;
+            ++total;
+            if (its > 60 || total > 60 * r) { failed = true; break; }
+            cf mu;
+            {
+                const cf a = T[hi - 1][hi - 1], b = T[hi - 1][hi], c = T[hi][hi - 1], dv = T[hi][hi];
+                if (its % 11 == 0) {
+                    mu = {dv.x + fabs1c(c), dv.y};
+                } else {
+                    // Wilkinson: the eigenvalue of the last 2 x 2 block nearer to dv
+                    const cf half = {0.5f * (a.x - dv.x), 0.5f * (a.y - dv.y)};
+                    const cf bc = fmulc(b, c);
+                    const cf disc = fsqrtc(faddc(fmulc(half, half), bc));
+                    const cf s1 = faddc(half, disc), s2 = fsubc(half, disc);
+                    const cf s = fabs2c(s1) >= fabs2c(s2) ? s1 : s2;
+                    mu = fabs2c(s) > 0.0f ? fsubc(dv, fmulc(bc, finvc(s))) : dv;
+                }
             }
-            __syncwarp();
-            const int row1 = min(q + 3, hi + 1);
-            if (lane < r) {
+            // bulge chase: rotation q acts on rows q, q+1 (lanes = columns), then
+            // on columns q, q+1 (lanes = rows) and on Z; the entry T[q+1][q-1]
+            // the row rotation zeroes is written 0 by its lane
+            cf x = fsubc(T[lo][lo], mu), y = T[lo + 1][lo];
+            for (int q = lo; q < hi; ++q) {
+                const int row1 = min(q + 3, hi + 1);
+                const cf a0 = T[q][lane], a1 = T[q + 1][lane];
+                const cf z0 = Zs[lane][q], z1 = Zs[lane][q + 1];
+                const float n2 = fabs2c(x) + fabs2c(y);
+                cf cg_ = {1.0f, 0.0f}, sg = {0.0f, 0.0f};
+                if (n2 > 1e-36f) {
+                    const float inv = rsqrtf(n2);
+                    cg_ = {x.x * inv, x.y * inv};
+                    sg = {y.x * inv, y.y * inv};
+                }
+                if (lane >= max(q - 1, 0)) {
+                    T[q][lane] = faddc(fmulc(fconjc(cg_), a0), fmulc(fconjc(sg), a1));
+                    T[q + 1][lane] =
+                        (q > lo && lane == q - 1) ? cf{0.0f, 0.0f} : fsubc(fmulc(cg_, a1), fmulc(sg, a0));
+                }
+                __syncwarp();
+                cf b0 = {0.0f, 0.0f};
                 if (lane < row1) {
                     const cf t0 = T[lane][q], t1 = T[lane][q + 1];
-                    T[lane][q] = faddc(fmulc(t0, cg_), fmulc(t1, sg));
+                    b0 = faddc(fmulc(t0, cg_), fmulc(t1, sg));
+                    T[lane][q] = b0;
                     T[lane][q + 1] = fsubc(fmulc(t1, fconjc(cg_)), fmulc(t0, fconjc(sg)));
                 }
-                const cf z0 = Zs[lane][q], z1 = Zs[lane][q + 1];
                 Zs[lane][q] = faddc(fmulc(z0, cg_), fmulc(z1, sg));
                 Zs[lane][q + 1] = fsubc(fmulc(z1, fconjc(cg_)), fmulc(z0, fconjc(sg)));
+                // the next rotation zeroes T[q+2][q] against T[q+1][q]
+                x = shfl_cf(b0, q + 1);
+                y = shfl_cf(b0, min(q + 2, 31));
+                __syncwarp();
             }
-            __syncwarp();
         }
-    }
-    // a failed FP32 iteration hands the whole problem to the FP64 QR fallback
-    if (lane == 0) *fallback = failed ? 1 : 0;
-    __syncwarp();
-    float tmax = 0.0f;
-    for (int i = 0; i < r; ++i)
-        for (int c = i; c < r; ++c) tmax = fmaxf(tmax, fabsc(T[i][c]));
-    const float small = eps32 * fmaxf(tmax, 1e-30f);
-    if (lane < r) {
-        const int j = lane;
-        for (int i = 0; i < r; ++i) X[i][j] = {i == j ? 1.0f : 0.0f, 0.0f};
-        for (int i = j - 1; i >= 0; --i) {
-            cf s = {0.0f, 0.0f};
-            for (int q = i + 1; q <= j; ++q) s = faddc(s, fmulc(T[i][q], X[q][j]));
-            cf den = fsubc(T[i][i], T[j][j]);
-            if (fabsc(den) < small) den = {small, 0.0f};
-            const cf v = fdivc(s, den);
-            X[i][j] = {-v.x, -v.y};
-        }
-    }
-    __syncwarp();
-    if (lane < r) {
-        const int j = lane;
-        cf tmp[kMaxR];
-        for (int i = 0; i < r; ++i) {
-            cf s = {0.0f, 0.0f};
-            for (int q = 0; q <= j; ++q) s = faddc(s, fmulc(Zs[i][q], X[q][j]));
-            tmp[i] = s;
-        }
-        for (int i = 0; i < r; ++i) {
-            float re = 0.0f, im = 0.0f;
-            for (int q = 0; q < r; ++q) {
-                re += Q[i][q] * tmp[q].x;
-                im += Q[i][q] * tmp[q].y;
+        // a failed FP32 iteration hands the whole problem to the FP64 QR fallback
+        if (lane == 0) clip.flag[0] = failed ? 1 : 0;
+        __syncwarp();
+        float tmax = 0.0f;
+        for (int i = 0; i <= lane && lane < r; ++i) tmax = fmaxf(tmax, fabs1c(T[i][lane]));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+        const float small = eps32 * fmaxf(tmax, 1e-30f);
+        // eigenvector `lane` of the triangular T, right-looking: entry q, once
+        // known, is taken into the sums of the rows above (kept in registers)
+        cf s[kMaxR];
+        const cf tjj = T[lane][lane];
+#pragma unroll
+        for (int i = 0; i < kMaxR; ++i) s[i] = {0.0f, 0.0f};
+#pragma unroll
+        for (int q = kMaxR - 1; q >= 0; --q) {
+            if (q < r) {
+                cf den = fsubc(T[q][q], tjj);
+                if (!(fabs1c(den) >= small)) den = {small, 0.0f};
+                const cf v = fmulc(s[q], finvc(den));
+                const cf xq = q == lane ? cf{1.0f, 0.0f} : q < lane ? cf{-v.x, -v.y} : cf{0.0f, 0.0f};
+                X[q][lane] = xq;
+#pragma unroll
+                for (int i = 0; i < q; ++i) s[i] = faddc(s[i], fmulc(T[i][q], xq));
+            } else {
+                X[q][lane] = {0.0f, 0.0f};
             }
-            W32[static_cast<int64_t>(j) * r + i] = make_float2(re, im);
         }
-        lam32[j] = make_float2(T[j][j].x, T[j][j].y);
+        if (lane < r) clip.lam32[lane] = make_float2(tjj.x, tjj.y);
+    }
+    __syncthreads();
+    // W = Q (Z X), column `lane`, rows dealt to the warps; Z X into T's place
+    {
+        cf x[kMaxR];
+#pragma unroll
+        for (int u = 0; u < kMaxR; ++u) x[u] = X[u][lane];
+        for (int i = wid; i < r; i += kEig32Threads / 32) {
+            cf a = {0.0f, 0.0f}, b = {0.0f, 0.0f};
+#pragma unroll
+            for (int u = 0; u < kMaxR; u += 2) {
+                a = faddc(a, fmulc(Zs[i][u], x[u]));
+                b = faddc(b, fmulc(Zs[i][u + 1], x[u + 1]));
+            }
+            T[i][lane] = faddc(a, b);
+        }
+        __syncthreads();
+        if (lane < r) {
+            for (int i = wid; i < r; i += kEig32Threads / 32) {
+                float re = 0.0f, im = 0.0f;
+                for (int u = 0; u < r; ++u) {
+                    re = fmaf(Q[i][u], T[u][lane].x, re);
+                    im = fmaf(Q[i][u], T[u][lane].y, im);
+                }
+                clip.W32[static_cast<int64_t>(lane) * r + i] = make_float2(re, im);
+            }
+        }
     }
 }
 
-__global__ void __launch_bounds__(32)
-eig_refine_kernel(const __grid_constant__ SolveBatch sb) {
-    const SolveClip& clip = sb.c[blockIdx.z];
-    const double* At = clip.At;
-    const int r = sb.r;
-    const float2 *lam32 = clip.lam32, *W32 = clip.W32;
-    double *lamR = clip.lamR, *WR = clip.WR;
-    int* fallback = clip.flag;
-    __shared__ double A[kMaxR][kMaxR + 1];
+// Newton's method of 6b with one FP64 elimination per step (one warp); w
+// (shared memory) and mu are updated in place, done says whether it settled.
+__device__ void eig_newton_fp64(const double (*A)[kMaxR + 1], int r, int pidx, cd& mu, cd* wv, bool& done) {
     __shared__ cd Mx[kMaxR][kMaxR + 1];
-    __shared__ cd wv[kMaxR];
     __shared__ cd rhs[kMaxR];
     __shared__ cd zz[kMaxR];
     __shared__ int perm[kMaxR];
-    const int j = blockIdx.x;
-    const int lane = threadIdx.x;
-    for (int idx = lane; idx < r * r; idx += 32) {
-        const int i = idx % r, c = idx / r;
-        A[i][c] = At[static_cast<int64_t>(c) * r + i];
-    }
-    cd mu = {static_cast<double>(lam32[j].x), static_cast<double>(lam32[j].y)};
-    cd w = {0.0, 0.0};
-    if (lane < r) {
-        const float2 v = W32[static_cast<int64_t>(j) * r + lane];
-        w = {static_cast<double>(v.x), static_cast<double>(v.y)};
-    }
-    // hold the largest entry of w at 1
-    double key = (lane < r) ? cabs2(w) : -1.0;
-    const double kmax = warp_max(key);
-    const unsigned at = __ballot_sync(0xffffffffu, key == kmax && lane < r);
-    const int pidx = at ? __ffs(at) - 1 : 0;   // no candidate only with non-finite entries
-    const cd wp = shfl_cd(w, pidx);
-    if (kmax > 0.0) w = cmul(w, cinv(wp));
-    if (lane == pidx) w = {1.0, 0.0};
-    if (lane < r) wv[lane] = w;
-    __syncwarp();
-    bool done = false;
+    const int lane = threadIdx.x & 31;
+    done = false;
     for (int it = 0; it < 4 && !done; ++it) {
         // residual and the bordered matrix: column pidx replaced by -w
         if (lane < r) {
@@ -1493,9 +1508,179 @@ eig_refine_kernel(const __grid_constant__ SolveBatch sb) {
         done = (cabs2(dmu) <= 1e-28 * cabs2(mu)) && (dw <= 1e-26) && it > 0;
         __syncwarp();
     }
-    // no quadratic convergence (a cluster or a nearly defective pair): the
-    // FP64 QR fallback recomputes every eigenpair
-    if (!done && lane == 0) atomicExch(fallback, 1);
+}
+
+constexpr int kRefThreads = 128;
+constexpr int kRefSteps = 8;      // refinement steps with the FP32 inverse before the FP64 elimination takes over
+
+// 6b. Eigenpair j: Newton's method on (A~ - mu I) w = 0 with the largest entry
+// of w held at 1, i.e. the bordered system whose column pidx is -w.
+// Fast path: the bordered matrix at the FP32 start is inverted once in FP32
+// (Gauss-Jordan, partial pivoting), and each step takes the residual in FP64
+// and the correction from that inverse: the error falls by the inverse's
+// relative error (about 1e-7 times the condition number) per step, to the same
+// fixed point.  A step costs the FP64 residual, a quarter of the columns per
+// warp, instead of an elimination (a DP instruction holds a scheduler 64
+// clocks).  A pair that has not settled in kRefSteps goes on with one FP64
+// elimination per Newton step, from the FP32 start; one that does not settle
+// there either raises the fallback flag.
+__global__ void __launch_bounds__(kRefThreads)
+eig_refine_kernel(const __grid_constant__ SolveBatch sb) {
+    const SolveClip& clip = sb.c[blockIdx.z];
+    const double* At = clip.At;
+    const int r = sb.r;
+    const float2 *lam32 = clip.lam32, *W32 = clip.W32;
+    double *lamR = clip.lamR, *WR = clip.WR;
+    __shared__ double A[kMaxR][kMaxR + 1];
+    __shared__ cf M[kMaxR][kMaxR + 1];       // bordered matrix, then its inverse
+    __shared__ cd wv[kMaxR], part[4][kMaxR];
+    __shared__ cf rowk[kMaxR], resf[kMaxR];
+    __shared__ int perm[kMaxR];
+    __shared__ int state;                    // 0: go on, 1: settled, 2: gave up
+    const int j = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    for (int idx = tid; idx < r * r; idx += kRefThreads) {
+        const int i = idx % r, c = idx / r;
+        A[i][c] = At[static_cast<int64_t>(c) * r + i];
+    }
+    cd mu = {static_cast<double>(lam32[j].x), static_cast<double>(lam32[j].y)};
+    const cf muf = {lam32[j].x, lam32[j].y};
+    // hold the largest entry of w at 1 (every warp finds the same)
+    cf wf = {0.0f, 0.0f};
+    if (lane < r) {
+        const float2 v = W32[static_cast<int64_t>(j) * r + lane];
+        wf = {v.x, v.y};
+    }
+    const float key = (lane < r) ? fabs2c(wf) : -1.0f;
+    float kmax = key;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) kmax = fmaxf(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
+    const unsigned at = __ballot_sync(0xffffffffu, key == kmax && lane < r);
+    const int pidx = at ? __ffs(at) - 1 : 0;   // no candidate only with non-finite entries
+    const cf wp = shfl_cf(wf, pidx);
+    if (kmax > 0.0f) wf = fmulc(wf, finvc(wp));
+    if (lane == pidx) wf = {1.0f, 0.0f};
+    if (lane < r && wid == 0) wv[lane] = {static_cast<double>(wf.x), static_cast<double>(wf.y)};
+    if (tid == 0) state = 0;
+    __syncthreads();
+    // FP32 inverse, warp 0: lane i holds row i in registers; step k scales the
+    // pivot row, passes it round through shared memory and clears column k
+    if (wid == 0) {
+        cf m[kMaxR];
+#pragma unroll
+        for (int c = 0; c < kMaxR; ++c) {
+            cf v = {lane == c ? 1.0f : 0.0f, 0.0f};      // identity past r
+            if (lane < r && c < r) {
+                v = {static_cast<float>(A[lane][c]), 0.0f};
+                if (c == lane) v = fsubc(v, muf);
+                if (c == pidx) v = {-wf.x, -wf.y};
+            }
+            m[c] = v;
+        }
+        bool used = lane >= r;
+        int mine = lane;                                  // the step this row was pivot of
+#pragma unroll
+        for (int k = 0; k < kMaxR; ++k) {
+            if (k < r) {
+                float mag = used ? -1.0f : fabs2c(m[k]);
+                float best = mag;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
+                const unsigned bb = __ballot_sync(0xffffffffu, !used && mag == best);
+                // no candidate only with non-finite entries: any unused row, the steps then do not settle
+                const int piv = bb ? __ffs(bb) - 1 : __ffs(__ballot_sync(0xffffffffu, !used)) - 1;
+                if (lane == piv) {
+                    used = true;
+                    mine = k;
+                    const cf inv = finvc(m[k]);
+                    m[k] = {1.0f, 0.0f};
+#pragma unroll
+                    for (int c = 0; c < kMaxR; ++c) {
+                        m[c] = fmulc(m[c], inv);
+                        rowk[c] = m[c];
+                    }
+                }
+                __syncwarp();
+                if (lane != piv) {
+                    const cf f = m[k];
+                    m[k] = {0.0f, 0.0f};
+#pragma unroll
+                    for (int c = 0; c < kMaxR; ++c) m[c] = fsubc(m[c], fmulc(f, rowk[c]));
+                }
+                __syncwarp();
+            }
+        }
+        // row `piv of step k` holds row k of P-permuted inverse: inverse[mine][piv of c] = m[c]
+        perm[mine] = lane;
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < kMaxR; ++c) M[mine][perm[c]] = m[c];
+    }
+    __syncthreads();
+    float dw_prev = 0.0f;
+    for (int it = 0; it < kRefSteps; ++it) {
+        // residual (A~ - mu) w: the warps share the columns
+        if (lane < r) {
+            double re = 0.0, im = 0.0;
+#pragma unroll 1
+            for (int c = wid; c < r; c += 4) {
+                re = fma(A[lane][c], wv[c].x, re);
+                im = fma(A[lane][c], wv[c].y, im);
+            }
+            part[wid][lane] = {re, im};
+        }
+        __syncthreads();
+        if (wid == 0) {
+            cd w = {0.0, 0.0};
+            if (lane < r) {
+                w = wv[lane];
+                const cd a = part[0][lane], b = part[1][lane], c = part[2][lane], d = part[3][lane];
+                const double re = fma(-mu.x, w.x, fma(mu.y, w.y, (a.x + b.x) + (c.x + d.x)));
+                const double im = fma(-mu.x, w.y, fma(-mu.y, w.x, (a.y + b.y) + (c.y + d.y)));
+                resf[lane] = {static_cast<float>(-re), static_cast<float>(-im)};
+            }
+            __syncwarp();
+            cf z = {0.0f, 0.0f};
+            if (lane < r) {
+                cf z1 = {0.0f, 0.0f};
+                int c = 0;
+                for (; c + 1 < r; c += 2) {
+                    z = faddc(z, fmulc(M[lane][c], resf[c]));
+                    z1 = faddc(z1, fmulc(M[lane][c + 1], resf[c + 1]));
+                }
+                if (c < r) z = faddc(z, fmulc(M[lane][c], resf[c]));
+                z = faddc(z, z1);
+            }
+            const cf dmu = shfl_cf(z, pidx);
+            mu = {mu.x + static_cast<double>(dmu.x), mu.y + static_cast<double>(dmu.y)};
+            float dw = 0.0f;
+            if (lane < r && lane != pidx) {
+                wv[lane] = {w.x + static_cast<double>(z.x), w.y + static_cast<double>(z.y)};
+                dw = fabs1c(z);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) dw = fmaxf(dw, __shfl_xor_sync(0xffffffffu, dw, o));
+            // settled: the last correction is at rounding level and the steps contract
+            const float am = static_cast<float>(fabs(mu.x) + fabs(mu.y));
+            if (lane == 0 && it > 0 && fabs1c(dmu) <= 1e-14f * am && dw <= 1e-13f &&
+                (dw <= 0.03f * dw_prev || dw <= 2e-15f))
+                state = 1;
+            dw_prev = dw;
+        }
+        __syncthreads();
+        if (state != 0) break;
+    }
+    if (wid != 0) return;
+    if (state != 1) {
+        mu = {static_cast<double>(muf.x), static_cast<double>(muf.y)};
+        if (lane < r) wv[lane] = {static_cast<double>(wf.x), static_cast<double>(wf.y)};
+        __syncwarp();
+        bool done = false;
+        eig_newton_fp64(A, r, pidx, mu, wv, done);
+        // no quadratic convergence (a cluster or a nearly defective pair): the
+        // FP64 QR fallback recomputes every eigenpair
+        if (!done && lane == 0) atomicExch(clip.flag, 1);
+    }
     if (lane == 0) {
         lamR[2 * j] = mu.x;
         lamR[2 * j + 1] = mu.y;
@@ -1533,16 +1718,13 @@ __device__ __forceinline__ cd csqrt_(cd a) {
     return {re, im};
 }
 
-constexpr int kQrThreads = 64;
+constexpr int kQrThreads = 128;
 constexpr size_t kQrSmem = 2 * kMaxR * (kMaxR + 1) * sizeof(double) + 3 * kMaxR * (kMaxR + 1) * sizeof(cd);
 
-__global__ void __launch_bounds__(kQrThreads)
-eig_qr64_kernel(const __grid_constant__ SolveBatch sb) {
-    const SolveClip& clip = sb.c[blockIdx.z];
+__device__ void eig_qr64_cta(const SolveClip& clip, int r, int* status) {
     const double* At = clip.At;
-    const int r = sb.r;
     double *lamR = clip.lamR, *WR = clip.WR;
-    int *fallback = clip.flag, *status = sb.status;
+    int* fallback = clip.flag;
     extern __shared__ double qsm[];
     typedef double RowD[kMaxR + 1];
     typedef cd RowC[kMaxR + 1];
@@ -1557,15 +1739,19 @@ eig_qr64_kernel(const __grid_constant__ SolveBatch sb) {
     __shared__ int flag[2];
     const int tid = threadIdx.x;
     const int nt = blockDim.x;
-    if (tid == 0) {
-        int go = *fallback;
-        for (int i = 0; i < r && !go; ++i)
-            for (int q = i + 1; q < r && !go; ++q) {
-                const cd li = {lamR[2 * i], lamR[2 * i + 1]}, lq = {lamR[2 * q], lamR[2 * q + 1]};
-                const double tol = 1e-8 * fmax(1.0, cabsd(li));
-                if (!(cabs2(csub(li, lq)) > tol * tol)) go = 1;   // coincident (or NaN) eigenvalues
-            }
-        flag[1] = go;
+    if (tid == 0) flag[1] = *fallback;
+    __syncthreads();
+    if (tid < r) {
+        const cd li = {lamR[2 * tid], lamR[2 * tid + 1]};
+        const float lx = static_cast<float>(li.x), ly = static_cast<float>(li.y);
+        const float far = 1e-5f * fmaxf(1.0f, fabsf(lx) + fabsf(ly));
+        for (int u = tid + 1; u < r; ++u) {
+            const cd lq = {lamR[2 * u], lamR[2 * u + 1]};
+            // well apart in FP32: no need to look closer (a NaN looks closer)
+            if (fabsf(static_cast<float>(lq.x) - lx) + fabsf(static_cast<float>(lq.y) - ly) > far) continue;
+            const double tol = 1e-8 * fmax(1.0, cabsd(li));
+            if (!(cabs2(csub(li, lq)) > tol * tol)) flag[1] = 1;   // coincident (or NaN) eigenvalues
+        }
     }
     __syncthreads();
     if (!flag[1]) return;
@@ -1740,92 +1926,124 @@ eig_qr64_kernel(const __grid_constant__ SolveBatch sb) {
     if (tid == 0) *fallback = 0;
 }
 
-__global__ void __launch_bounds__(32)
-eig_order_kernel(const __grid_constant__ SolveBatch sb) {
-    const SolveClip& clip = sb.c[blockIdx.z];
-    const double *lamR = clip.lamR, *WR = clip.WR;
-    const int r = sb.r;
-    double *lam_out = clip.lambda, *W_out = clip.W;
+// Unsigned 64-bit keys in the order of doubles (-0 and +0 alike).
+__device__ __forceinline__ unsigned long long order_key(double x) {
+    const long long b = __double_as_longlong(x + 0.0);
+    return static_cast<unsigned long long>(b) ^ (static_cast<unsigned long long>(b >> 63) | 0x8000000000000000ull);
+}
+// Lane that holds the largest (`least`: smallest) key among the lanes with
+// `in` (at least one), the lowest such lane.
+__device__ __forceinline__ int warp_pick(unsigned long long key, bool in, bool least) {
+    const unsigned hi = static_cast<unsigned>(key >> 32), lo = static_cast<unsigned>(key);
+    const unsigned fh = least ? ~hi : hi, fl = least ? ~lo : lo;
+    const unsigned bh = __reduce_max_sync(0xffffffffu, in ? fh : 0u);
+    const bool top = in && fh == bh;
+    const unsigned bl = __reduce_max_sync(0xffffffffu, top ? fl : 0u);
+    return __ffs(__ballot_sync(0xffffffffu, top && fl == bl)) - 1;
+}
+
+// 6c. Order and normalisation (all threads of the CTA): descending modulus,
+// conjugate pairs adjacent with the positive imaginary part first; unit
+// 2-norm, largest-modulus entry real positive.  Warp 0 pairs the eigenvalues
+// (the positive imaginary parts in descending order, each with the nearest
+// unused eigenvalue to its conjugate) and ranks them by integer keys; the
+// eigenvectors go through shared memory (Ws: r x 33 complex), a lane per
+// column and a quarter of the entries per warp.
+__device__ void eig_order_cta(const double* lamR, const double* WR, int r, double* lam_out, double* W_out, cd* Ws) {
+    constexpr int kLd = kMaxR + 1, kPart = kMaxR / (kQrThreads / 32);
     __shared__ int order[kMaxR];
-    const int lane = threadIdx.x;
-    if (lane == 0) {
-        bool used[kMaxR];
-        double key_abs[kMaxR], key_im[kMaxR];
-        int first[kMaxR], second[kMaxR];
-        int nu = 0;
-        for (int i = 0; i < r; ++i) used[i] = false;
-        for (int pass = 0; pass < r; ++pass) {
-            int i = -1;
-            for (int q = 0; q < r; ++q)
-                if (!used[q] && (i < 0 || lamR[2 * q + 1] > lamR[2 * i + 1])) i = q;
-            if (i < 0) break;
-            used[i] = true;
-            const cd li = {lamR[2 * i], lamR[2 * i + 1]};
-            int partner = -1;
-            if (li.y > 0.0) {
-                double bd = 1e300;
-                for (int q = 0; q < r; ++q) {
-                    if (used[q]) continue;
-                    const cd lq = {lamR[2 * q], lamR[2 * q + 1]};
-                    const double d2 = cabs2(csub(lq, cconj(li)));
-                    if (d2 < bd) { bd = d2; partner = q; }
-                }
-                const double tol = 1e-9 * fmax(1.0, sqrt(cabs2(li)));
-                if (partner >= 0 && !(bd <= tol * tol)) partner = -1;
-                if (partner >= 0) used[partner] = true;
+    __shared__ double n2s[4][kMaxR], bests[4][kMaxR];
+    __shared__ int bis[4][kMaxR];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    for (int idx = tid; idx < r * r; idx += kQrThreads)
+        Ws[(idx / r) * kLd + idx % r] = {WR[2 * idx], WR[2 * idx + 1]};
+    if (wid == 0) {
+        const bool live = lane < r;
+        const cd li = live ? cd{lamR[2 * lane], lamR[2 * lane + 1]} : cd{0.0, 0.0};
+        const unsigned long long kim = order_key(li.y), kabs = order_key(cabs2(li));
+        const unsigned long long zero = order_key(0.0);
+        bool used = !live, second = false;
+        int partner = -1;
+        for (;;) {
+            const bool in = !used && kim > zero;
+            if (!__any_sync(0xffffffffu, in)) break;
+            const int i = warp_pick(kim, in, false);
+            if (lane == i) used = true;
+            const cd l = shfl_cd(li, i);
+            const double d2 = cabs2(csub(li, cconj(l)));
+            if (!__any_sync(0xffffffffu, !used)) break;
+            const int m = warp_pick(order_key(d2), !used, true);
+            const double bd = __shfl_sync(0xffffffffu, d2, m);
+            const double tol = 1e-9 * fmax(1.0, sqrt(cabs2(l)));
+            if (bd <= tol * tol) {
+                if (lane == m) { used = true; second = true; partner = i; }
+                if (lane == i) partner = m;
             }
-            key_abs[nu] = cabs2(li);
-            key_im[nu] = li.y;
-            first[nu] = i;
-            second[nu] = partner;
-            ++nu;
         }
-        int perm[kMaxR];
-        for (int u = 0; u < nu; ++u) perm[u] = u;
-        for (int u = 1; u < nu; ++u) {
-            const int cur = perm[u];
-            int v = u - 1;
-            while (v >= 0) {
-                const int o = perm[v];
-                const bool before = (key_abs[cur] > key_abs[o]) || (key_abs[cur] == key_abs[o] && key_im[cur] > key_im[o]);
-                if (!before) break;
-                perm[v + 1] = perm[v];
-                --v;
-            }
-            perm[v + 1] = cur;
-        }
+        // position of every head: the heads before it and their partners
         int pos = 0;
-        for (int u = 0; u < nu; ++u) {
-            order[pos++] = first[perm[u]];
-            if (second[perm[u]] >= 0) order[pos++] = second[perm[u]];
+        for (int u = 0; u < r; ++u) {
+            const unsigned long long ua = __shfl_sync(0xffffffffu, kabs, u), ui = __shfl_sync(0xffffffffu, kim, u);
+            const int up = __shfl_sync(0xffffffffu, partner, u);
+            const bool us = __shfl_sync(0xffffffffu, static_cast<int>(second), u) != 0;
+            if (!us && (ua > kabs || (ua == kabs && (ui > kim || (ui == kim && u < lane))))) pos += up >= 0 ? 2 : 1;
+        }
+        const int head_pos = __shfl_sync(0xffffffffu, pos, partner >= 0 ? partner : lane);
+        if (second) pos = head_pos + 1;
+        if (live) {
+            order[pos] = lane;
+            lam_out[2 * pos] = li.x;
+            lam_out[2 * pos + 1] = li.y;
         }
     }
-    __syncwarp();
+    __syncthreads();
+    const int s = lane < r ? order[lane] : 0;
+    double n2 = 0.0, best = -1.0;
+    int bi = 0;
     if (lane < r) {
-        const int s = order[lane];
-        lam_out[2 * lane] = lamR[2 * s];
-        lam_out[2 * lane + 1] = lamR[2 * s + 1];
-        // unit 2-norm, largest-modulus entry real positive
-        double n2 = 0.0, best = -1.0;
-        int bi = 0;
-        for (int i = 0; i < r; ++i) {
-            const cd v = {WR[2 * (static_cast<int64_t>(s) * r + i)], WR[2 * (static_cast<int64_t>(s) * r + i) + 1]};
-            const double a2 = cabs2(v);
+#pragma unroll 1
+        for (int i = wid * kPart; i < min(r, (wid + 1) * kPart); ++i) {
+            const double a2 = cabs2(Ws[s * kLd + i]);
             n2 += a2;
-            if (a2 > best) { best = a2; bi = i; }
+            if (__double_as_longlong(a2) > __double_as_longlong(best)) { best = a2; bi = i; }   // a2 >= 0
         }
-        const cd vb = {WR[2 * (static_cast<int64_t>(s) * r + bi)], WR[2 * (static_cast<int64_t>(s) * r + bi) + 1]};
+        n2s[wid][lane] = n2;
+        bests[wid][lane] = best;
+        bis[wid][lane] = bi;
+    }
+    __syncthreads();
+    if (lane < r) {
+        n2 = (n2s[0][lane] + n2s[1][lane]) + (n2s[2][lane] + n2s[3][lane]);
+        best = -1.0;
+        bi = 0;
+        for (int w = 0; w < 4; ++w)
+            if (__double_as_longlong(bests[w][lane]) > __double_as_longlong(best)) {
+                best = bests[w][lane];
+                bi = bis[w][lane];
+            }
+        const cd vb = Ws[s * kLd + bi];
         const double inv_b = best > 0.0 ? rsqrt64(best) : 0.0;
         const double inv_n = n2 > 0.0 ? rsqrt64(n2) : 0.0;
-        const cd ph = {vb.x * inv_b * inv_n, -vb.y * inv_b * inv_n};   // conj(v_b)/|v_b| / ||v||
-        for (int i = 0; i < r; ++i) {
-            const cd v = {WR[2 * (static_cast<int64_t>(s) * r + i)], WR[2 * (static_cast<int64_t>(s) * r + i) + 1]};
-            cd o = cmul(v, ph);
+        const double inv = inv_b * inv_n;
+        const cd ph = {vb.x * inv, -vb.y * inv};   // conj(v_b)/|v_b| / ||v||
+#pragma unroll 1
+        for (int i = wid * kPart; i < min(r, (wid + 1) * kPart); ++i) {
+            cd o = cmul(Ws[s * kLd + i], ph);
             if (i == bi) o.y = 0.0;
             W_out[2 * (static_cast<int64_t>(lane) * r + i)] = o.x;
             W_out[2 * (static_cast<int64_t>(lane) * r + i) + 1] = o.y;
         }
     }
+}
+
+// The FP64 fallback where it is needed, then 6c; one CTA per clip.
+__global__ void __launch_bounds__(kQrThreads)
+eig_finish_kernel(const __grid_constant__ SolveBatch sb) {
+    extern __shared__ double qsm[];
+    const SolveClip& clip = sb.c[blockIdx.z];
+    eig_qr64_cta(clip, sb.r, sb.status);
+    __syncthreads();
+    eig_order_cta(clip.lamR, clip.WR, sb.r, clip.lambda, clip.W, reinterpret_cast<cd*>(qsm));
 }
 
 // 7. G[t][c] = sum_a V[t][a] / sigma_a * W[a][c]   (column-major complex)
@@ -2327,16 +2545,14 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
     CDMD_CHECK_LAUNCH("bmat_kernel");
     atilde_kernel<<<dim3(r, 1, nc), 32, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("atilde_kernel");
-    eig_f32_kernel<<<dim3(1, 1, nc), 32, 0, stream>>>(sb);
+    eig_f32_kernel<<<dim3(1, 1, nc), kEig32Threads, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("eig_f32_kernel");
-    eig_refine_kernel<<<dim3(r, 1, nc), 32, 0, stream>>>(sb);
+    eig_refine_kernel<<<dim3(r, 1, nc), kRefThreads, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("eig_refine_kernel");
-    CDMD_CHECK_CUDA(cudaFuncSetAttribute(eig_qr64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    CDMD_CHECK_CUDA(cudaFuncSetAttribute(eig_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(kQrSmem)));
-    eig_qr64_kernel<<<dim3(1, 1, nc), kQrThreads, kQrSmem, stream>>>(sb);
-    CDMD_CHECK_LAUNCH("eig_qr64_kernel");
-    eig_order_kernel<<<dim3(1, 1, nc), 32, 0, stream>>>(sb);
-    CDMD_CHECK_LAUNCH("eig_order_kernel");
+    eig_finish_kernel<<<dim3(1, 1, nc), kQrThreads, kQrSmem, stream>>>(sb);
+    CDMD_CHECK_LAUNCH("eig_finish_kernel");
     // 5. G, Gram-form quantities, selection
     gmat_kernel<<<dim3((p * r + 127) / 128, 1, nc), 128, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("gmat_kernel");
