@@ -234,18 +234,14 @@ namespace cdmd {
 constexpr int kMaxSolveClips = 8;   // clips whose small solves run side by side (cdmd_run_shared's limit)
 
 // Selector buffer: model blob (FP32, 2 KB slot), per clip of a call the pick
-// order (32 int32) and the accept flag (int), fallback count (uint64).
+// order (32 int32), fallback count (uint64).
 constexpr size_t kSelOrderOff = 2048;
-constexpr size_t kSelAcceptOff = kSelOrderOff + kMaxSolveClips * 32 * sizeof(int32_t);
-constexpr size_t kSelFallbackOff = kSelAcceptOff + kMaxSolveClips * sizeof(int32_t);
-constexpr size_t kSelBytes = kSelFallbackOff + 96;
+constexpr size_t kSelFallbackOff = kSelOrderOff + kMaxSolveClips * 32 * sizeof(int32_t);
+constexpr size_t kSelBytes = kSelFallbackOff + 128;
 static_assert(kSelFallbackOff % 8 == 0, "the fallback count is a 64-bit atomic");
 inline float* selector_blob(cdmd_ctx* ctx) { return static_cast<float*>(ctx->buf[BUF_SELECTOR].ptr); }
 inline int32_t* selector_order(cdmd_ctx* ctx, int clip) {
     return reinterpret_cast<int32_t*>(static_cast<char*>(ctx->buf[BUF_SELECTOR].ptr) + kSelOrderOff) + 32 * clip;
-}
-inline int* selector_accept(cdmd_ctx* ctx, int clip) {
-    return reinterpret_cast<int*>(static_cast<char*>(ctx->buf[BUF_SELECTOR].ptr) + kSelAcceptOff) + clip;
 }
 inline unsigned long long* selector_fallbacks(cdmd_ctx* ctx) {
     return reinterpret_cast<unsigned long long*>(static_cast<char*>(ctx->buf[BUF_SELECTOR].ptr) + kSelFallbackOff);
@@ -332,8 +328,12 @@ cdmd_status launch_selector_features(cdmd_ctx* ctx, const double* lambda, const 
 cdmd_status launch_selector_relabel(cdmd_ctx* ctx, const double* DY, int k, int n, const double* G,
                                     const double* lambda, int r, const double* y_target, int K, int32_t* sel,
                                     cudaStream_t stream);
-cdmd_status launch_mlp_select(cdmd_ctx* ctx, const double* lambda, const double* M, const double* cvec,
-                              const double* R, int r, int K, int32_t* order, cudaStream_t stream);
+// The learned pick order of each clip from its Gram quantities.
+struct MlpSelectIO {
+    const double *lambda, *M, *cvec, *R;
+    int32_t* order;
+};
+cdmd_status launch_mlp_select(cdmd_ctx* ctx, int nclips, const MlpSelectIO* io, int r, int K, cudaStream_t stream);
 cdmd_status launch_mlp_forward(cdmd_ctx* ctx, const float* blob, const float* X, int64_t N, int bf16,
                                float* s, float* p, cudaStream_t stream);
 cdmd_status launch_mlp_train(cdmd_ctx* ctx, int apply, float* blob, float* m, float* v, int step, float lr,

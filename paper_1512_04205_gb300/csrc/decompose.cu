@@ -65,13 +65,12 @@ struct SolveClip {
     int n, p;            // frames, p = n - 1
     double *gpart, *Rw;  // Gram partials; the Gram's own storage (NULL when R is given)
     double *Hv, *htau, *Tw, *dd, *ee;             // reflectors, their block factors, the tridiagonal form
-    double *lamT, *Z, *V, *B, *At, *W, *M, *WR, *lamR, *cvec;
+    double *lamT, *Z, *V, *B, *At, *Nm, *dv, *W, *M, *WR, *lamR, *cvec;
     float2 *lam32, *W32;
     int* flag;           // [0] eigen-solver fallback, [1] eigenvectors of T not orthogonal to kOrthTol
     double *sigma, *lambda, *G, *PhiY, *beta;     // the caller's outputs
     int32_t *sel, *nsel;
-    int32_t* order;      // learned pick order and its verdict
-    int* accept;
+    int32_t* order;      // learned pick order
 };
 struct SolveBatch {
     SolveClip c[kMaxSolveClips];
@@ -1124,49 +1123,66 @@ backtransform_kernel(const __grid_constant__ SolveBatch sb) {
     }
 }
 
-// 4c. B[a][c] = sum_b R[a][b+1] V[b][c] = ((Y^T Y') V)[a][c]; one warp per entry.
+// 4c. B[t][c] = sum_b R[t][b+1] V[b][c] for t < n: rows 0..p-1 are
+// ((Y^T Y') V), rows 1..n-1 are ((Y'^T Y') V).  One warp per row and four
+// columns, which share the row's loads and one shuffle reduction.
 __global__ void __launch_bounds__(256)
 bmat_kernel(const __grid_constant__ SolveBatch sb) {
     const SolveClip& q = sb.c[blockIdx.z];
-    const double *R = q.R, *V = q.V;
-    const int n = q.n, p = q.p;
-    double* B = q.B;
+    const int n = q.n, p = q.p, r = sb.r;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int a = blockIdx.x * 8 + wid;
-    const int c = blockIdx.y;
-    if (a >= p) return;   // also the rows a shorter clip does not have
-    const double* row = R + static_cast<int64_t>(a) * n + 1;
-    const double* vc = V + static_cast<int64_t>(c) * p;
-    double s0 = 0.0, s1 = 0.0;
-    int b = lane;
-    for (; b + 32 < p; b += 64) {
-        s0 = fma(row[b], vc[b], s0);
-        s1 = fma(row[b + 32], vc[b + 32], s1);
+    const int t = blockIdx.x * 8 + wid;
+    const int c0 = 4 * blockIdx.y;
+    if (t >= n) return;   // also the rows a shorter clip does not have
+    const double* row = q.R + static_cast<int64_t>(t) * n + 1;
+    const double* v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = q.V + static_cast<int64_t>(min(c0 + e, r - 1)) * p;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+    for (int b = lane; b < p; b += 32) {
+        const double x = row[b];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[e] = fma(x, v[e][b], s[e]);
     }
-    if (b < p) s0 = fma(row[b], vc[b], s0);
-    const double s = warp_sum(s0 + s1);
-    if (lane == 0) B[static_cast<int64_t>(c) * p + a] = s;
+    __syncwarp();
+    const double y = warp_sum4(s);
+    const int c = c0 + (lane >> 3);
+    if ((lane & 7) == 0 && c < r) q.B[static_cast<int64_t>(c) * n + t] = y;
 }
 
-// 5. A~[a][c] = V[:,a]^T B[:,c] / (sigma_a sigma_c), one CTA per column c.
-__global__ void __launch_bounds__(32)
+// 5. With B as above, one warp per four rows a of one column c:
+//   which = 0: A~[a][c] = V[:,a]^T B[0:p, c] / (sigma_a sigma_c)
+//   which = 1: N[a][c]  = V[:,a]^T B[1:n, c] / (sigma_a sigma_c), so that
+//              Phi_Y^H Phi_Y = W^H N W with Phi_Y = Y' V S^-1 W
+//   c = r (which = 1): d[a] = V[:,a]^T (Y'^T y1) / sigma_a, Phi_Y^H y1 = W^H d
+__global__ void __launch_bounds__(256)
 atilde_kernel(const __grid_constant__ SolveBatch sb) {
     const SolveClip& q = sb.c[blockIdx.z];
-    const double *V = q.V, *B = q.B, *sigma = q.sigma;
-    const int p = q.p, r = sb.r;
-    double* At = q.At;
-    const int c = blockIdx.x;
-    const int lane = threadIdx.x;
-    const double* bc = B + static_cast<int64_t>(c) * p;
-    for (int a = 0; a < r; ++a) {
-        const double* va = V + static_cast<int64_t>(a) * p;
-        double s = 0.0;
-        for (int i = lane; i < p; i += 32) s = fma(va[i], bc[i], s);
-        s = warp_sum(s);
-        if (lane == 0) {
-            const double den = sigma[a] * sigma[c];
-            At[static_cast<int64_t>(c) * r + a] = den > 0.0 ? s * rcp64(den) : 0.0;
-        }
+    const int n = q.n, p = q.p, r = sb.r;
+    const int c = blockIdx.x, which = blockIdx.y;
+    const int lane = threadIdx.x & 31, a0 = 4 * (threadIdx.x >> 5);
+    if (a0 >= r || (c == r && which == 0)) return;
+    const double* v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = q.V + static_cast<int64_t>(min(a0 + e, r - 1)) * p;
+    // column 0 of R is read along its row (R is symmetric)
+    const double* x = c < r ? q.B + static_cast<int64_t>(c) * n + which : q.R + 1;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+    for (int i = lane; i < p; i += 32) {
+        const double xi = x[i];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[e] = fma(v[e][i], xi, s[e]);
+    }
+    __syncwarp();
+    const double y = warp_sum4(s);
+    const int a = a0 + (lane >> 3);
+    if ((lane & 7) == 0 && a < r) {
+        const double den = q.sigma[a] * (c < r ? q.sigma[c] : 1.0);
+        const double val = den > 0.0 ? y * rcp64(den) : 0.0;
+        if (c == r) q.dv[a] = val;
+        else (which ? q.Nm : q.At)[static_cast<int64_t>(c) * r + a] = val;
     }
 }
 
@@ -2046,122 +2062,123 @@ eig_finish_kernel(const __grid_constant__ SolveBatch sb) {
     eig_order_cta(clip.lamR, clip.WR, sb.r, clip.lambda, clip.W, reinterpret_cast<cd*>(qsm));
 }
 
-// 7. G[t][c] = sum_a V[t][a] / sigma_a * W[a][c]   (column-major complex)
-__global__ void gmat_kernel(const __grid_constant__ SolveBatch sb) {
+// 7, 8. One CTA per mode c:
+//   G[:, c] = V S^-1 w_c   (warps 4..7, a frame per lane),
+//   M[:, c] = W^H (N w_c) = Phi_Y^H phi_c and cvec[c] = w_c^H d = phi_c^H y1
+//   (warps 0..3, a mode per lane, each warp a quarter of the sums).
+// The compressed modes' Gram comes from the r x r matrices N and d, not from
+// G: no pass over the n x n Gram is left after A~.
+__global__ void __launch_bounds__(256)
+modes_kernel(const __grid_constant__ SolveBatch sb) {
     const SolveClip& q = sb.c[blockIdx.z];
-    const double *V = q.V, *sigma = q.sigma, *W = q.W;
-    const int p = q.p, r = sb.r;
-    double* G = q.G;
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= p * r) return;
-    const int t = idx % p, c = idx / p;
-    double re = 0.0, im = 0.0;
-    for (int a = 0; a < r; ++a) {
-        const double va = V[static_cast<int64_t>(a) * p + t] / sigma[a];
-        re = fma(va, W[2 * (static_cast<int64_t>(c) * r + a)], re);
-        im = fma(va, W[2 * (static_cast<int64_t>(c) * r + a) + 1], im);
-    }
-    G[2 * static_cast<int64_t>(idx)] = re;
-    G[2 * static_cast<int64_t>(idx) + 1] = im;
-}
-
-// 8. h = (Y'^T Y') G[:, c];  M[a][c] = G[:,a]^H h;  cvec[c] = G[:,c]^H (Y'^T y1).
-// One CTA of 16 warps per column c, one warp per row of h, then per entry.
-__global__ void __launch_bounds__(512)
-hmat_kernel(const __grid_constant__ SolveBatch sb) {
-    const SolveClip& q = sb.c[blockIdx.z];
-    const double *R = q.R, *G = q.G;
-    const int n = q.n, p = q.p, r = sb.r;
-    double *M = q.M, *cvec = q.cvec;
-    extern __shared__ double hsm[];   // h: 2p
-    const int c = blockIdx.x;
-    const double* gc = G + 2 * static_cast<int64_t>(c) * p;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int t = wid; t < p; t += nw) {
-        const double* row = R + static_cast<int64_t>(t + 1) * n + 1;
-        double re = 0.0, im = 0.0;
-        for (int b = lane; b < p; b += 32) {
-            re = fma(row[b], gc[2 * b], re);
-            im = fma(row[b], gc[2 * b + 1], im);
-        }
-        re = warp_sum(re);
-        im = warp_sum(im);
-        if (lane == 0) { hsm[2 * t] = re; hsm[2 * t + 1] = im; }
+    const int p = q.p, r = sb.r, c = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    __shared__ cd Ws[kMaxR][kMaxR + 1];     // Ws[i][a] = W[i, a]
+    __shared__ double Ns[kMaxR][kMaxR + 1];
+    __shared__ cd part[4][kMaxR], h[kMaxR], wc[kMaxR], wsig[kMaxR];
+    for (int idx = tid; idx < r * r; idx += 256) {
+        const int i = idx % r, a = idx / r;
+        const cd w = {q.W[2 * idx], q.W[2 * idx + 1]};
+        Ws[i][a] = w;
+        Ns[i][a] = q.Nm[idx];
+        if (a == c) wc[i] = w;
     }
     __syncthreads();
-    for (int a = wid; a <= r; a += nw) {
-        // a < r: M[a][c]; a == r: cvec[c]
+    if (wid == 4 && lane < r) {
+        const double is = 1.0 / q.sigma[lane];
+        wsig[lane] = cscale(wc[lane], is);
+    }
+    if (wid < 4 && lane < r) {
         double re = 0.0, im = 0.0;
-        if (a < r) {
-            const double* ga = G + 2 * static_cast<int64_t>(a) * p;
-            for (int t = lane; t < p; t += 32) {
-                const double gr = ga[2 * t], gi = ga[2 * t + 1];
-                const double hr = hsm[2 * t], hi = hsm[2 * t + 1];
-                re += gr * hr + gi * hi;   // conj(g) h
-                im += gr * hi - gi * hr;
-            }
-        } else {
-            for (int t = lane; t < p; t += 32) {
-                const double y = R[static_cast<int64_t>(t + 1) * n];   // (Y'^T y1)_t
-                re += gc[2 * t] * y;
-                im -= gc[2 * t + 1] * y;
-            }
+#pragma unroll 1
+        for (int j = wid; j < r; j += 4) {
+            re = fma(Ns[lane][j], wc[j].x, re);
+            im = fma(Ns[lane][j], wc[j].y, im);
         }
-        re = warp_sum(re);
-        im = warp_sum(im);
+        part[wid][lane] = {re, im};
+    }
+    __syncthreads();
+    if (wid == 0 && lane < r) {
+        const cd a = part[0][lane], b = part[1][lane], d = part[2][lane], e = part[3][lane];
+        h[lane] = {(a.x + b.x) + (d.x + e.x), (a.y + b.y) + (d.y + e.y)};
+    }
+    if (wid >= 4) {
+#pragma unroll 1
+        for (int t = tid - 128; t < p; t += 128) {
+            double re = 0.0, im = 0.0;
+#pragma unroll 4
+            for (int a = 0; a < r; ++a) {
+                const double va = q.V[static_cast<int64_t>(a) * p + t];
+                re = fma(va, wsig[a].x, re);
+                im = fma(va, wsig[a].y, im);
+            }
+            q.G[2 * (static_cast<int64_t>(c) * p + t)] = re;
+            q.G[2 * (static_cast<int64_t>(c) * p + t) + 1] = im;
+        }
+    }
+    __syncthreads();
+    if (wid < 4 && lane < r) {
+        double re = 0.0, im = 0.0;
+#pragma unroll 1
+        for (int i = wid; i < r; i += 4) {
+            const cd w = Ws[i][lane], x = h[i];         // conj(w) h
+            re = fma(w.x, x.x, fma(w.y, x.y, re));
+            im = fma(w.x, x.y, fma(-w.y, x.x, im));
+        }
+        part[wid][lane] = {re, im};
+    }
+    if (wid == 4) {
+        const double d = lane < r ? q.dv[lane] : 0.0;
+        const double re = warp_sum(lane < r ? wc[lane].x * d : 0.0);
+        const double im = warp_sum(lane < r ? -wc[lane].y * d : 0.0);
         if (lane == 0) {
-            if (a < r) {
-                M[2 * (static_cast<int64_t>(c) * r + a)] = re;
-                M[2 * (static_cast<int64_t>(c) * r + a) + 1] = im;
-            } else {
-                cvec[2 * c] = re;
-                cvec[2 * c + 1] = im;
-            }
+            q.cvec[2 * c] = re;
+            q.cvec[2 * c + 1] = im;
         }
+    }
+    __syncthreads();
+    if (tid < r) {
+        const cd a = part[0][tid], b = part[1][tid], d = part[2][tid], e = part[3][tid];
+        q.M[2 * (static_cast<int64_t>(c) * r + tid)] = (a.x + b.x) + (d.x + e.x);
+        q.M[2 * (static_cast<int64_t>(c) * r + tid) + 1] = (a.y + b.y) + (d.y + e.y);
     }
 }
 
 // 9. OMP in Gram form, one warp (r <= 32; lane j owns mode j).  M = Phi_Y^H
 // Phi_Y (Hermitian, column-major), cvec = Phi_Y^H y1, ||y1||^2 = R[0][0].
-// Scores |phi_j^H rho|^2 / ||phi_j||^2 with phi_j^H rho = c_j - sum_q M[j][S_q]
-// beta_q; ties (relative 2e-9 on the squared score, i.e. 1e-9 on the score)
-// go to the largest Im(lambda), then the lowest index.  The least-squares fit
-// on the selected set solves M_SS beta = c_S through a Cholesky factor
-// M_SS = L L^H grown by one row per pick; every triangular solve is
-// right-looking (one row per lane, one broadcast per step).
-__device__ void omp_warp(const double* M, const double* cvec, const double* R, const double* lam, int r, int K,
+// Scores |g_j|^2 / ||phi_j||^2 with g_j = phi_j^H rho; ties (relative 2e-9 on
+// the squared score, i.e. 1e-9 on the score) go to the largest Im(lambda), then
+// the lowest index.  With the Cholesky factor M_SS = L L^H of the picks, every
+// lane keeps x_j = L^-1 M_Sj (one entry per pick) and the new entry of
+// y = L^-1 c_S updates g_j -= conj(x_j) y, ||phi_j||^2's remainder and the
+// residual's norm: a pick costs one length-ns sum on all lanes at once and no
+// triangular solve; the amplitudes L^H beta = y are solved for once, at the end.
+// order given: the picks are order's (learned selection); the result stands
+// when its relative residual is within blob's tolerance, else it returns false
+// and writes nothing.
+__device__ bool omp_warp(const double* M, const double* cvec, const double* R, const double* lam, int r, int K,
                          int lstsq, double* beta, int32_t* sel, int32_t* nsel_out, int* status,
-                         const int32_t* order, const float* blob, int* accept, unsigned long long* fallbacks) {
-    // Modes of operation:
-    //   order == nullptr, accept == nullptr   greedy OMP (or lstsq over all r)
-    //   order != nullptr                      least squares on the learned pick
-    //                                         order; accepted (outputs written,
-    //                                         *accept = 1) when the relative
-    //                                         residual is within the model's tol,
-    //                                         else *accept = 0 and one fallback
-    //                                         is counted
-    //   order == nullptr, accept != nullptr   greedy OMP unless *accept == 1
-    if (order == nullptr && accept != nullptr && *accept == 1) return;
-    __shared__ cd L[kMaxR][kMaxR + 1];   // L[u][q], u >= q
+                         const int32_t* order, const float* blob) {
+    __shared__ cd Ms[kMaxR][kMaxR + 1];   // Ms[j][i] = M[i][j]
+    __shared__ cd X[kMaxR][kMaxR + 1];    // X[q][j] = (x_j)_q
     __shared__ double invdiag[kMaxR];
-    __shared__ cd bsel[kMaxR];
+    __shared__ cd ys[kMaxR];
     __shared__ int S[kMaxR];
     const int lane = threadIdx.x;
-    auto Mel = [&](int i, int jj) -> cd {
-        return {M[2 * (static_cast<int64_t>(jj) * r + i)], M[2 * (static_cast<int64_t>(jj) * r + i) + 1]};
-    };
+    for (int idx = lane; idx < r * r; idx += 32) Ms[idx / r][idx % r] = {M[2 * idx], M[2 * idx + 1]};
+    __syncwarp();
     const bool live = lane < r;
-    const double mjj = live ? Mel(lane, lane).x : 0.0;
+    const double mjj = live ? Ms[lane][lane].x : 0.0;
     const double inv_m = (live && mjj > 0.0) ? rcp64(mjj) : 0.0;
-    const cd cj = live ? cd{cvec[2 * lane], cvec[2 * lane + 1]} : cd{0.0, 0.0};
-    const double imlam = live ? lam[2 * lane + 1] : 0.0;
-    bool used = false;
+    const unsigned long long kim = order_key(live ? lam[2 * lane + 1] : 0.0);
+    cd g = live ? cd{cvec[2 * lane], cvec[2 * lane + 1]} : cd{0.0, 0.0};
+    double rem = mjj;
+    bool used = !live || !(mjj > 0.0);
     const double y2 = R[0];
     const int kmax_steps = lstsq ? r : min(K, r);
     int ns = 0;
     double res2 = y2;
     for (int step = 0; step < kmax_steps; ++step) {
-        if (!lstsq && order == nullptr && res2 <= 1e-24 * y2) break;
         int best;
         if (order != nullptr) {
             best = order[step];
@@ -2169,76 +2186,49 @@ __device__ void omp_warp(const double* M, const double* cvec, const double* R, c
         } else if (lstsq) {
             best = step;
         } else {
-            double score = -1.0;
-            if (live && !used && mjj > 0.0) {
-                cd g = cj;
-                for (int q = 0; q < ns; ++q) g = csub(g, cmul(Mel(lane, S[q]), bsel[q]));
-                score = cabs2(g) * inv_m;
-            }
-            const double bmax = warp_max(score);
+            if (res2 <= 1e-24 * y2) break;
+            const double score = cabs2(g) * inv_m;
+            if (!__any_sync(0xffffffffu, !used)) break;
+            const int top = warp_pick(order_key(score), !used && score > 0.0, false);   // -1: nothing above zero
+            if (top < 0) break;                         // also non-finite scores: no pick
+            const double bmax = __shfl_sync(0xffffffffu, score, top);
             if (!(bmax > 0.0)) break;
-            const bool cand = score >= bmax * (1.0 - 2e-9);
-            const double key = cand ? imlam : -1e300;
-            const double kbest = warp_max(key);
-            const unsigned bb = __ballot_sync(0xffffffffu, cand && key == kbest);
-            if (bb == 0u) break;                    // non-finite scores: no pick
-            best = __ffs(bb) - 1;
+            best = warp_pick(kim, !used && score >= bmax * (1.0 - 2e-9), false);
+            if (best < 0) break;
         }
-        // new Cholesky row: solve L x = m (m_q = M[S_q][best]); row = conj(x)
-        cd t = (lane < ns) ? Mel(S[lane], best) : cd{0.0, 0.0};
-        double xs2 = 0.0;
-        for (int q = 0; q < ns; ++q) {
-            cd xq = {0.0, 0.0};
-            if (lane == q) xq = cscale(t, invdiag[q]);
-            xq = shfl_cd(xq, q);
-            if (lane == q) { L[ns][q] = cconj(xq); xs2 = cabs2(xq); }
-            if (lane > q && lane < ns) t = csub(t, cmul(L[lane][q], xq));
-        }
-        const double diag2 = Mel(best, best).x - warp_sum(xs2);
-        if (!(diag2 > kEps * Mel(best, best).x)) {
+        cd t = live ? Ms[lane][best] : cd{0.0, 0.0};    // M[best][lane]
+        for (int q = 0; q < ns; ++q) t = csub(t, cmul(cconj(X[q][best]), X[q][lane]));
+        const double diag2 = __shfl_sync(0xffffffffu, rem, best);
+        if (!(diag2 > kEps * Ms[best][best].x)) {
             if (lstsq && lane == 0) record_status(status, CDMD_ERR_RANK_DEFICIENT);
             break;
         }
         const double invd = rsqrt64(diag2);
+        const cd x = cscale(t, invd);
+        const cd y = cscale(shfl_cd(g, best), invd);
+        g = csub(g, cmul(cconj(x), y));
+        rem = fma(-x.x, x.x, fma(-x.y, x.y, rem));
+        res2 = fma(-y.x, y.x, fma(-y.y, y.y, res2));
+        X[ns][lane] = x;
         if (lane == 0) {
-            L[ns][ns] = {diag2 * invd, 0.0};
             invdiag[ns] = invd;
+            ys[ns] = y;
             S[ns] = best;
         }
         if (lane == best) used = true;
         ++ns;
         __syncwarp();
-        // beta: L y = c_S (forward), then L^H beta = y (backward); lane u owns row u
-        cd v = (lane < ns) ? cd{cvec[2 * S[lane]], cvec[2 * S[lane] + 1]} : cd{0.0, 0.0};
-        for (int q = 0; q < ns; ++q) {
-            cd yq = {0.0, 0.0};
-            if (lane == q) { yq = cscale(v, invdiag[q]); v = yq; }
-            yq = shfl_cd(yq, q);
-            if (lane > q && lane < ns) v = csub(v, cmul(L[lane][q], yq));
-        }
-        for (int q = ns - 1; q >= 0; --q) {
-            cd bq = {0.0, 0.0};
-            if (lane == q) { bq = cscale(v, invdiag[q]); v = bq; }
-            bq = shfl_cd(bq, q);
-            if (lane < q) v = csub(v, cmul(cconj(L[q][lane]), bq));
-        }
-        if (lane < ns) bsel[lane] = v;
-        __syncwarp();
-        double cb = 0.0;
-        if (lane < ns) {
-            const cd c = {cvec[2 * S[lane]], cvec[2 * S[lane] + 1]};
-            cb = fma(c.x, v.x, c.y * v.y);
-        }
-        res2 = y2 - warp_sum(cb);
     }
     if (order != nullptr) {
         const double tol = static_cast<double>(blob[8]);
-        const bool ok = tol >= 0.0 && res2 <= tol * tol * y2;   // a negative tol rejects every pick
-        if (lane == 0) {
-            *accept = ok ? 1 : 0;
-            if (!ok) atomicAdd(fallbacks, 1ull);
-        }
-        if (!ok) return;
+        if (!(tol >= 0.0 && res2 <= tol * tol * y2)) return false;   // a negative tol rejects every pick
+    }
+    // L^H beta = y, lane u owning row u: L[q][u] = conj((x_{S_q})_u)
+    cd v = lane < ns ? ys[lane] : cd{0.0, 0.0};
+    for (int q = ns - 1; q >= 0; --q) {
+        const cd bq = cscale(shfl_cd(v, q), invdiag[q]);
+        if (lane == q) v = bq;
+        else if (lane < q) v = csub(v, cmul(X[lane][S[q]], bq));
     }
     if (live) {
         beta[2 * lane] = 0.0;
@@ -2246,28 +2236,33 @@ __device__ void omp_warp(const double* M, const double* cvec, const double* R, c
     }
     __syncwarp();
     if (lane < ns) {
-        beta[2 * S[lane]] = bsel[lane].x;
-        beta[2 * S[lane] + 1] = bsel[lane].y;
+        beta[2 * S[lane]] = v.x;
+        beta[2 * S[lane] + 1] = v.y;
     }
     if (lane < K) sel[lane] = (lane < ns) ? S[lane] : -1;
     if (lane == 0) *nsel_out = ns;
+    return true;
 }
 
-// learned: 0 = OMP or lstsq, 1 = least squares on the learned pick order,
-// 2 = OMP unless that order was accepted
+// learned: least squares on the learned pick order, and OMP when that is
+// rejected (counted); else OMP, or least squares over all r modes
 __global__ void __launch_bounds__(32)
 omp_kernel(const __grid_constant__ SolveBatch sb, int lstsq, int learned, const float* blob,
            unsigned long long* fallbacks) {
     const SolveClip& q = sb.c[blockIdx.z];
-    omp_warp(q.M, q.cvec, q.R, q.lambda, sb.r, sb.K, lstsq, q.beta, q.sel, q.nsel, sb.status,
-             learned == 1 ? q.order : nullptr, blob, learned != 0 ? q.accept : nullptr, fallbacks);
+    if (learned) {
+        if (omp_warp(q.M, q.cvec, q.R, q.lambda, sb.r, sb.K, 0, q.beta, q.sel, q.nsel, sb.status, q.order, blob)) return;
+        if (threadIdx.x == 0) atomicAdd(fallbacks, 1ull);
+        __syncwarp();
+    }
+    omp_warp(q.M, q.cvec, q.R, q.lambda, sb.r, sb.K, lstsq, q.beta, q.sel, q.nsel, sb.status, nullptr, nullptr);
 }
 
 // OMP against another target (cvec and ||y||^2 of it) on the last decomposition
 __global__ void __launch_bounds__(32)
 relabel_omp_kernel(const double* M, const double* cvec, const double* y2, const double* lam, int r, int K,
                    double* beta, int32_t* sel, int32_t* nsel, int* status) {
-    omp_warp(M, cvec, y2, lam, r, K, 0, beta, sel, nsel, status, nullptr, nullptr, nullptr, nullptr);
+    omp_warp(M, cvec, y2, lam, r, K, 0, beta, sel, nsel, status, nullptr, nullptr);
 }
 
 // 10. Phi_Y[i][c] = sum_t DY[(t+1)*k + i] G[t][c]
@@ -2366,14 +2361,29 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
                            cdmd_selector selector, cudaStream_t stream, const AutoRank* autor = nullptr) {
     if (nclips < 1 || nclips > kMaxSolveClips) return fail(CDMD_ERR_INVALID_ARG, "%d clips in one solve", nclips);
     // ---- workspace layout (doubles), one region per clip ----
-    const int kchunk = 128;
+    // rows of the sketch per Gram CTA: the FP64 rate bounds the pass, so the
+    // multiple of 32 that leaves the least work to the busiest SM (and of two
+    // equal ones the larger, for fewer partials to add up)
+    int kchunk = 128;
+    if (io[0].R == nullptr) {
+        int64_t tiles = 0, best = INT64_MAX;
+        for (int i = 0; i < nclips; ++i) {
+            const int64_t nt = (io[i].n + kGT - 1) / kGT;
+            tiles += nt * (nt + 1) / 2;
+        }
+        for (int kc = 256; kc >= 64; kc -= 32) {
+            const int64_t ctas = tiles * ((k + kc - 1) / kc);
+            const int64_t load = (ctas + ctx->device_sms - 1) / ctx->device_sms * (std::min(kc, k) + 8);
+            if (load < best) { best = load; kchunk = kc; }
+        }
+    }
     const int splits = io[0].R != nullptr ? 0 : (k + kchunk - 1) / kchunk;
     size_t off[kMaxSolveClips + 1] = {0};
     int nmax = 0;
     for (int i = 0; i < nclips; ++i) {
         const size_t n = io[i].n, p = n - 1, rr = r;
         const size_t total = static_cast<size_t>(splits) * n * n + n * n + p * p + 32 * p + 1024 + 3 * p + rr +
-                             3 * p * rr + 10 * rr * rr + 6 * rr + 64;
+                             3 * p * rr + 12 * rr * rr + 8 * rr + 64;
         // + one slot for the eigen-solver's fallback flag and two for the rank
         // threshold's result; with an automatic rank, r is its upper bound here
         off[i + 1] = off[i] + total + 3;
@@ -2395,8 +2405,10 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
             q.Z = q.lamT + rr;
             q.V = q.Z + nz;
             q.B = q.V + nz;
-            q.At = q.B + nz;
-            q.W = q.At + ns;
+            q.At = q.B + nz + rr;                    // B: n x r
+            q.Nm = q.At + static_cast<size_t>(rr) * rr;
+            q.dv = q.Nm + static_cast<size_t>(rr) * rr;
+            q.W = q.dv + rr;
             q.M = q.W + ns;
             q.WR = q.M + ns;
             q.lamR = q.WR + ns;
@@ -2430,7 +2442,6 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
         q.nsel = io[i].nsel;
         if (selector == CDMD_SEL_MLP) {
             q.order = selector_order(ctx, i);
-            q.accept = selector_accept(ctx, i);
         }
         want_phiy = want_phiy || (q.PhiY != nullptr && q.DY != nullptr);
     }
@@ -2541,9 +2552,9 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
         CDMD_CHECK_LAUNCH("backtransform_kernel");
     }
     // 4. A~ and its eigen-decomposition
-    bmat_kernel<<<dim3((p + 7) / 8, r, nc), 256, 0, stream>>>(sb);
+    bmat_kernel<<<dim3((nmax + 7) / 8, (r + 3) / 4, nc), 256, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("bmat_kernel");
-    atilde_kernel<<<dim3(r, 1, nc), 32, 0, stream>>>(sb);
+    atilde_kernel<<<dim3(r + 1, 2, nc), 256, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("atilde_kernel");
     eig_f32_kernel<<<dim3(1, 1, nc), kEig32Threads, 0, stream>>>(sb);
     CDMD_CHECK_LAUNCH("eig_f32_kernel");
@@ -2554,10 +2565,8 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
     eig_finish_kernel<<<dim3(1, 1, nc), kQrThreads, kQrSmem, stream>>>(sb);
     CDMD_CHECK_LAUNCH("eig_finish_kernel");
     // 5. G, Gram-form quantities, selection
-    gmat_kernel<<<dim3((p * r + 127) / 128, 1, nc), 128, 0, stream>>>(sb);
-    CDMD_CHECK_LAUNCH("gmat_kernel");
-    hmat_kernel<<<dim3(r, 1, nc), 512, 2 * p * sizeof(double), stream>>>(sb);
-    CDMD_CHECK_LAUNCH("hmat_kernel");
+    modes_kernel<<<dim3(r, 1, nc), 256, 0, stream>>>(sb);
+    CDMD_CHECK_LAUNCH("modes_kernel");
     const SolveClip& last = sb.c[nclips - 1];
     ctx->last_M = last.M;
     ctx->last_cvec = last.cvec;
@@ -2565,14 +2574,14 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
     ctx->last_r = r;
     if (selector == CDMD_SEL_MLP) {
         // learned pick order -> least squares on it -> OMP only if rejected
+        MlpSelectIO mio[kMaxSolveClips];
         for (int i = 0; i < nclips; ++i) {
             const SolveClip& q = sb.c[i];
-            st = launch_mlp_select(ctx, q.lambda, q.M, q.cvec, q.R, r, K, q.order, stream);
-            if (st != CDMD_OK) return st;
+            mio[i] = {q.lambda, q.M, q.cvec, q.R, q.order};
         }
+        st = launch_mlp_select(ctx, nclips, mio, r, K, stream);
+        if (st != CDMD_OK) return st;
         omp_kernel<<<dim3(1, 1, nc), 32, 0, stream>>>(sb, 0, 1, selector_blob(ctx), selector_fallbacks(ctx));
-        CDMD_CHECK_LAUNCH("omp_kernel");
-        omp_kernel<<<dim3(1, 1, nc), 32, 0, stream>>>(sb, 0, 2, nullptr, nullptr);
     } else {
         omp_kernel<<<dim3(1, 1, nc), 32, 0, stream>>>(sb, selector == CDMD_SEL_LSTSQ ? 1 : 0, 0, nullptr, nullptr);
     }

@@ -198,13 +198,17 @@ selector_features_kernel(const double* __restrict__ lam, const double* __restric
 // Scores every mode (BF16 inference) and writes the pick order: order[q] is
 // the mode of rank q (descending logit, equal logits by index) for q < K,
 // -1 after.
+struct MlpSelectBatch {
+    MlpSelectIO c[kMaxSolveClips];
+};
+
 __global__ void __launch_bounds__(32)
-mlp_select_kernel(const float* __restrict__ blob, const double* __restrict__ lam, const double* __restrict__ M,
-                  const double* __restrict__ cvec, const double* __restrict__ R, int r, int K,
-                  int32_t* __restrict__ order) {
+mlp_select_kernel(const float* __restrict__ blob, const __grid_constant__ MlpSelectBatch mb, int r, int K) {
+    const MlpSelectIO& q = mb.c[blockIdx.x];
+    int32_t* order = q.order;
     const int lane = threadIdx.x;
     float f[kFeat], xh[kFeat];
-    lane_features(lane, r, lam, M, cvec, R, f);
+    lane_features(lane, r, q.lambda, q.M, q.cvec, q.R, f);
     float s = -INFINITY;
     if (lane < r) {
         normalise(blob, f, true, xh);
@@ -231,9 +235,10 @@ cdmd_status launch_selector_features(cdmd_ctx* ctx, const double* lambda, const 
     return CDMD_OK;
 }
 
-cdmd_status launch_mlp_select(cdmd_ctx* ctx, const double* lambda, const double* M, const double* cvec,
-                              const double* R, int r, int K, int32_t* order, cudaStream_t stream) {
-    mlp_select_kernel<<<1, 32, 0, stream>>>(selector_blob(ctx), lambda, M, cvec, R, r, K, order);
+cdmd_status launch_mlp_select(cdmd_ctx* ctx, int nclips, const MlpSelectIO* io, int r, int K, cudaStream_t stream) {
+    MlpSelectBatch mb = {};
+    std::copy(io, io + nclips, mb.c);
+    mlp_select_kernel<<<nclips, 32, 0, stream>>>(selector_blob(ctx), mb, r, K);
     CDMD_CHECK_LAUNCH("mlp_select_kernel");
     return CDMD_OK;
 }
