@@ -4,10 +4,9 @@
 //   bg_jt = | sum_c Phi_jc beta_{s_c} lambda_{s_c}^t |   (Eq. DMDTerms, MODULUS)
 //   mask_jt = |x_jt - bg_jt| > tau                       (Eq. thres, strict)
 //
-// subtract_table_kernel (one block: lane = selected column, eight warps =
-// eight blocks of frames) forms lambda^t for t < n in FP64, each warp from
-// lambda^t0 by binary powering and then by repeated multiplication, and the
-// amplitudes.  It also classifies the selected modes:
+// subtract_table_kernel (lane = selected column, a warp = kTableFrames frames)
+// forms lambda^t for t < n in FP64, each warp from lambda^t0 by binary powering
+// and then by repeated multiplication, and the amplitudes.  It also classifies the selected modes:
 // the video is real, so the modes of a real A~ come as real eigenvalues and
 // conjugate pairs with conjugate modes and (least-squares) amplitudes, and a
 // pair contributes phi b lambda^t + conj(phi b lambda^t) = 2 Re(phi b lambda^t).
@@ -27,7 +26,17 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kMaxCols = 32;
-constexpr int kTableThreads = 256;     // table kernel: 8 warps, one block of frames each
+// Table kernel: four warps a block (one per scheduler), a warp per kTableFrames
+// frames.  An FP64 instruction holds its scheduler 64 clocks, so the frames are
+// spread over SMs: n = 200 takes 25 warps on seven of them, about 45 FP64
+// instructions of powering and 4 a frame on each (one block of eight warps
+// took 35 us, as long as a sixth of the pass over a 1920x1080x200 clip).
+constexpr int kTableThreads = 128;
+constexpr int kTableFrames = 8;
+
+__host__ __device__ constexpr int table_blocks(int n) {
+    return (n + kTableFrames * (kTableThreads / 32) - 1) / (kTableFrames * (kTableThreads / 32));
+}
 
 // Table layout (one allocation):
 //   hdr[4] int32            nterms, real_only
@@ -63,12 +72,12 @@ __host__ __device__ inline Table table_views(void* base, int n, int nc_pad) {
 
 __device__ __forceinline__ void build_table(const int32_t* __restrict__ cols, int ncols, int nc_pad,
                                             const double* __restrict__ beta, const double* __restrict__ lambda, int r,
-                                            int n, const Table& tb) {
-    // lane c = selected column; warp w = block w of the frames (every warp
-    // classifies the columns the same way, warp 0 writes the per-column data)
+                                            int n, const Table& tb, int wb) {
+    // lane c = selected column; wb = the warp's block of kTableFrames frames
+    // (every warp classifies the columns the same way, warp 0 of the clip
+    // writes the per-column data)
     const int c = threadIdx.x & 31;
-    const int wb = threadIdx.x >> 5;
-    const int nwb = blockDim.x >> 5;
+    if (wb > 0 && wb * kTableFrames >= n) return;
     int s = -1;
     if (c < ncols) s = cols ? cols[c] : c;
     const bool ok = (s >= 0 && s < r);
@@ -77,18 +86,31 @@ __device__ __forceinline__ void build_table(const int32_t* __restrict__ cols, in
     const double br = ok ? beta[2 * s] : 0.0;
     const double bi = ok ? beta[2 * s + 1] : 0.0;
     // classify: real, lead of a pair (Im > 0), follower (Im < 0), or lone
-    const double mag = hypot(lr, li);
+    const double mag = ok ? hypot(lr, li) : 0.0;
     const bool is_real = ok && fabs(li) <= 1e-12 * fmax(mag, 1e-300);
     const double tol = 1e-9 * fmax(1.0, mag);
+    // columns near the conjugate by FP32 (far wider than tol), lowest first,
+    // are looked at in FP64
     int partner = -1;
-    for (int d = 0; d < 32; ++d) {
-        const double dr = __shfl_sync(0xffffffffu, lr, d);
-        const double di = __shfl_sync(0xffffffffu, li, d);
-        const bool dok = __shfl_sync(0xffffffffu, ok, d);
-        const bool dreal = __shfl_sync(0xffffffffu, is_real, d);
-        if (partner < 0 && ok && !is_real && dok && !dreal && d != c && (di > 0.0) != (li > 0.0) &&
-            hypot(dr - lr, di + li) <= tol)
-            partner = d;
+    {
+        const float lrf = static_cast<float>(lr), lif = static_cast<float>(li);
+        const float near_f = 1e-5f * fmaxf(1.0f, static_cast<float>(mag));
+        const bool cplx = ok && !is_real;
+        const unsigned cmask = __ballot_sync(0xffffffffu, cplx), pmask = __ballot_sync(0xffffffffu, li > 0.0);
+        const unsigned others = cmask & (li > 0.0 ? ~pmask : pmask) & ~(1u << c);
+        unsigned cand = 0u;
+        for (int d = 0; d < ncols; ++d) {
+            const float dr = __shfl_sync(0xffffffffu, lrf, d), di = __shfl_sync(0xffffffffu, lif, d);
+            if (cplx && ((others >> d) & 1u) &&
+                !(fabsf(dr - lrf) + fabsf(di + lif) > near_f))
+                cand |= 1u << d;
+        }
+        while (__any_sync(0xffffffffu, cand != 0u && partner < 0)) {
+            const int d = cand != 0u ? __ffs(cand) - 1 : c;
+            const double dr = __shfl_sync(0xffffffffu, lr, d), di = __shfl_sync(0xffffffffu, li, d);
+            if (cand != 0u && partner < 0 && hypot(dr - lr, di + li) <= tol) partner = d;
+            cand &= cand - 1u;
+        }
     }
     // a pair counts only when each side names the other and the amplitudes
     // are conjugate to working precision
@@ -124,9 +146,8 @@ __device__ __forceinline__ void build_table(const int32_t* __restrict__ cols, in
     }
     // frames t0 .. t1-1 of this warp: lambda^t0 by binary powering, then
     // repeated multiplication
-    const int per = (n + nwb - 1) / nwb;
-    const int t0 = wb * per;
-    const int t1 = t0 + per < n ? t0 + per : n;
+    const int t0 = wb * kTableFrames;
+    const int t1 = t0 + kTableFrames < n ? t0 + kTableFrames : n;
     double pr = 1.0, pi = 0.0;
     {
         double xr = lr, xi = li;
@@ -156,14 +177,15 @@ __device__ __forceinline__ void build_table(const int32_t* __restrict__ cols, in
 __global__ void __launch_bounds__(kTableThreads)
 subtract_table_kernel(const int32_t* __restrict__ cols, int ncols, int nc_pad, const double* __restrict__ beta,
                       const double* __restrict__ lambda, int r, int n, Table tb) {
-    build_table(cols, ncols, nc_pad, beta, lambda, r, n, tb);
+    build_table(cols, ncols, nc_pad, beta, lambda, r, n, tb, blockIdx.x * (kTableThreads / 32) + (threadIdx.x >> 5));
 }
 
-// Grouped: one block per clip, tables with the common column stride nc.
+// Grouped: blockIdx.y = clip, tables with the common column stride nc.
 __global__ void __launch_bounds__(kTableThreads)
 subtract_table_grouped_kernel(const SubtractClip* __restrict__ clips, int nc) {
-    const SubtractClip c = clips[blockIdx.x];
-    build_table(c.cols, c.ncols, nc, c.beta, c.lambda, c.r, c.n, table_views(c.table, c.n, nc));
+    const SubtractClip c = clips[blockIdx.y];
+    build_table(c.cols, c.ncols, nc, c.beta, c.lambda, c.r, c.n, table_views(c.table, c.n, nc),
+                blockIdx.x * (kTableThreads / 32) + (threadIdx.x >> 5));
 }
 
 // One pixel tile for every frame.  REAL: accumulate real terms only (the
@@ -661,7 +683,7 @@ cdmd_status launch_subtract(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, i
     cdmd_status st = ensure_buffer(ctx, BUF_SUBTRACT_TABLE, table_bytes(n, nc_pad), &tbl);
     if (st != CDMD_OK) return st;
     const Table tb = table_views(tbl, n, nc_pad);
-    subtract_table_kernel<<<1, kTableThreads, 0, stream>>>(cols, ncols, nc_pad, beta, lambda, r, n, tb);
+    subtract_table_kernel<<<table_blocks(n), kTableThreads, 0, stream>>>(cols, ncols, nc_pad, beta, lambda, r, n, tb);
     CDMD_CHECK_LAUNCH("subtract_table_kernel");
     if (subtract_tc_supported(n, ncols, mode, D, ldd, m, Phi, bg))
         return launch_subtract_tc(ctx, D, m, n, ldd, Phi, ncols, subtract_tc_table(tbl, n, nc_pad), nc_pad, tau, mode,
@@ -717,7 +739,8 @@ cdmd_status make_subtract_tmap(CUtensorMap* map, const uint8_t* D, int64_t m, in
 
 cdmd_status launch_subtract_grouped(const SubtractClip* clips, int nclips, const SubtractItem* items, int nitems,
                                     int nc, int max_n, cdmd_bgmode mode, float tau, int* status, cudaStream_t stream) {
-    subtract_table_grouped_kernel<<<static_cast<unsigned>(nclips), kTableThreads, 0, stream>>>(clips, nc);
+    subtract_table_grouped_kernel<<<dim3(table_blocks(max_n), static_cast<unsigned>(nclips)), kTableThreads, 0, stream>>>(
+        clips, nc);
     CDMD_CHECK_LAUNCH("subtract_table_grouped_kernel");
     if (nitems == 0) return CDMD_OK;
     const size_t smem = tma_smem_bytes(max_n, nc);
