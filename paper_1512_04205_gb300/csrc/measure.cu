@@ -152,6 +152,235 @@ sparse_sketch_kernel(const uint8_t* __restrict__ D, int64_t m, int n, int64_t ld
     }
 }
 
+// Packed form of the same pass, for 4-byte aligned frames and sparse enough C.
+// The kernel above spends a warp instruction per non-zero of its busiest pixel
+// and per frame, a quarter of the lanes live, and its adds collide in the banks.
+// Here lanes are frames: a warp copies 128 pixels x kFrames frames into its own
+// shared tile, transposed to [pixel][frame], and walks the pixels' non-zeros one
+// after another; a lane adds two frames of the pixel, packed into one word, to
+// its word of the row's accumulator: one conflict-free shared atomic of the warp
+// per 32 / kFrames x 2 non-zeros and kFrames frames.
+// A word holds two signed 16-bit sums (as lo + 65536 hi), so a row may take at
+// most 128 entries of 255 between two emptyings of the accumulators into the
+// FP64-reduced int32 partials.  The entries of a round (every warp's next 128
+// pixels) are therefore counted per row first, 32 lanes at a time; when a row
+// would pass 128 the accumulators are emptied before the round, and a round
+// that passes it by itself is added to the partials directly.
+// kFrames = 32, or 16 past 2048 rows: the accumulators take 2 kFrames bytes a
+// row, and the smaller they are the more warps (24 at k = 1000) hide the latency
+// of the entry's descriptor, word and atomic, which bounds the pass (issue 29 %,
+// DRAM 16 % with 64 frames and 11 warps).
+// Measured: 3840x2160x300, k = 1000, density 1/1000: 5.11 -> 2.15 ms (2.25 with
+// 64 frames); 1280x720x200: 417 -> 203 us (273); k = 3000, 1280x720x100:
+// 421 -> 321 us.
+constexpr int kPackPix = 128;            // pixels per warp tile
+constexpr int kPackLimit = 128;          // entries of 255 a signed 16-bit sum holds
+constexpr size_t kPackSmemMax = 232448;
+
+__host__ __device__ constexpr int pack_tile_words(int frames) { return kPackPix * (frames / 4 + 1) + 32 * 4; }
+
+template <int kFrames>
+__global__ void __launch_bounds__(768)
+sparse_packed_kernel(const uint8_t* __restrict__ D, int64_t m, int n, int64_t ldd, int k,
+                     const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
+                     int64_t pix_per_split, int fps, int32_t* part) {
+    constexpr int kQuads = kFrames / 4;          // words of one pixel in the tile
+    constexpr int kLd = kQuads + 1;              // tile row stride (odd)
+    constexpr int kWords = kFrames / 2;          // accumulator words of a row
+    constexpr int kSub = 32 / kWords;            // entries a warp adds at once
+    extern __shared__ int32_t psm[];
+    int32_t* acc = psm;                                          // k x kWords
+    int32_t* cnt = acc + static_cast<size_t>(k) * kWords;        // k: entries since the last emptying
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarps = blockDim.x >> 5;
+    uint32_t* tile = reinterpret_cast<uint32_t*>(cnt + (k + 3) / 4 * 4) + static_cast<size_t>(wid) * pack_tile_words(kFrames);
+    uint4* list = reinterpret_cast<uint4*>(tile + kPackPix * kLd);   // 32 entries: tile and accumulator address, sign
+    // 32-bit shared addresses: this lane's word of a tile row (its two frames are
+    // the low or the high half) and of an accumulator row
+    const uint32_t tile_s = static_cast<uint32_t>(__cvta_generic_to_shared(tile));
+    const uint32_t acc_s = static_cast<uint32_t>(__cvta_generic_to_shared(acc));
+    const uint32_t tcol = static_cast<uint32_t>((lane % kWords) >> 1) * 4u, acol = static_cast<uint32_t>(lane % kWords) * 4u;
+    const uint32_t half = (lane & 1) ? 0x4342u : 0x4140u;
+    __shared__ int over;
+    const int t0 = blockIdx.x * fps;             // fps <= kFrames frames per slab
+    const int nt = min(fps, n - t0);
+    int32_t* dst = part + static_cast<int64_t>(blockIdx.y) * k * n;
+    for (int idx = tid; idx < k * kWords; idx += blockDim.x) acc[idx] = 0;
+    for (int idx = tid; idx < k; idx += blockDim.x) cnt[idx] = 0;
+    for (int idx = tid; idx < k * nt; idx += blockDim.x)
+        dst[static_cast<int64_t>(idx / nt) * n + t0 + idx % nt] = 0;
+    if (tid == 0) over = 0;
+    const int64_t pbeg = static_cast<int64_t>(blockIdx.y) * pix_per_split;
+    const int64_t pend = min(m, pbeg + pix_per_split);
+    const int64_t rounds = (pend - pbeg + static_cast<int64_t>(nwarps) * kPackPix - 1) / (static_cast<int64_t>(nwarps) * kPackPix);
+    const uint8_t* Dt = D + static_cast<int64_t>(t0) * ldd;
+    __syncthreads();
+
+    // the accumulators into this CTA's partials, then zero; whole CTA
+    auto empty = [&]() {
+        for (int idx = tid; idx < k * kWords; idx += blockDim.x) {
+            const int i = idx / kWords, w = idx % kWords;
+            const int32_t v = acc[idx];
+            if (v != 0) {
+                const int32_t lo = static_cast<int16_t>(v & 0xffff), hi = (v - lo) >> 16;
+                int32_t* d = dst + static_cast<int64_t>(i) * n + t0 + 2 * w;
+                if (2 * w < nt) d[0] += lo;
+                if (2 * w + 1 < nt) d[1] += hi;
+                acc[idx] = 0;
+            }
+        }
+        for (int idx = tid; idx < k; idx += blockDim.x) cnt[idx] = 0;
+    };
+    // counts the entries [a, b) of this warp's pixels
+    auto count = [&](int64_t a, int64_t b) {
+        for (int64_t e = a + lane; e < b; e += 32) {
+            const int i = row_idx[e] & 0x7fffffff;
+            if (atomicAdd(cnt + i, 1) >= kPackLimit) over = 1;
+        }
+    };
+
+    // the words of a tile (lane: pixels 4 lane .. 4 lane + 3 of every frame),
+    // loaded one round ahead so that they arrive while the present one is added
+    uint32_t w[kFrames];
+    auto pixels = [&](int64_t rd) {
+        const int64_t j = pbeg + (rd * nwarps + wid) * kPackPix;
+        return static_cast<int>(max(static_cast<int64_t>(0), min(static_cast<int64_t>(kPackPix), pend - j)));
+    };
+    auto load = [&](int64_t rd) {
+        const int np = pixels(rd);
+        const uint8_t* src = Dt + pbeg + (rd * nwarps + wid) * kPackPix + 4 * lane;
+#pragma unroll
+        for (int t = 0; t < kFrames; ++t) w[t] = 0u;
+        if (4 * lane + 4 <= np) {
+#pragma unroll
+            for (int t = 0; t < kFrames; ++t)
+                if (t < nt) w[t] = __ldg(reinterpret_cast<const uint32_t*>(src + static_cast<int64_t>(t) * ldd));
+        } else if (4 * lane < np) {
+#pragma unroll
+            for (int t = 0; t < kFrames; ++t)
+                if (t < nt)
+                    for (int i = 0; 4 * lane + i < np; ++i)
+                        w[t] |= static_cast<uint32_t>(src[static_cast<int64_t>(t) * ldd + i]) << (8 * i);
+        }
+    };
+    load(0);
+    for (int64_t rd = 0; rd < rounds; ++rd) {
+        const int64_t j0 = pbeg + (rd * nwarps + wid) * kPackPix;
+        const int np = pixels(rd);
+        // 4 pixels x 4 frames at a time, transposed
+#pragma unroll
+        for (int fq = 0; fq < kQuads; ++fq) {
+            const uint32_t a01 = __byte_perm(w[4 * fq], w[4 * fq + 1], 0x5140);
+            const uint32_t b01 = __byte_perm(w[4 * fq], w[4 * fq + 1], 0x7362);
+            const uint32_t a23 = __byte_perm(w[4 * fq + 2], w[4 * fq + 3], 0x5140);
+            const uint32_t b23 = __byte_perm(w[4 * fq + 2], w[4 * fq + 3], 0x7362);
+            // pixel 4 lane + i in row 32 i + lane: the stores of a warp, an odd
+            // stride apart, meet no bank twice
+            uint32_t* o = tile + lane * kLd + fq;
+            o[0] = __byte_perm(a01, a23, 0x5410);
+            o[32 * kLd] = __byte_perm(a01, a23, 0x7632);
+            o[64 * kLd] = __byte_perm(b01, b23, 0x5410);
+            o[96 * kLd] = __byte_perm(b01, b23, 0x7632);
+        }
+        if (rd + 1 < rounds) load(rd + 1);
+        // column bounds of the lane's pixels, from the tile's first entry on
+        int64_t e0 = 0, e1 = 0;
+        int cp[4] = {0, 0, 0, 0};
+        if (np > 0) {
+            e0 = col_ptr[j0];
+            e1 = col_ptr[j0 + np];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) cp[i] = static_cast<int>(col_ptr[j0 + min(4 * lane + i, np)] - e0);
+            count(e0, e1);
+        }
+        __syncthreads();
+        bool direct = false;
+        if (over != 0) {                             // the same for every thread
+            empty();
+            __syncthreads();
+            if (tid == 0) over = 0;
+            __syncthreads();
+            if (np > 0) count(e0, e1);
+            __syncthreads();
+            direct = over != 0;
+            if (direct) {
+                __syncthreads();
+                for (int idx = tid; idx < k; idx += blockDim.x) cnt[idx] = 0;
+                if (tid == 0) over = 0;
+            }
+        }
+        if (np > 0) {
+            __syncwarp();
+            const int total = static_cast<int>(e1 - e0);
+            for (int base = 0; base < total; base += 32) {
+                // lane e: entry base + e, its row, sign and pixel
+                const int idx = base + lane;
+                uint32_t code = 0u;
+                int pix = 0;
+                if (idx < total) code = static_cast<uint32_t>(row_idx[e0 + idx]);
+                // the lane that holds the entry's pixel: the last whose first entry is not past it
+                {
+                    int lo = 0;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) {
+                        const int c = __shfl_sync(0xffffffffu, cp[0], lo + o);
+                        if (c <= idx) lo += o;
+                    }
+                    const int c1 = __shfl_sync(0xffffffffu, cp[1], lo), c2 = __shfl_sync(0xffffffffu, cp[2], lo),
+                              c3 = __shfl_sync(0xffffffffu, cp[3], lo);
+                    pix = 4 * lo + (c1 <= idx) + (c2 <= idx) + (c3 <= idx);
+                }
+                __syncwarp();
+                {
+                    const uint32_t row = code & 0x7fffffffu, trow = static_cast<uint32_t>((pix & 3) * 32 + (pix >> 2));
+                    list[lane] = make_uint4(tile_s + trow * (kLd * 4u), acc_s + row * (kWords * 4u),
+                                            (code & 0x80000000u) ? 0xffffffffu : 1u, row);
+                }
+                __syncwarp();
+                const int cntb = min(32, total - base);
+                if (!direct) {
+                    // eight entries at a time: their loads before their adds
+                    int e = lane / kWords;
+                    for (; e + 7 * kSub < cntb; e += 8 * kSub) {
+                        uint4 ds[8];
+                        uint32_t w8[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) ds[u] = list[e + u * kSub];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w8[u]) : "r"(ds[u].x + tcol) : "memory");
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(ds[u].y + acol),
+                                         "r"(__byte_perm(w8[u], 0u, half) * ds[u].z)
+                                         : "memory");
+                    }
+                    for (; e < cntb; e += kSub) {
+                        const uint4 d = list[e];
+                        uint32_t w1;
+                        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w1) : "r"(d.x + tcol) : "memory");
+                        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(d.y + acol),
+                                     "r"(__byte_perm(w1, 0u, half) * d.z)
+                                     : "memory");
+                    }
+                } else {
+                    const int l = lane % kWords;
+                    for (int e = lane / kWords; e < cntb; e += kSub) {
+                        const uint4 d = list[e];
+                        uint32_t w1;
+                        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w1) : "r"(d.x + tcol) : "memory");
+                        const uint32_t two = __byte_perm(w1, 0u, half);
+                        int32_t* g = dst + static_cast<int64_t>(d.w) * n + t0 + 2 * l;
+                        if (2 * l < nt) atomicAdd(g, static_cast<int32_t>((two & 0xffffu) * d.z));
+                        if (2 * l + 1 < nt) atomicAdd(g + 1, static_cast<int32_t>((two >> 16) * d.z));
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+    empty();
+}
+
 __global__ void sparse_reduce_kernel(const int32_t* __restrict__ part, int splits, int k, int n,
                                      double* __restrict__ DY) {
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -317,6 +546,41 @@ cdmd_status launch_sketch_gather(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int
         const int64_t tot = static_cast<int64_t>(k) * n;
         rowsample_sketch_kernel<<<static_cast<unsigned>((tot + 255) / 256), 256, 0, stream>>>(D, n, ldd, k, meas->rows, DY);
         CDMD_CHECK_LAUNCH("rowsample_sketch_kernel");
+        return CDMD_OK;
+    }
+    // The packed kernel wherever a 4-byte load cannot be misaligned and a round of
+    // it (every warp's 128 pixels) is expected to bring a row no more than a
+    // quarter of the entries its 16-bit sums hold (density up to 0.0104 with 24
+    // warps; at 0.01, 1280x720x64, 340 us against the plain kernel's 367); denser
+    // C takes the plain one.
+    const int frames = k <= 2048 ? 32 : 16;
+    const size_t tile = static_cast<size_t>(pack_tile_words(frames)) * sizeof(uint32_t);
+    const size_t fixed = static_cast<size_t>(k) * (2 * frames) + static_cast<size_t>((k + 3) / 4 * 4) * 4;
+    const int warps = static_cast<int>(std::min<size_t>(24, (kPackSmemMax - 256 - fixed) / tile));
+    if (reinterpret_cast<uintptr_t>(D) % 4 == 0 && ldd % 4 == 0 &&
+        meas->density * warps * kPackPix <= 0.25 * kPackLimit) {
+        const int slabs = (n + frames - 1) / frames;
+        const int fps = std::min(frames, ((n + slabs - 1) / slabs + 3) / 4 * 4);
+        const size_t smem = fixed + warps * tile;
+        const int per_sm = 2 * (smem + 1024) <= kPackSmemMax ? 2 : 1;
+        int64_t splits = std::max<int64_t>(1, static_cast<int64_t>(per_sm) * ctx->num_sms / slabs);
+        splits = std::min<int64_t>(splits, std::max<int64_t>(1, m / (2 * warps * kPackPix)));
+        const int64_t pps = ((m + splits - 1) / splits + 3) / 4 * 4;     // splits start on a 4-byte boundary
+        splits = (m + pps - 1) / pps;
+        int32_t* part = nullptr;
+        cdmd_status st = ensure_buffer(ctx, BUF_SKETCH_PARTIAL, static_cast<size_t>(splits) * k * n * sizeof(int32_t),
+                                       reinterpret_cast<void**>(&part));
+        if (st != CDMD_OK) return st;
+        auto kern = frames == 32 ? sparse_packed_kernel<32> : sparse_packed_kernel<16>;
+        CDMD_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             static_cast<int>(kPackSmemMax - 256)));
+        kern<<<dim3(slabs, static_cast<unsigned>(splits)), warps * 32, smem, stream>>>(
+            D, m, n, ldd, k, meas->col_ptr, meas->row_idx, pps, fps, part);
+        CDMD_CHECK_LAUNCH("sparse_packed_kernel");
+        const int64_t tot = static_cast<int64_t>(k) * n;
+        sparse_reduce_kernel<<<static_cast<unsigned>((tot + 255) / 256), 256, 0, stream>>>(
+            part, static_cast<int>(splits), k, n, DY);
+        CDMD_CHECK_LAUNCH("sparse_reduce_kernel");
         return CDMD_OK;
     }
     // frames per slab: 32 while the k x 33 integer tile fits, else 16
