@@ -46,35 +46,28 @@ __device__ __forceinline__ void record_status(int* status, int code) {
 // Philox4x32-10 (Salmon, Moraes, Dror & Shaw, SC'11): ten rounds of two
 // 32x32->64 bit products with Weyl-bumped round keys.
 // ---------------------------------------------------------------------------
-// 1/a and 1/sqrt(a) in FP64 by the Newton-Raphson method: start from the
-// hardware's approximate reciprocal (rcp.approx.ftz.f64) or reciprocal square
-// root (rsqrt.approx.ftz.f64) and take two Newton steps for the root of
-// f(x) = 1/x - a, x <- x (2 - a x) = x + x (1 - a x), or of f(y) = 1/y^2 - a,
-// y <- y (3 - a y^2) / 2 = y + y (1/2 - (a/2) y^2).  Each step roughly doubles
-// the number of correct bits, so two steps from the approximation reach FP64
+// 1/a and 1/sqrt(a) in FP64: the hardware's approximation (rcp.approx.ftz.f64,
+// rsqrt.approx.ftz.f64: about 20 bits) and one step of Householder's method of
+// third order, which triples the correct bits: with e = 1 - a x,
+// x <- x (1 + e + e^2); with e = 1 - a y^2, y <- y (1 + e/2 + 3 e^2 / 8).  Three
+// and five dependent FP64 instructions; two Newton steps, which reach the same
 // rounding level (a few ulp; bounded by a GPU test against IEEE division and
-// square root).  Zero and subnormal inputs are flushed (ftz); callers pass
-// normal positive values.  They replace a division or square root (hundreds of
-// cycles in FP64 on this GPU) on the latency-critical paths of the small solves.
+// square root), take four and seven, 64 clocks each.  Zero and subnormal inputs
+// are flushed (ftz); callers pass normal positive values (rcp64: of either
+// sign).  They replace a division or square root (hundreds of cycles in FP64 on
+// this GPU) on the latency-critical paths of the small solves.
 __device__ __forceinline__ double rcp64(double a) {
     double x;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(a));
-    double e = fma(-a, x, 1.0);
-    x = fma(x, e, x);
-    e = fma(-a, x, 1.0);
-    x = fma(x, e, x);
-    return x;
+    const double e = fma(-a, x, 1.0);
+    return fma(x, fma(e, e, e), x);
 }
 
 __device__ __forceinline__ double rsqrt64(double a) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    const double h = 0.5 * a;
-    double t = fma(-h * y, y, 0.5);
-    y = fma(y, t, y);
-    t = fma(-h * y, y, 0.5);
-    y = fma(y, t, y);
-    return y;
+    const double e = fma(-(a * y), y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 key) {

@@ -39,6 +39,7 @@
 #include <cooperative_groups.h>
 
 #include "cdmd_internal.cuh"
+#include "tc_common.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -210,16 +211,22 @@ __global__ void gram_reduce_kernel(const __grid_constant__ SolveBatch sb, int sp
 // the scalar chains.  Column c is reached with reflector c-1 = (v, tau) in
 // every CTA and, from the exchange, u = A v and the column a_l = A[l][c] of
 // the rows as updated before it.  One iteration:
-//   kc = tau^2/2 v^T u, w = tau u - kc v, and the column of the updated matrix
-//   x = a - v w_c - w (formed in every CTA, so no CTA has to announce it);
-//   the row warps apply A -= v w^T + w v^T to their rows i > c and take
+//   with t = tau u and k2 = tau^2 v^T u the update is
+//   A -= v t^T + (t - k2 v) v^T, so its column c is
+//   x = a - t_c v - t + k2 v (formed in every CTA: no CTA has to announce it);
+//   the row warps apply the update to their rows i > c and take
 //   s_i = (A x)_i in the same pass over shared memory, while the scalar warp
 //   turns x into reflector c: H = I - tau v v^T, v = (x - alpha e_1) / v0 with
 //   a leading 1, tau in [1, 2], neither growing however small the column is;
 //   u_i = (s_i - alpha A[i][c+1]) / v0 = (A v)_i and A[i][c+1] go to every
-//   CTA (one 16-byte distributed-shared-memory store per row and CTA).
-// One cluster barrier per column: the exchange buffer alternates, and every
-// CTA has read buffer c before it arrives at the barrier of c+1.
+//   CTA, one 16-byte asynchronous distributed-shared-memory store per row and
+//   CTA, counted on an mbarrier of the receiver.
+// No cluster barrier inside the loop: the exchange buffer alternates, and a CTA
+// that has every CTA's column c + 1 knows that they have all read column c,
+// whose buffer and barrier column c + 2 takes.  For that every CTA sends with
+// every column, one whose rows are all done a token of a row's size (without it
+// the others could run ahead of such a CTA by more than a column).  The waits
+// are bounded.
 // Bound by the FP64 unit.  A DP instruction holds its scheduler's port 64
 // clocks however many lanes are active or predicated off, and an SM retires one
 // per 19 clocks (micro-probe).  So a row is passed over once for update and
@@ -227,7 +234,8 @@ __global__ void gram_reduce_kernel(const __grid_constant__ SolveBatch sb, int sp
 // reduction (six additions instead of twenty), loops branch over idle rows and
 // lanes instead of predicating them, and the next reflector's norm and
 // reciprocals run on a warp of their own beside the pass.
-// Measured, p = 199: 0.70 ms on 16 CTAs, 0.86 ms on 8; 1.53 ms for a form with
+// Measured, p = 199: 0.68 ms on 16 CTAs; 0.73 ms with w = t - (k2 / 2) v
+// formed as a vector and a cluster barrier per column; 1.53 ms for a form with
 // the update and the product as two passes, one reduction per row and two
 // barriers per column.
 // Outputs: diagonal dd[p], off-diagonal ee[p-1], reflectors Hv[j*p + l]
@@ -235,12 +243,12 @@ __global__ void gram_reduce_kernel(const __grid_constant__ SolveBatch sb, int sp
 // ---------------------------------------------------------------------------
 constexpr int kTriRows = 4;                         // rows per row warp
 
-// Rows slot, slot + W, .. (NR of them) of this CTA: A -= v w^T + w v^T on the
-// columns past c, and the products of the updated rows with x, summed over the
+// Rows slot, slot + W, .. (NR of them) of this CTA: A -= v t^T + (t - k2 v) v^T
+// on the columns past c, and the products of the updated rows with x, summed over the
 // warp: lane group g of 32 / NR' lanes (NR' = 1, 2 or 4) ends with row g's.
 template <int NR>
 __device__ __forceinline__ double tri_pass(double* Aloc, int slot, int W, int rank, int P, int c, int p,
-                                           const double* v, const double* wv, const double* xv) {
+                                           const double* v, const double* tv, const double* xv, double k2) {
     const int lane = threadIdx.x & 31;
     double vi[NR], wi[NR], s[NR];
     double* a[NR];
@@ -248,16 +256,16 @@ __device__ __forceinline__ double tri_pass(double* Aloc, int slot, int W, int ra
     for (int e = 0; e < NR; ++e) {
         const int li = slot + W * e;
         vi[e] = v[rank + P * li];
-        wi[e] = wv[rank + P * li];
+        wi[e] = fma(-k2, vi[e], tv[rank + P * li]);
         a[e] = Aloc + static_cast<size_t>(li) * p;
         s[e] = 0.0;
     }
 #pragma unroll 1
     for (int l = c + 1 + lane; l < p; l += 32) {
-        const double vv = v[l], ww = wv[l], xx = xv[l];
+        const double vv = v[l], tt = tv[l], xx = xv[l];
 #pragma unroll
         for (int e = 0; e < NR; ++e) {
-            const double t = fma(-vi[e], ww, fma(-wi[e], vv, a[e][l]));
+            const double t = fma(-vi[e], tt, fma(-wi[e], vv, a[e][l]));
             a[e][l] = t;
             s[e] = fma(t, xx, s[e]);
         }
@@ -283,6 +291,17 @@ __device__ __forceinline__ double tri_pass(double* Aloc, int slot, int W, int ra
     return t;
 }
 
+// One row's (u, a) into the same place of CTA `rank`'s shared memory, counted
+// (16 bytes) on that CTA's mbarrier.
+__device__ __forceinline__ void store_async(double2* dst, uint64_t* bar, int rank, double u, double a) {
+    uint32_t d, m;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(tc::smem_u32(dst)), "r"(rank));
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(m) : "r"(tc::smem_u32(bar)), "r"(rank));
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(d), "d"(u),
+                 "d"(a), "r"(m)
+                 : "memory");
+}
+
 template <int W>
 __global__ void __launch_bounds__((W + 1) * 32)
 tridiag_kernel(const __grid_constant__ SolveBatch sb) {
@@ -295,13 +314,15 @@ tridiag_kernel(const __grid_constant__ SolveBatch sb) {
     const int P = static_cast<int>(cluster.num_blocks());
     const int rank = static_cast<int>(cluster.block_rank());
     const int rows_per = (p + P - 1) / P;
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) double sm[];
     double2* ua = reinterpret_cast<double2*>(sm);              // 2 x p: (u_l, A[l][c]) of every row, alternating
     double* v = sm + 4 * static_cast<size_t>(p);               // p
-    double* wv = v + p;                                        // p
-    double* xv = wv + p;                                       // p
-    double* scal = xv + p;                                     // kc, alpha, 1 / v0, tau
-    double* Aloc = scal + 4;                                   // rows_per x p
+    double* tv = v + p;                                        // p
+    double* xv = tv + p;                                       // p
+    double* scal = xv + p;                                     // k2, alpha, 1 / v0, tau, tau^2
+    uint64_t* full = reinterpret_cast<uint64_t*>(scal + 6);    // [2] a column's payload has landed
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(scal + 8);
+    double* Aloc = scal + 10;                                  // rows_per x p
     const int tid = threadIdx.x;
     const int lane = tid & 31, wid = tid >> 5;
     const bool scalar_warp = wid == W;
@@ -316,41 +337,49 @@ tridiag_kernel(const __grid_constant__ SolveBatch sb) {
         ua[l] = make_double2(0.0, R[static_cast<int64_t>(l) * n]);
         v[l] = 0.0;
     }
-    if (tid == 0) scal[3] = 0.0;
-    // every CTA of the cluster has started before any CTA writes into
-    // another's shared memory
+    if (tid == 0) {
+        scal[3] = scal[4] = 0.0;
+        tc::mbar_init(&full[0], 1);
+        tc::mbar_init(&full[1], 1);
+        *abort_flag = 0;
+        tc::fence_mbar_init();
+    }
+    // every CTA of the cluster has started (and set up its barriers) before
+    // any CTA writes into another's shared memory
     cluster.sync();
 
+    const int last_row = rank < p ? rank + P * ((p - 1 - rank) / P) : -1;
+    bool ok = true;
     for (int c = 0; c + 1 < p; ++c) {
         const double2* uc = ua + static_cast<size_t>(c & 1) * p;
-        const double tau_prev = scal[3];
-        // x = a - tau u - (tau u_c) v + 2 kc v and w = tau u - kc v: all but
-        // the kc terms while the scalar warp sums v^T u
+        // columns 1, 3, .. come on barrier 1, 2, 4, .. on barrier 0.  A thread
+        // whose wait ran out goes on to the end, so that every thread meets the
+        // same barriers, but announces and sends nothing any more.
+        if (c > 0) ok = ok && tc::mbar_wait_cl(&full[c & 1], static_cast<uint32_t>((c - 1) >> 1) & 1u, abort_flag, sb.status);
+        if (tid == kRowThreads && c + 2 < p && ok)
+            tc::mbar_arrive_expect_tx(&full[(c + 1) & 1], static_cast<uint32_t>(max(p - 1 - c, P)) * 16u);
+        // x: all but the k2 term while the scalar warp sums v^T u
         if (scalar_warp) {
             double s0 = 0.0;
 #pragma unroll 1
             for (int l = c + lane; l < p; l += 32) s0 = fma(v[l], uc[l].x, s0);
             __syncwarp();
             const double vtu = warp_sum(s0);
-            if (lane == 0) scal[0] = (0.5 * tau_prev * tau_prev) * vtu;
+            if (lane == 0) scal[0] = scal[4] * vtu;
         } else {
+            const double tau = scal[3], u0 = uc[c].x;
 #pragma unroll 1
             for (int l = c + tid; l < p; l += kRowThreads) {
                 const double2 g = uc[l];
-                const double tu = tau_prev * g.x;
-                wv[l] = tu;
-                xv[l] = fma(-(tau_prev * uc[c].x), v[l], g.y - tu);
+                tv[l] = tau * g.x;
+                xv[l] = fma(-tau, fma(u0, v[l], g.x), g.y);
             }
         }
         __syncthreads();
+        const double k2 = scal[0];
         if (!scalar_warp) {
-            const double kc = scal[0];
 #pragma unroll 1
-            for (int l = c + tid; l < p; l += kRowThreads) {
-                const double kv = kc * v[l];
-                wv[l] -= kv;
-                xv[l] = fma(2.0, kv, xv[l]);
-            }
+            for (int l = c + tid; l < p; l += kRowThreads) xv[l] = fma(k2, v[l], xv[l]);
         }
         __syncthreads();
         if (c + 2 >= p) break;
@@ -365,18 +394,24 @@ tridiag_kernel(const __grid_constant__ SolveBatch sb) {
             const double tail2 = warp_sum(t0);
             const double x0 = xv[c + 1];
             double alpha = x0, tau = 0.0, inv = 0.0;
-            if (tail2 > 1e-280) {             // else nothing below the sub-diagonal (or a subnormal remainder)
+            // tail2 > 1e-280 and finite, by the high word (an FP64 comparison
+            // costs as much as an FP64 addition); else nothing is left below
+            // the sub-diagonal (or a subnormal remainder)
+            constexpr int kTinyHi = 0x05d00000;            // 1.2e-280
+            if (static_cast<unsigned>(__double2hiint(tail2) - kTinyHi) < static_cast<unsigned>(0x7ff00000 - kTinyHi)) {
                 const double s2 = fma(x0, x0, tail2);
                 const double rs = rsqrt64(s2);
-                alpha = (x0 >= 0.0) ? -(s2 * rs) : s2 * rs;
-                const double v0 = x0 - alpha; // |v0| >= nrm > 0
+                alpha = copysign(s2 * rs, -x0);
+                const double v0 = x0 - alpha;              // |v0| >= nrm > 0
                 inv = rcp64(v0);
-                tau = fabs(v0) * rs;          // 2 v0^2 / (v0^2 + tail2), as v0^2 + tail2 = 2 nrm |v0|
+                tau = fabs(v0) * rs;                       // 2 v0^2 / (v0^2 + tail2), as v0^2 + tail2 = 2 nrm |v0|
             }
+            const double tau2 = tau * tau;
             if (lane == 0) {
                 scal[1] = alpha;
                 scal[2] = inv;
                 scal[3] = tau;
+                scal[4] = tau2;
                 if (rank == 0) {
                     q.dd[c] = xv[c];
                     q.ee[c] = alpha;
@@ -387,33 +422,39 @@ tridiag_kernel(const __grid_constant__ SolveBatch sb) {
             while (rank + P * slot <= c) slot += W;
             nr = (p - 1 - rank - P * slot + P * W) / (P * W);     // floor division: 0 when the first row is past p - 1
             if (rank + P * slot >= p) nr = 0;
-            if (nr == 1) s = tri_pass<1>(Aloc, slot, W, rank, P, c, p, v, wv, xv);
-            else if (nr == 2) s = tri_pass<2>(Aloc, slot, W, rank, P, c, p, v, wv, xv);
-            else if (nr == 3) s = tri_pass<3>(Aloc, slot, W, rank, P, c, p, v, wv, xv);
-            else if (nr == 4) s = tri_pass<4>(Aloc, slot, W, rank, P, c, p, v, wv, xv);
+            if (nr == 1) s = tri_pass<1>(Aloc, slot, W, rank, P, c, p, v, tv, xv, k2);
+            else if (nr == 2) s = tri_pass<2>(Aloc, slot, W, rank, P, c, p, v, tv, xv, k2);
+            else if (nr == 3) s = tri_pass<3>(Aloc, slot, W, rank, P, c, p, v, tv, xv, k2);
+            else if (nr == 4) s = tri_pass<4>(Aloc, slot, W, rank, P, c, p, v, tv, xv, k2);
         }
         __syncthreads();
         if (!scalar_warp) {
             const double alpha = scal[1], inv = scal[2];
             const int gs = nr <= 1 ? 32 : nr == 2 ? 16 : 8;       // lanes that hold one row's sum
             const int e = lane / gs;
-            if (e < nr) {
+            const int b = (c + 1) & 1;
+            if (!ok) {
+            } else if (last_row <= c) {
+                // no row left: a token in the row's place, in a slot that is not read
+                if (tid < P) store_async(ua + static_cast<size_t>(b) * p, &full[b], tid, 0.0, 0.0);
+            } else if (e < nr) {
                 const int li = slot + W * e;
                 const double a1 = Aloc[static_cast<size_t>(li) * p + c + 1];
-                const double2 g = make_double2(fma(-alpha, a1, s) * inv, a1);
-                double2* dst = ua + static_cast<size_t>((c & 1) ^ 1) * p + rank + P * li;
-                for (int rr = lane & (gs - 1); rr < P; rr += gs) *cluster.map_shared_rank(dst, rr) = g;
+                const double u = fma(-alpha, a1, s) * inv;
+                for (int rr = lane & (gs - 1); rr < P; rr += gs)
+                    store_async(ua + static_cast<size_t>(b) * p + rank + P * li, &full[b], rr, u, a1);
             }
             // reflector c into this CTA's v (every reader of the old one is past the barrier above)
+            const bool lead = (__double2hiint(inv) & 0x7fffffff) != 0;   // else tau = 0: the reflector is zero
 #pragma unroll 1
             for (int l = c + 1 + tid; l < p; l += kRowThreads) {
-                // tau = 0 comes with 1 / v0 = 0: the reflector is zero
-                const double val = (l == c + 1 && inv != 0.0) ? 1.0 : xv[l] * inv;
+                double val = xv[l] * inv;
+                if (l == c + 1 && lead) val = 1.0;
                 v[l] = val;
                 if (c % P == rank) q.Hv[static_cast<int64_t>(c) * p + l] = val;
             }
         }
-        cluster.sync();
+        __syncthreads();
     }
     // trailing 2 x 2 block: column p-2 is x, the last diagonal entry takes the last update
     if (tid == 0) {
@@ -424,10 +465,14 @@ tridiag_kernel(const __grid_constant__ SolveBatch sb) {
                 q.dd[p - 2] = xv[p - 2];
                 q.ee[p - 2] = xv[p - 1];
             }
-            if ((p - 1) % P == rank)
-                q.dd[p - 1] = fma(-2.0 * v[p - 1], wv[p - 1], Aloc[static_cast<size_t>((p - 1) / P) * p + p - 1]);
+            if ((p - 1) % P == rank) {
+                const double vl = v[p - 1], tl = tv[p - 1];
+                q.dd[p - 1] = fma(-vl, tl, fma(-fma(-scal[0], vl, tl), vl, Aloc[static_cast<size_t>((p - 1) / P) * p + p - 1]));
+            }
         }
     }
+    // no CTA leaves while another's stores to it, or its own, may be in flight
+    cluster.sync();
 }
 
 // ---------------------------------------------------------------------------
@@ -2470,7 +2515,7 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
             const int csize = ctas[ci];
             const int rows_per = (p + csize - 1) / csize;
             const int warps = rows_per <= 4 * kTriRows ? 4 : rows_per <= 8 * kTriRows ? 8 : 16;
-            const size_t smem = (static_cast<size_t>(rows_per) * p + 7 * static_cast<size_t>(p) + 4) * sizeof(double);
+            const size_t smem = (static_cast<size_t>(rows_per) * p + 7 * static_cast<size_t>(p) + 10) * sizeof(double);
             if (smem > kMaxOptInSmem || rows_per > warps * kTriRows) continue;
             void (*kern)(SolveBatch) = warps == 4   ? tridiag_kernel<4>
                                        : warps == 8 ? tridiag_kernel<8>
