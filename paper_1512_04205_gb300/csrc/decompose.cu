@@ -9,31 +9,36 @@
 //            compressed modes Phi_Y = Y' G (Remark 3)
 // so no kernel after the Gram touches the k-long sketch rows again.
 //
-// FP64 on this GPU is slow in both senses: about 1/64 of the FP32 FMA rate,
-// 64 cycles for a dependent FMA and ~640 for a division or square root.  So
-// the O(p^3) / O(p^2 r) stages are spread over SMs, serial chains are kept
-// short (several independent accumulators, more lanes), divisions and square
-// roots on critical paths become approximate reciprocals refined by Newton
-// steps, and the one iteration-heavy r x r stage runs in FP32 with an FP64
-// Newton correction per eigenpair:
+// FP64 on this GPU is slow in both senses (micro-probe): a DP instruction holds
+// its scheduler's port 64 clocks whatever its lanes do, an SM retires one per
+// 19 clocks, a division or square root takes ~640.  So
+// the O(p^3) / O(p^2 r) stages are spread over SMs and over the four
+// schedulers, serial chains are kept short, divisions and square
+// roots on critical paths become approximate reciprocals with one third-order
+// step, searches and factorisations run in FP32 or pairs of floats where
+// FP64 arithmetic decides the result afterwards, and the one iteration-heavy
+// r x r stage runs in FP32 with an FP64 Newton correction per eigenpair:
 //   gram_partial / gram_reduce   multi-CTA, split over the sketch rows
 //   tridiag                      Householder tridiagonalisation of Y^T Y on a
 //                                thread-block cluster, rows distributed over
-//                                the CTAs' shared memory, vectors exchanged
-//                                through distributed shared memory
+//                                the CTAs' shared memory, columns exchanged
+//                                by asynchronous stores into it
 //   tridiag_eigpair              one CTA per wanted eigenvalue: Sturm-count
-//                                multisection (64 shifts per pass), then
-//                                inverse iteration with reciprocal pivots
-//   orthonormalise               classical Gram-Schmidt, twice (one CTA)
+//                                multisection (128 shifts per pass), then
+//                                inverse iteration with reciprocal pivots;
+//                                further CTAs: blocks of reflectors as I - V T V^T
+//   orthogonality                one first-order Gram-Schmidt step, a CTA per column
 //   backtransform                one CTA per eigenvector: V = Q z
 //   bmat, atilde                 B = (Y^T Y') V, A~ = S^-1 V^T B S^-1
-//   eig_f32                      one warp: Hessenberg + complex-shift QR on A~
+//   eig_f32                      Hessenberg + complex-shift QR on A~
 //                                in FP32, eigenvectors by back-substitution
-//   eig_refine                   one CTA per eigenpair: FP64 Newton on
-//                                (A~ - mu) w = 0 with one entry of w fixed
-//   eig_order                    normalise, order (conjugate pairs adjacent)
-//   gmat                         G = V S^-1 W
-//   hmat                         H = (Y'^T Y') G, M = G^H H, c = G^H (Y'^T y1)
+//   eig_refine                   one CTA per eigenpair: FP64 residuals,
+//                                corrections from an FP32 inverse (Newton on
+//                                (A~ - mu) w = 0 with one entry of w fixed)
+//   eig_finish                   FP64 QR where a pair did not settle, then
+//                                normalise and order (conjugate pairs adjacent)
+//   modes                        G = V S^-1 W, and M = G^H H G, c from the
+//                                reduced matrices
 //   omp                          one warp: OMP / least squares in Gram form
 //   phiy (optional)              Phi_Y = Y' G
 #include <cooperative_groups.h>
@@ -537,6 +542,51 @@ __device__ __forceinline__ int sturm_count_f32(const float* d, const float* e2, 
     return c;
 }
 
+// The same count with entries, shift and minors as sums of two floats (about
+// 46 bits; Dekker's and Knuth's error-free transformations), for a second
+// bracket: some 30 FP32 instructions a step where the FP64 form holds the
+// scheduler 192 clocks.  Rescaled every two steps.
+__device__ __forceinline__ int sturm_count_2f(const float2* d, const float2* e2, int p, float xh, float xl) {
+    float ah = d[0].x - xh, al = 0.0f, bh = 1.0f, bl = 0.0f;
+    {
+        const float bb = ah - d[0].x;
+        al = ((d[0].x - (ah - bb)) + (-xh - bb)) + (d[0].y - xl);
+        const float t = ah + al;
+        al -= t - ah;
+        ah = t;
+    }
+    int c = static_cast<int>(__float_as_uint(ah) >> 31);
+    for (int i = 1; i < p; ++i) {
+        const float2 di = d[i], ei = e2[i - 1];
+        // s = d - x
+        const float sh = di.x - xh, sb = sh - di.x;
+        const float sl = ((di.x - (sh - sb)) + (-xh - sb)) + (di.y - xl);
+        // p = s a, q = e2 b
+        const float ph = sh * ah, pl = fmaf(sl, ah, fmaf(sh, al, fmaf(sh, ah, -ph)));
+        const float qh = ei.x * bh, ql = fmaf(ei.y, bh, fmaf(ei.x, bl, fmaf(ei.x, bh, -qh)));
+        // t = p - q
+        const float th = ph - qh, tb = th - ph;
+        const float tl = ((ph - (th - tb)) + (-qh - tb)) + (pl - ql);
+        const float t = th + tl;
+        c += static_cast<int>((__float_as_uint(t) ^ __float_as_uint(ah)) >> 31);
+        bh = ah;
+        bl = al;
+        ah = t;
+        al = tl - (t - th);
+        if ((i & 1) == 0) {
+            const int ex = static_cast<int>(__float_as_uint(ah) >> 23) & 0xff;
+            if (ex > 127 + 16 || (ex > 0 && ex < 127 - 16)) {
+                const float sc = __uint_as_float(static_cast<uint32_t>(254 - ex) << 23);
+                ah *= sc;
+                al *= sc;
+                bh *= sc;
+                bl *= sc;
+            }
+        }
+    }
+    return c;
+}
+
 __device__ __forceinline__ int sturm_count(const double* d, const double* e2, int p, double x) {
     double a = d[0] - x, b = 1.0;
     int c = static_cast<int>(static_cast<unsigned>(__double2hiint(a)) >> 31);
@@ -569,14 +619,17 @@ __device__ __forceinline__ int first_set(bool flag, unsigned* ball, int turn) {
 // Eigenpair `w` (descending) of T, one CTA of four warps, one per scheduler:
 // a DP instruction holds its scheduler 64 clocks whatever its lanes do, so four
 // warps of one shift each run a Sturm pass over 128 shifts in the time one
-// warp takes over 32.  Three passes in FP32 narrow the interval to 2 units of
-// 1e-6 of the norm (margin: 16 eps32, above the count's backward error);
-// FP64 passes, the first of which tests both ends of that bracket (else
-// everything is repeated from the Gershgorin interval), go on to eps.
+// warp takes over 32.  Three passes in FP32 narrow the interval to a few 1e-6 of the
+// norm (margin: 16 eps32, above the count's backward error), three on pairs of
+// floats to 3e-12 (margin 2^-42), and two in FP64 to eps; the first of those
+// tests both ends of the bracket (else everything is repeated from the
+// Gershgorin interval).
 // Inverse iteration: LU with partial pivoting and two solves by one thread,
 // each step one or two dependent DP instructions; everything that is not on
 // that chain (d - mu, the scaled rows of U, the divisions by the pivots) is
 // done by all threads between the chains.
+// p = 199, r = 20, one CTA per pair: 218 us; 265 with four FP64 passes in place of the pairs of
+// floats and a branch on every pivot; 0.62 ms on one warp per pair, all FP64.
 __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm) {
     const double *dd = q.dd, *ee = q.ee;
     const int p = q.p;
@@ -592,6 +645,9 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
     int* piv = reinterpret_cast<int*>(z + p);          // p
     float* d32 = reinterpret_cast<float*>(piv + p);    // p
     float* e32 = d32 + p;                              // p
+    // the pairs of floats take the places of what is filled after the search
+    float2* d2f = reinterpret_cast<float2*>(lmul);     // p
+    float2* e2f = reinterpret_cast<float2*>(udg);      // p
     __shared__ double red[12];
     __shared__ unsigned ball[8];
     __shared__ int flags[4];
@@ -635,9 +691,11 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
         const double sc = __hiloint2double((2046 - ex - 1) << 20, 0);     // tn sc in [1/2, 1)
         const double isc = __hiloint2double((ex + 1) << 20, 0);
         for (int i = tid; i < p; i += kEigThreads) {
-            const float ef = static_cast<float>(e[i] * sc);
-            d32[i] = static_cast<float>(d[i] * sc);
-            e32[i] = ef * ef;
+            const double ds = d[i] * sc, es = e2[i] * sc * sc;
+            d32[i] = static_cast<float>(ds);
+            e32[i] = static_cast<float>(es);
+            d2f[i] = make_float2(d32[i], static_cast<float>(ds - static_cast<double>(d32[i])));
+            e2f[i] = make_float2(e32[i], static_cast<float>(es - static_cast<double>(e32[i])));
         }
         __syncthreads();
         float flo = static_cast<float>(glo * sc), fhi = static_cast<float>(ghi * sc);
@@ -649,9 +707,21 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
             fhi = (f == kEigThreads) ? fhi : fmaf(step, static_cast<float>(f + 1), flo);
             flo = nlo;
         }
-        const double margin = 16.0 * 1.1920929e-07;
-        lo = (static_cast<double>(flo) - margin) * isc;
-        hi = (static_cast<double>(fhi) + margin) * isc;
+        const double margin = 16.0 * 1.1920929e-07, margin2 = 2.3e-13;
+        lo = static_cast<double>(flo) - margin;
+        hi = static_cast<double>(fhi) + margin;
+        for (int it = 0; it < 3; ++it) {
+            const double step = (hi - lo) * (1.0 / (kEigThreads + 1));
+            const double x = fma(step, static_cast<double>(tid + 1), lo);
+            const float xh = static_cast<float>(x), xl = static_cast<float>(x - static_cast<double>(xh));
+            const bool above = sturm_count_2f(d2f, e2f, p, xh, xl) > idx;
+            const int f = first_set(above, ball, turn++);
+            const double nlo = (f == 0) ? lo : fma(step, static_cast<double>(f), lo);
+            hi = (f == kEigThreads) ? hi : fma(step, static_cast<double>(f + 1), lo);
+            lo = nlo;
+        }
+        lo = (lo - margin2) * isc;
+        hi = (hi + margin2) * isc;
         // the ends of the bracket and 126 shifts between them
         const double step = (hi - lo) * (1.0 / (kEigThreads - 1));
         const bool above = sturm_count(d, e2, p, fma(step, static_cast<double>(tid), lo)) > idx;
@@ -710,29 +780,22 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
         int anyp = 0;
         for (int i = 0; i + 1 < p; ++i) {
             const double sub = e[i], nd = udg[i + 1], ns = e[i + 1];
-            // |cur| >= |sub| by the high words: at most 2^-20 off an exact comparison
-            if ((__double2hiint(cur) & 0x7fffffff) >= (__double2hiint(sub) & 0x7fffffff)) {
-                if ((__double2hiint(cur) & 0x7fffffff) == 0 && __double2loint(cur) == 0) cur = tiny;
-                const double inv = rcp64(cur);
-                const double f = sub * inv;
-                cur = fma(-f, sup, nd);
-                invd[i] = inv;
-                lmul[i] = f;
-                u1[i] = sup;
-                u2[i] = 0.0;
-                piv[i] = 0;
-                sup = ns;
-            } else {
-                const double inv = rcp64(sub);
-                const double f = cur * inv;
-                cur = fma(-f, nd, sup);
-                invd[i] = inv;
-                lmul[i] = f;
-                u1[i] = nd;
-                u2[i] = ns;
-                piv[i] = 1;
-                anyp = 1;
+            // |cur| < |sub| by the high words: at most 2^-20 off an exact comparison
+            const bool sw = (__double2hiint(cur) & 0x7fffffff) < (__double2hiint(sub) & 0x7fffffff);
+            if (!sw && (__double2hiint(cur) & 0x7fffffff) == 0 && __double2loint(cur) == 0) cur = tiny;
+            const double inv = rcp64(sw ? sub : cur);
+            const double f = (sw ? cur : sub) * inv;
+            const double up = sw ? nd : sup;
+            cur = fma(-f, up, sw ? sup : nd);
+            invd[i] = inv;
+            lmul[i] = f;
+            u1[i] = up;
+            u2[i] = sw ? ns : 0.0;
+            piv[i] = sw ? 1 : 0;
+            sup = ns;
+            if (sw) {
                 sup = -f * ns;
+                anyp = 1;
             }
         }
         if ((__double2hiint(cur) & 0x7fffffff) == 0 && __double2loint(cur) == 0) cur = tiny;
@@ -1595,7 +1658,7 @@ eig_refine_kernel(const __grid_constant__ SolveBatch sb) {
     __shared__ double A[kMaxR][kMaxR + 1];
     __shared__ cf M[kMaxR][kMaxR + 1];       // bordered matrix, then its inverse
     __shared__ cd wv[kMaxR], part[4][kMaxR];
-    __shared__ cf rowk[kMaxR], resf[kMaxR];
+    __shared__ cf rowk[kMaxR], resf[kMaxR], colk[2][kMaxR];
     __shared__ int perm[kMaxR];
     __shared__ int state;                    // 0: go on, 1: settled, 2: gave up
     const int j = blockIdx.x;
@@ -1624,58 +1687,66 @@ eig_refine_kernel(const __grid_constant__ SolveBatch sb) {
     if (lane < r && wid == 0) wv[lane] = {static_cast<double>(wf.x), static_cast<double>(wf.y)};
     if (tid == 0) state = 0;
     __syncthreads();
-    // FP32 inverse, warp 0: lane i holds row i in registers; step k scales the
-    // pivot row, passes it round through shared memory and clears column k
-    if (wid == 0) {
-        cf m[kMaxR];
+    // FP32 inverse: lane i of warp w holds columns 8w .. 8w + 7 of row i in
+    // registers.  Step k: the warp that holds column k picks the pivot row and
+    // passes the column round through shared memory; every warp scales the
+    // pivot row's part (passed round within the warp) and clears its columns.
+    // r = 20, whole kernel: 20 us; 66 with all columns in one warp's registers.
+    {
+        constexpr int kC = kMaxR / (kRefThreads / 32);
+        const int c0 = kC * wid;
+        cf m[kC];
 #pragma unroll
-        for (int c = 0; c < kMaxR; ++c) {
+        for (int e = 0; e < kC; ++e) {
+            const int c = c0 + e;
             cf v = {lane == c ? 1.0f : 0.0f, 0.0f};      // identity past r
             if (lane < r && c < r) {
                 v = {static_cast<float>(A[lane][c]), 0.0f};
                 if (c == lane) v = fsubc(v, muf);
                 if (c == pidx) v = {-wf.x, -wf.y};
             }
-            m[c] = v;
+            m[e] = v;
         }
         bool used = lane >= r;
         int mine = lane;                                  // the step this row was pivot of
 #pragma unroll
         for (int k = 0; k < kMaxR; ++k) {
-            if (k < r) {
-                float mag = used ? -1.0f : fabs2c(m[k]);
-                float best = mag;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-                const unsigned bb = __ballot_sync(0xffffffffu, !used && mag == best);
-                // no candidate only with non-finite entries: any unused row, the steps then do not settle
-                const int piv = bb ? __ffs(bb) - 1 : __ffs(__ballot_sync(0xffffffffu, !used)) - 1;
-                if (lane == piv) {
-                    used = true;
-                    mine = k;
-                    const cf inv = finvc(m[k]);
-                    m[k] = {1.0f, 0.0f};
-#pragma unroll
-                    for (int c = 0; c < kMaxR; ++c) {
-                        m[c] = fmulc(m[c], inv);
-                        rowk[c] = m[c];
-                    }
-                }
-                __syncwarp();
-                if (lane != piv) {
-                    const cf f = m[k];
-                    m[k] = {0.0f, 0.0f};
-#pragma unroll
-                    for (int c = 0; c < kMaxR; ++c) m[c] = fsubc(m[c], fmulc(f, rowk[c]));
-                }
-                __syncwarp();
+            if (k >= r) break;
+            const int kl = k % kC;
+            const bool owner = wid == k / kC;
+            if (owner) {
+                colk[k & 1][lane] = m[kl];
+                const unsigned mag = used ? 0u : __float_as_uint(fabs2c(m[kl])) + 1u;
+                const unsigned best = __reduce_max_sync(0xffffffffu, mag);
+                const int piv = __ffs(__ballot_sync(0xffffffffu, !used && mag == best)) - 1;   // r - k rows are unused
+                if (lane == 0) perm[k] = piv;
             }
-        }
-        // row `piv of step k` holds row k of P-permuted inverse: inverse[mine][piv of c] = m[c]
-        perm[mine] = lane;
-        __syncwarp();
+            __syncthreads();
+            const int piv = perm[k];
+            const cf f = colk[k & 1][lane], inv = finvc(colk[k & 1][piv]);
+            if (lane == piv) {
+                used = true;
+                mine = k;
 #pragma unroll
-        for (int c = 0; c < kMaxR; ++c) M[mine][perm[c]] = m[c];
+                for (int e = 0; e < kC; ++e) {
+                    m[e] = fmulc(owner && e == kl ? cf{1.0f, 0.0f} : m[e], inv);
+                    rowk[c0 + e] = m[e];
+                }
+            }
+            __syncwarp();
+            if (lane != piv) {
+#pragma unroll
+                for (int e = 0; e < kC; ++e)
+                    m[e] = fsubc(owner && e == kl ? cf{0.0f, 0.0f} : m[e], fmulc(f, rowk[c0 + e]));
+            }
+            __syncwarp();
+        }
+        // row `piv of step k` holds row k of the inverse with its columns in
+        // pivot order: inverse[mine][pivot of c] = m[c]
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < kC; ++e)
+            if (lane < r && c0 + e < r) M[mine][perm[c0 + e]] = m[e];
     }
     __syncthreads();
     float dw_prev = 0.0f;
