@@ -430,7 +430,7 @@ cdmd_status cdmd_median3x3(cdmd_ctx* ctx, const uint32_t* mask, int64_t W, int64
     const uintptr_t a = reinterpret_cast<uintptr_t>(mask), b = reinterpret_cast<uintptr_t>(out);
     CDMD_REQUIRE(a + bytes <= b || b + bytes <= a, "mask and out overlap");
     DeviceGuard g(ctx->device);
-    return launch_median3x3(mask, W, H, n, out, static_cast<cudaStream_t>(stream));
+    return launch_median3x3(ctx, mask, W, H, n, out, static_cast<cudaStream_t>(stream));
 }
 
 namespace {

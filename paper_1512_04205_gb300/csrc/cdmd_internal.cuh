@@ -294,7 +294,7 @@ cdmd_status launch_decompose(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, i
                              cdmd_selector selector, cudaStream_t stream);
 cdmd_status launch_decompose_auto(cdmd_ctx* ctx, const DecomposeIO& io, int k, int r_max, int K,
                                   cdmd_selector selector, int* r_out, double* tau_out, cudaStream_t stream);
-cdmd_status launch_median3x3(const uint32_t* mask, int64_t W, int64_t H, int n, uint32_t* out,
+cdmd_status launch_median3x3(cdmd_ctx* ctx, const uint32_t* mask, int64_t W, int64_t H, int n, uint32_t* out,
                              cudaStream_t stream);
 cdmd_status launch_sketch_gather(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, int64_t ldd,
                                  const cdmd_measure* meas, double* DY, cudaStream_t stream);

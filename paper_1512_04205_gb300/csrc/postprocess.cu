@@ -4,14 +4,10 @@
 // positives).  Pixel j of a frame sits at row j / W, column j % W; pixels
 // outside the frame count as background.
 //
-// On 0/1 values the median of nine is 1 iff at least five are 1, so each
-// thread filters 32 pixels at once: it forms the nine shifted 32-bit windows
-// (row above, same row, row below; left, centre, right), clears the
-// neighbours that would wrap across a row end, and counts the ones per bit
-// with a bit-sliced adder.  A thread keeps one word position for four frames,
-// so its row-edge masks are computed once, and loads all their words before
-// it uses any (36 loads in flight).  HBM traffic is one read and one write of
-// the mask; the row above and below come from L1/L2.
+// On 0/1 values the median of nine is 1 iff at least five are 1, so a thread
+// filters 32 pixels at once with bit-sliced sums.
+#include <algorithm>
+
 #include "cdmd_internal.cuh"
 
 namespace cdmd {
@@ -26,6 +22,69 @@ __device__ __forceinline__ void full_add(uint32_t a, uint32_t b, uint32_t c, uin
     carry = (a & b) | (t & c);
 }
 
+// count >= 5 of nine pixels from the three rows' horizontal sums (bit planes
+// s + 2 c each).
+__device__ __forceinline__ uint32_t five_of_nine(uint32_t s1, uint32_t c1, uint32_t s2, uint32_t c2, uint32_t s3,
+                                                 uint32_t c3) {
+    uint32_t S, C, t1, t2;
+    full_add(s1, s2, s3, S, C);   // count = S + 2 (C + c1 + c2 + c3)
+    full_add(c1, c2, c3, t1, t2); // c1 + c2 + c3 = t1 + 2 t2
+    // twos = C + t1 + 2 t2; count >= 5 iff twos >= 3, or twos >= 2 and S
+    const uint32_t ge3 = t2 & (C | t1);
+    const uint32_t ge2 = t2 | (C & t1);
+    return ge3 | (ge2 & S);
+}
+
+// Rows of whole words (W a multiple of 32: no word spans two rows, none has
+// spare bits).  A thread walks down one word column of a strip of rows and
+// keeps the last two rows' horizontal sums as bit planes: per word one new row
+// (the word and its two neighbours, from L1), four bit-sliced additions and
+// one store, some 20 instructions, where the kernel below shifts and sums
+// nine words per word (issue-bound, about 60).
+// 1920 x 1080 x 200 (104 MB moved, out of L2 mostly): 37 us, 55 with the kernel below.
+constexpr int kMedianRows = 32;    // rows per strip, at most
+
+__global__ void __launch_bounds__(kMedianThreads)
+median3x3_rows_kernel(const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int wpr, int H, int rows,
+                      int strips, int64_t total) {
+    const int64_t g = static_cast<int64_t>(blockIdx.x) * kMedianThreads + threadIdx.x;
+    if (g >= total) return;
+    const int col = static_cast<int>(g % wpr);
+    const int64_t fs = g / wpr;
+    const int strip = static_cast<int>(fs % strips);
+    const int64_t frame = fs / strips;
+    const int y0 = strip * rows, y1 = min(H, y0 + rows);
+    const bool has_prev = col > 0, has_next = col + 1 < wpr;
+    const uint32_t* src = in + (frame * H + y0) * wpr + col;      // row y0
+    uint32_t* dst = out + (frame * H + y0) * wpr + col;
+    // horizontal sums of the row at p
+    auto sums = [&](const uint32_t* p, uint32_t& s, uint32_t& c) {
+        const uint32_t x = __ldg(p), a = has_prev ? __ldg(p - 1) : 0u, b = has_next ? __ldg(p + 1) : 0u;
+        full_add(__funnelshift_l(a, x, 1), x, __funnelshift_r(x, b, 1), s, c);
+    };
+    uint32_t s0 = 0u, c0 = 0u, s1, c1;
+    if (y0 > 0) sums(src - wpr, s0, c0);
+    sums(src, s1, c1);
+    const int inner = min(y1, H - 1);       // rows with a row below
+#pragma unroll 4
+    for (int y = y0; y < inner; ++y) {
+        src += wpr;
+        uint32_t s2, c2;
+        sums(src, s2, c2);
+        *dst = five_of_nine(s0, c0, s1, c1, s2, c2);
+        dst += wpr;
+        s0 = s1;
+        c0 = c1;
+        s1 = s2;
+        c1 = c2;
+    }
+    if (inner < y1) *dst = five_of_nine(s0, c0, s1, c1, 0u, 0u);
+}
+
+// Other widths: a thread forms the nine shifted 32-bit windows of its word (row
+// above, same row, row below; left, centre, right) from nine words.  It keeps
+// one word position for four frames, so its row-edge masks are computed once,
+// and loads all their words before it uses any (36 loads in flight).
 __global__ void __launch_bounds__(kMedianThreads) median3x3_kernel(const uint32_t* __restrict__ in,
                                                                    uint32_t* __restrict__ out, uint32_t W,
                                                                    uint32_t m, int64_t nw, int n) {
@@ -102,24 +161,36 @@ __global__ void __launch_bounds__(kMedianThreads) median3x3_kernel(const uint32_
             v[3 * dy + 1] = __funnelshift_r(lo, hi, 1u);
             v[3 * dy + 2] = __funnelshift_r(lo, hi, 2u) & ~right;
         }
-        uint32_t s1, c1, s2, c2, s3, c3, S, C, t1, t2;
+        uint32_t s1, c1, s2, c2, s3, c3;
         full_add(v[0], v[1], v[2], s1, c1);
         full_add(v[3], v[4], v[5], s2, c2);
         full_add(v[6], v[7], v[8], s3, c3);
-        full_add(s1, s2, s3, S, C);   // count = S + 2 (C + c1 + c2 + c3)
-        full_add(c1, c2, c3, t1, t2); // c1 + c2 + c3 = t1 + 2 t2
-        // twos = C + t1 + 2 t2; count >= 5 iff twos >= 3, or twos >= 2 and S
-        const uint32_t ge3 = t2 & (C | t1);
-        const uint32_t ge2 = t2 | (C & t1);
-        if (i < nf) out[static_cast<int64_t>(f0 + i) * nw + w] = (ge3 | (ge2 & S)) & rmask;
+        if (i < nf) out[static_cast<int64_t>(f0 + i) * nw + w] = five_of_nine(s1, c1, s2, c2, s3, c3) & rmask;
     }
 }
 
 }  // namespace
 
-cdmd_status launch_median3x3(const uint32_t* mask, int64_t W, int64_t H, int n, uint32_t* out, cudaStream_t stream) {
+cdmd_status launch_median3x3(cdmd_ctx* ctx, const uint32_t* mask, int64_t W, int64_t H, int n, uint32_t* out,
+                             cudaStream_t stream) {
     const int64_t m = W * H;
     const int64_t nw = (m + 31) / 32;
+    // whole words per row: 37 us against 55 at 1920 x 1080 x 200, 16 against 27 at
+    // 1280 x 720 x 200; below some 30 Mpixel both end within the launch's own time
+    if (W % 32 == 0) {
+        const int wpr = static_cast<int>(W / 32), Hi = static_cast<int>(H);
+        // strips as long as they leave about 24 warps per SM, at least 4 rows
+        const int64_t want = 24LL * 32 * ctx->device_sms;
+        const int64_t fit = nw * n / want;
+        const int rows = static_cast<int>(std::max<int64_t>(4, std::min<int64_t>(kMedianRows, fit)));
+        const int strips = (Hi + rows - 1) / rows;
+        const int64_t total = static_cast<int64_t>(n) * strips * wpr;
+        const int64_t blocks = (total + kMedianThreads - 1) / kMedianThreads;
+        median3x3_rows_kernel<<<static_cast<unsigned>(blocks), kMedianThreads, 0, stream>>>(mask, out, wpr, Hi, rows,
+                                                                                            strips, total);
+        CDMD_CHECK_LAUNCH("median3x3_rows_kernel");
+        return CDMD_OK;
+    }
     const dim3 grid(static_cast<unsigned>((nw + kMedianThreads - 1) / kMedianThreads),
                     static_cast<unsigned>((n + kMedianFrames - 1) / kMedianFrames));
     median3x3_kernel<<<grid, kMedianThreads, 0, stream>>>(mask, out, static_cast<uint32_t>(W),
