@@ -21,7 +21,7 @@
 //              two 256-row slots; each segment's tensor copy lands in the B
 //              operand directly, so the conversion is done once per clip and
 //              not again in every row block.
-//   packed, Rademacher C   the same packing, but the +1 / -1 entries are
+//   packed, Rademacher C   (one clip or several) the same packing, but the +1 / -1 entries are
 //              exact in FP16: one product, and sixteen warps convert the
 //              uint8 bytes (loaded into registers two K steps ahead) to FP16
 //              B tiles in the kernel, so no BF16 copy is made.  With the
@@ -235,48 +235,12 @@ __device__ __forceinline__ void draw_c_tiles(uint8_t* a_stage, int gt, int mtile
     }
 }
 
-// One 128-row Rademacher tile of C (rows row0 .. row0 + 127, row0 a multiple
-// of 128; pixels j0 .. j0 + 63) as BF16 +1 / -1 in the 128-byte swizzled
-// K-major layout.  Entry (i, j) is bit (i % 128) % 32 of word (i % 128) / 32
-// of the Philox counter (j, i / 128, 1, 0): clear = +1, set = -1.  One counter
-// gives all 128 rows of a pixel, so generator warp gw (0 .. 7) covers the rows
-// of one word, 32 (gw & 3) .. +31, and 32 pixels, 32 (gw >> 2) .. +31: each
-// lane draws one pixel's counter and the warp passes the word round by
-// shuffles, lane l keeping bit l (its row).  Rows past k and pixels past m
-// are zero.  +1 and -1 are exact in BF16, so C needs no lo part.
-__device__ __forceinline__ void draw_rademacher_tile(uint8_t* a_tile, int gw, int lane, int row0, int k, int64_t j0,
-                                                     int64_t m, const PhiloxKeys& rk) {
-    const int wi = gw & 3;
-    const int64_t jb = j0 + 32 * (gw >> 2);
-    const uint4 w = philox4x32_10(
-        make_uint4(static_cast<uint32_t>(jb + lane), static_cast<uint32_t>(row0 >> 7), 1u, 0u), rk);
-    const uint32_t word = wi == 0 ? w.x : wi == 1 ? w.y : wi == 2 ? w.z : w.w;
-    const uint32_t row = static_cast<uint32_t>(32 * wi + lane);
-    const bool row_ok = row0 + static_cast<int>(row) < k;
-#pragma unroll
-    for (int gg = 0; gg < 4; ++gg) {
-        uint32_t out[4];
-#pragma unroll
-        for (int p2 = 0; p2 < 4; ++p2) {
-            const int src = gg * 8 + 2 * p2;
-            const uint32_t b0 = (__shfl_sync(0xffffffffu, word, src) >> lane) & 1u;
-            const uint32_t b1 = (__shfl_sync(0xffffffffu, word, src + 1) >> lane) & 1u;
-            const uint32_t e0 = (row_ok && jb + src < m) ? (0x3F80u | (b0 << 15)) : 0u;
-            const uint32_t e1 = (row_ok && jb + src + 1 < m) ? (0x3F80u | (b1 << 15)) : 0u;
-            out[p2] = e0 | (e1 << 16);
-        }
-        const uint32_t chunk = static_cast<uint32_t>(4 * (gw >> 2) + gg);   // 8 pixels per 16-byte chunk
-        *reinterpret_cast<uint4*>(a_tile + tc::sw128_offset(row, chunk)) = make_uint4(out[0], out[1], out[2], out[3]);
-    }
-}
-
 // One CTA's share of C D: the rows of C in row block U.rowblk (128 mtiles
 // rows) over the 64-pixel K steps step0 .. step0+nsteps-1, against each of
 // U.nclips clips, written to U.part[g][t * k + row] (this split's partial
 // sums).  Used by the per-clip and the grouped launch.
 // U.tmap[g] maps the uint8 frames; the bytes are staged and converted to BF16
 // by warps 2-11.
-template <bool kRad>
 __device__ __forceinline__ void sketch_tc_body(const SketchItem& U, int* status, uint8_t* smem) {
     const int nclips = U.nclips, mtiles = U.mtiles, k = U.k;
     const int n0 = U.n[0], n1 = nclips > 1 ? U.n[1] : 0;
@@ -370,7 +334,7 @@ __device__ __forceinline__ void sketch_tc_body(const SketchItem& U, int* status,
                         for (int kk = 0; kk < 4; ++kk) {
                             const uint64_t bdesc = tc::desc_sw128(b_base + (g ? L.b_clip[1] : 0u) + kk * 32);
 #pragma unroll
-                            for (int hl = 0; hl < (kRad ? 1 : 2); ++hl) {
+                            for (int hl = 0; hl < 2; ++hl) {
                                 const uint64_t adesc = tc::desc_sw128(a_base + (mt * 2 + hl) * kTileBytes + kk * 32);
                                 tc::mma_bf16(acc, adesc, bdesc, g ? idesc1 : idesc0, (ks | kk | hl) ? 1u : 0u);
                             }
@@ -393,15 +357,7 @@ __device__ __forceinline__ void sketch_tc_body(const SketchItem& U, int* status,
             const int s = static_cast<int>(ks % kStages);
             const uint32_t u = static_cast<uint32_t>(ks / kStages);
             if (u >= 1 && !tc::mbar_wait(&mma_done[s], (u - 1) & 1u, abort_flag, status)) break;
-            if (gen) {
-                if constexpr (kRad) {
-                    for (int mt = 0; mt < mtiles; ++mt)
-                        draw_rademacher_tile(A + s * L.a_stage + (mt * 2) * kTileBytes, warp - 4, lane,
-                                             row0 + 128 * mt, k, (U.step0 + ks) * kKStep, U.m, rk);
-                } else {
-                    draw_c_tiles(A + s * L.a_stage, gt, mtiles, row0, k, (U.step0 + ks) * kKStep, U.m, rk);
-                }
-            }
+            if (gen) draw_c_tiles(A + s * L.a_stage, gt, mtiles, row0, k, (U.step0 + ks) * kKStep, U.m, rk);
             // uint8 -> BF16: 8 pixels of one frame per item, over both clips
             if (!tc::mbar_wait(&tma_full[s], u & 1u, abort_flag, status)) break;
             const uint8_t* src_stage = Dst + s * L.dst_stage;
@@ -479,7 +435,6 @@ struct SketchArgs {
     uint2 key;
 };
 
-template <bool kRad>
 __global__ void __launch_bounds__(kThreads, 1)
 sketch_tc_kernel(const __grid_constant__ CUtensorMap tmap0, const __grid_constant__ CUtensorMap tmap1,
                  const SketchArgs a, int* status) {
@@ -503,7 +458,7 @@ sketch_tc_kernel(const __grid_constant__ CUtensorMap tmap0, const __grid_constan
     U.mtiles = a.mtiles;
     U.k = a.k;
     U.rowblk = blockIdx.x;
-    sketch_tc_body<kRad>(U, status, smem);
+    sketch_tc_body(U, status, smem);
 }
 
 // Grouped launch: CTA b runs work item items[b] (any clip or clip pair, frame
@@ -513,7 +468,7 @@ sketch_tc_grouped_kernel(const SketchItem* __restrict__ items, int* status) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const SketchItem it = items[blockIdx.x];
-    sketch_tc_body<false>(it, status, smem);
+    sketch_tc_body(it, status, smem);
 }
 
 // Grouped fixed-order reduce: element idx of the concatenated outputs belongs
@@ -1003,16 +958,22 @@ __global__ void widen_kernel(const uint8_t* __restrict__ D, int64_t m, int64_t l
 // are built in the kernel: each of warps 1-16 loads the bytes of four B rows
 // (16 pixels each) into registers two 64-pixel K steps ahead and converts
 // them to FP16 (the byte permute 0x6400 | b = 1024 + b, then one packed
-// subtract of 1024) in the 128-byte swizzled K-major layout.  With only a
-// Philox counter per 32 pixels to draw, the Gaussian form's widened BF16
-// copies would leave this kernel bound by their tensor copies (eight
-// row-block CTAs each read every BF16 tile); reading the bytes halves that
-// traffic and needs no copy of the frames.
+// subtract of 1024) in the 128-byte swizzled K-major layout.  The Gaussian
+// form's widened BF16 copies would leave this kernel bound by their tensor
+// copies (eight row-block CTAs each read every BF16 tile); reading the bytes
+// halves that traffic and needs no copy of the frames.  Bound by the issue of
+// the conversion and of the C tile's expansion: 1280x720x200, k = 1000: 0.71 ms;
+// about 1.0 with every warp drawing the words of its own rows.
 //   warp 0       tensor-memory allocation; lane 0 issues tcgen05.mma per K
 //                step (per slot four K16 quarters) into 2 x 256 FP32 columns
-//   warps 1-16   per K step: the C tile (row g / 4, 16 pixels) into the A
-//                stage, four B rows into the B stage; 2 operand stages.
-//                Lane 0 waits for a stage and arrives for its warp.
+//   warps 1-16   every 16 K steps: warp w draws the Philox words of step w for
+//                all of them (64 counters; each warp drawing its own words
+//                meant every counter 16 times over) into shared memory, two
+//                batches deep, one named barrier a batch.
+//                Per K step: the C tile (eight pixels of two rows each; a
+//                rotation and a mask per entry) into the A stage, four B rows
+//                into the B stage; 2 operand stages.  Lane 0 waits for a stage
+//                and arrives for its warp.
 //   warps 1-16   after the last K step: the accumulators to FP32 partials
 //                [split][B row][k]; a reduce per segment sums the splits in
 //                FP64 into the clip's DY columns f0 .. f0 + L - 1.
@@ -1025,6 +986,8 @@ constexpr int kRThreads = 544;                           // warp 0 + 16 generato
 constexpr int kRGenWarps = 16;                           // warps 1-16
 constexpr int kRKStep = 64;                              // pixels per K step
 constexpr int kRBuf = 2;                                 // operand stages = K steps of bytes in flight
+constexpr int kRBatch = kRGenWarps;                      // K steps whose words are drawn together, one per warp
+constexpr uint32_t kRWords = 288u;                       // Philox words of one K step: 4 per pixel, padded
 constexpr uint32_t kRAStage = 128u * 128u;               // 128 rows x 128 bytes of FP16
 constexpr uint32_t kRSlotBytes = 256u * 128u;            // one 256-row slot of B
 constexpr uint32_t kRBStage = 2u * kRSlotBytes;          // 512 rows x 128 bytes of FP16
@@ -1040,15 +1003,16 @@ struct RadSeg {
 struct RadArgs {
     RadSeg seg[kRadMaxSeg];
     PhiloxKeys rk;               // round keys of the seed (constant for the launch)
-    float* part;                 // [splits][kRadRows][k]
+    float* part;                 // [splits][part_rows][k]
     int nseg, k;
+    int part_rows;               // rows any launch of the call covers (at most kRadRows)
     int nslot[2];                // rows of each slot the MMAs cover (multiples of 16, 0 = unused)
     int64_t m;
     int steps_per_split, total_steps;
 };
 
 __host__ __device__ inline uint32_t rad_smem_bytes() {
-    return kRBuf * (kRAStage + kRBStage) + (2 * kRBuf + 1) * 8 + 64;
+    return kRBuf * (kRAStage + kRBStage) + 2u * kRBatch * kRWords * 4u + (2 * kRBuf + 1) * 8 + 64;
 }
 
 // 16 bytes of a B row at pixel j (16-byte aligned), streaming; pixels at or
@@ -1095,38 +1059,51 @@ __device__ __forceinline__ void convert_row16(uint8_t* b_stage, uint32_t off_a, 
     *reinterpret_cast<uint4*>(b_stage + off_b) = make_uint4(w[4], w[5], w[6], w[7]);
 }
 
-// One Rademacher item as FP16 +1 / -1: row r = g / 4 of the tile, pixels
-// j0 + 16 (g mod 4) .. + 15, two 16-byte chunks.  Entry (i, j) is bit
-// (i % 128) % 32 of word (i % 128) / 32 of the Philox counter (j, i / 128,
-// 1, 0): clear = +1, set = -1.  Lane l draws the counters of pixels j0 + l
-// and j0 + 32 + l (every row of a warp lies in one word) and the warp passes
-// the words round by shuffles.  Rows past k and pixels past m are zero.
-__device__ __forceinline__ void draw_rademacher_f16(uint8_t* a_stage, uint32_t off_a, uint32_t off_b, int lane, int r,
-                                                    int pg, int row0, int k, int64_t j0, int64_t m,
-                                                    const PhiloxKeys& rk) {
-    const uint32_t blk = static_cast<uint32_t>(row0 >> 7);
-    const uint4 wa = philox4x32_10(make_uint4(static_cast<uint32_t>(j0) + lane, blk, 1u, 0u), rk);
-    const uint4 wb = philox4x32_10(make_uint4(static_cast<uint32_t>(j0) + 32u + lane, blk, 1u, 0u), rk);
-    const int wi = r >> 5;
-    const uint32_t word_a = wi == 0 ? wa.x : wi == 1 ? wa.y : wi == 2 ? wa.z : wa.w;
-    const uint32_t word_b = wi == 0 ? wb.x : wi == 1 ? wb.y : wi == 2 ? wb.z : wb.w;
-    const bool row_ok = row0 + r < k;
-    const bool hi_half = pg >= 2;                   // pixels 32 .. 63 of the step
-    uint32_t out[8];
+// The Philox words of 64 pixels (one K step from pixel j0) of row block blk
+// into `bits`: word wi of pixel p at bits[72 wi + p + 4 (p / 32)]; one warp.
+// The gap of four words puts the eight lanes of a load phase (eight pixels
+// apart) in different banks.
+__device__ __forceinline__ void draw_rademacher_words(uint32_t* bits, int lane, uint32_t blk, int64_t j0,
+                                                      const PhiloxKeys& rk) {
 #pragma unroll
-    for (int p2 = 0; p2 < 8; ++p2) {
-        const int src = 16 * (pg & 1) + 2 * p2;     // lane of the counter
-        const uint32_t a0 = __shfl_sync(0xffffffffu, word_a, src), a1 = __shfl_sync(0xffffffffu, word_a, src + 1);
-        const uint32_t b0 = __shfl_sync(0xffffffffu, word_b, src), b1 = __shfl_sync(0xffffffffu, word_b, src + 1);
-        const uint32_t s0 = ((hi_half ? b0 : a0) >> (r & 31)) & 1u;
-        const uint32_t s1 = ((hi_half ? b1 : a1) >> (r & 31)) & 1u;
-        const int64_t jp = j0 + 16 * pg + 2 * p2;
-        const uint32_t e0 = (row_ok && jp < m) ? (0x3C00u | (s0 << 15)) : 0u;
-        const uint32_t e1 = (row_ok && jp + 1 < m) ? (0x3C00u | (s1 << 15)) : 0u;
-        out[p2] = e0 | (e1 << 16);
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t p = static_cast<uint32_t>(32 * h + lane);
+        const uint4 w = philox4x32_10(make_uint4(static_cast<uint32_t>(j0) + p, blk, 1u, 0u), rk);
+        uint32_t* b = bits + p + 4u * static_cast<uint32_t>(h);
+        b[0] = w.x;
+        b[72] = w.y;
+        b[144] = w.z;
+        b[216] = w.w;
     }
-    *reinterpret_cast<uint4*>(a_stage + off_a) = make_uint4(out[0], out[1], out[2], out[3]);
-    *reinterpret_cast<uint4*>(a_stage + off_b) = make_uint4(out[4], out[5], out[6], out[7]);
+}
+
+// One Rademacher item as FP16 +1 / -1: the 16-byte chunk of eight pixels (the
+// words w) in rows r and r + 16 of the tile, off and off + 2048 in the layout.
+// Entry (i, j) is bit (i % 128) % 32 of word (i % 128) / 32 of the Philox
+// counter (j, i / 128, 1, 0): clear = +1, set = -1.  One rotation (rot) brings
+// a word's bits of the two rows to the signs of its halves, and a byte permute
+// pairs the halves of two pixels.  one and sign are zero for rows past k; only
+// `left` pixels lie below m.
+__device__ __forceinline__ void expand_signs(uint8_t* a_stage, uint32_t off, const uint32_t* w, uint32_t rot,
+                                             const uint32_t (&one)[2], const uint32_t (&sign)[2], int left) {
+    const uint4 qa = *reinterpret_cast<const uint4*>(w), qb = *reinterpret_cast<const uint4*>(w + 4);
+    const uint32_t q[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
+    uint32_t out[2][4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        const uint32_t x = __funnelshift_l(q[2 * v], q[2 * v], rot), y = __funnelshift_l(q[2 * v + 1], q[2 * v + 1], rot);
+        out[0][v] = (__byte_perm(x, y, 0x5410) & sign[0]) | one[0];
+        out[1][v] = (__byte_perm(x, y, 0x7632) & sign[1]) | one[1];
+    }
+    if (left < 8) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                out[h][v] = 2 * v >= left ? 0u : 2 * v + 1 >= left ? out[h][v] & 0xffffu : out[h][v];
+    }
+    *reinterpret_cast<uint4*>(a_stage + off) = make_uint4(out[0][0], out[0][1], out[0][2], out[0][3]);
+    *reinterpret_cast<uint4*>(a_stage + off + 2048) = make_uint4(out[1][0], out[1][1], out[1][2], out[1][3]);
 }
 
 __global__ void __launch_bounds__(kRThreads, 1)
@@ -1135,7 +1112,8 @@ sketch_rad_u8_kernel(const __grid_constant__ RadArgs a, int* status) {
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint8_t* A = smem;                                   // kRBuf x C tiles
     uint8_t* B = smem + kRBuf * kRAStage;                // kRBuf x 512-row FP16 tiles
-    uint64_t* bars = reinterpret_cast<uint64_t*>(B + kRBuf * kRBStage);
+    uint32_t* bits = reinterpret_cast<uint32_t*>(B + kRBuf * kRBStage);   // 2 x kRBatch x kRWords
+    uint64_t* bars = reinterpret_cast<uint64_t*>(bits + 2 * kRBatch * kRWords);
     uint64_t* ab_full = bars;                            // [kRBuf] A and B written
     uint64_t* mma_done = bars + kRBuf;                   // [kRBuf] read by the MMAs
     uint64_t* accum_done = bars + 2 * kRBuf;
@@ -1229,6 +1207,17 @@ sketch_rad_u8_kernel(const __grid_constant__ RadArgs a, int* status) {
                 }
             }
         }
+        // C item: chunk cc (eight pixels) of rows cr and cr + 16
+        const int cc = g & 7, cr = 32 * (g >> 7) + ((g >> 3) & 15);
+        const uint32_t off_c = tc::sw128_offset(static_cast<uint32_t>(cr), static_cast<uint32_t>(cc));
+        const uint32_t rot = (15u - static_cast<uint32_t>(cr)) & 31u;
+        uint32_t one[2], sign[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const bool row_ok = row0 + cr + 16 * h < k;
+            one[h] = row_ok ? 0x3C003C00u : 0u;
+            sign[h] = row_ok ? 0x80008000u : 0u;
+        }
         const int64_t m = a.m;
         // no pixel of this split's K steps lies past m: loads need no tail checks
         const bool full = static_cast<int64_t>(step0 + nsteps) * kRKStep <= m;
@@ -1238,7 +1227,7 @@ sketch_rad_u8_kernel(const __grid_constant__ RadArgs a, int* status) {
         for (int d = 0; d < kRBuf; ++d)
 #pragma unroll
             for (int t = 0; t < 4; ++t)
-                buf[d][t] = d < nsteps ? load_row16(src[t], static_cast<int64_t>(step0 + d) * kRKStep, m)
+                buf[d][t] = d < nsteps ? load_row16(src[t], static_cast<int64_t>(step0 + d) * kRKStep, m - 16 * pg)
                                        : make_uint4(0u, 0u, 0u, 0u);
         uint32_t ph = 0;      // parity of the current use of the stages
         bool ok = true;
@@ -1259,10 +1248,24 @@ sketch_rad_u8_kernel(const __grid_constant__ RadArgs a, int* status) {
                     ok = __shfl_sync(0xffffffffu, free_ok ? 1 : 0, 0) != 0;
                 }
                 const int64_t j0 = static_cast<int64_t>(step0 + ks) * kRKStep;
+                if ((ks & (kRBatch - 1)) == 0) {
+                    // the batch before last, which this one overwrites, has been
+                    // read: every warp passed the last batch's barrier after it.
+                    // All sixteen warps run every step, so all come here.
+                    const int mine = ks + warp - 1;
+                    if (mine < nsteps)
+                        draw_rademacher_words(bits + (((ks / kRBatch) & 1) * kRBatch + warp - 1) * kRWords, lane,
+                                              static_cast<uint32_t>(row0 >> 7),
+                                              static_cast<int64_t>(step0 + mine) * kRKStep, a.rk);
+                    asm volatile("bar.sync 1, %0;" ::"n"(kRGenWarps * 32) : "memory");
+                }
+                const uint32_t* words = bits + ((ks / kRBatch & 1) * kRBatch + (ks & (kRBatch - 1))) * kRWords +
+                                        72 * (cr >> 5) + 8 * cc + 4 * (cc >> 2);
                 uint8_t* a_stage = A + s * kRAStage;
                 uint8_t* b_stage = B + s * kRBStage;
                 if (ok) {
-                    draw_rademacher_f16(a_stage, off_a, off_b, lane, r, pg, row0, k, j0, m, a.rk);
+                    expand_signs(a_stage, off_c, words, rot, one, sign,
+                                 full ? 8 : static_cast<int>(min(static_cast<int64_t>(8), max(static_cast<int64_t>(0), m - j0 - 8 * cc))));
 #pragma unroll
                     for (int t = 0; t < 4; ++t)
                         if (src[t] != nullptr)
@@ -1280,7 +1283,7 @@ sketch_rad_u8_kernel(const __grid_constant__ RadArgs a, int* status) {
                         for (int t = 0; t < 4; ++t) buf[s][t] = load_row16_full(src[t], j0 + kRBuf * kRKStep);
                     } else {
 #pragma unroll
-                        for (int t = 0; t < 4; ++t) buf[s][t] = load_row16(src[t], j0 + kRBuf * kRKStep, m);
+                        for (int t = 0; t < 4; ++t) buf[s][t] = load_row16(src[t], j0 + kRBuf * kRKStep, m - 16 * pg);
                     }
                 }
             }
@@ -1293,7 +1296,7 @@ sketch_rad_u8_kernel(const __grid_constant__ RadArgs a, int* status) {
             const int quarter = warp & 3;
             const int cg = (warp - 1) >> 2;                 // column group 0 .. 3
             const int row = row0 + quarter * 32 + lane;
-            float* part = a.part + static_cast<int64_t>(split) * kRadRows * k;
+            float* part = a.part + static_cast<int64_t>(split) * a.part_rows * k;
             for (int slot = 0; slot < 2; ++slot) {
                 for (int c0 = 16 * cg; c0 < (slot ? nslot1 : nslot0); c0 += 64) {
                     uint32_t v[16];
@@ -1325,7 +1328,7 @@ __global__ void sketch_rad_reduce_kernel(const __grid_constant__ RadArgs a, int 
     const int64_t total = static_cast<int64_t>(sg.L) * a.k;
     if (idx >= total) return;
     const int64_t src = static_cast<int64_t>(sg.row0) * a.k + idx;
-    const int64_t stride = static_cast<int64_t>(kRadRows) * a.k;
+    const int64_t stride = static_cast<int64_t>(a.part_rows) * a.k;
     double s = 0.0;
     for (int sp = 0; sp < splits; ++sp) s += static_cast<double>(a.part[sp * stride + src]);
     if (!isfinite(s)) record_status(status, CDMD_ERR_NONFINITE);
@@ -1362,7 +1365,7 @@ namespace {
 
 // One launch: nclips (1 or 2) clips of <= 256 frames, each its own DY.
 cdmd_status launch_sketch_tc_unit(cdmd_ctx* ctx, int nclips, const uint8_t* const* D, int64_t m, const int* n,
-                                  const int64_t* ldd, bool rad, int k, uint64_t seed, double* const* DY,
+                                  const int64_t* ldd, int k, uint64_t seed, double* const* DY,
                                   cudaStream_t stream) {
     const int mtiles = nclips == 1 ? 2 : 1;
     CUtensorMap tmap[2];
@@ -1396,9 +1399,9 @@ cdmd_status launch_sketch_tc_unit(cdmd_ctx* ctx, int nclips, const uint8_t* cons
     a.key = seed_key(seed);
     const size_t smem = smem_layout(mtiles, nclips, a.n[0], a.n[1]).total + 1024;
     if (smem > kMaxSmem) return fail(CDMD_ERR_UNSUPPORTED, "sketch: %zu bytes of shared memory per CTA", smem);
-    auto kern = rad ? sketch_tc_kernel<true> : sketch_tc_kernel<false>;
-    CDMD_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-    kern<<<dim3(rowblks, static_cast<unsigned>(splits)), kThreads, smem, stream>>>(tmap[0], tmap[1], a, ctx->d_status);
+    CDMD_CHECK_CUDA(cudaFuncSetAttribute(sketch_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(smem)));
+    sketch_tc_kernel<<<dim3(rowblks, static_cast<unsigned>(splits)), kThreads, smem, stream>>>(tmap[0], tmap[1], a, ctx->d_status);
     CDMD_CHECK_LAUNCH("sketch_tc_kernel");
     const int64_t tot = static_cast<int64_t>(k) * std::max(a.n[0], a.n[1]);
     sketch_tc_reduce_kernel<<<dim3(static_cast<unsigned>((tot + 255) / 256), nclips), 256, 0, stream>>>(
@@ -1411,16 +1414,18 @@ cdmd_status launch_sketch_tc_unit(cdmd_ctx* ctx, int nclips, const uint8_t* cons
 // (no BF16 copies); launches of up to 512 packed frames.
 cdmd_status launch_sketch_rad_u8(cdmd_ctx* ctx, int nclips, const uint8_t* const* D, int64_t m, const int* n,
                                  const int64_t* ldd, int k, uint64_t seed, double* const* DY, cudaStream_t stream) {
-    if (m > (static_cast<int64_t>(1) << 31) - kRKStep)
-        return fail(CDMD_ERR_UNSUPPORTED, "packed sketch: m = %lld pixels (at most 2^31 - 64)", static_cast<long long>(m));
     const int rowblks = (k + 127) / 128;
     const int64_t total_steps = (m + kRKStep - 1) / kRKStep;
     int64_t splits = std::max<int64_t>(1, ctx->num_sms / rowblks);
     splits = std::min<int64_t>(splits, total_steps);
     const int64_t steps_per_split = (total_steps + splits - 1) / splits;
     splits = (total_steps + steps_per_split - 1) / steps_per_split;
+    // every clip starts at a multiple of 8 rows, a launch covers multiples of 16
+    int64_t used = 0;
+    for (int i = 0; i < nclips; ++i) used += (n[i] + 7) / 8 * 8;
+    const int part_rows = static_cast<int>(std::min<int64_t>(kRadRows, (used + 15) / 16 * 16));
     float* part = nullptr;
-    cdmd_status st = ensure_buffer(ctx, BUF_SKETCH_PARTIAL, static_cast<size_t>(splits) * kRadRows * k * sizeof(float),
+    cdmd_status st = ensure_buffer(ctx, BUF_SKETCH_PARTIAL, static_cast<size_t>(splits) * part_rows * k * sizeof(float),
                                    reinterpret_cast<void**>(&part));
     if (st != CDMD_OK) return st;
     const size_t smem = rad_smem_bytes() + 1024;
@@ -1432,6 +1437,7 @@ cdmd_status launch_sketch_rad_u8(cdmd_ctx* ctx, int nclips, const uint8_t* const
     RadArgs a{};
     a.part = part;
     a.k = k;
+    a.part_rows = part_rows;
     a.m = m;
     a.steps_per_split = static_cast<int>(steps_per_split);
     a.total_steps = static_cast<int>(total_steps);
@@ -1490,12 +1496,19 @@ cdmd_status launch_sketch_tc(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, 
         return fail(CDMD_ERR_UNSUPPORTED, "BF16X2 sketch generates GAUSSIAN or RADEMACHER C");
     cdmd_status st = check_tc_video(D, ldd);
     if (st != CDMD_OK) return st;
+    // +1 / -1 C: the packed kernel also for one clip.  Its 128-row CTAs take the
+    // uint8 frames as they are, 512 rows of them at most, and one product per
+    // step: 0.71 ms at 1280x720x200, k = 1000 (0.95 for the Gaussian kernel's
+    // form with 256 rows of BF16 C and staged, converted tiles); 0.44 against
+    // 0.96 at n = 300, k = 500 (one launch, not two); 38 us against 60 at
+    // 320x240x100, k = 300
+    if (ctype == CDMD_C_RADEMACHER) return launch_sketch_rad_u8(ctx, 1, &D, m, &n, &ldd, k, seed, &DY, stream);
     // the sketch is linear in the frames: DY[t0:t1] = C D[:, t0:t1]
     for (int t0 = 0; t0 < n; t0 += kMaxFrames) {
         const int nc = std::min(kMaxFrames, n - t0);
         const uint8_t* Dc = D + static_cast<int64_t>(t0) * ldd;
         double* DYc = DY + static_cast<int64_t>(t0) * k;
-        st = launch_sketch_tc_unit(ctx, 1, &Dc, m, &nc, &ldd, ctype == CDMD_C_RADEMACHER, k, seed, &DYc, stream);
+        st = launch_sketch_tc_unit(ctx, 1, &Dc, m, &nc, &ldd, k, seed, &DYc, stream);
         if (st != CDMD_OK) return st;
     }
     return CDMD_OK;
@@ -1509,7 +1522,12 @@ cdmd_status launch_sketch_tc_shared(cdmd_ctx* ctx, int nclips, const uint8_t* co
         if (st != CDMD_OK) return st;
     }
     if (nclips == 1) return launch_sketch_tc(ctx, D[0], m, n[0], ldd[0], ctype, k, seed, DY[0], stream);
-    if (ctype == CDMD_C_RADEMACHER) return launch_sketch_rad_u8(ctx, nclips, D, m, n, ldd, k, seed, DY, stream);
+    if (ctype == CDMD_C_RADEMACHER) {
+        if (m > (static_cast<int64_t>(1) << 31) - kRKStep)
+            return fail(CDMD_ERR_UNSUPPORTED, "packed sketch: m = %lld pixels (at most 2^31 - 64)",
+                        static_cast<long long>(m));
+        return launch_sketch_rad_u8(ctx, nclips, D, m, n, ldd, k, seed, DY, stream);
+    }
     // BF16 copies of every clip's frames (one HBM-bound pass each)
     const int64_t ldw = (m + 15) / 16 * 16;
     size_t elems = 0;
