@@ -70,6 +70,25 @@ __device__ __forceinline__ double rsqrt64(double a) {
     return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 
+// Two FP32 values in one 64-bit register: an f32x2 instruction issues once for
+// both and rounds each half as the scalar one does.
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ void fma_f32x2(uint64_t& d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 key) {
 #pragma unroll
     for (int rnd = 0; rnd < 10; ++rnd) {
