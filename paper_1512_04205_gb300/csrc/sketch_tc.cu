@@ -126,8 +126,11 @@ constexpr size_t kMaxSmem = 232448;         // opt-in shared memory per CTA
 // mean ~128 grey levels turns into ~1e-4 relative.
 __device__ __forceinline__ void box_muller_fast(uint32_t wa, uint32_t wb, float& zc, float& zs) {
     const float u = fmaf(__uint2float_rn(wa), 2.3283064365386963e-10f, 1.1641532182693481e-10f);
-    const float x = -1.3862943611198906f * __log2f(u);   // -2 ln u
-    float rad;
+    // u >= 2^-33: the flush-to-zero form of the logarithm gives the same value
+    // without __log2f's scaling for subnormal arguments
+    float lg, rad;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(u));
+    const float x = -1.3862943611198906f * lg;           // -2 ln u
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rad) : "f"(x));
     const float f = __uint_as_float(0x3F800000u | ((wb >> 7) & 0x7FFFFFu)) - (1.0f - 5.9604645e-08f);
     float s, c;
@@ -261,11 +264,17 @@ __device__ __forceinline__ void sketch_tc_body(const SketchItem& U, int* status,
     const int warp = tid >> 5;
     const int lane = tid & 31;
     const int64_t nsteps = U.nsteps < 0 ? 0 : U.nsteps;
+    // Two row tiles (one clip): the generator warps draw 16384 Gaussians a step
+    // and set its length, so warps 2-3, which have nothing to draw, convert all
+    // of the step's bytes.  One row tile and two clips: half the draws and up to
+    // twice the bytes, shared by all ten warps.  1920x1080x200, k = 1000, one
+    // clip: 3.02 ms (3.15 with the conversion spread over all ten warps).
+    const int converters = mtiles == 2 ? 64 : kWorkers;
 
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             tc::mbar_init(&tma_full[s], 1);
-            tc::mbar_init(&d_free[s], kWorkers);
+            tc::mbar_init(&d_free[s], converters);
             tc::mbar_init(&ab_full[s], kWorkers);
             tc::mbar_init(&mma_done[s], 1);
         }
@@ -358,11 +367,17 @@ __device__ __forceinline__ void sketch_tc_body(const SketchItem& U, int* status,
             const uint32_t u = static_cast<uint32_t>(ks / kStages);
             if (u >= 1 && !tc::mbar_wait(&mma_done[s], (u - 1) & 1u, abort_flag, status)) break;
             if (gen) draw_c_tiles(A + s * L.a_stage, gt, mtiles, row0, k, (U.step0 + ks) * kKStep, U.m, rk);
+            if (wt >= converters) {
+                tc::fence_proxy_async_smem();
+                tc::mbar_arrive(&ab_full[s]);
+                continue;
+            }
             // uint8 -> BF16: 8 pixels of one frame per item, over both clips
             if (!tc::mbar_wait(&tma_full[s], u & 1u, abort_flag, status)) break;
             const uint8_t* src_stage = Dst + s * L.dst_stage;
             uint8_t* b_stage = B + s * L.b_stage;
-            for (int it = wt; it < conv_total; it += kWorkers) {
+#pragma unroll 2
+            for (int it = wt; it < conv_total; it += converters) {
                 const int g = it >= conv0 ? 1 : 0;
                 const int li = it - (g ? conv0 : 0);
                 const int t = li >> 3, c8 = li & 7;
@@ -374,8 +389,11 @@ __device__ __forceinline__ void sketch_tc_body(const SketchItem& U, int* status,
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         // byte b of the word into a float with exponent 2^23: 2^23 + b, exact
-                        const float f0 = __uint_as_float(__byte_perm(word, 0x4B000000u, 0x7540u + 2u * e)) - 8388608.0f;
-                        const float f1 = __uint_as_float(__byte_perm(word, 0x4B000000u, 0x7541u + 2u * e)) - 8388608.0f;
+                        float f0, f1;
+                        unpack_f32x2(add_f32x2(pack_f32x2(__uint_as_float(__byte_perm(word, 0x4B000000u, 0x7540u + 2u * e)),
+                                                          __uint_as_float(__byte_perm(word, 0x4B000000u, 0x7541u + 2u * e))),
+                                               pack_f32x2(-8388608.0f, -8388608.0f)),
+                                     f0, f1);
                         w[h * 2 + e] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
                     }
                 }
