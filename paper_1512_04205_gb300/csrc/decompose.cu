@@ -600,6 +600,7 @@ __device__ __forceinline__ int sturm_count(const double* d, const double* e2, in
     return c;
 }
 
+constexpr double kSearchTol = 256.0 * kEps;
 constexpr int kEigThreads = 128;   // one warp per scheduler; one shift per thread
 
 // The first of the block's kEigThreads flags that is set (kEigThreads if
@@ -619,17 +620,23 @@ __device__ __forceinline__ int first_set(bool flag, unsigned* ball, int turn) {
 // Eigenpair `w` (descending) of T, one CTA of four warps, one per scheduler:
 // a DP instruction holds its scheduler 64 clocks whatever its lanes do, so four
 // warps of one shift each run a Sturm pass over 128 shifts in the time one
-// warp takes over 32.  Three passes in FP32 narrow the interval to a few 1e-6 of the
-// norm (margin: 16 eps32, above the count's backward error), three on pairs of
-// floats to 3e-12 (margin 2^-42), and two in FP64 to eps; the first of those
-// tests both ends of the bracket (else everything is repeated from the
-// Gershgorin interval).
+// warp takes over 32.  Three passes in FP32 narrow the interval to a few 1e-6
+// of the norm (margin: 16 eps32, above the count's backward error), three on
+// pairs of floats to 3e-12 (margin 2^-42), and one in FP64, which tests both
+// ends of the bracket (else everything is repeated from the Gershgorin
+// interval), to kSearchTol: the inverse iteration's shift needs no more (two
+// solves leave the square of shift error / gap of other vectors).  The Rayleigh
+// quotient of its vector then gives the eigenvalue to rounding level, which
+// errs with z's share of the norm where a Sturm count errs with the norm itself.
+// sigma and G at n = 300, r = 30, against LAPACK in FP64: off by 3.7e-16 and
+// 4.5e-13; 8.9e-15 and 4.9e-12 with the search carried on to eps.
 // Inverse iteration: LU with partial pivoting and two solves by one thread,
 // each step one or two dependent DP instructions; everything that is not on
 // that chain (d - mu, the scaled rows of U, the divisions by the pivots) is
 // done by all threads between the chains.
-// p = 199, r = 20, one CTA per pair: 218 us; 265 with four FP64 passes in place of the pairs of
-// floats and a branch on every pivot; 0.62 ms on one warp per pair, all FP64.
+// p = 199, r = 20, one CTA per pair: 192 us; 218 with the search carried on to
+// eps in FP64, 265 with four FP64 passes in place of the pairs of floats and a
+// branch on every pivot; 0.62 ms on one warp per pair, all FP64.
 __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm) {
     const double *dd = q.dd, *ee = q.ee;
     const int p = q.p;
@@ -739,7 +746,7 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
     bool converged = false;
     for (int it = 0; it < 40; ++it) {
         const double width = hi - lo;
-        if (width <= 2.0 * kEps * fmax(fabs(lo), fabs(hi)) + kEps * tn + 1e-300) { converged = true; break; }
+        if (width <= kSearchTol * tn + 1e-300) { converged = true; break; }
         const double step = width * (1.0 / (kEigThreads + 1));
         const bool above = sturm_count(d, e2, p, fma(step, static_cast<double>(tid + 1), lo)) > idx;
         const int f = first_set(above, ball, turn++);
@@ -858,10 +865,22 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
             for (int i = tid; i < p; i += kEigThreads) z[i] *= sc;
         }
     }
-    double s0 = 0.0;
-    for (int i = tid; i < p; i += kEigThreads) s0 = fma(z[i], z[i], s0);
-    s0 = warp_sum(s0);
-    if (lane == 0) red[wid] = s0;
+    // z^T z and z^T (T - lambda) z
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll 1
+    for (int i = tid; i < p; i += kEigThreads) {
+        const double zi = z[i], zm = i > 0 ? z[i - 1] : 0.0, zp = i + 1 < p ? z[i + 1] : 0.0, em = i > 0 ? e[i - 1] : 0.0;
+        s0 = fma(zi, zi, s0);
+        s1 = fma(zi, fma(d[i] - lambda, zi, fma(em, zm, e[i] * zp)), s1);
+    }
+    __syncwarp();
+    {
+        const bool hi_half = (lane & 16) != 0;
+        double t = (hi_half ? s1 : s0) + __shfl_xor_sync(0xffffffffu, hi_half ? s0 : s1, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if ((lane & 15) == 0) red[wid + (hi_half ? 4 : 0)] = t;      // their last readers are past many barriers
+    }
     __syncthreads();
     const double nrm2 = (red[0] + red[1]) + (red[2] + red[3]);
     if (!(nrm2 > 0.0) || !isfinite(nrm2)) {
@@ -871,6 +890,12 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
     }
     const double inv = rsqrt64(nrm2);
     for (int i = tid; i < p; i += kEigThreads) Z[i] = z[i] * inv;
+    if (tid == 0) {
+        // the Rayleigh quotient: its error is the square of z's.  Within a
+        // cluster z may mix neighbours; the search's interval bounds the step.
+        const double step = ((red[4] + red[5]) + (red[6] + red[7])) * inv * inv;
+        if (fabs(step) <= 2.0 * kSearchTol * tn) q.lamT[w] = lambda + step;
+    }
 }
 
 // Reflectors j0 .. j0 + NB - 1 as one block I - V T V^T (compact WY form,
