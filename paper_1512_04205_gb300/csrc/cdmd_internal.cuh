@@ -150,23 +150,21 @@ __device__ __forceinline__ void box_muller_accurate(uint32_t wa, uint32_t wb, fl
         ln_u = log1pf(-((__uint2float_rn(~wa) + 0.5f) * two_m32));
     }
     const float radius = sqrtf(-2.0f * ln_u);
-    const uint32_t quarter = wb >> 30;
     const float f = (__uint2float_rn(wb & 0x3fffffffu) + 0.5f) * 9.313225746154785e-10f;   // 2^-30
     float s, c;
     sincospif(0.5f * f, &s, &c);
-    float cs, sn;   // rotate by quarter * pi/2
-    switch (quarter) {
-        case 0: cs = c; sn = s; break;
-        case 1: cs = -s; sn = c; break;
-        case 2: cs = -c; sn = -s; break;
-        default: cs = s; sn = -c; break;
-    }
-    z_cos = radius * cs;
-    z_sin = radius * sn;
+    // quarter turns q = top two bits: (c, s), (-s, c), (-c, -s), (s, -c); the
+    // signs go to the radius (bit 31 for the second value, 31 ^ 30 for the first)
+    const uint32_t w2 = wb << 1;
+    const float rs = __uint_as_float(__float_as_uint(radius) ^ (wb & 0x80000000u));
+    const float rc = __uint_as_float(__float_as_uint(rs) ^ (w2 & 0x80000000u));
+    const bool odd = static_cast<int32_t>(w2) < 0;
+    z_cos = rc * (odd ? s : c);
+    z_sin = rs * (odd ? c : s);
 }
 
 // Four Gaussian entries C[4q + 0..3, j] from counter (j, q, 0, 0).
-__device__ __forceinline__ float4 gaussian_quad(uint2 key, uint32_t j, uint32_t q) {
+__device__ __forceinline__ float4 gaussian_quad(const PhiloxKeys& key, uint32_t j, uint32_t q) {
     const uint4 w = philox4x32_10(make_uint4(j, q, 0u, 0u), key);
     float4 z;
     box_muller_accurate(w.x, w.y, z.x, z.y);

@@ -634,7 +634,7 @@ __device__ __forceinline__ int first_set(bool flag, unsigned* ball, int turn) {
 // each step one or two dependent DP instructions; everything that is not on
 // that chain (d - mu, the scaled rows of U, the divisions by the pivots) is
 // done by all threads between the chains.
-// p = 199, r = 20, one CTA per pair: 192 us; 218 with the search carried on to
+// p = 199, r = 20, one CTA per pair: 203 us; 218 with the search carried on to
 // eps in FP64, 265 with four FP64 passes in place of the pairs of floats and a
 // branch on every pivot; 0.62 ms on one warp per pair, all FP64.
 __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm) {

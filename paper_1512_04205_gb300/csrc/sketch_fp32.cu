@@ -6,6 +6,14 @@
 // Philox into shared memory, stages the 32 pixels of every frame (uint8 ->
 // float) and accumulates a 64 x (frames) tile in registers: warp w owns rows
 // 8w..8w+7, lane l owns frames l, l+32, ...  Every C entry is drawn once.
+// Two chunks of shared memory: between two barriers, half of the warps draw the
+// next chunk's block and then multiply this one's, the others multiply and
+// then draw, so that on every scheduler the generator's long dependent chains
+// run beside multiply-adds; the frames' bytes are loaded a chunk ahead of their
+// conversion.  Bound by instruction issue (about 80% of it):
+// 720x480x200, k = 400: 1.77 ms; 2.13 with a barrier between drawing and
+// multiplying.  Rows in pairs through fma.rn.f32x2 halve the multiply-adds but
+// not the time (1.92 ms): the second operand has to be doubled in registers.
 // Partial sums (one per split) are written as float [split][k][n] and summed
 // in FP64 by sketch_reduce_kernel in a fixed order (deterministic).
 #include "cdmd_internal.cuh"
@@ -17,15 +25,22 @@ constexpr int kRowsPerCta = 64;
 constexpr int kPixPerChunk = 32;
 constexpr int kThreads = 256;
 
+// two chunks of C and of the frames
+constexpr size_t fp32_smem_bytes(int tq) {
+    return 2 * static_cast<size_t>(kPixPerChunk) * (kRowsPerCta + 32 * tq + 1) * sizeof(float);
+}
+
 template <int TQ, int CTYPE>
 __global__ void __launch_bounds__(kThreads, 2)
 sketch_fp32_kernel(const uint8_t* __restrict__ D, int64_t m, int n_slab, int t0, int64_t ldd,
-                   int k, uint2 key, int64_t pix_per_split, int n_total,
+                   int k, const __grid_constant__ PhiloxKeys key, int64_t pix_per_split, int n_total,
                    float* __restrict__ part) {
     constexpr int NP = 32 * TQ;      // padded frames of the slab
     constexpr int DS = NP + 1;       // shared row stride (odd: fewer conflicts)
-    __shared__ __align__(16) float Cs[kPixPerChunk][kRowsPerCta];
-    extern __shared__ float Ds[];    // [kPixPerChunk][DS]
+    constexpr int kCs = kPixPerChunk * kRowsPerCta, kDs = kPixPerChunk * DS;
+    extern __shared__ __align__(16) float fsm[];
+    float* Cs = fsm;                 // 2 x [kPixPerChunk][kRowsPerCta]
+    float* Ds = fsm + 2 * kCs;       // 2 x [kPixPerChunk][DS]
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
@@ -34,7 +49,7 @@ sketch_fp32_kernel(const uint8_t* __restrict__ D, int64_t m, int n_slab, int t0,
     const int64_t pbeg = static_cast<int64_t>(blockIdx.y) * pix_per_split;
     const int64_t pend = min(m, pbeg + pix_per_split);
 
-    for (int idx = tid; idx < kPixPerChunk * DS; idx += kThreads) Ds[idx] = 0.0f;
+    for (int idx = tid; idx < 2 * kDs; idx += kThreads) Ds[idx] = 0.0f;
 
     float acc[8][TQ];
 #pragma unroll
@@ -44,9 +59,8 @@ sketch_fp32_kernel(const uint8_t* __restrict__ D, int64_t m, int n_slab, int t0,
 
     const bool vec_ok = ((ldd & 3) == 0) && ((reinterpret_cast<uintptr_t>(D) & 3) == 0);
 
-    for (int64_t j0 = pbeg; j0 < pend; j0 += kPixPerChunk) {
-        __syncthreads();   // previous chunk fully consumed
-        // C block: 16 quads of rows x 32 pixels = 512 Philox calls.
+    // C block of the pixels from j0: 16 quads of rows x 32 pixels = 512 Philox calls
+    auto draw = [&](float* Cd, int64_t j0) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int c = tid + kThreads * h;
@@ -57,41 +71,83 @@ sketch_fp32_kernel(const uint8_t* __restrict__ D, int64_t m, int n_slab, int t0,
             if (j < pend && row0 + 4 * quad < k) {
                 const uint32_t q = static_cast<uint32_t>((row0 >> 2) + quad);
                 z = (CTYPE == CDMD_C_GAUSSIAN) ? gaussian_quad(key, static_cast<uint32_t>(j), q)
-                                               : rademacher_quad(key, static_cast<uint32_t>(j), q);
+                                               : rademacher_quad(make_uint2(key.x[0], key.y[0]), static_cast<uint32_t>(j), q);
             }
-            *reinterpret_cast<float4*>(&Cs[jj][4 * quad]) = z;
+            *reinterpret_cast<float4*>(&Cd[jj * kRowsPerCta + 4 * quad]) = z;
         }
-        // D block: frames t0 .. t0+n_slab-1, pixels j0 .. j0+31 (4 per thread).
+    };
+    // bytes of frames t0 .. t0+n_slab-1, pixels j0 .. j0+31: 4 pixels per word
+    uint32_t raw[TQ];
+    auto load = [&](int64_t j0) {
         const bool full = vec_ok && (j0 + kPixPerChunk <= pend);
-        for (int idx = tid; idx < n_slab * 8; idx += kThreads) {
+#pragma unroll
+        for (int i = 0; i < TQ; ++i) {
+            const int idx = tid + kThreads * i;
             const int t = idx >> 3;
             const int g = idx & 7;
-            const uint8_t* src = D + static_cast<int64_t>(t0 + t) * ldd + j0 + 4 * g;
             uint32_t w = 0;
-            if (full) {
-                w = __ldg(reinterpret_cast<const uint32_t*>(src));
-            } else {
+            if (t < n_slab && j0 < pend) {
+                const uint8_t* src = D + static_cast<int64_t>(t0 + t) * ldd + j0 + 4 * g;
+                if (full) {
+                    w = __ldg(reinterpret_cast<const uint32_t*>(src));
+                } else {
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (j0 + 4 * g + e < pend) w |= static_cast<uint32_t>(src[e]) << (8 * e);
+                    for (int e = 0; e < 4; ++e)
+                        if (j0 + 4 * g + e < pend) w |= static_cast<uint32_t>(src[e]) << (8 * e);
+                }
             }
-            float* dst = Ds + (4 * g) * DS + t;
-            dst[0] = static_cast<float>(w & 255u);
-            dst[DS] = static_cast<float>((w >> 8) & 255u);
-            dst[2 * DS] = static_cast<float>((w >> 16) & 255u);
-            dst[3 * DS] = static_cast<float>(w >> 24);
+            raw[i] = w;
         }
-        __syncthreads();
+    };
+    auto store = [&](float* Dd) {
+#pragma unroll
+        for (int i = 0; i < TQ; ++i) {
+            const int idx = tid + kThreads * i;
+            const int t = idx >> 3;
+            const int g = idx & 7;
+            if (t < n_slab) {
+                float* dst = Dd + (4 * g) * DS + t;
+                const uint32_t w = raw[i];
+                dst[0] = static_cast<float>(w & 255u);
+                dst[DS] = static_cast<float>((w >> 8) & 255u);
+                dst[2 * DS] = static_cast<float>((w >> 16) & 255u);
+                dst[3 * DS] = static_cast<float>(w >> 24);
+            }
+        }
+    };
+
+    load(pbeg);
+    draw(Cs, pbeg);
+    __syncthreads();                 // the buffers are cleared
+    store(Ds);
+    load(pbeg + kPixPerChunk);
+    int cur = 0;
+    for (int64_t j0 = pbeg; j0 < pend; j0 += kPixPerChunk, cur ^= 1) {
+        __syncthreads();             // this chunk is staged, the other buffer consumed
+        const float* Cc = Cs + cur * kCs;
+        const float* Dc = Ds + cur * kDs;
+        const int64_t jn = j0 + kPixPerChunk;
+        if (jn < pend) {
+            store(Ds + (cur ^ 1) * kDs);
+            load(jn + kPixPerChunk);
+        }
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+            if (half == (warp >> 2)) {
+                if (jn < pend) draw(Cs + (cur ^ 1) * kCs, jn);
+                continue;
+            }
 #pragma unroll 4
-        for (int jj = 0; jj < kPixPerChunk; ++jj) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&Cs[jj][warp * 8]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&Cs[jj][warp * 8 + 4]);
-            const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            for (int jj = 0; jj < kPixPerChunk; ++jj) {
+                const float4 a0 = *reinterpret_cast<const float4*>(&Cc[jj * kRowsPerCta + warp * 8]);
+                const float4 a1 = *reinterpret_cast<const float4*>(&Cc[jj * kRowsPerCta + warp * 8 + 4]);
+                const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
 #pragma unroll
-            for (int q = 0; q < TQ; ++q) {
-                const float b = Ds[jj * DS + lane + 32 * q];
+                for (int q = 0; q < TQ; ++q) {
+                    const float b = Dc[jj * DS + lane + 32 * q];
 #pragma unroll
-                for (int a = 0; a < 8; ++a) acc[a][q] = fmaf(av[a], b, acc[a][q]);
+                    for (int a = 0; a < 8; ++a) acc[a][q] = fmaf(av[a], b, acc[a][q]);
+                }
             }
         }
     }
@@ -124,7 +180,7 @@ __global__ void sketch_reduce_kernel(const float* __restrict__ part, int splits,
 
 template <int CTYPE>
 cdmd_status launch_slab(int tq, dim3 grid, size_t smem, cudaStream_t stream, const uint8_t* D,
-                        int64_t m, int n_slab, int t0, int64_t ldd, int k, uint2 key,
+                        int64_t m, int n_slab, int t0, int64_t ldd, int k, const PhiloxKeys& key,
                         int64_t pps, int n_total, float* part) {
 #define CDMD_SKETCH_CASE(TQV)                                                                    \
     case TQV: {                                                                                  \
@@ -172,11 +228,11 @@ cdmd_status launch_sketch_fp32(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n
                                    static_cast<size_t>(splits) * k * n * sizeof(float),
                                    reinterpret_cast<void**>(&part));
     if (st != CDMD_OK) return st;
-    const uint2 key = seed_key(seed);
+    const PhiloxKeys key = philox_round_keys(seed_key(seed));
     for (int t0 = 0; t0 < n; t0 += kMaxSlab) {
         const int n_slab = std::min(kMaxSlab, n - t0);
         const int tq = (n_slab + 31) / 32;
-        const size_t smem = static_cast<size_t>(kPixPerChunk) * (32 * tq + 1) * sizeof(float);
+        const size_t smem = fp32_smem_bytes(tq);
         const dim3 grid(row_tiles, static_cast<unsigned>(splits));
         st = (ctype == CDMD_C_GAUSSIAN)
                  ? launch_slab<CDMD_C_GAUSSIAN>(tq, grid, smem, stream, D, m, n_slab, t0, ldd, k, key, pps, n, part)
@@ -270,11 +326,11 @@ extern "C" cdmd_status cdmd_sketch_noalloc(const uint8_t* D, int64_t m, int n, i
     const int64_t chunks_per_split = (chunks + splits - 1) / splits;
     const int64_t pps = chunks_per_split * kPixPerChunk;
     splits = (m + pps - 1) / pps;   // never more than before: every split gets pixels
-    const uint2 key = seed_key(seed);
+    const PhiloxKeys key = philox_round_keys(seed_key(seed));
     for (int t0 = 0; t0 < n; t0 += kMaxSlab) {
         const int n_slab = std::min(kMaxSlab, n - t0);
         const int tq = (n_slab + 31) / 32;
-        const size_t smem = static_cast<size_t>(kPixPerChunk) * (32 * tq + 1) * sizeof(float);
+        const size_t smem = fp32_smem_bytes(tq);
         const dim3 grid(row_tiles, static_cast<unsigned>(splits));
         const cdmd_status s2 =
             (ctype == CDMD_C_GAUSSIAN)
