@@ -1,28 +1,46 @@
 // Pass (b), plain form: full-state modes Phi = X' G with G = V S^-1 W
 // (Algorithm 1 step 8, Eq. cDMDModes), FP32 CUDA-core FMA.
 //
-// Each thread owns 4 consecutive pixels (one 32-bit load per frame) and a
-// tile of 8 complex modes; G for the tile is converted FP64 -> FP32 into
-// shared memory by the CTA.  Grid: (pixel blocks of 1024) x (mode tiles).
+// Each thread owns four consecutive pixels (one 32-bit load per frame) and a
+// tile of CT complex modes; G for the tile is converted FP64 -> FP32 into
+// shared memory by the CTA, and the bytes of eight frames are loaded while the
+// eight before are multiplied.  Grid: (pixel blocks of 512) x (mode tiles).
+// The modes go in tiles of equal size, at most eight (ten in two tiles of five:
+// tiles of eight and eight would multiply for six that do not exist).  Bound by the
+// multiply-adds at 1920x1080x200, 10 modes: 0.52 ms; 1.15 with a load per frame
+// at its use and tiles of eight.  By the latency of a chain of loads at
+// 160x120x100: 17 us; 40 so.  CTAs of 128 threads spread small frames over
+// more SMs (480x360x100, 8 modes: 34 us; 42 with 256).
 #include "cdmd_internal.cuh"
 
 namespace cdmd {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 128;
 constexpr int kPx = 4;
-constexpr int kCt = 8;
+constexpr int kBatch = 8;        // frames loaded together
 
+// Four pixels of a frame, as bytes of a word; those at or past m read as zero
+__device__ __forceinline__ uint32_t load_pixels(const uint8_t* src, int64_t j0, int64_t m, bool vec) {
+    if (vec) return __ldg(reinterpret_cast<const uint32_t*>(src));
+    uint32_t w = 0;
+#pragma unroll
+    for (int e = 0; e < kPx; ++e)
+        if (j0 + e < m) w |= static_cast<uint32_t>(src[e]) << (8 * e);
+    return w;
+}
+
+template <int CT>
 __global__ void __launch_bounds__(kThreads)
 lift_fp32_kernel(const uint8_t* __restrict__ D, int64_t m, int n, int64_t ldd,
                  const double* __restrict__ G, int r, const int32_t* __restrict__ cols, int ncols,
                  float* __restrict__ Phi) {
-    extern __shared__ float2 Gs[];   // [(n-1)][kCt]
+    extern __shared__ __align__(16) float2 Gs[];   // [(n-1)][CT]
     const int p = n - 1;
-    const int c0 = blockIdx.y * kCt;
-    for (int idx = threadIdx.x; idx < p * kCt; idx += kThreads) {
-        const int t = idx / kCt;
-        const int c = idx % kCt;
+    const int c0 = blockIdx.y * CT;
+    for (int idx = threadIdx.x; idx < p * CT; idx += kThreads) {
+        const int c = idx / p;
+        const int t = idx % p;
         float2 g = make_float2(0.f, 0.f);
         if (c0 + c < ncols) {
             const int s = cols ? cols[c0 + c] : c0 + c;
@@ -31,52 +49,72 @@ lift_fp32_kernel(const uint8_t* __restrict__ D, int64_t m, int n, int64_t ldd,
                 g = make_float2(static_cast<float>(src[0]), static_cast<float>(src[1]));
             }
         }
-        Gs[idx] = g;
+        Gs[t * CT + c] = g;
     }
     __syncthreads();
 
     const int64_t j0 = (static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x) * kPx;
     if (j0 >= m) return;
     const bool vec = (j0 + kPx <= m) && ((ldd & 3) == 0) && ((reinterpret_cast<uintptr_t>(D) & 3) == 0);
-    float2 acc[kPx][kCt];
+    float2 acc[kPx][CT];
 #pragma unroll
     for (int e = 0; e < kPx; ++e)
 #pragma unroll
-        for (int c = 0; c < kCt; ++c) acc[e][c] = make_float2(0.f, 0.f);
+        for (int c = 0; c < CT; ++c) acc[e][c] = make_float2(0.f, 0.f);
 
-    for (int t = 0; t < p; ++t) {
-        const uint8_t* src = D + static_cast<int64_t>(t + 1) * ldd + j0;
-        uint32_t w = 0;
-        if (vec) {
-            w = __ldg(reinterpret_cast<const uint32_t*>(src));
-        } else {
+    const uint8_t* src = D + ldd + j0;
+    uint32_t next[kBatch];
 #pragma unroll
-            for (int e = 0; e < kPx; ++e)
-                if (j0 + e < m) w |= static_cast<uint32_t>(src[e]) << (8 * e);
-        }
-        float x[kPx];
+    for (int u = 0; u < kBatch; ++u) next[u] = u < p ? load_pixels(src + u * ldd, j0, m, vec) : 0u;
+    for (int t0 = 0; t0 < p; t0 += kBatch) {
+        uint32_t w[kBatch];
 #pragma unroll
-        for (int e = 0; e < kPx; ++e) x[e] = static_cast<float>((w >> (8 * e)) & 255u);
-        const float2* gt = Gs + t * kCt;
+        for (int u = 0; u < kBatch; ++u) w[u] = next[u];
+        src += kBatch * ldd;
 #pragma unroll
-        for (int c = 0; c < kCt; ++c) {
-            const float2 g = gt[c];
+        for (int u = 0; u < kBatch; ++u)
+            if (t0 + kBatch + u < p) next[u] = load_pixels(src + u * ldd, j0, m, vec);
 #pragma unroll
-            for (int e = 0; e < kPx; ++e) {
-                acc[e][c].x = fmaf(x[e], g.x, acc[e][c].x);
-                acc[e][c].y = fmaf(x[e], g.y, acc[e][c].y);
+        for (int u = 0; u < kBatch; ++u) {
+            if (t0 + u >= p) break;
+            float x[kPx];
+#pragma unroll
+            for (int e = 0; e < kPx; ++e) x[e] = static_cast<float>((w[u] >> (8 * e)) & 255u);
+            const float2* gt = Gs + (t0 + u) * CT;
+#pragma unroll
+            for (int c = 0; c < CT; ++c) {
+                const float2 g = gt[c];
+#pragma unroll
+                for (int e = 0; e < kPx; ++e) {
+                    acc[e][c].x = fmaf(x[e], g.x, acc[e][c].x);
+                    acc[e][c].y = fmaf(x[e], g.y, acc[e][c].y);
+                }
             }
         }
     }
-    const int cn = min(kCt, ncols - c0);
+    const int cn = min(CT, ncols - c0);
 #pragma unroll
     for (int e = 0; e < kPx; ++e) {
         if (j0 + e >= m) break;
         float2* dst = reinterpret_cast<float2*>(Phi) + (j0 + e) * ncols + c0;
 #pragma unroll
-        for (int c = 0; c < kCt; ++c)
+        for (int c = 0; c < CT; ++c)
             if (c < cn) dst[c] = acc[e][c];
     }
+}
+
+template <int CT>
+cdmd_status launch_tile(const uint8_t* D, int64_t m, int n, int64_t ldd, const double* G, int r, const int32_t* cols,
+                        int ncols, float* Phi, cudaStream_t stream) {
+    const int64_t pix = static_cast<int64_t>(kThreads) * kPx;
+    const dim3 grid(static_cast<unsigned>((m + pix - 1) / pix), static_cast<unsigned>((ncols + CT - 1) / CT));
+    auto kern = lift_fp32_kernel<CT>;
+    // the attribute covers eight modes whatever CT is: the longest clip stays the same
+    CDMD_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(static_cast<size_t>(n - 1) * 8 * sizeof(float2))));
+    kern<<<grid, kThreads, static_cast<size_t>(n - 1) * CT * sizeof(float2), stream>>>(D, m, n, ldd, G, r, cols, ncols, Phi);
+    CDMD_CHECK_LAUNCH("lift_fp32_kernel");
+    return CDMD_OK;
 }
 
 }  // namespace
@@ -85,15 +123,15 @@ cdmd_status launch_lift_fp32(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, 
                              const double* G, int r, const int32_t* cols, int ncols, float* Phi,
                              cudaStream_t stream) {
     (void)ctx;
-    const int64_t pix_per_cta = static_cast<int64_t>(kThreads) * kPx;
-    const dim3 grid(static_cast<unsigned>((m + pix_per_cta - 1) / pix_per_cta),
-                    static_cast<unsigned>((ncols + kCt - 1) / kCt));
-    const size_t smem = static_cast<size_t>(n - 1) * kCt * sizeof(float2);
-    CDMD_CHECK_CUDA(cudaFuncSetAttribute(lift_fp32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem)));
-    lift_fp32_kernel<<<grid, kThreads, smem, stream>>>(D, m, n, ldd, G, r, cols, ncols, Phi);
-    CDMD_CHECK_LAUNCH("lift_fp32_kernel");
-    return CDMD_OK;
+    const int tiles = (ncols + 7) / 8;
+#define CDMD_LIFT_TILE(CT) \
+    case CT: return launch_tile<CT>(D, m, n, ldd, G, r, cols, ncols, Phi, stream);
+    switch ((ncols + tiles - 1) / tiles) {
+        CDMD_LIFT_TILE(1) CDMD_LIFT_TILE(2) CDMD_LIFT_TILE(3) CDMD_LIFT_TILE(4)
+        CDMD_LIFT_TILE(5) CDMD_LIFT_TILE(6) CDMD_LIFT_TILE(7)
+        default: return launch_tile<8>(D, m, n, ldd, G, r, cols, ncols, Phi, stream);
+    }
+#undef CDMD_LIFT_TILE
 }
 
 }  // namespace cdmd
