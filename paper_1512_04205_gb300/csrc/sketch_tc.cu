@@ -503,8 +503,7 @@ __global__ void sketch_reduce_grouped_kernel(const ReduceChunk* __restrict__ chu
     }
     const ReduceChunk c = chunks[lo];
     const int64_t e = idx - prefix[lo];
-    double s = 0.0;
-    for (int sp = 0; sp < c.splits; ++sp) s += static_cast<double>(c.part[static_cast<int64_t>(sp) * c.elems + e]);
+    const double s = sum_partials(c.part + e, c.elems, c.splits);
     if (!isfinite(s)) record_status(status, CDMD_ERR_NONFINITE);
     c.DY[e] = s;
 }
@@ -928,8 +927,7 @@ __global__ void sketch_packed_reduce_kernel(const __grid_constant__ PackArgs a, 
     const int64_t total = static_cast<int64_t>(sg.L) * a.k;
     if (idx >= total) return;
     const int64_t src = static_cast<int64_t>(sg.row0) * a.k + idx;
-    double s = 0.0;
-    for (int sp = 0; sp < splits; ++sp) s += static_cast<double>(a.part[static_cast<int64_t>(sp) * kPackRows * a.k + src]);
+    const double s = sum_partials(a.part + src, static_cast<int64_t>(kPackRows) * a.k, splits);
     if (!isfinite(s)) record_status(status, CDMD_ERR_NONFINITE);
     sg.DY[static_cast<int64_t>(sg.f0) * a.k + idx] = s;
 }
@@ -1347,8 +1345,7 @@ __global__ void sketch_rad_reduce_kernel(const __grid_constant__ RadArgs a, int 
     if (idx >= total) return;
     const int64_t src = static_cast<int64_t>(sg.row0) * a.k + idx;
     const int64_t stride = static_cast<int64_t>(a.part_rows) * a.k;
-    double s = 0.0;
-    for (int sp = 0; sp < splits; ++sp) s += static_cast<double>(a.part[sp * stride + src]);
+    const double s = sum_partials(a.part + src, stride, splits);
     if (!isfinite(s)) record_status(status, CDMD_ERR_NONFINITE);
     sg.DY[static_cast<int64_t>(sg.f0) * a.k + idx] = s;
 }
@@ -1360,8 +1357,7 @@ __global__ void sketch_tc_reduce_kernel(const SketchArgs a, int splits, double* 
     const int64_t total = static_cast<int64_t>(a.k) * (g ? a.n[1] : a.n[0]);
     if (idx >= total) return;
     const float* part = g ? a.part[1] : a.part[0];
-    double s = 0.0;
-    for (int sp = 0; sp < splits; ++sp) s += static_cast<double>(part[static_cast<int64_t>(sp) * total + idx]);
+    const double s = sum_partials(part + idx, total, splits);
     if (!isfinite(s)) record_status(status, CDMD_ERR_NONFINITE);
     (g ? DY1 : DY0)[idx] = s;
 }
@@ -1422,7 +1418,7 @@ cdmd_status launch_sketch_tc_unit(cdmd_ctx* ctx, int nclips, const uint8_t* cons
     sketch_tc_kernel<<<dim3(rowblks, static_cast<unsigned>(splits)), kThreads, smem, stream>>>(tmap[0], tmap[1], a, ctx->d_status);
     CDMD_CHECK_LAUNCH("sketch_tc_kernel");
     const int64_t tot = static_cast<int64_t>(k) * std::max(a.n[0], a.n[1]);
-    sketch_tc_reduce_kernel<<<dim3(static_cast<unsigned>((tot + 255) / 256), nclips), 256, 0, stream>>>(
+    sketch_tc_reduce_kernel<<<dim3(static_cast<unsigned>((tot + kReduceThreads - 1) / kReduceThreads), nclips), kReduceThreads, 0, stream>>>(
         a, static_cast<int>(splits), DY[0], nclips > 1 ? DY[1] : nullptr, ctx->d_status);
     CDMD_CHECK_LAUNCH("sketch_tc_reduce_kernel");
     return CDMD_OK;
@@ -1470,7 +1466,7 @@ cdmd_status launch_sketch_rad_u8(cdmd_ctx* ctx, int nclips, const uint8_t* const
         sketch_rad_u8_kernel<<<dim3(rowblks, static_cast<unsigned>(splits)), kRThreads, smem, stream>>>(a, ctx->d_status);
         CDMD_CHECK_LAUNCH("sketch_rad_u8_kernel");
         const int64_t tot = static_cast<int64_t>(maxL) * k;
-        sketch_rad_reduce_kernel<<<dim3(static_cast<unsigned>((tot + 255) / 256), a.nseg), 256, 0, stream>>>(
+        sketch_rad_reduce_kernel<<<dim3(static_cast<unsigned>((tot + kReduceThreads - 1) / kReduceThreads), a.nseg), kReduceThreads, 0, stream>>>(
             a, static_cast<int>(splits), ctx->d_status);
         CDMD_CHECK_LAUNCH("sketch_rad_reduce_kernel");
         a.nseg = 0;
@@ -1611,7 +1607,7 @@ cdmd_status launch_sketch_tc_shared(cdmd_ctx* ctx, int nclips, const uint8_t* co
         }
         CDMD_CHECK_LAUNCH("sketch_tc_packed_kernel");
         const int64_t tot = static_cast<int64_t>(maxL) * k;
-        sketch_packed_reduce_kernel<<<dim3(static_cast<unsigned>((tot + 255) / 256), a.nseg), 256, 0, stream>>>(
+        sketch_packed_reduce_kernel<<<dim3(static_cast<unsigned>((tot + kReduceThreads - 1) / kReduceThreads), a.nseg), kReduceThreads, 0, stream>>>(
             a, static_cast<int>(splits), ctx->d_status);
         CDMD_CHECK_LAUNCH("sketch_packed_reduce_kernel");
         a.nseg = 0;
@@ -1650,7 +1646,7 @@ cdmd_status launch_sketch_grouped(const SketchItem* items, int nitems, size_t sm
                                          static_cast<int>(smem)));
     sketch_tc_grouped_kernel<<<static_cast<unsigned>(nitems), kThreads, smem, stream>>>(items, status);
     CDMD_CHECK_LAUNCH("sketch_tc_grouped_kernel");
-    sketch_reduce_grouped_kernel<<<static_cast<unsigned>((total + 255) / 256), 256, 0, stream>>>(chunks, prefix, nchunks,
+    sketch_reduce_grouped_kernel<<<static_cast<unsigned>((total + kReduceThreads - 1) / kReduceThreads), kReduceThreads, 0, stream>>>(chunks, prefix, nchunks,
                                                                                                 total, status);
     CDMD_CHECK_LAUNCH("sketch_reduce_grouped_kernel");
     return CDMD_OK;
