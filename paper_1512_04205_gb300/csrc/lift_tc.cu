@@ -92,8 +92,12 @@ __device__ __forceinline__ void split_f16(double g, int sh, uint16_t& hb, uint16
     const uint32_t sign = static_cast<uint32_t>(b >> 32) & 0x80000000u;
     uint64_t u = b & 0x7fffffffffffffffull;
     const int e = static_cast<int>(u >> 52), es = e + sh;
-    if (e == 0x7ff) {                              // infinity or NaN
-        hb = lb = f16_rn_bits(static_cast<float>(g));
+    if (e == 0x7ff || es > 1023 + 126) {
+        // infinity, NaN, or a number the clamped scale leaves at the end of
+        // FP32's range or past it: in FP64, whose conversions overflow to infinity
+        const double gs = g * __hiloint2double((1023 + sh) << 20, 0);
+        hb = f16_rn_bits(static_cast<float>(gs));
+        lb = f16_rn_bits(static_cast<float>(gs - static_cast<double>(f16_to_f32(hb))));
         return;
     }
     hb = lb = 0;
