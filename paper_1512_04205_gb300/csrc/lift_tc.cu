@@ -169,19 +169,26 @@ lift_tc_kernel(const __grid_constant__ CUtensorMap tmap, int64_t m, int n, const
     }
     // Scale of mode c: 2^s with max_t max(|Re G|, |Im G|) * 2^s in [2^14, 2^15),
     // so the FP16 hi and lo parts stay normal and far from overflow; only the
-    // maximum's exponent is needed, so the high words are compared.
+    // maximum's exponent is needed, so the high words are compared.  NaN is not
+    // counted, and a mode with an entry past 1e300 takes the scale of a maximum in
+    // [1/2, 1): the other part (Re or Im) of such a mode keeps its precision.
     for (int c = warp; c < kMaxModes; c += kThreads / 32) {
+        constexpr unsigned kPast = 0x7ff00000u;        // stands for every magnitude past 1e300
         unsigned mx = 0u;
         const int s = (c < nmodes) ? (cols ? cols[col0 + c] : col0 + c) : -1;
         if (s >= 0 && s < r) {
             const double* g = G + 2 * static_cast<int64_t>(s) * ldg;
-            for (int t = lane; t < 2 * p; t += 32)
-                mx = max(mx, static_cast<unsigned>(__double2hiint(g[t])) & 0x7fffffffu);
+            for (int t = lane; t < 2 * p; t += 32) {
+                const uint64_t b = static_cast<uint64_t>(__double_as_longlong(g[t])) & 0x7fffffffffffffffull;
+                unsigned h = static_cast<unsigned>(b >> 32);
+                if (b > static_cast<uint64_t>(__double_as_longlong(1.0e300))) h = b > (0x7ffull << 52) ? 0u : kPast;
+                mx = max(mx, h);
+            }
         }
         mx = __reduce_max_sync(0xffffffffu, mx);
         if (lane == 0) {
             int e = 0;
-            if (mx >= 0x00100000u && mx <= static_cast<unsigned>(__double2hiint(1.0e300)))
+            if (mx >= 0x00100000u && mx < kPast)
                 e = static_cast<int>(mx >> 20) - 1022;
             else if (mx < 0x00100000u && mx > 0u)
                 e = -1022;
