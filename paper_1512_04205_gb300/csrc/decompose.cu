@@ -601,6 +601,11 @@ __device__ __forceinline__ int sturm_count(const double* d, const double* e2, in
 }
 
 constexpr double kSearchTol = 256.0 * kEps;
+// Neighbours nearer than this (of the norm) make a cluster, whose eigenvalues are
+// searched to eps.  Past it a shift off by kSearchTol / 2 = 128 eps leaves a share of
+// (128 eps / gap)^2 < 1e-4 of the neighbour in the vector after two solves, and the
+// Rayleigh quotient is off by the gap times that share squared, below 2e-4 eps.
+constexpr double kClusterGap = 16384.0 * kEps;
 constexpr int kEigThreads = 128;   // one warp per scheduler; one shift per thread
 
 // The first of the block's kEigThreads flags that is set (kEigThreads if
@@ -628,6 +633,9 @@ __device__ __forceinline__ int first_set(bool flag, unsigned* ball, int turn) {
 // solves leave the square of shift error / gap of other vectors).  The Rayleigh
 // quotient of its vector then gives the eigenvalue to rounding level, which
 // errs with z's share of the norm where a Sturm count errs with the norm itself.
+// With a neighbour within kClusterGap (counted by the same FP64 pass) neither
+// holds: the search goes on to eps, and the quotient moves the eigenvalue by no
+// more than the count's own error.
 // sigma and G at n = 300, r = 30, against LAPACK in FP64: off by 3.7e-16 and
 // 4.5e-13; 8.9e-15 and 4.9e-12 with the search carried on to eps.
 // Inverse iteration: LU with partial pivoting and two solves by one thread,
@@ -694,6 +702,7 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
     // FP32 bracket (skipped when the scale factor would leave the range)
     const int ex = (__double2hiint(tn) >> 20) & 0x7ff;
     bool bracket = ex > 64 && ex < 1983;
+    bool cluster = true;         // unless the FP64 pass counts no neighbour
     if (bracket) {
         const double sc = __hiloint2double((2046 - ex - 1) << 20, 0);     // tn sc in [1/2, 1)
         const double isc = __hiloint2double((ex + 1) << 20, 0);
@@ -729,14 +738,21 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
         }
         lo = (lo - margin2) * isc;
         hi = (hi + margin2) * isc;
-        // the ends of the bracket and 126 shifts between them
-        const double step = (hi - lo) * (1.0 / (kEigThreads - 1));
-        const bool above = sturm_count(d, e2, p, fma(step, static_cast<double>(tid), lo)) > idx;
-        const int f = first_set(above, ball, turn++);
-        bracket = f > 0 && f < kEigThreads;
+        // threads 1 .. 126: the ends of the bracket and 124 shifts between them;
+        // 0 and 127: kClusterGap outside, to count the neighbours
+        const double step = (hi - lo) * (1.0 / (kEigThreads - 3));
+        const double x = tid == 0                 ? lo - kClusterGap * tn
+                         : tid == kEigThreads - 1 ? hi + kClusterGap * tn
+                                                  : fma(step, static_cast<double>(tid - 1), lo);
+        const int count = sturm_count(d, e2, p, x);
+        if (tid == 0) flags[2] = count;
+        if (tid == kEigThreads - 1) flags[3] = count;
+        const int f = first_set(count > idx, ball, turn++);
+        bracket = f > 1 && f < kEigThreads - 1;
         if (bracket) {
-            hi = fma(step, static_cast<double>(f), lo);
-            lo = fma(step, static_cast<double>(f - 1), lo);
+            hi = fma(step, static_cast<double>(f - 1), lo);
+            lo = fma(step, static_cast<double>(f - 2), lo);
+            cluster = flags[3] - flags[2] > 1;
         }
     }
     if (!bracket) {
@@ -746,7 +762,8 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
     bool converged = false;
     for (int it = 0; it < 40; ++it) {
         const double width = hi - lo;
-        if (width <= kSearchTol * tn + 1e-300) { converged = true; break; }
+        const double tol = cluster ? 2.0 * kEps * fmax(fabs(lo), fabs(hi)) + kEps * tn : kSearchTol * tn;
+        if (width <= tol + 1e-300) { converged = true; break; }
         const double step = width * (1.0 / (kEigThreads + 1));
         const bool above = sturm_count(d, e2, p, fma(step, static_cast<double>(tid + 1), lo)) > idx;
         const int f = first_set(above, ball, turn++);
@@ -891,10 +908,10 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
     const double inv = rsqrt64(nrm2);
     for (int i = tid; i < p; i += kEigThreads) Z[i] = z[i] * inv;
     if (tid == 0) {
-        // the Rayleigh quotient: its error is the square of z's.  Within a
-        // cluster z may mix neighbours; the search's interval bounds the step.
+        // the Rayleigh quotient: its error is the square of z's.  Where z may mix
+        // neighbours, the search's interval (and the count's error) bounds the step.
         const double step = ((red[4] + red[5]) + (red[6] + red[7])) * inv * inv;
-        if (fabs(step) <= 2.0 * kSearchTol * tn) q.lamT[w] = lambda + step;
+        if (fabs(step) <= (cluster ? 8.0 * kEps : 2.0 * kSearchTol) * tn) q.lamT[w] = lambda + step;
     }
 }
 
@@ -1258,7 +1275,11 @@ backtransform_kernel(const __grid_constant__ SolveBatch sb) {
     for (int i = tid; i < p; i += kOrthThreads) clip.V[static_cast<int64_t>(c) * p + i] = y[i];
     if (tid == 0) {
         const double l0 = clip.lamT[0];
-        const double lc = clip.lamT[c];
+        double lc = clip.lamT[c];
+        // within a cluster the quotients' rounding may leave neighbours out of order
+        if (clip.flag[1] != 0)
+            for (int u = 0; u < c; ++u)
+                if (clip.lamT[u] < lc) lc = clip.lamT[u];
         if (!(lc > kRankTol * static_cast<double>(p) * kEps * fabs(l0)))
             record_status(sb.status, CDMD_ERR_RANK_DEFICIENT);
         clip.sigma[c] = lc > 0.0 ? lc * rsqrt64(lc) : 0.0;
