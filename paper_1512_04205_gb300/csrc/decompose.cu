@@ -69,6 +69,7 @@ struct SolveClip {
     const double* DY;    // k x n sketch; NULL when R is given
     const double* R;     // n x n Gram
     int n, p;            // frames, p = n - 1
+    int kchunk, splits;  // sketch rows per Gram CTA, and how many such chunks (0 when R is given)
     double *gpart, *Rw;  // Gram partials; the Gram's own storage (NULL when R is given)
     double *Hv, *htau, *Tw, *dd, *ee;             // reflectors, their block factors, the tridiagonal form
     double *lamT, *Z, *V, *B, *At, *Nm, *dv, *W, *M, *WR, *lamR, *cvec;
@@ -152,9 +153,29 @@ __device__ __forceinline__ cd shfl_cd(cd v, int src) {
 // ---------------------------------------------------------------------------
 constexpr int kGT = 32;
 
+// Rows of the sketch per CTA: the FP64 rate bounds the pass, so the multiple of 32
+// that leaves the least work to the busiest SM (and of two equal ones the larger,
+// for fewer partials to add up).  The choice decides the order of the sums, so it
+// looks at this clip's n and k alone, and at a fixed number of SMs: a clip's Gram
+// has the same bits whichever clips share the launch, and on every device.
+constexpr int kGramSms = 152;
+int gram_chunk(int n, int k) {
+    const int64_t nt = (n + kGT - 1) / kGT, tiles = nt * (nt + 1) / 2;
+    int64_t best = INT64_MAX;
+    int kchunk = 256;
+    for (int kc = 256; kc >= 64; kc -= 32) {
+        const int64_t ctas = tiles * ((k + kc - 1) / kc);
+        const int64_t load = (ctas + kGramSms - 1) / kGramSms * (std::min(kc, k) + 8);
+        if (load < best) { best = load; kchunk = kc; }
+    }
+    return kchunk;
+}
+
 __global__ void __launch_bounds__(256)
-gram_partial_kernel(const __grid_constant__ SolveBatch sb, int kchunk) {
+gram_partial_kernel(const __grid_constant__ SolveBatch sb) {
     const SolveClip& q = sb.c[blockIdx.y];
+    if (static_cast<int>(blockIdx.z) >= q.splits) return;
+    const int kchunk = q.kchunk;
     const double* DY = q.DY;
     const int k = sb.k, n = q.n;
     // blockIdx.x counts the tile pairs ta <= tb row by row
@@ -195,8 +216,9 @@ gram_partial_kernel(const __grid_constant__ SolveBatch sb, int kchunk) {
     }
 }
 
-__global__ void gram_reduce_kernel(const __grid_constant__ SolveBatch sb, int splits) {
+__global__ void gram_reduce_kernel(const __grid_constant__ SolveBatch sb) {
     const SolveClip& q = sb.c[blockIdx.y];
+    const int splits = q.splits;
     const double* part = q.gpart;
     const int n = q.n;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2537,28 +2559,16 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
                            cdmd_selector selector, cudaStream_t stream, const AutoRank* autor = nullptr) {
     if (nclips < 1 || nclips > kMaxSolveClips) return fail(CDMD_ERR_INVALID_ARG, "%d clips in one solve", nclips);
     // ---- workspace layout (doubles), one region per clip ----
-    // rows of the sketch per Gram CTA: the FP64 rate bounds the pass, so the
-    // multiple of 32 that leaves the least work to the busiest SM (and of two
-    // equal ones the larger, for fewer partials to add up)
-    int kchunk = 128;
-    if (io[0].R == nullptr) {
-        int64_t tiles = 0, best = INT64_MAX;
-        for (int i = 0; i < nclips; ++i) {
-            const int64_t nt = (io[i].n + kGT - 1) / kGT;
-            tiles += nt * (nt + 1) / 2;
-        }
-        for (int kc = 256; kc >= 64; kc -= 32) {
-            const int64_t ctas = tiles * ((k + kc - 1) / kc);
-            const int64_t load = (ctas + ctx->device_sms - 1) / ctx->device_sms * (std::min(kc, k) + 8);
-            if (load < best) { best = load; kchunk = kc; }
-        }
-    }
-    const int splits = io[0].R != nullptr ? 0 : (k + kchunk - 1) / kchunk;
     size_t off[kMaxSolveClips + 1] = {0};
-    int nmax = 0;
+    SolveBatch sb = {};
+    int nmax = 0, splits = 0;
     for (int i = 0; i < nclips; ++i) {
         const size_t n = io[i].n, p = n - 1, rr = r;
-        const size_t total = static_cast<size_t>(splits) * n * n + n * n + p * p + 32 * p + 1024 + 3 * p + rr +
+        SolveClip& q = sb.c[i];
+        q.kchunk = io[i].R != nullptr ? 0 : gram_chunk(io[i].n, k);
+        q.splits = io[i].R != nullptr ? 0 : (k + q.kchunk - 1) / q.kchunk;
+        splits = std::max(splits, q.splits);
+        const size_t total = static_cast<size_t>(q.splits) * n * n + n * n + p * p + 32 * p + 1024 + 3 * p + rr +
                              3 * p * rr + 12 * rr * rr + 8 * rr + 64;
         // + one slot for the eigen-solver's fallback flag and two for the rank
         // threshold's result; with an automatic rank, r is its upper bound here
@@ -2568,7 +2578,6 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
     double* ws = nullptr;
     cdmd_status st = ensure_buffer(ctx, BUF_EIG, off[nclips] * sizeof(double), reinterpret_cast<void**>(&ws));
     if (st != CDMD_OK) return st;
-    SolveBatch sb = {};
     sb.k = k;
     sb.status = ctx->d_status;
     bool want_phiy = false;
@@ -2600,7 +2609,7 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
         q.n = io[i].n;
         q.p = q.n - 1;
         q.gpart = ws + off[i];
-        q.Rw = q.gpart + static_cast<size_t>(splits) * q.n * q.n;
+        q.Rw = q.gpart + static_cast<size_t>(q.splits) * q.n * q.n;
         q.R = io[i].R != nullptr ? io[i].R : q.Rw;
         q.Hv = q.Rw + static_cast<size_t>(q.n) * q.n;
         q.htau = q.Hv + static_cast<size_t>(q.p) * q.p;
@@ -2629,9 +2638,9 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
     // 1. Gram
     if (splits > 0) {
         const int ntiles = (nmax + kGT - 1) / kGT;
-        gram_partial_kernel<<<dim3(ntiles * (ntiles + 1) / 2, nc, splits), 256, 0, stream>>>(sb, kchunk);
+        gram_partial_kernel<<<dim3(ntiles * (ntiles + 1) / 2, nc, splits), 256, 0, stream>>>(sb);
         CDMD_CHECK_LAUNCH("gram_partial_kernel");
-        gram_reduce_kernel<<<dim3((nmax * nmax + 255) / 256, nc), 256, 0, stream>>>(sb, splits);
+        gram_reduce_kernel<<<dim3((nmax * nmax + 255) / 256, nc), 256, 0, stream>>>(sb);
         CDMD_CHECK_LAUNCH("gram_reduce_kernel");
     }
 
