@@ -60,6 +60,12 @@ constexpr double kRankTol = 64.0;
 constexpr int kMaxR = 32;
 constexpr size_t kMaxOptInSmem = 232448;      // opt-in shared memory per CTA
 
+// Reflectors go in blocks of 32 while two of them fit the back-transform's shared
+// memory, else 16.  Per clip: a longer one in the same call does not change a
+// clip's blocks, and with them its bits; each of the two kernels passes over the
+// other width's clips.
+__host__ __device__ constexpr int wy_width(int p) { return p <= 256 ? 32 : 16; }
+
 // One launch of each kernel below serves every clip of a call (up to
 // kMaxSolveClips clips under one C, their own n, the same k, r, K): the chain
 // is bound by dependent FP64 latency and leaves the device mostly idle, so the
@@ -1000,12 +1006,14 @@ __device__ void wy_cta(const SolveClip& q, int blk, double* tsm) {
     for (int idx = tid; idx < NB * NB; idx += kEigThreads) T[idx] = Ts[(idx % NB) * NB + idx / NB];
 }
 
-// blockIdx.x < r: eigenpair blockIdx.x; above: block blockIdx.x - r of reflectors
+// blockIdx.x < r: eigenpair blockIdx.x; above: block blockIdx.x - r of reflectors.
+// The clips whose reflectors go NB at a time.
 template <int NB>
 __global__ void __launch_bounds__(kEigThreads)
 tridiag_eigpair_kernel(const __grid_constant__ SolveBatch sb) {
     extern __shared__ double tsm[];
     const SolveClip& q = sb.c[blockIdx.z];
+    if (wy_width(q.p) != NB) return;
     const int b = static_cast<int>(blockIdx.x);
     if (b == 0 && threadIdx.x == 0) q.flag[1] = 0;      // set by orthogonality_kernel
     if (b < sb.r) eigpair_cta(q, b, sb.status, tsm);
@@ -1229,6 +1237,7 @@ backtransform_kernel(const __grid_constant__ SolveBatch sb) {
     constexpr int kWarps = kOrthThreads / 32;
     static_assert(NB % kWarps == 0 && NB <= 32, "rows per warp");
     const SolveClip& clip = sb.c[blockIdx.z];
+    if (wy_width(clip.p) != NB) return;
     const int p = clip.p, c = blockIdx.x;
     extern __shared__ double ysm[];
     double* y = ysm;                              // p
@@ -2716,25 +2725,34 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
         lay_out(r);
     }
     // 3. eigenpairs of T and, beside them, the reflectors' block factors; one
-    // step of orthogonalisation; back-transform.  Blocks of 32 reflectors while
-    // two of them fit the shared memory (p <= 256), else 16
-    const bool wide = p <= 256;
+    // step of orthogonalisation; back-transform.  One launch per width of
+    // reflector blocks that the call's clips have, sized for the longest of them
     {
-        const int nb = wide ? 32 : 16;
-        const int nblk = p > 2 ? (p - 2 + nb - 1) / nb : 0;
-        const size_t esm = std::max(84 * static_cast<size_t>(p),
-                                    (2 * nb + static_cast<size_t>(p)) * nb * sizeof(double));
-        const size_t bsm = (2 * nb + 1) * static_cast<size_t>(p) * sizeof(double);
-        void (*ek)(SolveBatch) = wide ? tridiag_eigpair_kernel<32> : tridiag_eigpair_kernel<16>;
-        void (*bk)(SolveBatch) = wide ? backtransform_kernel<32> : backtransform_kernel<16>;
-        for (auto kern : {ek, bk})
-            CDMD_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
-        ek<<<dim3(r + nblk, 1, nc), kEigThreads, esm, stream>>>(sb);
-        CDMD_CHECK_LAUNCH("tridiag_eigpair_kernel");
+        int pw[2] = {0, 0};          // longest p of the clips with blocks of 16, of 32
+        for (int i = 0; i < nclips; ++i) {
+            int& w = pw[wy_width(sb.c[i].p) == 32];
+            w = std::max(w, sb.c[i].p);
+        }
+        void (*const ek[2])(SolveBatch) = {tridiag_eigpair_kernel<16>, tridiag_eigpair_kernel<32>};
+        void (*const bk[2])(SolveBatch) = {backtransform_kernel<16>, backtransform_kernel<32>};
+        for (int w = 0; w < 2; ++w) {
+            if (pw[w] == 0) continue;
+            const size_t nb = w ? 32 : 16, pc = pw[w];
+            const int nblk = pc > 2 ? static_cast<int>((pc - 2 + nb - 1) / nb) : 0;
+            const size_t esm = std::max(84 * pc, (2 * nb + pc) * nb * sizeof(double));
+            for (auto kern : {ek[w], bk[w]})
+                CDMD_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
+            ek[w]<<<dim3(r + nblk, 1, nc), kEigThreads, esm, stream>>>(sb);
+            CDMD_CHECK_LAUNCH("tridiag_eigpair_kernel");
+        }
         orthogonality_kernel<<<dim3(r, 1, nc), kOrthThreads, 0, stream>>>(sb);
         CDMD_CHECK_LAUNCH("orthogonality_kernel");
-        bk<<<dim3(r, 1, nc), kOrthThreads, bsm, stream>>>(sb);
-        CDMD_CHECK_LAUNCH("backtransform_kernel");
+        for (int w = 0; w < 2; ++w) {
+            if (pw[w] == 0) continue;
+            const size_t bsm = (2 * (w ? 32 : 16) + 1) * static_cast<size_t>(pw[w]) * sizeof(double);
+            bk[w]<<<dim3(r, 1, nc), kOrthThreads, bsm, stream>>>(sb);
+            CDMD_CHECK_LAUNCH("backtransform_kernel");
+        }
     }
     // 4. A~ and its eigen-decomposition
     bmat_kernel<<<dim3((nmax + 7) / 8, (r + 3) / 4, nc), 256, 0, stream>>>(sb);

@@ -1,7 +1,8 @@
 """A clip's small solves give the same bits whichever clips share the launches
 (FP32 sketches are per clip, so every stage sees the same inputs).  Unlike a k of
 one Gram block, these k are summed in several, whose size must not follow the
-companions' lengths; each clip takes its turn as the last, whose results the
+companions' lengths, and clips on both sides of 257 frames apply their reflectors
+in blocks of 32 and of 16; each clip takes its turn as the last, whose results the
 context shows."""
 import numpy as np
 import pytest
@@ -23,7 +24,8 @@ def C():
 
 
 @pytest.mark.parametrize("ns,k", [((200, 200, 200), 1000), ((200, 61, 130), 1000), ((40, 256, 33, 90, 100), 333),
-                                  ((100,) * 8, 700), ((120, 120), 4099)])
+                                  ((100,) * 8, 700), ((120, 120), 4099),
+                                  ((30, 260), 300), ((257, 130, 258), 200)])
 def test_solves_keep_their_bits_in_company(C, ns, k):
     w, h, r, K = 64, 48, 8, 4
     ctx = C.Context(0)
