@@ -164,19 +164,44 @@ constexpr int kGT = 32;
 // for fewer partials to add up).  The choice decides the order of the sums, so it
 // looks at this clip's n and k alone, and at a fixed number of SMs: a clip's Gram
 // has the same bits whichever clips share the launch, and on every device.
+// Some 16 CTAs an SM are enough, so a long sketch takes longer chunks; within one
+// the sums start anew every 256 rows, which keeps their rounding.
 constexpr int kGramSms = 152;
+constexpr int kGramRows = 256;
+constexpr int64_t gram_tiles(int n) { return static_cast<int64_t>((n + kGT - 1) / kGT) * ((n + kGT - 1) / kGT + 1) / 2; }
+constexpr int64_t gram_max_splits(int n) { return (16 * kGramSms + gram_tiles(n) - 1) / gram_tiles(n); }
 int gram_chunk(int n, int k) {
-    const int64_t nt = (n + kGT - 1) / kGT, tiles = nt * (nt + 1) / 2;
+    const int64_t tiles = gram_tiles(n), most = gram_max_splits(n);
     int64_t best = INT64_MAX;
-    int kchunk = 256;
-    for (int kc = 256; kc >= 64; kc -= 32) {
+    int kchunk = static_cast<int>(std::max<int64_t>(kGramRows, ((k + most - 1) / most + 31) / 32 * 32));
+    for (int kc = kchunk; kc >= 64 && (k + kc - 1) / kc <= most; kc -= 32) {
         const int64_t ctas = tiles * ((k + kc - 1) / kc);
         const int64_t load = (ctas + kGramSms - 1) / kGramSms * (std::min(kc, k) + 8);
         if (load < best) { best = load; kchunk = kc; }
     }
     return kchunk;
 }
+// Room for the partials (doubles): at least splits x n x n for the rule above, and
+// never less for a larger n or k, so that a workspace sized by the largest problem
+// serves every smaller one (a stream capture cannot grow it).  n <= 512: at most
+// 39 MB.
+constexpr int kMaxFrames = 512;
+constexpr int64_t gram_room_most() {
+    int64_t most = 0;
+    for (int n = 1; n <= kMaxFrames; ++n) {
+        const int64_t room = gram_max_splits(n) * n * n;
+        most = room > most ? room : most;
+    }
+    return most;
+}
+int64_t gram_room(int n, int k) {
+    constexpr int64_t most = gram_room_most();
+    return std::min<int64_t>(most, static_cast<int64_t>((k + 63) / 64) * n * n);
+}
 
+// kLong: for chunks past kGramRows; the sums so far take eight registers, which cost
+// the short form a quarter of its warps (n = 200, k = 20000: 2% of the whole call).
+template <bool kLong>
 __global__ void __launch_bounds__(256)
 gram_partial_kernel(const __grid_constant__ SolveBatch sb) {
     const SolveClip& q = sb.c[blockIdx.y];
@@ -197,8 +222,15 @@ gram_partial_kernel(const __grid_constant__ SolveBatch sb) {
     const int a0 = ta * kGT, b0 = tb * kGT;
     const int ibeg = blockIdx.z * kchunk;
     const int iend = min(k, ibeg + kchunk);
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    double acc[4] = {0.0, 0.0, 0.0, 0.0}, sum[4] = {0.0, 0.0, 0.0, 0.0};
     for (int i0 = ibeg; i0 < iend; i0 += kGT) {
+        if (kLong && (i0 - ibeg) % kGramRows == 0) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                sum[e] += acc[e];
+                acc[e] = 0.0;
+            }
+        }
         for (int idx = tid; idx < kGT * kGT; idx += 256) {
             const int ii = idx & 31, cc = idx >> 5;
             const int i = i0 + ii;
@@ -214,6 +246,9 @@ gram_partial_kernel(const __grid_constant__ SolveBatch sb) {
         }
         __syncthreads();
     }
+    if (kLong)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[e] += sum[e];
     double* dst = q.gpart + static_cast<int64_t>(blockIdx.z) * n * n;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -2577,7 +2612,8 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
         q.kchunk = io[i].R != nullptr ? 0 : gram_chunk(io[i].n, k);
         q.splits = io[i].R != nullptr ? 0 : (k + q.kchunk - 1) / q.kchunk;
         splits = std::max(splits, q.splits);
-        const size_t total = static_cast<size_t>(q.splits) * n * n + n * n + p * p + 32 * p + 1024 + 3 * p + rr +
+        const size_t room = io[i].R != nullptr ? 0 : gram_room(io[i].n, k);
+        const size_t total = room + n * n + p * p + 32 * p + 1024 + 3 * p + rr +
                              3 * p * rr + 12 * rr * rr + 8 * rr + 64;
         // + one slot for the eigen-solver's fallback flag and two for the rank
         // threshold's result; with an automatic rank, r is its upper bound here
@@ -2618,7 +2654,7 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
         q.n = io[i].n;
         q.p = q.n - 1;
         q.gpart = ws + off[i];
-        q.Rw = q.gpart + static_cast<size_t>(q.splits) * q.n * q.n;
+        q.Rw = q.gpart + (io[i].R != nullptr ? 0 : gram_room(q.n, k));
         q.R = io[i].R != nullptr ? io[i].R : q.Rw;
         q.Hv = q.Rw + static_cast<size_t>(q.n) * q.n;
         q.htau = q.Hv + static_cast<size_t>(q.p) * q.p;
@@ -2647,7 +2683,10 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
     // 1. Gram
     if (splits > 0) {
         const int ntiles = (nmax + kGT - 1) / kGT;
-        gram_partial_kernel<<<dim3(ntiles * (ntiles + 1) / 2, nc, splits), 256, 0, stream>>>(sb);
+        bool longer = false;
+        for (int i = 0; i < nclips; ++i) longer = longer || sb.c[i].kchunk > kGramRows;
+        auto gram = longer ? gram_partial_kernel<true> : gram_partial_kernel<false>;
+        gram<<<dim3(ntiles * (ntiles + 1) / 2, nc, splits), 256, 0, stream>>>(sb);
         CDMD_CHECK_LAUNCH("gram_partial_kernel");
         gram_reduce_kernel<<<dim3((nmax * nmax + 255) / 256, nc), 256, 0, stream>>>(sb);
         CDMD_CHECK_LAUNCH("gram_reduce_kernel");
