@@ -37,6 +37,14 @@ void clear_error();
         if (!(cond)) return ::cdmd::fail(CDMD_ERR_INVALID_ARG, __VA_ARGS__); \
     } while (0)
 
+// Opt-in to dynamic shared memory beyond 48 KB.  The limit belongs to the function,
+// not to a context or a thread, so it is the device's maximum on every call: a limit
+// of this call's own size, set by one thread between another's opt-in and its
+// launch, would have that launch refused.  (Kernels without static shared memory.)
+constexpr int kMaxDynamicSmem = 232448;
+#define CDMD_ALLOW_SMEM(kern)                                                                              \
+    CDMD_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ::cdmd::kMaxDynamicSmem))
+
 // Device status word: the first numerical error recorded wins.
 __device__ __forceinline__ void record_status(int* status, int code) {
     if (status != nullptr) atomicCAS(status, 0, code);

@@ -109,9 +109,7 @@ cdmd_status launch_tile(const uint8_t* D, int64_t m, int n, int64_t ldd, const d
     const int64_t pix = static_cast<int64_t>(kThreads) * kPx;
     const dim3 grid(static_cast<unsigned>((m + pix - 1) / pix), static_cast<unsigned>((ncols + CT - 1) / CT));
     auto kern = lift_fp32_kernel<CT>;
-    // the attribute covers eight modes whatever CT is: the longest clip stays the same
-    CDMD_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(static_cast<size_t>(n - 1) * 8 * sizeof(float2))));
+    // at most 511 frames of eight modes: 32 KB, no opt-in
     kern<<<grid, kThreads, static_cast<size_t>(n - 1) * CT * sizeof(float2), stream>>>(D, m, n, ldd, G, r, cols, ncols, Phi);
     CDMD_CHECK_LAUNCH("lift_fp32_kernel");
     return CDMD_OK;

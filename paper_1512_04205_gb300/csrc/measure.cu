@@ -504,9 +504,7 @@ cdmd_status launch_measure_build(cdmd_ctx* ctx, cdmd_measure* meas, cudaStream_t
             m, k, seed_key(meas->seed), srft ? kStreamSrftFreq : kStreamRowsample, draws);
         CDMD_CHECK_LAUNCH("rowsample_draw_kernel");
         const size_t smem = in_smem ? slots * sizeof(int64_t) : 0;
-        if (smem > 48 * 1024)
-            CDMD_CHECK_CUDA(cudaFuncSetAttribute(rowsample_floyd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 static_cast<int>(smem)));
+        CDMD_ALLOW_SMEM(rowsample_floyd_kernel);
         rowsample_floyd_kernel<<<1, 1024, smem, stream>>>(m, k, draws, table, bits, picks);
         CDMD_CHECK_LAUNCH("rowsample_floyd_kernel");
         rank_sort_kernel<<<static_cast<unsigned>((k + 255) / 256), 256, 0, stream>>>(picks, k, meas->rows);

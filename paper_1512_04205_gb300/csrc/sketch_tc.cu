@@ -1413,8 +1413,7 @@ cdmd_status launch_sketch_tc_unit(cdmd_ctx* ctx, int nclips, const uint8_t* cons
     a.key = seed_key(seed);
     const size_t smem = smem_layout(mtiles, nclips, a.n[0], a.n[1]).total + 1024;
     if (smem > kMaxSmem) return fail(CDMD_ERR_UNSUPPORTED, "sketch: %zu bytes of shared memory per CTA", smem);
-    CDMD_CHECK_CUDA(cudaFuncSetAttribute(sketch_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem)));
+    CDMD_ALLOW_SMEM(sketch_tc_kernel);
     sketch_tc_kernel<<<dim3(rowblks, static_cast<unsigned>(splits)), kThreads, smem, stream>>>(tmap[0], tmap[1], a, ctx->d_status);
     CDMD_CHECK_LAUNCH("sketch_tc_kernel");
     const int64_t tot = static_cast<int64_t>(k) * std::max(a.n[0], a.n[1]);
@@ -1642,8 +1641,7 @@ cdmd_status launch_sketch_tc_shared(cdmd_ctx* ctx, int nclips, const uint8_t* co
 cdmd_status launch_sketch_grouped(const SketchItem* items, int nitems, size_t smem, const ReduceChunk* chunks,
                                   const int64_t* prefix, int nchunks, int64_t total, int* status, cudaStream_t stream) {
     if (smem > kMaxSmem) return fail(CDMD_ERR_UNSUPPORTED, "grouped sketch: %zu bytes of shared memory per CTA", smem);
-    CDMD_CHECK_CUDA(cudaFuncSetAttribute(sketch_tc_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem)));
+    CDMD_ALLOW_SMEM(sketch_tc_grouped_kernel);
     sketch_tc_grouped_kernel<<<static_cast<unsigned>(nitems), kThreads, smem, stream>>>(items, status);
     CDMD_CHECK_LAUNCH("sketch_tc_grouped_kernel");
     sketch_reduce_grouped_kernel<<<static_cast<unsigned>((total + kReduceThreads - 1) / kReduceThreads), kReduceThreads, 0, stream>>>(chunks, prefix, nchunks,

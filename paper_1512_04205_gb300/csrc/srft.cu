@@ -301,8 +301,7 @@ cdmd_status launch_sketch_srft(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n
                                    reinterpret_cast<void**>(&part));
     if (st != CDMD_OK) return st;
     const size_t smem = fixed + static_cast<size_t>(S) * per_col;
-    CDMD_CHECK_CUDA(cudaFuncSetAttribute(srft_partial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem)));
+    CDMD_ALLOW_SMEM(srft_partial_kernel);
     srft_partial_kernel<<<dim3(groups, fgroups), kSrftThreads, smem, stream>>>(
         D, m, n, ldd, N1, static_cast<int>(N2), S, srft_stages(N2), seed_key(meas->seed), meas->rows, nf, tiles,
         tiles_per_group, fpc, reinterpret_cast<float2*>(part));

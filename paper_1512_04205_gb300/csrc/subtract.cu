@@ -640,8 +640,7 @@ cdmd_status launch_nc_tma(cdmd_ctx* ctx, cdmd_bgmode mode, const uint8_t* D, int
 #define CDMD_SUBT_MODE(MV)                                                                              \
     {                                                                                                   \
         auto kern = subtract_tma_kernel<NC, MV>;                                                        \
-        CDMD_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,         \
-                                             static_cast<int>(smem)));                                  \
+        CDMD_ALLOW_SMEM(kern);                                                                          \
         kern<<<static_cast<unsigned>(blocks), kTmaThreads, smem, stream>>>(tmap, m, n, Phi, ncols, tb, tau, \
                                                                            mask, wpf, bg, ctx->d_status); \
     }
@@ -666,8 +665,7 @@ cdmd_status launch_nc(cdmd_bgmode mode, const uint8_t* D, int64_t m, int n, int6
 #define CDMD_SUB_MODE(MV)                                                                         \
     {                                                                                             \
         auto kern = subtract_kernel<NC, PX, MV>;                                                  \
-        CDMD_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                                             static_cast<int>(smem)));                            \
+        CDMD_ALLOW_SMEM(kern);                                                                    \
         kern<<<static_cast<unsigned>(blocks), kThreads, smem, stream>>>(D, m, n, ldd, Phi, ncols, \
                                                                         tb, tau, mask, wpf, bg);  \
     }
@@ -762,8 +760,7 @@ cdmd_status launch_subtract_grouped(const SubtractClip* clips, int nclips, const
 #define CDMD_SUBG(NCV, MV)                                                                                   \
     {                                                                                                        \
         auto kern = subtract_tma_grouped_kernel<NCV, MV>;                                                    \
-        CDMD_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,              \
-                                             static_cast<int>(smem)));                                       \
+        CDMD_ALLOW_SMEM(kern);                                                                               \
         kern<<<static_cast<unsigned>(nitems), kTmaThreads, smem, stream>>>(clips, items, tau, status);       \
     }
 #define CDMD_SUBG_NC(MV)                                \
