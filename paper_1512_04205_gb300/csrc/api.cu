@@ -11,12 +11,14 @@ namespace cdmd {
 namespace {
 thread_local char g_last_error[512] = "";
 
-// Restores the caller's current device on scope exit.
+// Restores the caller's current device on scope exit.  The device is set even when
+// it is the current one already: in a host thread that has made no CUDA call yet,
+// that is what gives it the context the tensor maps' driver call needs.
 struct DeviceGuard {
     int prev = -1;
     explicit DeviceGuard(int dev) {
         if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
-        if (prev != dev) cudaSetDevice(dev);
+        cudaSetDevice(dev);
     }
     ~DeviceGuard() {
         int cur = -1;

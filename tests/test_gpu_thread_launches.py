@@ -72,3 +72,31 @@ def test_calls_of_two_threads(C, what):
     for ctx in ctxs:
         C.cdmd_status_sync(ctx)
     assert not errors, (len(errors), errors[0])
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16x2"])
+def test_first_call_of_a_thread(C, prec):
+    # a thread's first CUDA call may be the library's: a sketch whose workspace exists
+    # starts with the tensor map of the video
+    ctx = C.Context(0)
+    D = _video(40, 640, 640)
+    DY = torch.empty((40, 64), dtype=torch.float64, device="cuda")
+    stream = torch.cuda.current_stream()
+    C.cdmd_sketch(ctx, D, 64, 3, prec=prec, DY=DY, stream=stream)
+    torch.cuda.synchronize()
+    want, errors = DY.clone(), []
+    DY.zero_()
+
+    def work():
+        try:
+            C.cdmd_sketch(ctx, D, 64, 3, prec=prec, DY=DY, stream=stream)
+        except C.CdmdError as e:
+            errors.append(str(e))
+
+    torch.cuda.synchronize()
+    t = threading.Thread(target=work)
+    t.start()
+    t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    assert torch.equal(DY, want)
