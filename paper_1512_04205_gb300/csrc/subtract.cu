@@ -180,12 +180,13 @@ subtract_table_kernel(const int32_t* __restrict__ cols, int ncols, int nc_pad, c
     build_table(cols, ncols, nc_pad, beta, lambda, r, n, tb, blockIdx.x * (kTableThreads / 32) + (threadIdx.x >> 5));
 }
 
-// Grouped: blockIdx.y = clip, tables with the common column stride nc.
+// Grouped: blockIdx.x = clip (a batch may hold more clips than a grid has rows),
+// tables with the common column stride nc.
 __global__ void __launch_bounds__(kTableThreads)
 subtract_table_grouped_kernel(const SubtractClip* __restrict__ clips, int nc) {
-    const SubtractClip c = clips[blockIdx.y];
+    const SubtractClip c = clips[blockIdx.x];
     build_table(c.cols, c.ncols, nc, c.beta, c.lambda, c.r, c.n, table_views(c.table, c.n, nc),
-                blockIdx.x * (kTableThreads / 32) + (threadIdx.x >> 5));
+                blockIdx.y * (kTableThreads / 32) + (threadIdx.x >> 5));
 }
 
 // One pixel tile for every frame.  REAL: accumulate real terms only (the
@@ -752,7 +753,7 @@ cdmd_status make_subtract_tmap(CUtensorMap* map, const uint8_t* D, int64_t m, in
 
 cdmd_status launch_subtract_grouped(const SubtractClip* clips, int nclips, const SubtractItem* items, int nitems,
                                     int nc, int max_n, cdmd_bgmode mode, float tau, int* status, cudaStream_t stream) {
-    subtract_table_grouped_kernel<<<dim3(table_blocks(max_n), static_cast<unsigned>(nclips)), kTableThreads, 0, stream>>>(
+    subtract_table_grouped_kernel<<<dim3(static_cast<unsigned>(nclips), table_blocks(max_n)), kTableThreads, 0, stream>>>(
         clips, nc);
     CDMD_CHECK_LAUNCH("subtract_table_grouped_kernel");
     if (nitems == 0) return CDMD_OK;
