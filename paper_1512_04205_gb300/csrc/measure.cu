@@ -536,6 +536,66 @@ cdmd_status launch_measure_build(cdmd_ctx* ctx, cdmd_measure* meas, cudaStream_t
     return CDMD_OK;
 }
 
+namespace {
+
+// The packed pass's shape for a call, and whether it is the faster one.
+struct GatherPlan {
+    int frames, fps, slabs, warps;   // accumulator frames, frames of a slab, slabs, warps per CTA
+    int64_t splits, pps;             // CTAs per slab, pixels of each
+    size_t smem;
+    bool packed;
+};
+
+// One CTA an SM (the accumulators and the warps' tiles fill its shared memory), each
+// with at least one round of pixels: with two rounds asked for, clips below some
+// 150,000 pixels left half of the SMs idle (153168x61, k = 960, density 7.5e-4: 58 us,
+// 49 so, 50 for the plain kernel).
+//
+// The packed kernel pays for its accumulators (two passes over k x frames words) and
+// handles 32 (16) frames per entry whatever the slab holds; the plain one pays per
+// entry and frame, for the busiest lane of a warp, and skips the pixels without an
+// entry.  So the packed one is taken
+//   - within its sums' range: a round is expected to bring a row no more than a
+//     quarter of the entries its 16-bit sums hold (density up to 0.0104 with 24 warps);
+//   - when a CTA's pixels x frames outweigh its accumulators: `fill` = pixels / k x
+//     slab frames / 32 at least 2 (111370x3, k = 3156, 1.3e-3, fill 0.1: 48 us plain, 67
+//     packed), or 0.15 and pixels 1.5 k where the grid fills the device and the plain
+//     one, with twice the CTAs, takes two turns (921600x8, k = 3400, 1e-4, fill 0.4:
+//     83 us, 64); with 18 .. 23 warps (k of 1750 to 2048) always 2;
+//   - while C has neither too few entries per pixel (below 0.005 the plain one reads
+//     next to nothing: 17633x301, k = 33, 1.5e-4: 21 us, 26) nor too many (the plain
+//     one's lanes are then all busy: 2073600x300, k = 2100, 9e-3, 19 per pixel: 6.0 ms,
+//     8.7), the more the fewer warps and frames the packed one runs with.
+// Both were timed over 2,304 calls (4,800 .. 2,073,600 pixels, 2 .. 300 frames, k = 20
+// .. 3,400, densities 1e-4 .. 9e-3) and 520 random ones, from which the figures above
+// are.  With this rule 31 of the 2,304 are more than 5 % slower than on the plain kernel
+// alone (20 % at most); 1,009, up to 3.2 times as slow, when it asked for no more
+// than the sums' range and two rounds a CTA.
+GatherPlan gather_plan(int64_t m, int n, int k, double density, int sms) {
+    GatherPlan g;
+    g.frames = k <= 2048 ? 32 : 16;
+    const size_t tile = static_cast<size_t>(pack_tile_words(g.frames)) * sizeof(uint32_t);
+    const size_t fixed = static_cast<size_t>(k) * (2 * g.frames) + static_cast<size_t>((k + 3) / 4 * 4) * 4;
+    g.warps = static_cast<int>(std::min<size_t>(24, (kPackSmemMax - 256 - fixed) / tile));
+    g.slabs = (n + g.frames - 1) / g.frames;
+    g.fps = std::min(g.frames, ((n + g.slabs - 1) / g.slabs + 3) / 4 * 4);
+    g.smem = fixed + g.warps * tile;
+    g.splits = std::max<int64_t>(1, static_cast<int64_t>(sms) / g.slabs);
+    g.splits = std::min<int64_t>(g.splits, std::max<int64_t>(1, m / (g.warps * kPackPix)));
+    g.pps = ((m + g.splits - 1) / g.splits + 3) / 4 * 4;     // splits start on a 4-byte boundary
+    g.splits = (m + g.pps - 1) / g.pps;
+    const double slab = static_cast<double>(n) / g.slabs, per_pixel = density * k;
+    const double fill = static_cast<double>(g.pps) / k * slab / 32.0;
+    const bool full = g.slabs * g.splits >= 0.9 * sms;
+    const bool slim = g.warps < 24 || g.frames < 32;         // k past 1750
+    const bool turns = full && g.warps == 24 && 2 * g.pps >= 3 * static_cast<int64_t>(k);
+    g.packed = density * g.warps * kPackPix <= 0.25 * kPackLimit && fill >= (turns ? 0.15 : 2.0) &&
+               per_pixel >= 0.005 && per_pixel <= (slim ? 3.5 : slab >= 24.0 ? 14.0 : 6.0);
+    return g;
+}
+
+}  // namespace
+
 cdmd_status launch_sketch_gather(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, int64_t ldd,
                                  const cdmd_measure* meas, double* DY, cudaStream_t stream) {
     const int k = meas->k;
@@ -546,38 +606,21 @@ cdmd_status launch_sketch_gather(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int
         CDMD_CHECK_LAUNCH("rowsample_sketch_kernel");
         return CDMD_OK;
     }
-    // The packed kernel wherever a 4-byte load cannot be misaligned and a round of
-    // it (every warp's 128 pixels) is expected to bring a row no more than a
-    // quarter of the entries its 16-bit sums hold (density up to 0.0104 with 24
-    // warps; at 0.01, 1280x720x64, 340 us against the plain kernel's 367); denser
-    // C takes the plain one.
-    const int frames = k <= 2048 ? 32 : 16;
-    const size_t tile = static_cast<size_t>(pack_tile_words(frames)) * sizeof(uint32_t);
-    const size_t fixed = static_cast<size_t>(k) * (2 * frames) + static_cast<size_t>((k + 3) / 4 * 4) * 4;
-    const int warps = static_cast<int>(std::min<size_t>(24, (kPackSmemMax - 256 - fixed) / tile));
-    if (reinterpret_cast<uintptr_t>(D) % 4 == 0 && ldd % 4 == 0 &&
-        meas->density * warps * kPackPix <= 0.25 * kPackLimit) {
-        const int slabs = (n + frames - 1) / frames;
-        const int fps = std::min(frames, ((n + slabs - 1) / slabs + 3) / 4 * 4);
-        const size_t smem = fixed + warps * tile;
-        const int per_sm = 2 * (smem + 1024) <= kPackSmemMax ? 2 : 1;
-        int64_t splits = std::max<int64_t>(1, static_cast<int64_t>(per_sm) * ctx->num_sms / slabs);
-        splits = std::min<int64_t>(splits, std::max<int64_t>(1, m / (2 * warps * kPackPix)));
-        const int64_t pps = ((m + splits - 1) / splits + 3) / 4 * 4;     // splits start on a 4-byte boundary
-        splits = (m + pps - 1) / pps;
+    const GatherPlan g = gather_plan(m, n, k, meas->density, ctx->num_sms);
+    if (reinterpret_cast<uintptr_t>(D) % 4 == 0 && ldd % 4 == 0 && g.packed) {
         int32_t* part = nullptr;
-        cdmd_status st = ensure_buffer(ctx, BUF_SKETCH_PARTIAL, static_cast<size_t>(splits) * k * n * sizeof(int32_t),
+        cdmd_status st = ensure_buffer(ctx, BUF_SKETCH_PARTIAL, static_cast<size_t>(g.splits) * k * n * sizeof(int32_t),
                                        reinterpret_cast<void**>(&part));
         if (st != CDMD_OK) return st;
-        auto kern = frames == 32 ? sparse_packed_kernel<32> : sparse_packed_kernel<16>;
+        auto kern = g.frames == 32 ? sparse_packed_kernel<32> : sparse_packed_kernel<16>;
         CDMD_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(kPackSmemMax - 256)));
-        kern<<<dim3(slabs, static_cast<unsigned>(splits)), warps * 32, smem, stream>>>(
-            D, m, n, ldd, k, meas->col_ptr, meas->row_idx, pps, fps, part);
+        kern<<<dim3(g.slabs, static_cast<unsigned>(g.splits)), g.warps * 32, g.smem, stream>>>(
+            D, m, n, ldd, k, meas->col_ptr, meas->row_idx, g.pps, g.fps, part);
         CDMD_CHECK_LAUNCH("sparse_packed_kernel");
         const int64_t tot = static_cast<int64_t>(k) * n;
         sparse_reduce_kernel<<<static_cast<unsigned>((tot + 255) / 256), 256, 0, stream>>>(
-            part, static_cast<int>(splits), k, n, DY);
+            part, static_cast<int>(g.splits), k, n, DY);
         CDMD_CHECK_LAUNCH("sparse_reduce_kernel");
         return CDMD_OK;
     }
