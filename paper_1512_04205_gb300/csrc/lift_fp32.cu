@@ -121,10 +121,20 @@ cdmd_status launch_lift_fp32(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, 
                              const double* G, int r, const int32_t* cols, int ncols, float* Phi,
                              cudaStream_t stream) {
     (void)ctx;
+    // Equal tiles, unless there is little to multiply: with few frames the pass is its
+    // stores, and rows of 64 bytes are whole sectors where 40 to 56 are not (10^6
+    // pixels, 5 frames, 28 modes: 187 us; 385 in tiles of seven).  The narrower the
+    // equal tiles, the more tiles of eight would multiply in vain, so those of
+    // five (nine or ten modes) are given up for fewer frames only (17 frames, 10 modes:
+    // 83 us in fives, 87 in eights; 5 frames: 77 and 70).  Longest where whole rows are
+    // whole sectors (33 frames, 28 modes: 248 us, 367 in sevens; 17 modes: 214, 212).
+    // Small outputs are latency, for which more and narrower tiles are better.
     const int tiles = (ncols + 7) / 8;
+    int ct = (ncols + tiles - 1) / tiles;
+    if (tiles > 1 && m * ncols >= (1 << 20) && n <= (ct < 6 ? 12 : ncols % 4 ? 24 : 40)) ct = 8;
 #define CDMD_LIFT_TILE(CT) \
     case CT: return launch_tile<CT>(D, m, n, ldd, G, r, cols, ncols, Phi, stream);
-    switch ((ncols + tiles - 1) / tiles) {
+    switch (ct) {
         CDMD_LIFT_TILE(1) CDMD_LIFT_TILE(2) CDMD_LIFT_TILE(3) CDMD_LIFT_TILE(4)
         CDMD_LIFT_TILE(5) CDMD_LIFT_TILE(6) CDMD_LIFT_TILE(7)
         default: return launch_tile<8>(D, m, n, ldd, G, r, cols, ncols, Phi, stream);
