@@ -11,6 +11,10 @@
 // at its use and tiles of eight.  By the latency of a chain of loads at
 // 160x120x100: 17 us; 40 so.  CTAs of 128 threads spread small frames over
 // more SMs (480x360x100, 8 modes: 34 us; 42 with 256).
+// Frames that are not 4-byte aligned are read byte by byte, one frame ahead: the
+// bytes come from L1 after the first, and eight frames of four loads each crowd out
+// the multiply-adds' registers (480x480x200, 13 modes: 129 us; 226 eight frames
+// ahead; 148 with a frame's bytes loaded at their use).
 #include "cdmd_internal.cuh"
 
 namespace cdmd {
@@ -18,7 +22,6 @@ namespace {
 
 constexpr int kThreads = 128;
 constexpr int kPx = 4;
-constexpr int kBatch = 8;        // frames loaded together
 
 // Four pixels of a frame, as bytes of a word; those at or past m read as zero
 __device__ __forceinline__ uint32_t load_pixels(const uint8_t* src, int64_t j0, int64_t m, bool vec) {
@@ -30,7 +33,8 @@ __device__ __forceinline__ uint32_t load_pixels(const uint8_t* src, int64_t j0, 
     return w;
 }
 
-template <int CT>
+// kBatch: frames loaded together
+template <int CT, int kBatch>
 __global__ void __launch_bounds__(kThreads)
 lift_fp32_kernel(const uint8_t* __restrict__ D, int64_t m, int n, int64_t ldd,
                  const double* __restrict__ G, int r, const int32_t* __restrict__ cols, int ncols,
@@ -108,7 +112,8 @@ cdmd_status launch_tile(const uint8_t* D, int64_t m, int n, int64_t ldd, const d
                         int ncols, float* Phi, cudaStream_t stream) {
     const int64_t pix = static_cast<int64_t>(kThreads) * kPx;
     const dim3 grid(static_cast<unsigned>((m + pix - 1) / pix), static_cast<unsigned>((ncols + CT - 1) / CT));
-    auto kern = lift_fp32_kernel<CT>;
+    const bool vec = (ldd & 3) == 0 && (reinterpret_cast<uintptr_t>(D) & 3) == 0;
+    auto kern = vec ? lift_fp32_kernel<CT, 8> : lift_fp32_kernel<CT, 1>;
     // at most 511 frames of eight modes: 32 KB, no opt-in
     kern<<<grid, kThreads, static_cast<size_t>(n - 1) * CT * sizeof(float2), stream>>>(D, m, n, ldd, G, r, cols, ncols, Phi);
     CDMD_CHECK_LAUNCH("lift_fp32_kernel");

@@ -1,7 +1,7 @@
 """Tile width and frame batches of the FP32 lift: results where the rule takes tiles
 of eight (few frames, a large output) are those of the equal tiles, bit for bit
 (a sum runs over the frames in order whatever the tile), aligned or not, and
-few frames with many modes do not cost more than their stores."""
+neither few frames with many modes nor unaligned frames cost what they do not have to."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -65,3 +65,13 @@ def test_a_few_more_modes_cost_a_little_more(C, n, few, many):
         Phi = torch.empty((1000000, ncols, 2), device="cuda")
         us.append(_median_us(lambda: C.cdmd_lift(ctx, D, G, prec="fp32", Phi=Phi)))
     assert us[1] <= 1.4 * us[0] * many / few, us
+
+
+def test_unaligned_frames(C):
+    ctx = C.Context(0)
+    us = []
+    for pad in (4, 1):
+        D, G = _inputs(230401, 200, 13, pad)
+        Phi = torch.empty((230401, 13, 2), device="cuda")
+        us.append(_median_us(lambda: C.cdmd_lift(ctx, D, G, prec="fp32", Phi=Phi)))
+    assert us[1] <= 1.15 * us[0], us
