@@ -2840,7 +2840,14 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
 
 cdmd_status launch_decompose(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int k, int r, int K,
                              cdmd_selector selector, cudaStream_t stream) {
-    return decompose_impl(ctx, nclips, io, k, r, K, selector, stream);
+    cdmd_status st = decompose_impl(ctx, nclips, io, k, r, K, selector, stream);
+    if (st == CDMD_ERR_NOMEM && nclips > 1) {
+        // no room for all clips at once (nothing has been launched): one after another
+        clear_error();
+        st = CDMD_OK;
+        for (int i = 0; i < nclips && st == CDMD_OK; ++i) st = decompose_impl(ctx, 1, io + i, k, r, K, selector, stream);
+    }
+    return st;
 }
 
 cdmd_status launch_decompose_auto(cdmd_ctx* ctx, const DecomposeIO& io, int k, int r_max, int K,
