@@ -411,9 +411,17 @@ cdmd_status cdmd_run_host(cdmd_ctx* ctx, const uint8_t* D_host, int64_t m, int n
                           const cdmd_params* p, uint32_t* mask_host, void* stream);
 
 /* cdmd_run for 1..8 clips of the same pixel count and parameters (one
- * measurement matrix): the sketches go through cdmd_sketch_shared, then each
- * clip's small solves, lift and subtract run in order on `stream`, reusing
- * the context's workspace (cdmd_workspace_views then shows the last clip).
+ * measurement matrix): the sketches go through cdmd_sketch_shared, then, with
+ * a fixed rank, the small solves of all clips run side by side in shared
+ * launches, and the lift and the subtract follow clip by clip on `stream`
+ * (with an automatic rank the solves too go clip by clip).  A clip's
+ * results are those of its own run up to rounding: the FP64 sums over the
+ * sketch rows are split by the tiles of all clips of the call and by the
+ * device's SMs, so their order depends on both (with BF16X2 the packed sketch
+ * rounds in another order too).  The small solves hold every clip's workspace at once (for 512
+ * frames and k = 1000 about 40 MB a clip); where the device has no room for
+ * that they run one after another.  cdmd_workspace_views then shows the last
+ * clip.
  * D, n, ldd and mask are host arrays of nclips entries; each clip as for
  * cdmd_run.  CDMD_ERR_INVALID_ARG (naming the clip) as cdmd_run would, or for
  * nclips outside [1, 8]. */

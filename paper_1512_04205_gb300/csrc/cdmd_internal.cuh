@@ -246,7 +246,7 @@ enum BufferId {
     BUF_RUN_VIDEO,            // cdmd_run_host device copy of the video
     BUF_RUN_MASK,
     BUF_SUBTRACT_TABLE,       // lambda^t table and amplitudes for pass (c)
-    BUF_SELECTOR,             // selector model blob, pick order, accept flag, fallback count
+    BUF_SELECTOR,             // selector model blob, pick order of each clip, fallback count
     BUF_MLP_PARTS,            // selector training: per-warp partial gradients
     BUF_RELABEL,              // selector training: OMP against a second target
     BUF_RUN_GRAM,             // cdmd_run_exact: the n x n snapshot Gram (double)

@@ -75,7 +75,6 @@ struct SolveClip {
     const double* DY;    // k x n sketch; NULL when R is given
     const double* R;     // n x n Gram
     int n, p;            // frames, p = n - 1
-    int kchunk, splits;  // sketch rows per Gram CTA, and how many such chunks (0 when R is given)
     double *gpart, *Rw;  // Gram partials; the Gram's own storage (NULL when R is given)
     double *Hv, *htau, *Tw, *dd, *ee;             // reflectors, their block factors, the tridiagonal form
     double *lamT, *Z, *V, *B, *At, *Nm, *dv, *W, *M, *WR, *lamR, *cvec;
@@ -161,22 +160,28 @@ constexpr int kGT = 32;
 
 // Rows of the sketch per CTA: the FP64 rate bounds the pass, so the multiple of 32
 // that leaves the least work to the busiest SM (and of two equal ones the larger,
-// for fewer partials to add up).  The choice decides the order of the sums, so it
-// looks at this clip's n and k alone, and at a fixed number of SMs: a clip's Gram
-// has the same bits whichever clips share the launch, and on every device.
-// Some 16 CTAs an SM are enough, so a long sketch takes longer chunks; within one
-// the sums start anew every 256 rows, which keeps their rounding.
+// for fewer partials to add up), counted over the tiles of all clips of the call and
+// the device's SMs (n = 200, k = 1000: 64 rows alone, 256 beside four others).  The
+// order of a clip's sums, and with it the last bits of its Gram, follows that
+// choice; everything after the Gram looks at the clip alone.
+// Some 16 CTAs an SM are enough for the longest clip, so a long sketch takes longer
+// chunks; within one the sums start anew every 256 rows, which keeps their rounding.
 constexpr int kGramSms = 152;
 constexpr int kGramRows = 256;
 constexpr int64_t gram_tiles(int n) { return static_cast<int64_t>((n + kGT - 1) / kGT) * ((n + kGT - 1) / kGT + 1) / 2; }
 constexpr int64_t gram_max_splits(int n) { return (16 * kGramSms + gram_tiles(n) - 1) / gram_tiles(n); }
-int gram_chunk(int n, int k) {
-    const int64_t tiles = gram_tiles(n), most = gram_max_splits(n);
-    int64_t best = INT64_MAX;
+int gram_chunk(const DecomposeIO* io, int nclips, int k, int sms) {
+    int64_t tiles = 0, best = INT64_MAX;
+    int nmax = 0;
+    for (int i = 0; i < nclips; ++i) {
+        tiles += gram_tiles(io[i].n);
+        nmax = std::max(nmax, io[i].n);
+    }
+    const int64_t most = gram_max_splits(nmax);
     int kchunk = static_cast<int>(std::max<int64_t>(kGramRows, ((k + most - 1) / most + 31) / 32 * 32));
     for (int kc = kchunk; kc >= 64 && (k + kc - 1) / kc <= most; kc -= 32) {
         const int64_t ctas = tiles * ((k + kc - 1) / kc);
-        const int64_t load = (ctas + kGramSms - 1) / kGramSms * (std::min(kc, k) + 8);
+        const int64_t load = (ctas + sms - 1) / sms * (std::min(kc, k) + 8);
         if (load < best) { best = load; kchunk = kc; }
     }
     return kchunk;
@@ -203,10 +208,8 @@ int64_t gram_room(int n, int k) {
 // the short form a quarter of its warps (n = 200, k = 20000: 2% of the whole call).
 template <bool kLong>
 __global__ void __launch_bounds__(256)
-gram_partial_kernel(const __grid_constant__ SolveBatch sb) {
+gram_partial_kernel(const __grid_constant__ SolveBatch sb, int kchunk) {
     const SolveClip& q = sb.c[blockIdx.y];
-    if (static_cast<int>(blockIdx.z) >= q.splits) return;
-    const int kchunk = q.kchunk;
     const double* DY = q.DY;
     const int k = sb.k, n = q.n;
     // blockIdx.x counts the tile pairs ta <= tb row by row
@@ -257,9 +260,8 @@ gram_partial_kernel(const __grid_constant__ SolveBatch sb) {
     }
 }
 
-__global__ void gram_reduce_kernel(const __grid_constant__ SolveBatch sb) {
+__global__ void gram_reduce_kernel(const __grid_constant__ SolveBatch sb, int splits) {
     const SolveClip& q = sb.c[blockIdx.y];
-    const int splits = q.splits;
     const double* part = q.gpart;
     const int n = q.n;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2605,13 +2607,11 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
     // ---- workspace layout (doubles), one region per clip ----
     size_t off[kMaxSolveClips + 1] = {0};
     SolveBatch sb = {};
-    int nmax = 0, splits = 0;
+    const int kchunk = io[0].R != nullptr ? 0 : gram_chunk(io, nclips, k, ctx->device_sms);
+    const int splits = io[0].R != nullptr ? 0 : (k + kchunk - 1) / kchunk;
+    int nmax = 0;
     for (int i = 0; i < nclips; ++i) {
         const size_t n = io[i].n, p = n - 1, rr = r;
-        SolveClip& q = sb.c[i];
-        q.kchunk = io[i].R != nullptr ? 0 : gram_chunk(io[i].n, k);
-        q.splits = io[i].R != nullptr ? 0 : (k + q.kchunk - 1) / q.kchunk;
-        splits = std::max(splits, q.splits);
         const size_t room = io[i].R != nullptr ? 0 : gram_room(io[i].n, k);
         const size_t total = room + n * n + p * p + 32 * p + 1024 + 3 * p + rr +
                              3 * p * rr + 12 * rr * rr + 8 * rr + 64;
@@ -2683,12 +2683,10 @@ cdmd_status decompose_impl(cdmd_ctx* ctx, int nclips, const DecomposeIO* io, int
     // 1. Gram
     if (splits > 0) {
         const int ntiles = (nmax + kGT - 1) / kGT;
-        bool longer = false;
-        for (int i = 0; i < nclips; ++i) longer = longer || sb.c[i].kchunk > kGramRows;
-        auto gram = longer ? gram_partial_kernel<true> : gram_partial_kernel<false>;
-        gram<<<dim3(ntiles * (ntiles + 1) / 2, nc, splits), 256, 0, stream>>>(sb);
+        auto gram = kchunk > kGramRows ? gram_partial_kernel<true> : gram_partial_kernel<false>;
+        gram<<<dim3(ntiles * (ntiles + 1) / 2, nc, splits), 256, 0, stream>>>(sb, kchunk);
         CDMD_CHECK_LAUNCH("gram_partial_kernel");
-        gram_reduce_kernel<<<dim3((nmax * nmax + 255) / 256, nc), 256, 0, stream>>>(sb);
+        gram_reduce_kernel<<<dim3((nmax * nmax + 255) / 256, nc), 256, 0, stream>>>(sb, splits);
         CDMD_CHECK_LAUNCH("gram_reduce_kernel");
     }
 
