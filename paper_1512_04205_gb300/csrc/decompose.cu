@@ -666,11 +666,11 @@ __device__ __forceinline__ int sturm_count(const double* d, const double* e2, in
 }
 
 constexpr double kSearchTol = 256.0 * kEps;
-// Neighbours nearer than this (of the norm) make a cluster, whose eigenvalues are
-// searched to eps.  Past it a shift off by kSearchTol / 2 = 128 eps leaves a share of
-// (128 eps / gap)^2 < 1e-4 of the neighbour in the vector after two solves, and the
-// Rayleigh quotient is off by the gap times that share squared, below 2e-4 eps.
-constexpr double kClusterGap = 16384.0 * kEps;
+// Neighbours nearer than this (of a norm between 1/2 and 1) make a cluster, whose
+// eigenvalues are searched to eps.  Past it a shift off by kSearchTol / 2 = 128 eps
+// leaves a share of (128 eps / gap)^2 < 4e-4 of the neighbour in the vector after two
+// solves, and the Rayleigh quotient is off by the gap times that share squared.
+constexpr double kClusterGap = 7168.0 * kEps;
 constexpr int kEigThreads = 128;   // one warp per scheduler; one shift per thread
 
 // The first of the block's kEigThreads flags that is set (kEigThreads if
@@ -698,9 +698,11 @@ __device__ __forceinline__ int first_set(bool flag, unsigned* ball, int turn) {
 // solves leave the square of shift error / gap of other vectors).  The Rayleigh
 // quotient of its vector then gives the eigenvalue to rounding level, which
 // errs with z's share of the norm where a Sturm count errs with the norm itself.
-// With a neighbour within kClusterGap (counted by the same FP64 pass) neither
-// holds: the search goes on to eps, and the quotient moves the eigenvalue by no
-// more than the count's own error.
+// With a neighbour within kClusterGap neither holds: the last pass on pairs of
+// floats counts the eigenvalues one of its shifts (as far apart or further) to either
+// side (with one more count where the eigenvalue is at the edge and the pass before
+// does not tell), and where there is another the search goes on to eps, and the
+// quotient moves the eigenvalue by no more than the count's own error.
 // sigma and G at n = 300, r = 30, against LAPACK in FP64: off by 3.7e-16 and
 // 4.5e-13; 8.9e-15 and 4.9e-12 with the search carried on to eps.
 // Inverse iteration: LU with partial pivoting and two solves by one thread,
@@ -731,6 +733,7 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
     __shared__ double red[12];
     __shared__ unsigned ball[8];
     __shared__ int flags[4];
+    __shared__ int counts[2][kEigThreads];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     double lo = 1e300, hi = -1e300, tn = 0.0;
     for (int i = tid; i < p; i += kEigThreads) {
@@ -767,7 +770,7 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
     // FP32 bracket (skipped when the scale factor would leave the range)
     const int ex = (__double2hiint(tn) >> 20) & 0x7ff;
     bool bracket = ex > 64 && ex < 1983;
-    bool cluster = true;         // unless the FP64 pass counts no neighbour
+    bool near = true, cluster = true;     // another eigenvalue within kClusterGap; unless none is counted
     if (bracket) {
         const double sc = __hiloint2double((2046 - ex - 1) << 20, 0);     // tn sc in [1/2, 1)
         const double isc = __hiloint2double((ex + 1) << 20, 0);
@@ -791,33 +794,50 @@ __device__ void eigpair_cta(const SolveClip& q, int w, int* status, double* tsm)
         const double margin = 16.0 * 1.1920929e-07, margin2 = 2.3e-13;
         lo = static_cast<double>(flo) - margin;
         hi = static_cast<double>(fhi) + margin;
+        bool seen = false;
+        int f1 = 0;                          // of the pass before
         for (int it = 0; it < 3; ++it) {
             const double step = (hi - lo) * (1.0 / (kEigThreads + 1));
             const double x = fma(step, static_cast<double>(tid + 1), lo);
             const float xh = static_cast<float>(x), xl = static_cast<float>(x - static_cast<double>(xh));
-            const bool above = sturm_count_2f(d2f, e2f, p, xh, xl) > idx;
-            const int f = first_set(above, ball, turn++);
+            const int count = sturm_count_2f(d2f, e2f, p, xh, xl);
+            counts[it & 1][tid] = count;
+            const int f = first_set(count > idx, ball, turn++);
+            // the eigenvalue lies between shifts f - 1 and f: is it the only one between
+            // f - 2 and f + 1?  The ends of this pass are shifts f1 - 1 and f1 of the one
+            // before; one step outside them its next ones, far out, may tell as well
+            if (it == 2 && step >= kClusterGap) {
+                const int below = f >= 2 ? counts[0][f - 2] : f1 - 2 + f >= 0 ? counts[1][f1 - 2 + f] : -1;
+                const int g = f + 1 - kEigThreads;
+                const int above = g < 0 ? counts[0][f + 1] : f1 + g < kEigThreads ? counts[1][f1 + g] : -1;
+                near = above - below > 1;
+                seen = below >= 0 && above >= 0 && !(near && (f == 0 || f == kEigThreads));
+            }
+            f1 = f;
             const double nlo = (f == 0) ? lo : fma(step, static_cast<double>(f), lo);
             hi = (f == kEigThreads) ? hi : fma(step, static_cast<double>(f + 1), lo);
             lo = nlo;
         }
+        if (!seen) {                         // the same for every thread
+            const double x = tid == 0 ? lo - kClusterGap : hi + kClusterGap;
+            const float xh = static_cast<float>(x), xl = static_cast<float>(x - static_cast<double>(xh));
+            const int count = sturm_count_2f(d2f, e2f, p, xh, xl);
+            __syncthreads();                 // the counts have been read
+            counts[1][tid] = count;
+            __syncthreads();
+            near = counts[1][1] - counts[1][0] > 1;
+        }
         lo = (lo - margin2) * isc;
         hi = (hi + margin2) * isc;
-        // threads 1 .. 126: the ends of the bracket and 124 shifts between them;
-        // 0 and 127: kClusterGap outside, to count the neighbours
-        const double step = (hi - lo) * (1.0 / (kEigThreads - 3));
-        const double x = tid == 0                 ? lo - kClusterGap * tn
-                         : tid == kEigThreads - 1 ? hi + kClusterGap * tn
-                                                  : fma(step, static_cast<double>(tid - 1), lo);
-        const int count = sturm_count(d, e2, p, x);
-        if (tid == 0) flags[2] = count;
-        if (tid == kEigThreads - 1) flags[3] = count;
-        const int f = first_set(count > idx, ball, turn++);
-        bracket = f > 1 && f < kEigThreads - 1;
+        // the ends of the bracket and 126 shifts between them
+        const double step = (hi - lo) * (1.0 / (kEigThreads - 1));
+        const bool above = sturm_count(d, e2, p, fma(step, static_cast<double>(tid), lo)) > idx;
+        const int f = first_set(above, ball, turn++);
+        bracket = f > 0 && f < kEigThreads;
         if (bracket) {
-            hi = fma(step, static_cast<double>(f - 1), lo);
-            lo = fma(step, static_cast<double>(f - 2), lo);
-            cluster = flags[3] - flags[2] > 1;
+            hi = fma(step, static_cast<double>(f), lo);
+            lo = fma(step, static_cast<double>(f - 1), lo);
+            cluster = near;
         }
     }
     if (!bracket) {
