@@ -132,7 +132,9 @@ def compare_with_golden(gold, form, lam, sel, bg_at, F):
 
 
 def launches_per_step(selector, K, clips=1, n=200):
-    """Kernels one pipeline step over `clips` clips of n frames launches:
+    """Kernels of one pipeline step over `clips` clips of n frames when every
+    clip's small solves were launches of their own (the count the library is
+    compared with; kernels_per_step counts what it launches now):
     sketch 2 for one clip (tiles + fixed-order reduce), or for several clips
     under one C a widen pass per clip and 2 per packed launch of up to 512
     frames; per clip: decompose 15 (Gram 2, tridiagonalisation 1, eigenpairs 1,
