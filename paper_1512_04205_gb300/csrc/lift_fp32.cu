@@ -13,8 +13,8 @@
 // more SMs (480x360x100, 8 modes: 34 us; 42 with 256).
 // Frames that are not 4-byte aligned are read byte by byte, one frame ahead: the
 // bytes come from L1 after the first, and eight frames of four loads each crowd out
-// the multiply-adds' registers (480x480x200, 13 modes: 129 us; 226 eight frames
-// ahead; 148 with a frame's bytes loaded at their use).
+// the multiply-adds' registers (230401 pixels, 200 frames, 13 modes: 136 us; 226 eight
+// frames ahead; 148 with a frame's bytes loaded at their use).
 #include "cdmd_internal.cuh"
 
 namespace cdmd {
@@ -131,7 +131,7 @@ cdmd_status launch_lift_fp32(cdmd_ctx* ctx, const uint8_t* D, int64_t m, int n, 
     // pixels, 5 frames, 28 modes: 187 us; 385 in tiles of seven).  The narrower the
     // equal tiles, the more tiles of eight would multiply in vain, so those of
     // five (nine or ten modes) are given up for fewer frames only (17 frames, 10 modes:
-    // 83 us in fives, 87 in eights; 5 frames: 77 and 70).  Longest where whole rows are
+    // 89 us in fives, 93 in eights; 5 frames: 92 and 85).  Longest where whole rows are
     // whole sectors (33 frames, 28 modes: 248 us, 367 in sevens; 17 modes: 214, 212).
     // Small outputs are latency, for which more and narrower tiles are better.
     const int tiles = (ncols + 7) / 8;

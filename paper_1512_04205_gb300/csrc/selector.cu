@@ -195,13 +195,13 @@ selector_features_kernel(const double* __restrict__ lam, const double* __restric
     }
 }
 
-// Scores every mode (BF16 inference) and writes the pick order: order[q] is
-// the mode of rank q (descending logit, equal logits by index) for q < K,
-// -1 after.
 struct MlpSelectBatch {
     MlpSelectIO c[kMaxSolveClips];
 };
 
+// Scores every mode of clip blockIdx.x (BF16 inference) and writes its pick
+// order: order[q] is the mode of rank q (descending logit, equal logits by index)
+// for q < K, -1 after.
 __global__ void __launch_bounds__(32)
 mlp_select_kernel(const float* __restrict__ blob, const __grid_constant__ MlpSelectBatch mb, int r, int K) {
     const MlpSelectIO& q = mb.c[blockIdx.x];

@@ -243,7 +243,7 @@ __device__ __forceinline__ void draw_c_tiles(uint8_t* a_stage, int gt, int mtile
 // U.nclips clips, written to U.part[g][t * k + row] (this split's partial
 // sums).  Used by the per-clip and the grouped launch.
 // U.tmap[g] maps the uint8 frames; the bytes are staged and converted to BF16
-// by warps 2-11.
+// by warps 2-3 (two row tiles) or 2-11.
 __device__ __forceinline__ void sketch_tc_body(const SketchItem& U, int* status, uint8_t* smem) {
     const int nclips = U.nclips, mtiles = U.mtiles, k = U.k;
     const int n0 = U.n[0], n1 = nclips > 1 ? U.n[1] : 0;
@@ -355,7 +355,7 @@ __device__ __forceinline__ void sketch_tc_body(const SketchItem& U, int* status,
             tc::mma_commit(accum_done);   // fires once every MMA issued above has finished
         }
     } else {
-        // ---------------- workers: C generators (warps 4-11) and converters (warps 2-11) ----------------
+        // ------- workers: C generators (warps 4-11) and converters (warps 2-3 with two row tiles, else 2-11) -------
         const int wt = tid - 64;
         const bool gen = warp >= 4;
         const int gt = tid - 128;
