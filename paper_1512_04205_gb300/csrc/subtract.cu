@@ -516,6 +516,8 @@ __device__ __forceinline__ void tma_consume(const uint8_t* stages, uint64_t* ful
                 const int64_t wi = tile * (kTmaTile / 32) + warp * kTmaPxl + (lane & 1);
                 if (t < n && wi < words_per_frame) mask[static_cast<int64_t>(t) * words_per_frame + wi] = keep;
             }
+            // the next tensor copies into the stage write through the async proxy
+            tc::fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&empty[s]);
         }

@@ -501,8 +501,13 @@ __device__ __forceinline__ void subtract_tc_body(const CUtensorMap* tmap, const 
             for (int64_t u = g; u < my_units; u += 2) {
                 const int64_t i2 = upt == 2 ? (u >> 1) : u;       // the 128-pixel tile
                 const int sub = upt == 2 ? g : 0;
-                if (!tc::mbar_wait(&x_full[s], px, abort_flag, status)) break;
+                // the accumulators first: this group sees every phase of its own
+                // accumulators, but with an odd S only every other one of a
+                // stage, whose parity alone could be that of the phase before;
+                // once the accumulators are there (the builders waited for the
+                // tile) it is this tile's, and the second wait orders its bytes
                 if (!tc::mbar_wait(&acc_full[sa], pa, abort_flag, status)) break;
+                if (!tc::mbar_wait(&x_full[s], px, abort_flag, status)) break;
                 tc::tc_fence_after();
                 const uint8_t* row = X + s * L.x_stage + t * kTile;
                 const uint32_t sw = static_cast<uint32_t>(t) & 7u;
@@ -526,14 +531,25 @@ __device__ __forceinline__ void subtract_tc_body(const CUtensorMap* tmap, const 
                     }
                     if (V == 2) tmem_wait_ld32(re, im);
                     else tmem_wait_ld32(re);
+                    if (c == kWords - 1) {
+                        // this warp is done with the accumulators and the bytes.
+                        // The next tensor copy into the stage writes through the
+                        // async proxy: the fence keeps it behind the reads above,
+                        // which an arrival alone does not (a row's last 16 bytes
+                        // could be another tile's where something stalled the loads
+                        // in flight, such as the host mapping memory).  1080p, 200
+                        // frames: 208 us; 211 with the arrivals after the last
+                        // word's decisions, 206 without the fence and this order
+                        // of the waits
+                        tc::fence_proxy_async_smem();
+                        tc::tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) {
+                            tc::mbar_arrive(&acc_free[sa]);
+                            tc::mbar_arrive(&x_free[s]);
+                        }
+                    }
                     word[c] = decide32<V>(x0, x1, re, V == 2 ? im : re, tau);
-                }
-                // this warp is done with the accumulators and the bytes
-                tc::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) {
-                    tc::mbar_arrive(&acc_free[sa]);
-                    tc::mbar_arrive(&x_free[s]);
                 }
                 if ((sa += 2) >= nacc) {
                     sa -= nacc;
