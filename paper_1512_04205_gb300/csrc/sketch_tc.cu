@@ -12,7 +12,7 @@
 // CTA draws is applied to as many frames as fit there.
 //   per clip   two 128-row tiles of C against one clip's frames (n <= 256 per
 //              launch).  Warp 0 TMA-loads the uint8 bytes (64 pixels x n
-//              frames per K step) into a staging buffer and warps 2-11
+//              frames per K step) into a staging buffer and warps 2-3
 //              convert them to BF16 B tiles in the 128-byte swizzled layout.
 //   packed     one 128-row tile of C against up to 512 frames of several
 //              clips under the same C (same pixel count, k and seed: windows
